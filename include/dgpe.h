@@ -289,9 +289,8 @@ typedef struct dgpe_tuning {
   int plan_style[3];     /* FFT radix order per axis: 0 radix-8 first, 1 radix-4, 2 radix-3 first */
   int ylines;            /* lines per CTA of the y transforms: 2, 4, 8, 16 or 32 */
   int fft_threads;       /* threads per CTA of the y/x transforms: 128 or 256 */
-  int cn_per_sm;         /* CTAs per SM of the persistent Crank-Nicolson sweeps: 1 or 2 (an upper
-                            bound: the FP32 sweeps of 512-thread CTAs fit one per SM by registers;
-                            those of short lines run four per SM regardless) */
+  int cn_per_sm;         /* FP32 x and y sweeps: persistent threads per SM in units of 256, 1 or 2 (at
+                            least one CTA) */
   double step_ms_default, step_ms_tuned;  /* measured by dgpe_autotune (0 otherwise) */
 } dgpe_tuning;
 

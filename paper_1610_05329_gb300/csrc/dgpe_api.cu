@@ -92,6 +92,28 @@ int cn_chunk(int n) {
   return c;
 }
 
+// Interior points per thread of the FP32 x and y sweeps (k_cn_reg): 16 (the least fix-up and
+// scan work per point), or 12 where that keeps the columns per tile: the same tile on more
+// threads with shorter chains (n = 3 2^k, 288 to 386: e.g. 256 threads instead of 192 at 96,
+// 192 and 384).  Chunks of 8 and 4 were slower from 96^3 on (16 members of 128^3: 752 and 860
+// against 705 us a step).
+int sweep_chunk(int n) {
+  const int q12 = (n - 2 + 11) / 12, q16 = (n - 2 + 15) / 16;
+  return q12 <= kWarp && cnr_cols(q12) == cnr_cols(q16) ? 12 : 16;
+}
+
+// The same for the differentiation calls: the chunks of the 32-lane (a power of two) and 8-lane
+// (n = 8 CH) solvers.  A gradient is a small difference of FP32 values, so another chunking
+// shows in its seventh digit; dgpe_grad_z2 and dgpe_adjoint_step keep these, on which their
+// stored results rest.
+int diff_chunk(int n) { return n == 32 || n == 48 || n == 64 || n == 96 || n == 128 ? n / 8 : cn_chunk(n); }
+
+// The chunk of the tables of axis d: the sweeps' own in FP32 along x and y, else cn_chunk.
+int axis_chunk(const dgpe_params *p, int d) {
+  const int n = d == 0 ? p->nx : d == 1 ? p->ny : p->nz;
+  return p->precision == DGPE_MIXED && d < 2 ? sweep_chunk(n) : cn_chunk(n);
+}
+
 int log2_int(int v) {
   int l = 0;
   while ((1 << l) < v) ++l;
@@ -124,7 +146,7 @@ int check_physics(const dgpe_params *p) {
 }
 
 struct Layout {
-  size_t state, partials, tw[3], cn[3], cn_adj[3], cnz, cn8[3], cn8_adj[2], dtv[3], psi, spec, utab, ybuf, total;
+  size_t state, partials, tw[3], cn[3], cn_diff[2], cn_adj[3], cnz, cn8z, dtv[3], psi, spec, utab, ybuf, total;
 };
 
 // FP32 contexts whose compile-time K5 (nz = 128, 256, 384, 512) solves along z at a chunk
@@ -151,30 +173,29 @@ Layout layout_of(const dgpe_params *p, const KernelSet *ks, int max_blocks) {
   for (int d = 0; d < 3; ++d) {
     L.cn[d] = off;
     // lane-interleaved tables, scan factors, then the twist pivot of the two-thread sweeps
-    off += align_up((size_t)(4 * cn_chunk(n[d]) + 11) * kWarp * e);
-    L.cn_adj[d] = off;   // the same for dt -> -dt (adjoint)
-    off += align_up((size_t)(4 * cn_chunk(n[d]) + 11) * kWarp * e);
+    off += align_up((size_t)(4 * axis_chunk(p, d) + 11) * kWarp * e);
+    // the same at the chunk of the differentiation calls, and for dt -> -dt (adjoint)
+    const int dc = p->precision == DGPE_MIXED && d < 2 ? diff_chunk(n[d]) : axis_chunk(p, d);
+    if (d < 2) {
+      L.cn_diff[d] = L.cn[d];
+      if (dc != axis_chunk(p, d)) {
+        L.cn_diff[d] = off;
+        off += align_up((size_t)(4 * dc + 11) * kWarp * e);
+      }
+    }
+    L.cn_adj[d] = off;
+    off += align_up((size_t)(4 * dc + 11) * kWarp * e);
   }
   L.cnz = 0;   // K5's z tables at their own chunk (FP32 where the compile-time K5 needs them)
   if (needs_cnz(p)) {
     L.cnz = off;
     off += align_up((size_t)(4 * k5_chunk(p->nz) + 11) * kWarp * e);
   }
-  // tables in the 8-lane layout: the x and y sweeps' (FP32 short lines), K5's z solve (FP32,
-  // the compile-time K5 of nz = 64, 96, 128)
-  for (int d = 0; d < 3; ++d) {
-    L.cn8[d] = 0;
-    if (p->precision == DGPE_MIXED && (d < 2 ? short_cn_chunk(n[d]) != 0 : k5_short_z(n[d]))) {
-      L.cn8[d] = off;
-      off += align_up((size_t)(4 * 8 * short_cn_chunk(n[d]) + 49) * e);
-    }
-  }
-  for (int d = 0; d < 2; ++d) {   // the same for dt -> -dt (the adjoint x and y sweeps)
-    L.cn8_adj[d] = 0;
-    if (L.cn8[d]) {
-      L.cn8_adj[d] = off;
-      off += align_up((size_t)(4 * 8 * short_cn_chunk(n[d]) + 49) * e);
-    }
+  // K5's z tables in the 8-lane layout (FP32, the compile-time K5 of nz = 64, 96, 128)
+  L.cn8z = 0;
+  if (p->precision == DGPE_MIXED && k5_short_z(p->nz)) {
+    L.cn8z = off;
+    off += align_up((size_t)(4 * p->nz + 49) * e);
   }
   for (int d = 0; d < 3; ++d) {
     L.dtv[d] = off;
@@ -213,7 +234,7 @@ KArgs base_args(const dgpe_params *p) {
     const int n = d == 0 ? p->nx : d == 1 ? p->ny : p->nz;
     a.plan[d] = make_plan(n, 0);
     a.cn[d].m = n - 2;
-    a.cn[d].chunk = cn_chunk(n);
+    a.cn[d].chunk = axis_chunk(p, d);
     a.cn[d].lchunk = log2_int(a.cn[d].chunk);
   }
   return a;
@@ -392,8 +413,22 @@ int enqueue_potential_transforms(dgpe_ctx *c, cudaStream_t st) {
   return DGPE_OK;
 }
 
+int diff_axis_chunk(const dgpe_ctx *c, int d);
+
+// The step's arguments; within dgpe_grad_z2 (FP32-mixed without norm restoration) the sweeps'
+// tables are those of the differentiation calls.
+KArgs step_args(dgpe_ctx *c) {
+  KArgs a = c->args;
+  if (c->p.precision == DGPE_MIXED && !c->restore_norm)
+    for (int d = 0; d < 2; ++d) {
+      a.cn[d].tab = at(c, c->L.cn_diff[d]);
+      a.cn[d].chunk = diff_axis_chunk(c, d);
+    }
+  return a;
+}
+
 int enqueue_step(dgpe_ctx *c, cudaStream_t st) {
-  const KArgs &a = c->args;
+  const KArgs a = step_args(c);
   const KernelSet *ks = c->ks;
   int rc;
   if ((rc = enqueue_potential_transforms(c, st))) return rc;
@@ -450,6 +485,11 @@ int build_graph(dgpe_ctx *c) {
   return DGPE_OK;
 }
 
+// Chunk of the differentiation calls' tables of axis d.
+int diff_axis_chunk(const dgpe_ctx *c, int d) {
+  return c->p.precision == DGPE_MIXED && d < 2 ? diff_chunk(d == 0 ? c->p.nx : c->p.ny) : c->args.cn[d].chunk;
+}
+
 // Per-axis tables of the physics: dt v_d x^2 (always), the Crank-Nicolson factor tables
 // (only when dt, h or the mode changed, or on the first call) and the dipolar kernel on the
 // half spectrum (only when h or the cutoff changed, or on the first call).
@@ -465,12 +505,15 @@ int setup_tables(dgpe_ctx *c, bool cn_changed, bool ut_changed) {
     if (rc) return rc;
     if (!cn_changed) continue;
     jobs.job[jobs.n++] = {at(c, c->L.cn[d]), c->args.cn[d].m, c->args.cn[d].chunk, c->args.cn_r[d], kWarp};
-    if (p->mode == DGPE_REAL_TIME)   // the adjoint sweep is the sweep with dt -> -dt
-      jobs.job[jobs.n++] = {at(c, c->L.cn_adj[d]), c->args.cn[d].m, c->args.cn[d].chunk, -c->args.cn_r[d], kWarp};
-    if (c->L.cn8[d]) jobs.job[jobs.n++] = {at(c, c->L.cn8[d]), c->args.cn[d].m, n[d] / 8, c->args.cn_r[d], 8};
-    if (d < 2 && c->L.cn8_adj[d] && p->mode == DGPE_REAL_TIME)
-      jobs.job[jobs.n++] = {at(c, c->L.cn8_adj[d]), c->args.cn[d].m, n[d] / 8, -c->args.cn_r[d], 8};
+    if (p->mode == DGPE_REAL_TIME) {   // the adjoint sweep is the sweep with dt -> -dt
+      const int dc = diff_axis_chunk(c, d);
+      jobs.job[jobs.n++] = {at(c, c->L.cn_adj[d]), c->args.cn[d].m, dc, -c->args.cn_r[d], kWarp};
+      if (dc != c->args.cn[d].chunk)
+        jobs.job[jobs.n++] = {at(c, c->L.cn_diff[d]), c->args.cn[d].m, dc, c->args.cn_r[d], kWarp};
+    }
   }
+  if (cn_changed && c->L.cn8z)
+    jobs.job[jobs.n++] = {at(c, c->L.cn8z), c->args.cn[2].m, n[2] / 8, c->args.cn_r[2], 8};
   if (cn_changed && c->L.cnz)
     jobs.job[jobs.n++] = {at(c, c->L.cnz), c->args.cn[2].m, k5_chunk(p->nz), c->args.cn_r[2], kWarp};
   if (jobs.n) {
@@ -501,9 +544,7 @@ KArgs adjoint_sweep_args(dgpe_ctx *c, void *gbar) {
   a.psi = gbar;
   for (int d = 0; d < 3; ++d) {
     a.cn[d].tab = at(c, c->L.cn_adj[d]);
-    // the adjoint x and y sweeps of short lines on their own 8-lane tables; K5's z solve does
-    // not run in the adjoint step
-    a.cn8_tab[d] = d < 2 && c->L.cn8_adj[d] ? at(c, c->L.cn8_adj[d]) : nullptr;
+    a.cn[d].chunk = diff_axis_chunk(c, d);
     a.cn_r[d] = -a.cn_r[d];
     a.cn_rf[d] = -a.cn_rf[d];
     a.cn_rl[d] = -a.cn_rl[d];
@@ -714,7 +755,7 @@ int dgpe_create(const dgpe_params *p, void *cuda_stream, dgpe_ctx **out) {
   a.utab = at(c, c->L.utab);
   a.ybuf = at(c, c->L.ybuf);
   a.cnz_tab = c->L.cnz ? at(c, c->L.cnz) : nullptr;
-  for (int d = 0; d < 3; ++d) a.cn8_tab[d] = c->L.cn8[d] ? at(c, c->L.cn8[d]) : nullptr;
+  a.cn8z_tab = c->L.cn8z ? at(c, c->L.cn8z) : nullptr;
   const int n[3] = {p->nx, p->ny, p->nz};
   rc = map_cuda(cudaMemsetAsync(a.psi, 0, (size_t)p->nx * p->ny * p->nz * c->ks->elem_bytes, c->stream));
   if (!rc) rc = map_cuda(c->ks->reset_state(a.state, c->stream));

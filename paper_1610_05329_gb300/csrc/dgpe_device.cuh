@@ -286,8 +286,6 @@ struct Tiles<double> {
   static constexpr int kZThreads = 256;   // 8 warps: one z-line per warp in the CN-z solve
   static constexpr int kZMinBlocks = 2;   // K5: two CTAs per SM (at most 128 registers)
   static constexpr int kXCols = 4;        // consecutive y columns per K3 tile
-  static constexpr int kCnCols = 8;       // consecutive z columns per K6/K7 tile (128 B rows)
-  static constexpr int kCnThreads = 128;  // 4 warps, two lines per warp
   static constexpr int kYBudget = 1024;   // K2/K4: lines per CTA ~ budget / ny
 };
 template <>
@@ -298,8 +296,6 @@ struct Tiles<float> {
   static constexpr int kZThreads = 256;
   static constexpr int kZMinBlocks = 2;
   static constexpr int kXCols = 8;
-  static constexpr int kCnCols = 16;
-  static constexpr int kCnThreads = 512;  // 16 warps, one line per warp
   static constexpr int kYBudget = 4096;
 };
 // z-lines per K1 and K5 tile: 32 for the FP32 compile-time lengths of at most 128 points
@@ -418,13 +414,6 @@ struct SlotWalkP {
   __device__ __forceinline__ int operator()(int j, int o) const { return (o | j) == 0 ? 0 : base + j * step; }
 };
 __host__ __device__ constexpr int gcd_c(int a, int b) { return b == 0 ? a : gcd_c(b, a % b); }
-
-template <int W>
-struct SlotWalk {
-  int base, step;
-  __device__ __forceinline__ SlotWalk(int k0, int lchunk) : base(k0 + ((k0 - 1) >> lchunk)), step(W + (W >> lchunk)) {}
-  __device__ __forceinline__ int operator()(int j, int k0) const { return (k0 | j) == 0 ? 0 : base + j * step; }
-};
 
 // ---------------------------------------------------------------------------------------
 // FFT: radix-2/3/4/5/7/8 butterflies (DIR = -1 forward e^{-i..}, +1 inverse, unnormalised)
@@ -1039,18 +1028,6 @@ __device__ __forceinline__ void cn_line_any(cplx<R> *__restrict__ buf, int es, i
     default: cn_line<R, Coef, 16, SHARED_TAB, FULL>(buf, es, m, lchunk, tab, scan_s, c); break;
   }
 }
-// cn_line2 (two lines in lockstep, padded to 32 whole chunks) at the chunk 2^lchunk
-template <typename R, typename Coef>
-__device__ __forceinline__ void cn_line2_any(cplx<R> *b1, cplx<R> *b2, int es, int lchunk, const Coef *tab,
-                                             const Coef *scan_s, Coef c) {
-  switch (lchunk) {
-    case 1: cn_line2<R, Coef, 2>(b1, b2, es, tab, scan_s, c); break;
-    case 2: cn_line2<R, Coef, 4>(b1, b2, es, tab, scan_s, c); break;
-    case 3: cn_line2<R, Coef, 8>(b1, b2, es, tab, scan_s, c); break;
-    default: cn_line2<R, Coef, 16>(b1, b2, es, tab, scan_s, c); break;
-  }
-}
-
 template <typename R, typename Coef>
 struct CnCoef;
 template <typename R>
@@ -1097,54 +1074,113 @@ __device__ __forceinline__ R scale_sq_of(const DevState *st) {
 }
 
 // ---------------------------------------------------------------------------------------
-// Reductions (FP64): warp shuffle, then across warps; deterministic order.
+// Reductions, in a fixed order.  The tail of a kernel that ends with one is latency: GB300
+// issues an FP64 warp instruction in 64 cycles per SM sub-partition, so summing NV values over
+// a block by NV x 5 shuffle steps per warp, twice, took about 8 us at the end of each step (the
+// x sweep of 64^3 FP32: 16 us against 7 us for the y sweep).  Here the lanes first trade
+// values (transposing butterfly: NV/2 + NV/4 + .. + 1 + 1 .. additions per warp instead of
+// 5 NV), FP32 kernels sum within the block on the FP32 pipe (double-float pairs), and the last
+// block's threads read the partial sums with several loads in flight.
 // ---------------------------------------------------------------------------------------
-template <int NV>
-__device__ __forceinline__ void block_sum(double (&v)[NV], double (*red)[NV]) {
-  const int lane = threadIdx.x & (kWarp - 1), warp = threadIdx.x / kWarp;
-  const int nwarps = (blockDim.x + kWarp - 1) / kWarp;
+// A (hi, lo) sum that can be traded between lanes.
+__device__ __forceinline__ DFAcc merged(DFAcc a, const DFAcc &b) {
+  a.add(b.hi);
+  a.lo = __fadd_rn(a.lo, b.lo);
+  return a;
+}
+__device__ __forceinline__ double merged(double a, double b) { return a + b; }
+__device__ __forceinline__ DFAcc lane_xor(const DFAcc &v, int m) {
+  DFAcc r;
+  r.hi = shfl_xor(v.hi, m);
+  r.lo = shfl_xor(v.lo, m);
+  return r;
+}
+__device__ __forceinline__ double lane_xor(double v, int m) { return shfl_xor(v, m); }
+
+// Sums of v[0..NV) over the warp (NV = 4 or 8): lane l ends with the total of v[l / (32 / NV)].
+template <int NV, typename S>
+__device__ __forceinline__ S warp_sums(S (&v)[NV]) {
+  const int lane = threadIdx.x & (kWarp - 1);
+  int m = kWarp / 2;
 #pragma unroll
-  for (int q = 0; q < NV; ++q)
-    for (int d = kWarp / 2; d > 0; d >>= 1) v[q] += __shfl_down_sync(0xffffffffu, v[q], d);
-  __syncthreads();
-  if (lane == 0)
+  for (int h = NV / 2; h > 0; h >>= 1, m >>= 1) {   // keep half of the values, hand over the others
+    const bool upper = lane & m;
 #pragma unroll
-    for (int q = 0; q < NV; ++q) red[warp][q] = v[q];
-  __syncthreads();
-  if (warp == 0) {
-#pragma unroll
-    for (int q = 0; q < NV; ++q) {
-      v[q] = lane < nwarps ? red[lane][q] : 0.0;
-      for (int d = kWarp / 2; d > 0; d >>= 1) v[q] += __shfl_down_sync(0xffffffffu, v[q], d);
+    for (int q = 0; q < h; ++q) {
+      const S keep = upper ? v[q + h] : v[q], give = upper ? v[q] : v[q + h];
+      v[q] = merged(keep, lane_xor(give, m));
     }
   }
+#pragma unroll
+  for (int k = kWarp / (2 * NV); k > 0; k >>= 1) v[0] = merged(v[0], lane_xor(v[0], k));
+  return v[0];
 }
 
-// Store this block's partial sums; the last block to finish adds all partials in block
-// order and returns true (in every thread of that block) with the totals in thread 0.
-template <int NV>
-__device__ bool reduce_across_blocks(double (&v)[NV], double *partials, unsigned int *ticket) {
-  __shared__ double red[32][NV];
+// Totals over the block: lane l of warp 0 ends with the total of value l / (32 / NV) (the other
+// warps' results are partial).  red: 32 warps x NV entries.
+template <int NV, typename S>
+__device__ __forceinline__ S block_sums(S (&v)[NV], S *red) {
+  constexpr int G = kWarp / NV;   // lanes per value
+  const int lane = threadIdx.x & (kWarp - 1), warp = threadIdx.x / kWarp;
+  const int nwarps = (blockDim.x + kWarp - 1) / kWarp;
+  S t = warp_sums<NV>(v);
+  if (lane % G == 0) red[warp * NV + lane / G] = t;
+  __syncthreads();
+  if (warp == 0) {
+    t = S{};
+    for (int w = lane % G; w < nwarps; w += G) t = merged(t, red[w * NV + lane / G]);
+#pragma unroll
+    for (int k = G / 2; k > 0; k >>= 1) t = merged(t, lane_xor(t, k));
+  }
+  return t;
+}
+
+__device__ __forceinline__ double as_double(double v) { return v; }
+__device__ __forceinline__ double as_double(const DFAcc &v) { return v.value(); }
+
+// Store this block's partial sums; the last block to finish adds all partials
+// and returns true (in every thread of that block) with the totals in tot[0..NV) of thread 0.
+template <int NV, typename S>
+__device__ bool reduce_across_blocks(S (&v)[NV], double (&tot)[NV], double *partials, unsigned int *ticket) {
+  static_assert(NV == 4 || NV == 8, "values a warp can trade");
+  constexpr int G = kWarp / NV;
+  __shared__ S red[32 * NV];
+  __shared__ double redd[32 * NV];
   __shared__ bool last;
   const int nblocks = gridDim.x * gridDim.y;
   const int bid = blockIdx.y * gridDim.x + blockIdx.x;
-  block_sum<NV>(v, red);
-  if (threadIdx.x == 0) {
-#pragma unroll
-    for (int q = 0; q < NV; ++q) partials[(size_t)bid * NV + q] = v[q];
+  const int lane = threadIdx.x & (kWarp - 1), warp = threadIdx.x / kWarp;
+  const S t = block_sums<NV>(v, red);
+  if (warp == 0) {
+    if (lane % G == 0) partials[(size_t)bid * NV + lane / G] = as_double(t);
     __threadfence();
-    const unsigned int prev = atomicAdd(ticket, 1u);
-    last = (prev == (unsigned int)nblocks - 1);
+    __syncwarp();
+    if (lane == 0) last = atomicAdd(ticket, 1u) == (unsigned int)nblocks - 1;
   }
   __syncthreads();
   if (!last) return false;
   __threadfence();
+  // thread t: value t mod NV of the blocks t / NV + k (blockDim / NV)
+  const int q = threadIdx.x % NV, bs = blockDim.x / NV;
+  double s[4] = {0.0, 0.0, 0.0, 0.0};
+  for (int b0 = threadIdx.x / NV; b0 < nblocks; b0 += 4 * bs)
 #pragma unroll
-  for (int q = 0; q < NV; ++q) v[q] = 0.0;
-  for (int b = threadIdx.x; b < nblocks; b += blockDim.x)
+    for (int u = 0; u < 4; ++u)
+      if (b0 + u * bs < nblocks) s[u] += __ldcg(partials + (size_t)(b0 + u * bs) * NV + q);
+  double d = (s[0] + s[1]) + (s[2] + s[3]);
 #pragma unroll
-    for (int q = 0; q < NV; ++q) v[q] += __ldcg(partials + (size_t)b * NV + q);
-  block_sum<NV>(v, red);
+  for (int k = NV; k < kWarp; k <<= 1) d += shfl_xor(d, k);
+  if (lane < NV) redd[warp * NV + lane] = d;
+  __syncthreads();
+  if (warp == 0) {
+    const int nwarps = (blockDim.x + kWarp - 1) / kWarp;
+    d = 0.0;
+    for (int w = lane % G; w < nwarps; w += G) d += redd[w * NV + lane / G];
+#pragma unroll
+    for (int k = G / 2; k > 0; k >>= 1) d += shfl_xor(d, k);
+#pragma unroll
+    for (int r = 0; r < NV; ++r) tot[r] = __shfl_sync(0xffffffffu, d, r * G);
+  }
   if (threadIdx.x == 0) *ticket = 0u;
   return true;
 }
@@ -1872,7 +1908,7 @@ __device__ __forceinline__ void k5_zline_body(const KArgs &a, const KArgs *ga) {
   if (phase) dtvx = reinterpret_cast<const R *>(a.dtv[0])[i];
   // the z solve's tables: K5's own at CHZ points per lane where that is not the sweeps' chunk
   const Coef *ztab_g = reinterpret_cast<const Coef *>(
-      LZ == 8 ? a.cn8_tab[2] : (kWalk && a.cnz_tab ? a.cnz_tab : a.cn[2].tab));
+      LZ == 8 ? a.cn8z_tab : (kWalk && a.cnz_tab ? a.cnz_tab : a.cn[2].tab));
   const int zmp = kWalk ? LZ * CHZ : (kWarp << lc);
   if (zmode == kZStep || zmode == kZCnOnly) {
     const Coef *gscan = ztab_g + 4 * zmp;
@@ -2203,7 +2239,9 @@ __device__ __forceinline__ void k5_zline_body(const KArgs &a, const KArgs *ga) {
         v[7] += w * zc * zc * dens;
       }
     }
-    if (reduce_across_blocks<8>(v, a.partials, &a.state->ticket) && threadIdx.x == 0) {
+    double tot[8];
+    if (reduce_across_blocks<8>(v, tot, a.partials, &a.state->ticket) && threadIdx.x == 0) {
+      for (int q = 0; q < 8; ++q) v[q] = tot[q];
       const double dv = a.hx * a.hy * a.hz;
       DevState *st = a.state;
       const double s2 = st->s * st->s;
@@ -2369,7 +2407,7 @@ __global__ void __launch_bounds__(Tiles<R>::kZThreads,
 
 // ---------------------------------------------------------------------------------------
 // K6 / K7: Crank-Nicolson along y (AXIS = 1, lines psi[i][:][k]) or x (AXIS = 0, lines
-// psi[:][j][k]) for kCnCols consecutive k per CTA (one warp per line).  K7 (x) also sums
+// psi[:][j][k]).  K7 (x) also sums
 // n, x^2 n, y^2 n, z^2 n (FP64 totals) and, in the last block, sets the norm and the pending
 // renormalisation factor s = 1/sqrt(norm) (imaginary time) or 1 (real time).  The x^2 n
 // sum is not taken (nothing reads it: the observables take their own FP64 sums).  FP64
@@ -2405,8 +2443,14 @@ struct SumAcc<df> {
 // real-time step conserves the norm; the FP32-rounded Crank-Nicolson factor tables make
 // each sweep non-unitary by about 1e-7 (the same rounding at every point of a line, so it
 // adds up instead of averaging out), and this undoes that drift from the FP64-class sum.
-__device__ __forceinline__ void finish_sweep_sums(const KArgs &a, double (&v)[4], int renorm) {
-  if (reduce_across_blocks<4>(v, a.partials, &a.state->ticket) && threadIdx.x == 0) {
+// acc: this thread's sums (times w = 1, wy, wz for the three used: n, y^2 n, z^2 n).
+template <typename S>
+__device__ __forceinline__ void finish_sweep_sums(const KArgs &a, S (&acc)[4], double w0, double wy, double wz, int renorm) {
+  double v[4];
+  if (reduce_across_blocks<4>(acc, v, a.partials, &a.state->ticket) && threadIdx.x == 0) {
+    v[0] *= w0;
+    v[2] *= wy;
+    v[3] *= wz;
     DevState *st = a.state;
     const double norm = a.hx * a.hy * a.hz * v[0];
     for (int q = 0; q < 4; ++q) st->sums[q] = v[q];
@@ -2429,273 +2473,212 @@ __device__ __forceinline__ void finish_sweep_sums(const KArgs &a, double (&v)[4]
   }
 }
 
-// Persistent, double-buffered: each CTA walks the tiles (fixed index, k-tile)
-// blockIdx.x, blockIdx.x + gridDim.x, ...; the cp.async copies of the next tile are in
-// flight while the current tile is solved and stored.
-// B columns (z) per tile, NT threads (B divides NT; one or two lines per warp).
-template <typename R, typename Coef, int AXIS, int B = Tiles<R>::kCnCols, int NT = Tiles<R>::kCnThreads,
-          bool FULL = false>
-__device__ __forceinline__ void k_cn_body(const KArgs &a, int reduce, int renorm) {
-  static_assert(std::is_same<R, float>::value, "the chunked sweeps serve FP32 data");
-  using C = cplx<R>;
+// FP32 sweeps along y (AXIS = 1) and x (AXIS = 0), every line length: the chunked Thomas solve
+// of cn_line with the line in registers.  Thread (column b, chunk q) of a tile of B columns
+// holds the CH interior points q CH .. q CH + CH - 1 of its line: it reads them from the tile's
+// copy in shared memory, runs both recurrences and the fix-up on them in registers and stores
+// them to global memory.  The factor tables are read as broadcasts (the threads of a row of
+// columns share their chunk), and one carry per chunk and direction passes through shared
+// memory: it is scanned across the chunks by warps, lane t the chunk t of a column, log2 steps.
+// Columns are taken over the flattened index of the contiguous columns (y z-planes for x lines,
+// per x the z index for y lines), so no tile is ragged and a row of B columns is one segment
+// of 8 B bytes.  Persistent CTAs with two tile buffers: a tile is in registers as soon as it
+// has been read, so the copies of the two tiles after it are in flight while it is solved.
+// Long x lines (PAIR: more than 16 chunks; rows a whole x plane apart) take two tiles of 16
+// columns at a time, copied together as rows of 256 bytes into two of three tile buffers while
+// the tiles before them are solved one after the other, one CTA per SM: a plain copy in rows of
+// 64 or 128 bytes a plane apart reaches 0.84 of the copy bandwidth at 512 x 196608, in rows of
+// 256 bytes 0.92.
+// Bound by HBM (y) and by the latency between two loads of a pair (x).  One sweep, real time,
+// us (of 16 bytes per point at 6784 GB/s), against the solver before it (a warp per line in
+// shared memory): 512x512x384 y 358 -> 292 (0.81), x with its sums 414 -> 363 (0.65); 480x480x500
+// y 566 -> 352 (0.77), x 582 -> 404 (0.67, without its sums); 384^3 294 -> 188, 317 -> 210; 240^3
+// 81 -> 45, 97 -> 60; 128^3 12.2 -> 12.3, 24.4 -> 20.4.
+constexpr int kCnrThreads = 512;   // persistent threads per SM (up to 128 registers each)
+template <typename Coef>
+struct alignas(2 * sizeof(Coef)) CoefPair {
+  Coef h, g;
+};
+// slot of (interior point i, column b) of a tile: rows of B columns; where a row is 64 bytes,
+// one more after each chunk (half-warps then read two rows of different banks)
+template <int CH>
+__host__ __device__ constexpr int cnr_row(int i, int cols) { return (i + (cols == 8 ? i / CH : 0)) * cols; }
+// shared memory: the two tiles, alpha, beta, (H, G) with one pad entry per chunk (threads of
+// neighbouring chunks then read different banks), the scan factors, two carry buffers, the x
+// weights
+__host__ __device__ constexpr size_t smem_cnr(int n, int ch, size_t coef, bool pair) {
+  const int q = (n - 2 + ch - 1) / ch, b = pair ? 16 : cnr_cols(q);
+  return (pair ? 3 : 2) * (size_t)q * (ch + (b == 8 ? 1 : 0)) * b * 8 + (size_t)4 * q * (ch + 1) * coef + 10 * kWarp * coef +
+         2 * (size_t)q * (b + 1) * 8 + (size_t)(q * ch + 1) * 4;
+}
+
+template <typename Coef, int AXIS, int CH, bool PAIR>
+__device__ __forceinline__ void k_cn_reg_body(const KArgs &a, int reduce, int renorm) {
+  using R = float;
+  using C = cplx<float>;
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  constexpr int SB = B + 1;
-  const int N = AXIS == 0 ? a.nx : a.ny;
-  const int nfixed = AXIS == 0 ? a.ny : a.nx;
-  const int nkt = (a.nz + B - 1) / B;
-  const int ntiles = nfixed * nkt;
-  const int lc = a.cn[AXIS].lchunk;
-  // FULL: the lines padded to 32 chunks of unknowns (grid indices up to m_pad + 1)
-  const int m_pad = kWarp << lc;
-  const int slots = FULL ? cn_slots(m_pad + 2, lc) : cn_slots(N, lc);
-  C *cur = reinterpret_cast<C *>(smem_raw);
-  C *nxt = cur + slots * SB;
-  Coef *stab = reinterpret_cast<Coef *>(nxt + slots * SB);     // factor tables, staged once
-  const int ntab = 4 * (kWarp << lc) + 10 * kWarp;
-  float *wxtab = reinterpret_cast<float *>(stab + ntab);        // W_x(i) = 3 x the weight (or 1)
+  const int n = AXIS == 0 ? a.nx : a.ny, m = n - 2;
+  const int Q = (m + CH - 1) / CH;
+  constexpr int S = PAIR ? 2 : 1, NBUF = S + 1;   // tiles copied together, tile buffers
+  const int B = PAIR ? 16 : cnr_cols(Q), lb = 31 - __clz(B), SB = B + 1;
+  const int tabn = Q * (CH + 1);
+  C *tiles = reinterpret_cast<C *>(smem_raw);
+  const int tile_slots = cnr_row<CH>(Q * CH, B);
+  CoefPair<Coef> *hg = reinterpret_cast<CoefPair<Coef> *>(tiles + NBUF * tile_slots);
+  Coef *al = reinterpret_cast<Coef *>(hg + tabn), *be = al + tabn;
+  Coef *scan_s = be + tabn;
+  C *car1 = reinterpret_cast<C *>(scan_s + 10 * kWarp), *car2 = car1 + Q * SB;
+  float *wxtab = reinterpret_cast<float *>(car2 + Q * SB);   // W_x(i) = 3 x the weight (or 1)
+  const bool do_reduce = AXIS == 0 && reduce;
+  {
+    const Coef *g = reinterpret_cast<const Coef *>(a.cn[AXIS].tab);
+    constexpr int mp = kWarp * CH;
+    for (int i = threadIdx.x; i < Q * CH; i += blockDim.x) {
+      const int t = i % Q, e = i / Q, d = t * (CH + 1) + e, s = e * kWarp + t;
+      al[d] = g[s];
+      be[d] = g[mp + s];
+      hg[d] = {g[2 * mp + s], g[3 * mp + s]};
+    }
+    for (int i = threadIdx.x; i < 10 * kWarp; i += blockDim.x) scan_s[i] = g[4 * mp + i];
+  }
+  if (do_reduce)
+    for (int i = threadIdx.x; i <= Q * CH; i += blockDim.x) wxtab[i] = (float)quad_weight3(i, a.nx, a.simpson);
+  const Coef c = CnCoef<R, Coef>::make(a.cn_rf[AXIS]);
+  const int b = threadIdx.x & (B - 1), q = threadIdx.x >> lb;
+  const int len = q < Q ? min(CH, m - q * CH) : 0;
+  const int tq = min(q, Q - 1) * (CH + 1);   // (the odd half-warp of an odd Q solves nothing)
+  const int lane = threadIdx.x & (kWarp - 1), warp = threadIdx.x / kWarp;
+  const int lq = Q > 1 ? 32 - __clz(Q - 1) : 0;   // 2^lq lanes per column in the scans
+  const int st = lane & ((1 << lq) - 1);
+  const int ncols = (AXIS == 0 ? a.ny : a.nx) * a.nz;
+  const int ntiles = (ncols + B - 1) >> lb;
   const size_t stride = AXIS == 1 ? (size_t)a.nz : (size_t)a.ny * a.nz;
   C *gpsi = reinterpret_cast<C *>(a.psi);
-  const int b = threadIdx.x % B;   // B divides the block size: the column is fixed per thread
-  const int n0 = threadIdx.x / B;
-  constexpr int nstep = NT / B;   // the launch has NT threads
-  const bool do_reduce = AXIS == 0 && reduce;
+  DFAcc acc[4];   // n, nothing (x^2 n is not taken), j'^2 n, k'^2 n
 
-  auto tile_origin = [&](int tile, int &fixed, int &k0) -> size_t {
-    fixed = tile / nkt;
-    k0 = (tile - fixed * nkt) * B;
-    return AXIS == 1 ? (size_t)fixed * a.ny * a.nz + k0 : (size_t)fixed * a.nz + k0;
+  // inclusive scan of the chunk carries of every column, in place
+  auto scan = [&](C *car, bool up) {
+    const Coef *f = scan_s + (up ? 0 : 5 * kWarp) + st;
+    for (int c0 = warp << (5 - lq); c0 < B; c0 += (blockDim.x / kWarp) << (5 - lq)) {
+      C *slot = car + st * SB + c0 + (lane >> lq);
+      C v = st < Q ? *slot : czero<R>();
+#pragma unroll
+      for (int k = 0; k < 5; ++k) {
+        if (k >= lq) break;
+        const C o = up ? shfl_up(v, 1 << k) : shfl_down(v, 1 << k);
+        if (up ? st >= (1 << k) : st + (1 << k) < (1 << lq)) v = cfma(f[k * kWarp], o, v);
+      }
+      if (st < Q) *slot = v;
+    }
   };
-  auto issue = [&](int tile, C *buf) {
-    int fixed, k0;
-    const size_t base = tile_origin(tile, fixed, k0);
-    if (b < min(B, a.nz - k0)) {
-      const C *src = gpsi + base + b + (size_t)n0 * stride;
-      const SlotWalk<NT / B> w(n0, lc);
-      // (FULL: not the far wall, whose slot stays zero, as the padding's do)
-      const int nload = FULL ? N - 1 : N;
-#pragma unroll 4
-      for (int j = 0; n0 + (NT / B) * j < nload; ++j, src += (NT / B) * stride) cp_async(buf + w(j, n0) * SB + b, src);
+
+  // unit u of this CTA: tile S (blockIdx.x + (u / S) gridDim.x) + u % S, in buffer u % NBUF.
+  // issue: the interior rows of the S tiles from unit u on, by 16-byte copies of column pairs
+  // (the columns of a pair share their x or y index and are 16-byte aligned, nz being even,
+  // unless the field itself is a caller's that is not: the adjoint's cotangent)
+  const bool wide = (reinterpret_cast<uintptr_t>(gpsi) & 15) == 0;
+  auto tile_of = [&](int u) { return S * (int)(blockIdx.x + (u / S) * gridDim.x) + u % S; };
+  auto issue = [&](int u) {
+    const int lp = lb - 1 + (S - 1), piece = threadIdx.x & ((1 << lp) - 1);
+    const int half = piece >> (lb - 1), c0 = 2 * (piece & ((B >> 1) - 1));   // (half: the second tile of a pair)
+    const int col = ((tile_of(u) + half) << lb) + c0;
+    if (col < ncols) {
+      C *buf = tiles + (u + half) % NBUF * tile_slots + c0;
+      const int fixed = col / a.nz, k = col - fixed * a.nz;
+      const C *src = gpsi + (AXIS == 0 ? (size_t)col : (size_t)fixed * a.ny * a.nz + k) + stride;
+      const int step = blockDim.x >> lp;
+      if (wide) {
+        for (int i = threadIdx.x >> lp; i < m; i += step)
+          cp_async(reinterpret_cast<float4 *>(buf + cnr_row<CH>(i, B)), reinterpret_cast<const float4 *>(src + i * stride));
+      } else {
+        for (int i = threadIdx.x >> lp; i < m; i += step) {
+          cp_async(buf + cnr_row<CH>(i, B), src + i * stride);
+          cp_async(buf + cnr_row<CH>(i, B) + 1, src + i * stride + 1);
+        }
+      }
     }
     cp_async_commit();
   };
 
-  if (do_reduce)
-    for (int n = threadIdx.x; n < N; n += blockDim.x) {
-      wxtab[n] = (float)quad_weight3(n, a.nx, a.simpson);
-    }
-  const Coef c = CnCoef<R, Coef>::make(pick<R>(a.cn_r[AXIS], a.cn_rf[AXIS], a.cn_rl[AXIS]));
-  {
-    const Coef *gtab = reinterpret_cast<const Coef *>(a.cn[AXIS].tab);
-    for (int q = threadIdx.x; q < ntab; q += blockDim.x) stab[q] = gtab[q];
-  }
-  const Coef *tab = stab;
-  DFAcc acc[4];
-  if constexpr (FULL) {   // the far wall and the padding: zero in both buffers, once
-    for (int q = threadIdx.x; q < (m_pad + 2 - N) * SB; q += blockDim.x) {
-      const int g = N - 1 + q / SB, col = q % SB;
-      cur[cn_slot(g, lc) * SB + col] = czero<R>();
-      nxt[cn_slot(g, lc) * SB + col] = czero<R>();
-    }
-  }
-
-  int tile = blockIdx.x;
-  if (tile < ntiles) issue(tile, cur);
-  for (; tile < ntiles; tile += gridDim.x) {
-    const int next = tile + gridDim.x;
-    if (next < ntiles) {
-      issue(next, nxt);
-      cp_async_wait_group<1>();
-    } else {
-      cp_async_wait_group<0>();
-    }
+  issue(0);
+  if (!PAIR) issue(1);
+  for (int u = 0, tile; (tile = tile_of(u)) < ntiles; ++u) {
+    if (!PAIR) cp_async_wait_group<1>();
+    else if (u % 2 == 0) cp_async_wait_group<0>();
     __syncthreads();
-    int fixed, k0;
-    const size_t base = tile_origin(tile, fixed, k0);
-    const int nb = min(B, a.nz - k0);
-    if constexpr (FULL && NT == 8 * kWarp && B == 16) {
-      // 8 warps, two columns each in lockstep (w, w + 8): each table value read once for both;
-      // columns past nb are solved too (their padding is zero) and not stored
-      const int w = threadIdx.x / kWarp;
-      cn_line2_any<R, Coef>(cur + w, cur + w + 8, SB, lc, tab, tab + 4 * (kWarp << lc), c);
-    } else {
-      for (int l = threadIdx.x / kWarp; l < nb; l += blockDim.x / kWarp)
-        cn_line_any<R, Coef, true, FULL>(cur + l, SB, FULL ? m_pad : a.cn[AXIS].m, lc, tab, tab + 4 * (kWarp << lc), c);
-    }
+    const int col = (tile << lb) + b;
+    const bool on = q < Q && col < ncols;
+    const int fixed = col / a.nz, k = col - fixed * a.nz;   // (x lines: the y index; y lines: the x index)
+    C *p = gpsi + (AXIS == 0 ? (size_t)col : (size_t)fixed * a.ny * a.nz + k) + (size_t)(q * CH + 1) * stride;
+    C v[CH], y[CH];
+    const C *row = tiles + u % NBUF * tile_slots + cnr_row<CH>(min(q, Q - 1) * CH, B) + b;
+#pragma unroll
+    for (int e = 0; e < CH; ++e) v[e] = e < len ? row[e * B] : czero<R>();
+    C s = czero<R>();
+#pragma unroll
+    for (int e = 0; e < CH; ++e) y[e] = s = cfma(al[tq + e], s, v[e]);
+    if (q < Q) car1[q * SB + b] = s;
+    __syncthreads();   // (every thread has read its points: the buffer can be filled again)
+    if (!PAIR || u % 2 == 0) issue(u + 2);
+    scan(car1, true);
     __syncthreads();
-    if (b < nb) {
-      DFAcc s0;   // this thread's share of the column: sum W_x n
-      C *dst = gpsi + base + b + (size_t)n0 * stride;
-      const SlotWalk<NT / B> walk(n0, lc);
-#pragma unroll 4
-      for (int j = 0, n = n0; n < N; ++j, n += nstep, dst += nstep * stride) {
-        const C w = cur[walk(j, n0) * SB + b];
-        *dst = w;
-        if (do_reduce) {
-          const float d = fmaf(w.re, w.re, w.im * w.im);
-          s0.add(a.simpson ? wxtab[n] * d : d);   // exact: W_x is 0, 1, 2 or 4 (1 without Simpson)
-        }
+    const C Y = q > 0 && q < Q ? car1[(q - 1) * SB + b] : czero<R>();
+    s = czero<R>();
+#pragma unroll
+    for (int e = CH - 1; e >= 0; --e) y[e] = s = mul(be[tq + e], cfma_c(c, s, y[e]));
+    if (q < Q) car2[q * SB + b] = cfma(hg[tq].h, Y, s);
+    __syncthreads();
+    scan(car2, false);
+    __syncthreads();
+    const C X = q < Q - 1 ? car2[(q + 1) * SB + b] : czero<R>();
+#pragma unroll
+    for (int e = 0; e < CH; ++e) {
+      const CoefPair<Coef> f = hg[tq + e];
+      const C chi = cfma(f.h, Y, cfma(f.g, X, y[e]));
+      v[e] = {twice_minus(chi.re, v[e].re), twice_minus(chi.im, v[e].im)};
+    }
+    if (on) {
+      if (len == CH) {
+#pragma unroll
+        for (int e = 0; e < CH; ++e) p[e * stride] = v[e];
+      } else {
+#pragma unroll
+        for (int e = 0; e < CH; ++e)
+          if (e < len) p[e * stride] = v[e];
       }
+      if (q == 0) p[-(ptrdiff_t)stride] = czero<R>();   // the walls
+      if (q == Q - 1) p[(size_t)len * stride] = czero<R>();
       if (do_reduce) {
+        DFAcc s0;   // this thread's share of the column: sum W_x n
+        // (the points past the line's end, in the last chunk, are zero)
+        if (a.simpson) {
+          const float *wx = wxtab + q * CH + 1;   // exact products: W_x is 0, 1, 2 or 4
+#pragma unroll
+          for (int e = 0; e < CH; ++e) s0.add(wx[e] * fmaf(v[e].re, v[e].re, v[e].im * v[e].im));
+        } else {
+#pragma unroll
+          for (int e = 0; e < CH; ++e) s0.add(fmaf(v[e].re, v[e].re, v[e].im * v[e].im));
+        }
         // W_y W_z is 0 or a power of two up to 16; j'^2 W_y W_z <= 2^20: exact floats
-        const int jj = fixed - a.ny / 2, kk = k0 + b - a.nz / 2;
-        const int wyz = quad_weight3(fixed, a.ny, a.simpson) * quad_weight3(k0 + b, a.nz, a.simpson);
+        const int jj = fixed - a.ny / 2, kk = k - a.nz / 2;
+        const int wyz = quad_weight3(fixed, a.ny, a.simpson) * quad_weight3(k, a.nz, a.simpson);
         acc[0].add_scaled((float)wyz, s0);
         acc[2].add_scaled((float)(jj * jj * wyz), s0);
         acc[3].add_scaled((float)(kk * kk * wyz), s0);
       }
     }
-    __syncthreads();   // `cur` is refilled by the prefetch two tiles ahead
-    C *t = cur;
-    cur = nxt;
-    nxt = t;
   }
   if (do_reduce) {
     const double w = a.simpson ? 1.0 / 27.0 : 1.0;   // (1/3)^3 of the integer Simpson weights
-    double v[4] = {acc[0].value() * w, 0.0, acc[2].value() * (w * a.hy * a.hy), acc[3].value() * (w * a.hz * a.hz)};
-    finish_sweep_sums(a, v, renorm);
+    finish_sweep_sums(a, acc, w, w * a.hy * a.hy, w * a.hz * a.hz, renorm);
   }
 }
 // one condensate (G = false, its arguments passed by value), or condensate blockIdx.z of
 // a group of same-shaped condensates (G = true, the arguments from the device array ga)
-template <typename R, typename Coef, int AXIS, int B = Tiles<R>::kCnCols, int NT = Tiles<R>::kCnThreads, bool G = false,
-          bool FULL = false>
-__global__ void __launch_bounds__(NT, (FULL && NT == 256) ? 1 : 512 / NT) k_cn(KArgs a, const KArgs *ga, int reduce, int renorm) {
-  if constexpr (G) k_cn_body<R, Coef, AXIS, B, NT, FULL>(ga[blockIdx.z], reduce, renorm);
-  else k_cn_body<R, Coef, AXIS, B, NT, FULL>(a, reduce, renorm);
-}
-
-// K6 / K7 for short FP32 lines of n = 8 CH points (CH = short_cn_chunk(n) = 4 .. 16): the
-// chunked solve on 8 lanes per line, CH points each (three scan steps instead of five, whose
-// cost per point on 32 lanes of 4 points outweighed the solve), four lines per warp, 4 warps
-// and 16 columns per tile, up to four CTAs per SM; persistent and double-buffered as k_cn.
-// The line is padded to the 8 CH unknowns of grid indices 1 .. n: the far wall n - 1 and the
-// slot n beyond it hold zero, and the tables (8-lane layout) decouple them.  Slot of grid
-// index g: g + (g - 1) / CH (slot 0 the wall g = 0).  The four lines of warp w are the columns
-// 2w, 2w + 8, 2w + 1 and 2w + 9: the two lines of a half-warp fall on distinct banks.
-template <typename Coef, int AXIS, int CH>
-__device__ __forceinline__ void k_cn_short_body(const KArgs &a, int reduce, int renorm) {
-  using R = float;
-  using C = cplx<float>;
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  constexpr int L = 8, B = 16, NT = 128, SB = B + 1;
-  constexpr int N = L * CH;                     // the line length
-  constexpr int SLOTS = N + 2 + N / CH;         // grid indices 0 .. N + 1
-  constexpr int W = NT / B;                     // rows per pass of the tile loops
-  constexpr int P = W / gcd_c(W, CH) * CH;      // lcm(W, CH): the rows' slot walk period
-  constexpr int NTAB = 4 * L * CH + 6 * L;      // alpha, beta, H, G, then the scan factors
-  static_assert(N % P == 0 && P % W == 0, "whole periods per line");
-  const int nkt = (a.nz + B - 1) / B;
-  const int ntiles = (AXIS == 0 ? a.ny : a.nx) * nkt;
-  C *cur = reinterpret_cast<C *>(smem_raw);
-  C *nxt = cur + SLOTS * SB;
-  Coef *stab = reinterpret_cast<Coef *>(nxt + SLOTS * SB);
-  float *wxtab = reinterpret_cast<float *>(stab + NTAB);   // W_x(i) = 3 x the weight (or 1)
-  const size_t stride = AXIS == 1 ? (size_t)a.nz : (size_t)a.ny * a.nz;
-  C *gpsi = reinterpret_cast<C *>(a.psi);
-  const int b = threadIdx.x % B, n0 = threadIdx.x / B;
-  const bool do_reduce = AXIS == 0 && reduce;
-
-  auto tile_origin = [&](int tile, int &fixed, int &k0) -> size_t {
-    fixed = tile / nkt;
-    k0 = (tile - fixed * nkt) * B;
-    return AXIS == 1 ? (size_t)fixed * a.ny * a.nz + k0 : (size_t)fixed * a.nz + k0;
-  };
-  // rows 0 .. N - 2 (not the far wall, whose slot stays zero)
-  auto issue = [&](int tile, C *buf) {
-    int fixed, k0;
-    const size_t base = tile_origin(tile, fixed, k0);
-    if (b < min(B, a.nz - k0)) {
-      const C *src = gpsi + base + b;
-#pragma unroll
-      for (int sub = 0; sub < P / W; ++sub) {
-        const int o = n0 + W * sub;
-        const SlotWalkP<P, CH> w(o);
-#pragma unroll
-        for (int j = 0; j < N / P; ++j)
-          if (o + P * j < N - 1) cp_async(buf + w(j, o) * SB + b, src + (size_t)(o + P * j) * stride);
-      }
-    }
-    cp_async_commit();
-  };
-
-  for (int q = threadIdx.x; q < 3 * SB; q += NT) {   // grid indices N - 1 .. N + 1: zero, once
-    const int g = N - 1 + q / SB, col = q % SB;
-    cur[(g + (g - 1) / CH) * SB + col] = czero<R>();
-    nxt[(g + (g - 1) / CH) * SB + col] = czero<R>();
-  }
-  {
-    const Coef *gtab = reinterpret_cast<const Coef *>(a.cn8_tab[AXIS]);
-    for (int q = threadIdx.x; q < NTAB; q += NT) stab[q] = gtab[q];
-  }
-  if (do_reduce)
-    for (int n = threadIdx.x; n < N; n += NT) wxtab[n] = (float)quad_weight3(n, a.nx, a.simpson);
-  const Coef c = CnCoef<R, Coef>::make(a.cn_rf[AXIS]);
-  const int warp = threadIdx.x / kWarp, grp = (threadIdx.x & (kWarp - 1)) >> 3;
-  const int col = 2 * warp + (grp >> 1) + 8 * (grp & 1);
-  DFAcc acc[4];
-
-  int tile = blockIdx.x;
-  if (tile < ntiles) issue(tile, cur);
-  for (; tile < ntiles; tile += gridDim.x) {
-    const int next = tile + gridDim.x;
-    if (next < ntiles) {
-      issue(next, nxt);
-      cp_async_wait_group<1>();
-    } else {
-      cp_async_wait_group<0>();
-    }
-    __syncthreads();
-    int fixed, k0;
-    const size_t base = tile_origin(tile, fixed, k0);
-    const int nb = min(B, a.nz - k0);
-    // every column is solved (all lanes take part in the scans); those past nb are not stored
-    cn_line<R, Coef, CH, true, true, L>(cur + col, SB, N, 0, stab, stab + 4 * L * CH, c);
-    __syncthreads();
-    if (b < nb) {
-      DFAcc s0;   // this thread's share of the column: sum W_x n
-      C *dst = gpsi + base + b;
-#pragma unroll
-      for (int sub = 0; sub < P / W; ++sub) {
-        const int o = n0 + W * sub;
-        const SlotWalkP<P, CH> w(o);
-#pragma unroll
-        for (int j = 0; j < N / P; ++j) {
-          const int n = o + P * j;
-          const C v = cur[w(j, o) * SB + b];
-          dst[(size_t)n * stride] = v;
-          if (do_reduce) {
-            const float d = fmaf(v.re, v.re, v.im * v.im);
-            s0.add(a.simpson ? wxtab[n] * d : d);   // exact: W_x is 0, 1, 2 or 4 (1 without Simpson)
-          }
-        }
-      }
-      if (do_reduce) {
-        const int jj = fixed - a.ny / 2, kk = k0 + b - a.nz / 2;
-        const int wyz = quad_weight3(fixed, a.ny, a.simpson) * quad_weight3(k0 + b, a.nz, a.simpson);
-        acc[0].add_scaled((float)wyz, s0);
-        acc[2].add_scaled((float)(jj * jj * wyz), s0);
-        acc[3].add_scaled((float)(kk * kk * wyz), s0);
-      }
-    }
-    __syncthreads();   // `cur` is refilled by the prefetch two tiles ahead
-    C *t = cur;
-    cur = nxt;
-    nxt = t;
-  }
-  if (do_reduce) {
-    const double w = a.simpson ? 1.0 / 27.0 : 1.0;   // (1/3)^3 of the integer Simpson weights
-    double v[4] = {acc[0].value() * w, 0.0, acc[2].value() * (w * a.hy * a.hy), acc[3].value() * (w * a.hz * a.hz)};
-    finish_sweep_sums(a, v, renorm);
-  }
-}
-template <typename Coef, int AXIS, int CH, bool G = false>
-__global__ void __launch_bounds__(128, 4) k_cn_short(KArgs a, const KArgs *ga, int reduce, int renorm) {
-  if constexpr (G) k_cn_short_body<Coef, AXIS, CH>(ga[blockIdx.z], reduce, renorm);
-  else k_cn_short_body<Coef, AXIS, CH>(a, reduce, renorm);
-}
-// shared memory of k_cn_short at chunk CH: two tile buffers, the tables, the x weights
-__host__ __device__ constexpr size_t smem_cn_short(int ch) {
-  return 2 * (size_t)(8 * ch + 2 + 8) * 17 * 8 + (size_t)(4 * 8 * ch + 48) * 8 + (size_t)8 * ch * 4;
+template <typename Coef, int AXIS, int CH, bool PAIR, bool G = false>
+__global__ void __launch_bounds__(kCnrThreads, 1) k_cn_reg(KArgs a, const KArgs *ga, int reduce, int renorm) {
+  if constexpr (G) k_cn_reg_body<Coef, AXIS, CH, PAIR>(ga[blockIdx.z], reduce, renorm);
+  else k_cn_reg_body<Coef, AXIS, CH, PAIR>(a, reduce, renorm);
 }
 
 // FP64-class sweeps: two threads per line, the twisted ("burn at both ends") factorization.
@@ -2852,7 +2835,7 @@ __global__ void __launch_bounds__(128, 7) k_cn_twisted(KArgs a, int reduce, int 
   }
   if (do_reduce) {
     double v[4] = {acc[0].value(), acc[1].value(), acc[2].value(), acc[3].value()};
-    finish_sweep_sums(a, v, renorm);
+    finish_sweep_sums(a, v, 1.0, 1.0, 1.0, renorm);
   }
 }
 
@@ -3005,8 +2988,8 @@ __global__ void __launch_bounds__(Tiles<R>::kZThreads) k5_adj_phase(KArgs a) {
   const C *res2 = fft_lines_n<R, -1, N, PZ, SB, Tiles<R>::kZThreads>(sbuf, res, a.plan[2], np, reinterpret_cast<const C *>(a.tw[2]));
   store_half_spectrum_column<R>(a, res2, i, j0, np);
   for (int e = threadIdx.x; e < nl * nz; e += blockDim.x) gb[e] = gt[e];
-  double v3[3] = {acc.get(0), acc.get(1), acc.get(2)};
-  if (reduce_across_blocks<3>(v3, a.partials, &a.state->ticket) && threadIdx.x == 0) {
+  double v4[4] = {acc.get(0), acc.get(1), acc.get(2), 0.0}, v3[4];
+  if (reduce_across_blocks<4>(v4, v3, a.partials, &a.state->ticket) && threadIdx.x == 0) {
     a.state->grads[0] += a.dt * v3[0];
     a.state->grads[1] += a.dt * v3[1];
     a.state->grads[2] += a.dt_nuz * v3[2];
@@ -3102,13 +3085,8 @@ struct Impl {
   static constexpr bool kCtSizes = !std::is_same<R, df>::value;
   // FP32 also at nz = 96 and 64 (K1, K5; the batched small grids)
   static constexpr bool kShortCt = std::is_same<R, float>::value;
-  // the padded (FULL) chunked sweeps: the y sweep on 8 warps, two columns each in lockstep
-  // (one CTA per SM); the x sweep, whose store also takes the norm sums (a longer serial chain
-  // per thread at half the threads), on 16 warps of one column each
-  template <int AXIS>
-  static constexpr int cn_full_threads() { return AXIS == 1 ? 256 : T::kCnThreads; }
   // the FP64-class sweeps run a Thomas solve per line on two threads (k_cn_twisted), the
-  // FP32 ones the chunked solver in persistent tiles (k_cn)
+  // FP32 ones the chunked solver in registers (k_cn_reg)
   static constexpr bool kCnThread = Fp64Class<R>::value;
   // and the z sweep too, after a phase-only K5 pass: the per-line solve's fewer arithmetic
   // instructions win over the extra pass through HBM
@@ -3128,14 +3106,7 @@ struct Impl {
   }
   static size_t smem_y(const KArgs &a) { return 2 * (size_t)a.ny * (a.ylines + 1) * E; }
   static size_t smem_x(const KArgs &a) { return 2 * (size_t)a.nx * T::kXCols * E; }
-  static size_t smem_cn(int n, int lchunk, int cols = T::kCnCols) {
-    return 2 * (size_t)cn_slots(n, lchunk) * (cols + 1) * E + (size_t)(4 * (kWarp << lchunk) + 10 * kWarp) * E +
-           2 * (size_t)n * sizeof(R);
-  }
-
-
   static dim3 grid_z(const KArgs &a) { return dim3((a.ny + T::kZLines - 1) / T::kZLines, a.nx); }
-  // persistent grid of the CN kernels: all tiles, capped at the number of co-resident CTAs
   static int sm_count() {
     static int n = 0;
     if (!n) {
@@ -3146,24 +3117,6 @@ struct Impl {
     }
     return n;
   }
-  // the chunked sweeps pad a line to 32 whole chunks (no per-point guard) when that adds at
-  // most two unknowns (the power-of-two lengths); the tile line then has 32 chunk + 2 points
-  static bool cn_full(const KArgs &a, int axis) { return (kWarp << a.cn[axis].lchunk) <= a.cn[axis].m + 2; }
-  static int cn_len(const KArgs &a, int axis) {
-    return cn_full(a, axis) ? (kWarp << a.cn[axis].lchunk) + 2 : a.cn[axis].m + 2;
-  }
-  static dim3 grid_cn(const KArgs &a, int axis, int cols = T::kCnCols) {
-    const int tiles = ((a.nz + cols - 1) / cols) * (axis == 0 ? a.ny : a.nx);
-    const int n = cn_len(a, axis);
-    const size_t sm = smem_cn(n, a.cn[axis].lchunk, cols);
-    // co-resident CTAs per SM: by shared memory, and by registers (NT threads of up to 128)
-    const int fit_regs = 65536 / (T::kCnThreads * 128) < 1 ? 1 : 65536 / (T::kCnThreads * 128);
-    const int fit = std::min(sm * 2 + 4096 <= 227 * 1024 ? 2 : 1, fit_regs);
-    const int per_sm = a.cn_per_sm < fit ? (a.cn_per_sm < 1 ? 1 : a.cn_per_sm) : fit;
-    const int cap = sm_count() * per_sm;
-    return dim3(tiles < cap ? tiles : cap);
-  }
-
   // Allow each kernel the device's opt-in shared memory minus its static shared memory.
   template <typename K>
   static cudaError_t allow_smem(K kernel) {
@@ -3193,6 +3146,48 @@ struct Impl {
     chk(allow_smem(static_cast<K>(k3_reg<512>)));
     chk(allow_smem(static_cast<K>(k3_reg<256>)));
     chk(allow_smem(static_cast<K>(k3_reg<128>)));
+    return e;
+  }
+
+  // Calls f with the kernel k_cn_reg<Coef, AXIS, CH, PAIR, GRP> of these arguments: 12 or 16
+  // points per thread; the smaller chunks serve the differentiation calls (real time, single
+  // contexts).  f(kernel) for one launch, or for every instance when ch = 0 (init).
+  template <int AXIS, bool GRP, typename F>
+  static void cn_reg_kernel(int ch, bool imag, bool pair, F &&f) {
+    using K = void (*)(KArgs, const KArgs *, int, int);
+    auto chunk = [&](auto chc) {
+      constexpr int CH = decltype(chc)::value;
+      if (ch != CH && ch != 0) return;
+      constexpr bool kMain = CH >= 12;
+      if constexpr (kMain || !GRP) {
+        if ((!imag && !pair) || ch == 0) f((K)k_cn_reg<C, AXIS, CH, false, GRP>);
+        if constexpr (kMain) {
+          if ((imag && !pair) || ch == 0) f((K)k_cn_reg<float, AXIS, CH, false, GRP>);
+        }
+        if constexpr (AXIS == 0) {
+          if ((!imag && pair) || ch == 0) f((K)k_cn_reg<C, 0, CH, true, GRP>);
+          if constexpr (kMain) {
+            if ((imag && pair) || ch == 0) f((K)k_cn_reg<float, 0, CH, true, GRP>);
+          }
+        }
+      }
+    };
+    using std::integral_constant;
+    chunk(integral_constant<int, 16>{});
+    chunk(integral_constant<int, 12>{});
+    chunk(integral_constant<int, 8>{});
+    chunk(integral_constant<int, 6>{});
+    chunk(integral_constant<int, 4>{});
+    chunk(integral_constant<int, 2>{});
+  }
+  template <bool GRP>
+  static cudaError_t init_sweeps() {
+    cudaError_t e = cudaSuccess;
+    auto f = [&](auto k) {
+      if (e == cudaSuccess) e = allow_smem(k);
+    };
+    cn_reg_kernel<0, GRP>(0, false, false, f);
+    cn_reg_kernel<1, GRP>(0, false, false, f);
     return e;
   }
 
@@ -3249,17 +3244,7 @@ struct Impl {
         chk(allow_smem(k5_zline<R, C, kZFast, 64>));
       }
     }
-    if constexpr (!kCnThread) {
-      constexpr int B = T::kCnCols, NT = T::kCnThreads;
-      chk(allow_smem(k_cn<R, R, 0>));
-      chk(allow_smem(k_cn<R, R, 1>));
-      chk(allow_smem(k_cn<R, C, 0>));
-      chk(allow_smem(k_cn<R, C, 1>));
-      chk(allow_smem(k_cn<R, R, 0, B, cn_full_threads<0>(), false, true>));
-      chk(allow_smem(k_cn<R, R, 1, B, cn_full_threads<1>(), false, true>));
-      chk(allow_smem(k_cn<R, C, 0, B, cn_full_threads<0>(), false, true>));
-      chk(allow_smem(k_cn<R, C, 1, B, cn_full_threads<1>(), false, true>));
-    }
+    if constexpr (!kCnThread) chk(init_sweeps<false>());
     if constexpr (kRegFft) chk(init_reg());
     if constexpr (kAdjoint) chk(allow_smem(k5_adj_phase<R>));
     if constexpr (kAdjoint) chk(allow_smem(k5_adj_combine<R>));
@@ -3437,9 +3422,9 @@ struct Impl {
       if (plan_ct(a.plan[2], 512)) go(integral_constant<int, 512>{});
       else if (plan_ct(a.plan[2], 384)) go(integral_constant<int, 384>{});
       else if (plan_ct(a.plan[2], 256)) go(integral_constant<int, 256>{});
-      else if (plan_ct(a.plan[2], 128) && (!kShortCt || a.cn8_tab[2])) go(integral_constant<int, 128>{});
-      else if (kShortCt && plan_ct(a.plan[2], 96) && a.cn8_tab[2]) go(integral_constant<int, kShortCt ? 96 : 0>{});
-      else if (kShortCt && plan_ct(a.plan[2], 64) && a.cn8_tab[2]) go(integral_constant<int, kShortCt ? 64 : 0>{});
+      else if (plan_ct(a.plan[2], 128) && (!kShortCt || a.cn8z_tab)) go(integral_constant<int, 128>{});
+      else if (kShortCt && plan_ct(a.plan[2], 96) && a.cn8z_tab) go(integral_constant<int, kShortCt ? 96 : 0>{});
+      else if (kShortCt && plan_ct(a.plan[2], 64) && a.cn8z_tab) go(integral_constant<int, kShortCt ? 64 : 0>{});
       else go(integral_constant<int, 0>{});
     } else {
       go(integral_constant<int, 0>{});
@@ -3483,35 +3468,21 @@ struct Impl {
     }
     return cudaGetLastError();
   }
-  // The short-line sweep (FP32, x or y lines of short_cn_chunk(n) != 0 with their 8-lane
-  // tables): launched for `members` condensates (blockIdx.z; ga their arguments when GRP) on
-  // one resident wave of persistent CTAs, four per SM.  False when the line takes k_cn.
+  // The FP32 x and y sweeps, for `members` condensates (blockIdx.z; ga their arguments when
+  // GRP): one resident wave of persistent CTAs, 512 threads per SM, shared out between the
+  // members.
   template <int AXIS, bool GRP>
-  static bool cn_short(const KArgs &a, const KArgs *ga, unsigned members, int reduce, int renorm, cudaStream_t st) {
-    if constexpr (!std::is_same<R, float>::value) {
-      return false;
-    } else {
-      const int n = AXIS == 0 ? a.nx : a.ny;
-      const int ch = short_cn_chunk(n);
-      if (!ch || !a.cn8_tab[AXIS]) return false;
-      const int tiles = ((a.nz + 15) / 16) * (AXIS == 0 ? a.ny : a.nx);
-      const int per = std::max(1, sm_count() * 4 / (int)members);
-      const dim3 g(std::min(tiles, per), 1, members);
-      const size_t sm = smem_cn_short(ch);
-      auto go = [&](auto chc) {
-        constexpr int CH = decltype(chc)::value;
-        if (a.imag) k_cn_short<R, AXIS, CH, GRP><<<g, 128, sm, st>>>(a, ga, reduce, renorm);
-        else k_cn_short<C, AXIS, CH, GRP><<<g, 128, sm, st>>>(a, ga, reduce, renorm);
-      };
-      switch (ch) {
-        case 4: go(std::integral_constant<int, 4>{}); break;
-        case 6: go(std::integral_constant<int, 6>{}); break;
-        case 8: go(std::integral_constant<int, 8>{}); break;
-        case 12: go(std::integral_constant<int, 12>{}); break;
-        default: go(std::integral_constant<int, 16>{}); break;
-      }
-      return true;
-    }
+  static void cn_reg(const KArgs &a, const KArgs *ga, unsigned members, int reduce, int renorm, cudaStream_t st) {
+    const int n = AXIS == 0 ? a.nx : a.ny, ch = a.cn[AXIS].chunk, q = (n - 2 + ch - 1) / ch;
+    const bool pair = AXIS == 0 && n > 258;
+    const int cols = pair ? 32 : cnr_cols(q);
+    const int nt = ((pair ? 16 : cols) * q + kWarp - 1) / kWarp * kWarp;
+    const int tiles = ((AXIS == 0 ? a.ny : a.nx) * a.nz + cols - 1) / cols;
+    const size_t sm = smem_cnr(n, ch, a.imag ? sizeof(float) : sizeof(C), pair);
+    const int per_sm = std::max(1, std::min(kCnrThreads * a.cn_per_sm / 2 / nt, (int)(220 * 1024 / (sm + 2048))));
+    const int share = std::max(1, sm_count() * per_sm / (int)members);
+    const dim3 g(std::min(tiles, share), 1, members);
+    cn_reg_kernel<AXIS, GRP>(ch, a.imag != 0, pair, [&](auto k) { k<<<g, nt, sm, st>>>(a, ga, reduce, renorm); });
   }
   template <int AXIS>
   static cudaError_t cn(const KArgs &a, int reduce, int renorm, cudaStream_t st) {
@@ -3523,20 +3494,7 @@ struct Impl {
       if (a.imag) k_cn_twisted<R, R, AXIS><<<blocks, 128, sm, st>>>(a, reduce, renorm);
       else k_cn_twisted<R, C, AXIS><<<blocks, 128, sm, st>>>(a, reduce, renorm);
     } else {
-      if constexpr (AXIS < 2) {
-        if (cn_short<AXIS, false>(a, nullptr, 1, reduce, renorm, st)) return cudaGetLastError();
-      }
-      constexpr int B = T::kCnCols, NT = T::kCnThreads;
-      const size_t sm = smem_cn(cn_len(a, AXIS), a.cn[AXIS].lchunk);
-      const dim3 g = grid_cn(a, AXIS);
-      if (cn_full(a, AXIS)) {
-        constexpr int NF = cn_full_threads<AXIS>();
-        if (a.imag) k_cn<R, R, AXIS, B, NF, false, true><<<g, NF, sm, st>>>(a, nullptr, reduce, renorm);
-        else k_cn<R, C, AXIS, B, NF, false, true><<<g, NF, sm, st>>>(a, nullptr, reduce, renorm);
-      } else {
-        if (a.imag) k_cn<R, R, AXIS><<<g, NT, sm, st>>>(a, nullptr, reduce, renorm);
-        else k_cn<R, C, AXIS><<<g, NT, sm, st>>>(a, nullptr, reduce, renorm);
-      }
+      if constexpr (AXIS < 2) cn_reg<AXIS, false>(a, nullptr, 1, reduce, renorm, st);
     }
     return cudaGetLastError();
   }
@@ -3607,7 +3565,7 @@ struct Impl {
   static int max_blocks(const KArgs &a) {
     const dim3 z = grid_z(a);
     const int bz = (int)(z.x * z.y);
-    const int bx = ((a.nz + T::kCnCols - 1) / T::kCnCols) * a.ny;
+    const int bx = (a.ny * a.nz + 7) / 8;   // the FP32 x sweep's tiles of at least 8 columns
     const int bt = (int)(((long long)a.ny * a.nz + 63) / 64);   // the two-thread sweep along x
     return std::max(bz, std::max(bx, bt));
   }
@@ -3683,14 +3641,7 @@ struct GroupLaunch {
     attr(k5_zline<R, C, kZStep, 128, true>, e);
     attr(k5_zline<R, R, kZStep, 0, true>, e);
     attr(k5_zline<R, C, kZStep, 0, true>, e);
-    attr(k_cn<R, R, 0, T::kCnCols, T::kCnThreads, true>, e);
-    attr(k_cn<R, R, 1, T::kCnCols, T::kCnThreads, true>, e);
-    attr(k_cn<R, C, 0, T::kCnCols, T::kCnThreads, true>, e);
-    attr(k_cn<R, C, 1, T::kCnCols, T::kCnThreads, true>, e);
-    attr(k_cn<R, R, 0, T::kCnCols, I::template cn_full_threads<0>(), true, true>, e);
-    attr(k_cn<R, R, 1, T::kCnCols, I::template cn_full_threads<1>(), true, true>, e);
-    attr(k_cn<R, C, 0, T::kCnCols, I::template cn_full_threads<0>(), true, true>, e);
-    attr(k_cn<R, C, 1, T::kCnCols, I::template cn_full_threads<1>(), true, true>, e);
+    if (e == cudaSuccess) e = I::template init_sweeps<true>();
     return e;
   }
 
@@ -3739,24 +3690,10 @@ struct GroupLaunch {
     if (I::plan_ct(a.plan[2], 512)) go(integral_constant<int, 512>{});
     else if (I::plan_ct(a.plan[2], 384)) go(integral_constant<int, 384>{});
     else if (I::plan_ct(a.plan[2], 256)) go(integral_constant<int, 256>{});
-    else if (I::plan_ct(a.plan[2], 128) && a.cn8_tab[2]) go(integral_constant<int, 128>{});
-    else if (I::plan_ct(a.plan[2], 96) && a.cn8_tab[2]) go(integral_constant<int, 96>{});
-    else if (I::plan_ct(a.plan[2], 64) && a.cn8_tab[2]) go(integral_constant<int, 64>{});
+    else if (I::plan_ct(a.plan[2], 128) && a.cn8z_tab) go(integral_constant<int, 128>{});
+    else if (I::plan_ct(a.plan[2], 96) && a.cn8z_tab) go(integral_constant<int, 96>{});
+    else if (I::plan_ct(a.plan[2], 64) && a.cn8z_tab) go(integral_constant<int, 64>{});
     else go(integral_constant<int, 0>{});
-  }
-  template <typename Co, int AXIS>
-  static void cn(const KArgs &a, const KArgs *ga, unsigned n, int reduce, int renorm, cudaStream_t st) {
-    if (I::template cn_short<AXIS, true>(a, ga, n, reduce, renorm, st)) return;
-    // one resident wave for the whole group: each member's share of the persistent CTAs,
-    // so that every CTA stages the factor tables once for many tiles and prefetches
-    dim3 g = I::grid_cn(a, AXIS);
-    g.x = g.x / n < 1 ? 1 : g.x / n;
-    g.z = n;
-    const size_t sm = I::smem_cn(I::cn_len(a, AXIS), a.cn[AXIS].lchunk);
-    if (I::cn_full(a, AXIS))
-      k_cn<R, Co, AXIS, T::kCnCols, I::template cn_full_threads<AXIS>(), true, true><<<g, I::template cn_full_threads<AXIS>(), sm, st>>>(a, ga, reduce, renorm);
-    else
-      k_cn<R, Co, AXIS, T::kCnCols, T::kCnThreads, true><<<g, T::kCnThreads, sm, st>>>(a, ga, reduce, renorm);
   }
   static cudaError_t step(const KArgs &a, const KArgs *ga, int count, int renorm, cudaStream_t st) {
     if (count < 1 || count > 65535) return cudaErrorInvalidValue;
@@ -3781,15 +3718,10 @@ struct GroupLaunch {
     ffty<-1>(a, ga, n, st);
     k3(a, ga, n, st);
     ffty<+1>(a, ga, n, st);
-    if (a.imag) {
-      k5<R>(a, ga, n, st);
-      cn<R, 1>(a, ga, n, 0, 0, st);
-      cn<R, 0>(a, ga, n, 1, renorm, st);
-    } else {
-      k5<C>(a, ga, n, st);
-      cn<C, 1>(a, ga, n, 0, 0, st);
-      cn<C, 0>(a, ga, n, 1, renorm, st);
-    }
+    if (a.imag) k5<R>(a, ga, n, st);
+    else k5<C>(a, ga, n, st);
+    I::template cn_reg<1, true>(a, ga, n, 0, 0, st);
+    I::template cn_reg<0, true>(a, ga, n, 1, renorm, st);
     return cudaGetLastError();
   }
 };

@@ -33,17 +33,15 @@ struct CnJob {
   void *tab;
   int m, chunk;
   double r;    // dt / (4 h^2), negated for the adjoint tables
-  int lanes;   // lanes per line of the layout: 32, or 8 (the short-line sweeps)
+  int lanes;   // lanes per line of the layout: 32, or 8 (K5's z solve of short lines)
 };
-constexpr int kMaxCnJobs = 12;
+constexpr int kMaxCnJobs = 12;   // forward, differentiation and adjoint per axis, two for K5's z solve
 
-// FP32 sweeps of short lines: n = 8 CH points (CH = 4, 6, 8, 12 or 16) are solved on 8 lanes
-// per line, CH points each; 0 where the line takes the 32-lane solver.
-__host__ __device__ constexpr int short_cn_chunk(int n) {
-  return (n == 32 || n == 48 || n == 64 || n == 96 || n == 128) ? n / 8 : 0;
-}
 // FP32 compile-time K5 lengths whose z solve runs on 8 lanes per line (8-lane z tables)
 __host__ __device__ constexpr bool k5_short_z(int n) { return n == 64 || n == 96 || n == 128; }
+
+// FP32 x and y sweeps: columns per tile at q chunks per line (CTAs of up to 256 threads)
+__host__ __device__ constexpr int cnr_cols(int q) { return q > 16 ? 8 : q > 8 ? 16 : q > 4 ? 32 : 64; }
 
 // Interior points per lane of K5's z solve at a compile-time length n: the least chunk with
 // 32 chunks covering the n - 2 unknowns (12 for n = 384; the sweeps' power of two for 128,
@@ -58,8 +56,8 @@ struct CnJobs {
 struct CnTab {
   const void *tab;
   int m;
-  int chunk;    // interior points per lane, a power of two
-  int lchunk;   // log2(chunk)
+  int chunk;    // interior points per lane, a power of two (FP32 x and y sweeps: per thread, 12 or 16; 2 to 16 in the differentiation calls)
+  int lchunk;   // log2(chunk), of a power of two
 };
 
 // Device-resident solver state (lives in the workspace).
@@ -111,8 +109,7 @@ struct KArgs {
   CnTab cn[3];
   const void *cnz_tab;         // K5's z tables at k5_chunk(nz) points per lane, where that is not
                                // cn[2].chunk (FP32, compile-time nz); else null
-  const void *cn8_tab[3];      // tables in the 8-lane layout: the x and y sweeps' (FP32 lines of
-                               // short_cn_chunk(n) != 0) and K5's z solve (FP32, k5_short_z(nz)); else null
+  const void *cn8z_tab;        // K5's z tables in the 8-lane layout (FP32, k5_short_z(nz)); else null
   void *out;                   // optional output (Phi for get_phi)
   // adjoint step
   void *gbar;                  // cotangent field (same layout as psi)
@@ -122,7 +119,7 @@ struct KArgs {
   // launch shapes (defaults set at create; dgpe_autotune may change them)
   int ylines;                  // K2/K4 lines per CTA (power of two, <= 32)
   int fft_threads;             // K2/K3/K4 threads per CTA (128 or 256)
-  int cn_per_sm;               // K6/K7 persistent CTAs per SM (1 or 2; capped by shared memory)
+  int cn_per_sm;               // K6/K7 (FP32): persistent threads per SM in units of 256 (1 or 2)
   int nsm;                     // SMs of the device: the FP32 tile kernels prefetch into L2 the tile of
                                // the CTA one resident wave ahead (residency x nsm; 0: no prefetch)
 };

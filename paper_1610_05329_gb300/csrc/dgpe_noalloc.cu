@@ -88,7 +88,9 @@ __global__ void __launch_bounds__(kNoAllocThreads)
     v[2] += y * y * t;
     v[3] += quad_weight(i, nx, simpson) * quad_weight(j, ny, simpson) * sz;
   }
-  if (reduce_across_blocks<4>(v, scr->partials, &scr->ticket) && threadIdx.x == 0) {
+  double sum[4];
+  if (reduce_across_blocks<4>(v, sum, scr->partials, &scr->ticket) && threadIdx.x == 0) {
+    for (int q = 0; q < 4; ++q) v[q] = sum[q];
     out[0] = hx * hy * hz * v[0];
     out[1] = sqrt(v[1] / v[0]);
     out[2] = sqrt(v[2] / v[0]);
