@@ -146,7 +146,7 @@ int check_physics(const dgpe_params *p) {
 }
 
 struct Layout {
-  size_t state, partials, tw[3], cn[3], cn_diff[2], cn_adj[3], cnz, cn8z, dtv[3], psi, spec, utab, ybuf, total;
+  size_t state, partials, tw[3], tw_st[2], cn[3], cn_diff[2], cn_adj[3], cnz, cn8z, dtv[3], psi, spec, utab, ybuf, total;
 };
 
 // FP32 contexts whose compile-time K5 (nz = 128, 256, 384, 512) solves along z at a chunk
@@ -169,6 +169,10 @@ Layout layout_of(const dgpe_params *p, const KernelSet *ks, int max_blocks) {
   for (int d = 0; d < 3; ++d) {
     L.tw[d] = off;
     off += align_up((size_t)n[d] * e);
+  }
+  for (int d = 0; d < 2; ++d) {   // the staged x and y transforms' twiddles (FP32)
+    L.tw_st[d] = off;
+    if (p->precision == DGPE_MIXED) off += align_up(2 * (size_t)n[d] * e);
   }
   for (int d = 0; d < 3; ++d) {
     L.cn[d] = off;
@@ -419,11 +423,13 @@ int diff_axis_chunk(const dgpe_ctx *c, int d);
 // tables are those of the differentiation calls.
 KArgs step_args(dgpe_ctx *c) {
   KArgs a = c->args;
-  if (c->p.precision == DGPE_MIXED && !c->restore_norm)
+  if (c->p.precision == DGPE_MIXED && !c->restore_norm) {
+    a.diff = 1;
     for (int d = 0; d < 2; ++d) {
       a.cn[d].tab = at(c, c->L.cn_diff[d]);
       a.cn[d].chunk = diff_axis_chunk(c, d);
     }
+  }
   return a;
 }
 
@@ -542,6 +548,7 @@ namespace {
 KArgs adjoint_sweep_args(dgpe_ctx *c, void *gbar) {
   KArgs a = c->args;
   a.psi = gbar;
+  a.diff = 1;
   for (int d = 0; d < 3; ++d) {
     a.cn[d].tab = at(c, c->L.cn_adj[d]);
     a.cn[d].chunk = diff_axis_chunk(c, d);
@@ -566,6 +573,7 @@ int enqueue_adjoint_step(dgpe_ctx *c, const void *psi_k, void *gbar, double *nu_
   fa.psi = const_cast<void *>(psi_k);
   fa.gbar = gbar;
   fa.unit_scale = 1;
+  fa.diff = 1;
   fa.grad_nu_slot = nu_slot;
   if ((rc = launch(c, st, kK1DensityR2Cz, [&] { return ks->k1(fa, st); }))) return rc;
   if ((rc = launch(c, st, kK2FftY, [&] { return ks->k2(fa, st); }))) return rc;
@@ -727,6 +735,7 @@ int dgpe_create(const dgpe_params *p, void *cuda_stream, dgpe_ctx **out) {
       c->args.nsm = nsm;
   }
   rc = map_cuda(c->ks->init());
+  if (!rc && p->precision == DGPE_MIXED) rc = map_cuda(stage_init(p->nx, p->ny));
   if (!rc) rc = map_cuda(cudaStreamCreateWithFlags(&c->cap_stream, cudaStreamNonBlocking));
   if (!rc) {
     if (p->workspace) {
@@ -760,7 +769,10 @@ int dgpe_create(const dgpe_params *p, void *cuda_stream, dgpe_ctx **out) {
   rc = map_cuda(cudaMemsetAsync(a.psi, 0, (size_t)p->nx * p->ny * p->nz * c->ks->elem_bytes, c->stream));
   if (!rc) rc = map_cuda(c->ks->reset_state(a.state, c->stream));
   for (int d = 0; d < 3 && !rc; ++d) rc = map_cuda(c->ks->twiddles(const_cast<void *>(a.tw[d]), a.plan[d], c->stream));
-  (void)n;
+  for (int d = 0; d < 2 && !rc && p->precision == DGPE_MIXED; ++d) {
+    a.tw_st[d] = at(c, c->L.tw_st[d]);
+    rc = map_cuda(stage_tables(const_cast<void *>(a.tw_st[d]), n[d], c->stream));
+  }
   if (!rc) rc = setup_tables(c, true, true);
   if (rc) {
     dgpe_destroy(c);

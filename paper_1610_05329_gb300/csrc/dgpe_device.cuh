@@ -3347,6 +3347,9 @@ struct Impl {
   static bool y_fixed(const KArgs &a, int n) {
     return a.ylines == y_lines_per_cta<R>(n) && a.fft_threads == kFftThreads && plan_ct(a.plan[1], n);
   }
+  // the staged FP32 transforms: where the radix order is the default one, outside the
+  // differentiation calls
+  static bool staged(const KArgs &a, int d) { return !a.diff && plan_ct(a.plan[d], d == 0 ? a.nx : a.ny); }
   // the register-resident FP32 transforms (default plans of length 128, 256, 512)
   static constexpr bool kRegFft = std::is_same<R, float>::value;
   static constexpr size_t kRegYSmem = 2 * (256 / 64) * (size_t)RegFft<512>::SLOTS * sizeof(cplx<float>);
@@ -3368,6 +3371,7 @@ struct Impl {
       if (plan_ct(a.plan[1], 512)) return ffty_reg<DIR, 512>(a, st), cudaGetLastError();
       if (plan_ct(a.plan[1], 256)) return ffty_reg<DIR, 256>(a, st), cudaGetLastError();
       if (plan_ct(a.plan[1], 128)) return ffty_reg<DIR, 128>(a, st), cudaGetLastError();
+      if (staged(a, 1) && stage_y(DIR, a, nullptr, 1, st)) return cudaGetLastError();
     }
     const size_t lines = (size_t)a.nzh * a.nx;
     const int L = a.ylines;
@@ -3390,6 +3394,7 @@ struct Impl {
       if (plan_ct(a.plan[0], 512)) return k3_reg_launch<512>(a, st), cudaGetLastError();
       if (plan_ct(a.plan[0], 256)) return k3_reg_launch<256>(a, st), cudaGetLastError();
       if (plan_ct(a.plan[0], 128)) return k3_reg_launch<128>(a, st), cudaGetLastError();
+      if (staged(a, 0) && stage_x(a, nullptr, 1, st)) return cudaGetLastError();
     }
     dim3 grid((a.ny + T::kXCols - 1) / T::kXCols, a.nzh);
     const size_t sm = smem_x(a);
@@ -3656,6 +3661,7 @@ struct GroupLaunch {
     if (I::plan_ct(a.plan[1], 512)) return reg(std::integral_constant<int, 512>{});
     if (I::plan_ct(a.plan[1], 256)) return reg(std::integral_constant<int, 256>{});
     if (I::plan_ct(a.plan[1], 128)) return reg(std::integral_constant<int, 128>{});
+    if (I::staged(a, 1) && stage_y(DIR, a, ga, n, st)) return;
     const int L = a.ylines;
     const dim3 g((unsigned)((lines + L - 1) / L), 1, n);
     const size_t sm = I::smem_y(a);
@@ -3670,6 +3676,7 @@ struct GroupLaunch {
     if (I::plan_ct(a.plan[0], 512)) return reg(std::integral_constant<int, 512>{});
     if (I::plan_ct(a.plan[0], 256)) return reg(std::integral_constant<int, 256>{});
     if (I::plan_ct(a.plan[0], 128)) return reg(std::integral_constant<int, 128>{});
+    if (I::staged(a, 0) && stage_x(a, ga, n, st)) return;
     const dim3 g((a.ny + T::kXCols - 1) / T::kXCols, a.nzh, n);
     const size_t sm = I::smem_x(a);
     if (a.fft_threads == kFftThreads && I::plan_ct(a.plan[0], 384))

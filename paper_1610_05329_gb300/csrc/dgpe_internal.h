@@ -104,6 +104,9 @@ struct KArgs {
   float kf[3];                 // 2 pi / (n_d h_d): wavenumber per frequency index (FP32 K3)
   DevState *state;
   double *partials;            // per-block reduction partials
+  const void *tw_st[2];        // twiddles of the staged FP32 x and y transforms (layout in dgpe_stages.cuh)
+  int diff;                    // 1: within the differentiation calls (FP32: the transforms and chunks whose
+                               // roundings their results rest on)
   const void *tw[3];           // per-stage twiddle tables of plan[d] (layout in FftPlan), d = x, y, z
   FftPlan plan[3];
   CnTab cn[3];
@@ -186,6 +189,37 @@ struct KernelSet {
   cudaError_t (*init_group)();
   cudaError_t (*step_group)(const KArgs &a, const KArgs *ga, int n, int renorm, cudaStream_t st);
 };
+
+// The staged FP32 transforms of the general line lengths (dgpe_stages.cuh), the lengths spread
+// over four translation units: y transforms (dir = -1, +1) and x transforms with the dipolar
+// kernel for `members` condensates (ga their arguments in device memory, or null for one); false
+// where the unit has no kernel of that length.
+#define DGPE_STAGE_UNIT(i)                                                                              \
+  bool stage_y##i(int dir, const KArgs &a, const KArgs *ga, unsigned members, cudaStream_t st);         \
+  bool stage_x##i(const KArgs &a, const KArgs *ga, unsigned members, cudaStream_t st);                  \
+  cudaError_t stage_init##i(int nx, int ny);
+DGPE_STAGE_UNIT(0)
+DGPE_STAGE_UNIT(1)
+DGPE_STAGE_UNIT(2)
+DGPE_STAGE_UNIT(3)
+#undef DGPE_STAGE_UNIT
+inline bool stage_y(int dir, const KArgs &a, const KArgs *ga, unsigned members, cudaStream_t st) {
+  return stage_y0(dir, a, ga, members, st) || stage_y1(dir, a, ga, members, st) ||
+         stage_y2(dir, a, ga, members, st) || stage_y3(dir, a, ga, members, st);
+}
+inline bool stage_x(const KArgs &a, const KArgs *ga, unsigned members, cudaStream_t st) {
+  return stage_x0(a, ga, members, st) || stage_x1(a, ga, members, st) || stage_x2(a, ga, members, st) ||
+         stage_x3(a, ga, members, st);
+}
+inline cudaError_t stage_init(int nx, int ny) {
+  cudaError_t e = stage_init0(nx, ny);
+  if (e == cudaSuccess) e = stage_init1(nx, ny);
+  if (e == cudaSuccess) e = stage_init2(nx, ny);
+  if (e == cudaSuccess) e = stage_init3(nx, ny);
+  return e;
+}
+// the twiddles of length n (2 n values; nothing where n has no staged transform)
+cudaError_t stage_tables(void *tw, int n, cudaStream_t st);
 
 cudaError_t group_init_f32();
 cudaError_t group_step_f32(const KArgs &a, const KArgs *ga, int n, int renorm, cudaStream_t st);

@@ -10,6 +10,7 @@
 // without ordering between them) race on it and give wrong results.
 #include <cuda_runtime.h>
 #include <math.h>
+#include <stdint.h>
 
 #include <algorithm>
 #include <mutex>
@@ -98,6 +99,210 @@ __global__ void __launch_bounds__(kNoAllocThreads)
   }
 }
 
+// FP32 data.  The kernel above spends six to eight FP64-pipe instructions per point (two
+// conversions among them; GB300 issues 2 per clock per SM): 1.42 ms at 512x512x384 against 0.12 ms
+// of HBM time.  Here the densities and the weighted sums of a warp's lines are FP32 pairs:
+//   - each lane's points are scaled by a power of two taken from the largest of them, so no
+//     square leaves the FP32 range and what underflows is below 2^-100 of the sum;
+//   - re^2 + im^2 is exact to 2^-48 (FMA residuals of both squares and of their sum);
+//   - the weights are exact integers (3 x the quadrature weights, squared signed indices), their
+//     products by the density carry the FMA residual, the sums are TwoSums, renormalised line
+//     by line; a warp passes its pairs on to FP64 once per unit of up to 8 lines
+//     (or where the x index or the scale changes).
+// The result is as near to extended-precision sums as the FP64 kernel's (1e-16).  Lanes that meet an infinity or a NaN take those points in FP64.  Bound by FP32 issue (about 40
+// instructions per point): 1.42 -> 0.245 ms at 512x512x384 (0.49 of HBM).
+constexpr int kMomentPairs = 4;   // pairs of points in a lane's registers
+
+// a + b, |a| >= |b| or a = 0
+__device__ __forceinline__ void renorm(DFAcc &a) {
+  const float t = __fadd_rn(a.hi, a.lo);
+  a.lo = __fsub_rn(a.lo, __fsub_rn(t, a.hi));
+  a.hi = t;
+}
+// a += w (h + l), exactly up to the rounding of the low part
+__device__ __forceinline__ void add_weighted(DFAcc &a, float w, float h, float l) {
+  const float p = __fmul_rn(w, h);
+  const float e = __fmaf_rn(w, l, __fmaf_rn(w, h, -p));
+  a.add(p);
+  a.lo = __fadd_rn(a.lo, e);
+}
+
+template <bool WIDE>
+__global__ void __launch_bounds__(kNoAllocThreads, 3)
+    k_moments_f32(const float2 *__restrict__ psi, int nx, int ny, int nz, double hx, double hy, double hz, int simpson,
+                  int lines_per_unit, NoAllocScratch *scr, double *out) {
+  __shared__ float4 wz[kNoAllocMaxN / 2];   // W and W k'^2 of two consecutive points
+  for (int p = threadIdx.x; p < nz / 2; p += blockDim.x) {
+    const int k0 = 2 * p - nz / 2, k1 = k0 + 1;
+    const float w0 = (float)quad_weight3(2 * p, nz, simpson), w1 = (float)quad_weight3(2 * p + 1, nz, simpson);
+    wz[p] = make_float4(w0, w0 * (float)(k0 * k0), w1, w1 * (float)(k1 * k1));
+  }
+  __syncthreads();
+  const int lane = threadIdx.x & (kWarp - 1), np = nz / 2;
+  const int nlines = nx * ny;
+  const int nwarps = gridDim.x * (blockDim.x / kWarp);
+  const int nunits = (nlines + lines_per_unit - 1) / lines_per_unit;
+  double v[4] = {0.0, 0.0, 0.0, 0.0};   // sums of W n, i'^2 W n, j'^2 W n, k'^2 W n
+  // the pairs of one run of lines of equal x index, over 2^-2(sb - 127)
+  DFAcc s0, sy, sz;
+  int sb = 0;   // 0: empty
+  auto flush = [&](int i) {
+    if (!sb) return;
+    const double un = __hiloint2double((1023 - 2 * (sb - 127)) << 20, 0);
+    const int ii = i - nx / 2;
+    const double wx = (double)quad_weight3(i, nx, simpson) * un;
+    const double t = wx * s0.value();
+    v[0] += t;
+    v[1] = fma((double)(ii * ii), t, v[1]);
+    v[2] = fma(wx, sy.value(), v[2]);
+    v[3] = fma(wx, sz.value(), v[3]);
+    s0 = sy = sz = DFAcc{};
+    sb = 0;
+  };
+  auto load = [&](int l, int p0, float4 (&c)[kMomentPairs]) {
+#pragma unroll
+    for (int u = 0; u < kMomentPairs; ++u) {
+      const int p = p0 + u * kWarp + lane;
+      if (p < np) {
+        const float2 *q = psi + (size_t)l * nz + 2 * p;
+        if constexpr (WIDE) {
+          c[u] = __ldg(reinterpret_cast<const float4 *>(q));
+        } else {
+          const float2 a = __ldg(q), b = __ldg(q + 1);
+          c[u] = make_float4(a.x, a.y, b.x, b.y);
+        }
+      } else {
+        c[u] = make_float4(0.f, 0.f, 0.f, 0.f);
+      }
+    }
+  };
+  for (int unit = blockIdx.x * (blockDim.x / kWarp) + threadIdx.x / kWarp; unit < nunits; unit += nwarps) {
+    const int l0 = unit * lines_per_unit, l1 = min(nlines, l0 + lines_per_unit);
+    int i = l0 / ny, j = l0 - i * ny;
+    float4 c[kMomentPairs], nxt[kMomentPairs];
+    load(l0, 0, nxt);
+    for (int l = l0; l < l1; ++l) {
+      const float wy = (float)quad_weight3(j, ny, simpson);
+      const int jj = j - ny / 2;
+      DFAcc t0, tz;   // this line's sums
+      for (int p0 = 0; p0 < np; p0 += kMomentPairs * kWarp) {
+#pragma unroll
+        for (int u = 0; u < kMomentPairs; ++u) c[u] = nxt[u];
+        // the next points of the line, or the next line's first
+        if (p0 + kMomentPairs * kWarp < np) load(l, p0 + kMomentPairs * kWarp, nxt);
+        else if (l + 1 < l1) load(l + 1, 0, nxt);
+        unsigned m = 0u;   // twice the bits of the largest magnitude
+#pragma unroll
+        for (int u = 0; u < kMomentPairs; ++u)
+          m = max(max(m, max(__float_as_uint(c[u].x) << 1, __float_as_uint(c[u].y) << 1)),
+                  max(__float_as_uint(c[u].z) << 1, __float_as_uint(c[u].w) << 1));
+        if (m == 0u) continue;
+        const int e = (int)(m >> 24);
+        if (e == 255) {   // an infinity or a NaN: in FP64
+          const int ii = i - nx / 2;
+          const double wxy = (double)(quad_weight3(i, nx, simpson) * quad_weight3(j, ny, simpson));
+#pragma unroll 1
+          for (int u = 0; u < 2 * kMomentPairs; ++u) {
+            const int p = p0 + (u >> 1) * kWarp + lane;
+            if (p >= np) break;
+            const float2 z = psi[(size_t)l * nz + 2 * p + (u & 1)];
+            const int k = 2 * p + (u & 1), kk = k - nz / 2;
+            const double t = wxy * quad_weight3(k, nz, simpson) * ((double)z.x * z.x + (double)z.y * z.y);
+            v[0] += t;
+            v[1] += (double)(ii * ii) * t;
+            v[2] += (double)(jj * jj) * t;
+            v[3] += (double)(kk * kk) * t;
+          }
+          continue;
+        }
+        // scale 2^(sb - 127): the largest magnitude of the run so far in [1, 2), later ones up to
+        // 2^20 larger before the run is passed on
+        const int want = max(254 - e, 1);
+        if (!sb || want < sb - 20) {
+          // the sums of the lines before stay at the old scale: pass them and this line's on
+          s0.add(__fmul_rn(wy, t0.hi));
+          s0.lo = __fadd_rn(s0.lo, __fmul_rn(wy, t0.lo));
+          add_weighted(sy, wy * (float)(jj * jj), t0.hi, t0.lo);
+          add_weighted(sz, wy, tz.hi, tz.lo);
+          t0 = tz = DFAcc{};
+          flush(i);
+          sb = want;
+        }
+        const float sc = __int_as_float(sb << 23);
+#pragma unroll
+        for (int u = 0; u < kMomentPairs; ++u) {
+          const int p = p0 + u * kWarp + lane;
+          const float4 w = wz[min(p, np - 1)];   // (past the line's end the density is zero)
+#pragma unroll
+          for (int h = 0; h < 2; ++h) {
+            const float re = __fmul_rn(h ? c[u].z : c[u].x, sc), im = __fmul_rn(h ? c[u].w : c[u].y, sc);
+            const float a = __fmul_rn(re, re), b = __fmul_rn(im, im);
+            DFAcc d;
+            d.hi = a;
+            d.lo = __fadd_rn(__fmaf_rn(re, re, -a), __fmaf_rn(im, im, -b));
+            d.add(b);
+            const float w0 = h ? w.z : w.x, w2 = h ? w.w : w.y;
+            t0.add(__fmul_rn(w0, d.hi));
+            t0.lo = __fmaf_rn(w0, d.lo, t0.lo);
+            add_weighted(tz, w2, d.hi, d.lo);
+          }
+        }
+      }
+      renorm(t0);
+      renorm(tz);
+      s0.add(__fmul_rn(wy, t0.hi));   // exact: W_y is 0, 1, 2 or 4
+      s0.lo = __fmaf_rn(wy, t0.lo, s0.lo);
+      add_weighted(sy, wy * (float)(jj * jj), t0.hi, t0.lo);
+      add_weighted(sz, wy, tz.hi, tz.lo);
+      renorm(s0);
+      renorm(sy);
+      renorm(sz);
+      if (++j == ny) {
+        flush(i);
+        j = 0;
+        ++i;
+      }
+    }
+    if (j) flush(i);
+  }
+  double sum[4];
+  if (reduce_across_blocks<4>(v, sum, scr->partials, &scr->ticket) && threadIdx.x == 0) {
+    // the factors with their rounding errors carried along, so that the results keep the
+    // sums' own accuracy: norm = hx hy hz sum / 27 (the integer Simpson weights' (1/3)^3) ...
+    const double a = hx * hy, b = a * hz, c = b * sum[0];
+    const double eb = fma(a, hz, -b) + fma(hx, hy, -a) * hz, ec = fma(b, sum[0], -c) + eb * sum[0];
+    const double q = c / (simpson ? 27.0 : 1.0);
+    out[0] = isfinite(c) ? q + (fma(-q, simpson ? 27.0 : 1.0, c) + ec) / (simpson ? 27.0 : 1.0) : c;
+    // ... and rms_d = h_d sqrt(sum_d / sum)
+    const double h[3] = {hx, hy, hz};
+    for (int d = 0; d < 3; ++d) {
+      const double r = sum[1 + d] / sum[0], t = sqrt(r), u = h[d] * t;
+      out[1 + d] = t > 0.0 ? u + (fma(h[d], t, -u) + h[d] * (fma(-t, t, r) / (2.0 * t))) : u;
+    }
+  }
+}
+
+// One resident wave of CTAs (three of 256 threads per SM); a warp takes up to 8 lines at a time,
+// fewer where that leaves warps without work.
+int moments_f32(const void *psi, const dgpe_params *p, int simpson, long long nlines, NoAllocScratch *scr, double *out,
+                cudaStream_t st) {
+  int dev = 0, nsm = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess ||
+      cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || nsm < 1)
+    return DGPE_ECUDA;
+  const long long warps = (long long)nsm * 3 * (kNoAllocThreads / kWarp);
+  const int lines = (int)std::max<long long>(1, std::min<long long>(8, nlines / (warps * 4)));
+  const long long units = (nlines + lines - 1) / lines, per_block = kNoAllocThreads / kWarp;
+  const unsigned blocks = (unsigned)std::min<long long>((units + per_block - 1) / per_block,
+                                                        std::min<long long>(nsm * 3, kNoAllocMaxBlocks));
+  const float2 *q = static_cast<const float2 *>(psi);
+  if (reinterpret_cast<uintptr_t>(psi) % 16 == 0)
+    k_moments_f32<true><<<blocks, kNoAllocThreads, 0, st>>>(q, p->nx, p->ny, p->nz, p->hx, p->hy, p->hz, simpson, lines, scr, out);
+  else   // (8-byte aligned)
+    k_moments_f32<false><<<blocks, kNoAllocThreads, 0, st>>>(q, p->nx, p->ny, p->nz, p->hx, p->hy, p->hz, simpson, lines, scr, out);
+  return cudaGetLastError() == cudaSuccess ? DGPE_OK : DGPE_ECUDA;
+}
+
 }  // namespace
 
 extern "C" int dgpe_moments_noalloc(const void *psi, const dgpe_params *p, double *out, void *cuda_stream) {
@@ -123,6 +328,11 @@ extern "C" int dgpe_moments_noalloc(const void *psi, const dgpe_params *p, doubl
     k_moments_noalloc<double><<<blocks, kNoAllocThreads, 0, st>>>(static_cast<const cplx<double> *>(psi), p->nx,
                                                                   p->ny, p->nz, p->hx, p->hy, p->hz, simpson,
                                                                   scr, out);
+  // FP32 pairs where the time is the arithmetic's.  Below 2^17 points the FP64 kernel takes under
+  // 2 us of its pipe, and the pairs' rounding (2^-48 a point) does not yet average out below the
+  // FP64 sums' own.  Odd lines have no pairs of points.
+  else if (p->nz % 2 == 0 && nlines * p->nz >= (1 << 17))
+    return moments_f32(psi, p, simpson, nlines, scr, out, st);
   else
     k_moments_noalloc<float><<<blocks, kNoAllocThreads, 0, st>>>(static_cast<const cplx<float> *>(psi), p->nx,
                                                                  p->ny, p->nz, p->hx, p->hy, p->hz, simpson,

@@ -74,3 +74,89 @@ def test_adjoint_cotangent_of_any_alignment():
     gpu.adjoint_step(psi, odd)
     assert torch.equal(a.reshape(-1), odd)
     gpu.close()
+
+
+def exact_moments(psi, h, simpson):
+    """norm and rms in extended precision (64 or 113 bits)."""
+    L = np.longdouble
+    n = psi.shape
+    dens = psi.real.astype(L) ** 2 + psi.imag.astype(L) ** 2
+    w, x2 = [], []
+    for d in range(3):
+        q = np.ones(n[d], dtype=L)
+        if simpson:
+            q[1::2], q[::2] = L(4) / 3, L(2) / 3
+            q[0] = q[n[d] - 2] = L(1) / 3
+            q[n[d] - 1] = 0
+        w.append(q)
+        x2.append(((np.arange(n[d]) - n[d] // 2).astype(L) * L(h[d])) ** 2)
+    dens = dens * w[0][:, None, None] * w[1][None, :, None] * w[2][None, None, :]
+    tot = dens.sum()
+    rms = [np.sqrt((dens.sum(axis=tuple(k for k in range(3) if k != d)) * x2[d]).sum() / tot) for d in range(3)]
+    return np.array([L(h[0]) * L(h[1]) * L(h[2]) * tot, *rms], dtype=L)
+
+
+def moments(psi_d, shape, h, simpson):
+    import torch
+    out = torch.zeros(4, dtype=torch.float64, device="cuda")
+    params = abi.make_params(shape, h, 0.01, precision=abi.DGPE_MIXED,
+                             integration=abi.DGPE_SIMPSON if simpson else abi.DGPE_RECTANGLE)
+    abi.dgpe_moments_noalloc(psi_d.data_ptr(), params, out.data_ptr(), torch.cuda.current_stream().cuda_stream)
+    return out.cpu().numpy()
+
+
+@pytest.mark.parametrize("shape", [(2, 3, 2), (5, 4, 24), (7, 9, 62), (6, 40, 250), (33, 17, 258), (40, 41, 512), (3, 4, 5),
+                                   (64, 64, 64), (3, 400, 250), (300, 5, 100), (100, 90, 24), (64, 512, 4)])
+@pytest.mark.parametrize("simpson", [False, True])
+@pytest.mark.parametrize("scale", [1.0, 1e-24, 1e17])
+def test_moments_of_fp32_states(shape, simpson, scale):
+    """The FP32 moments call is an FP64-quality sum: within 2e-15 (a few roundings of 1.1e-16 in
+    the totals, the quotient and the root) of extended precision, also where the squares leave
+    the FP32 range and where the field spans many powers of ten."""
+    import torch
+    h = (0.3, 0.25, 0.2)
+    psi = (inputs.random_psi(shape, seed=11) * scale).astype(np.complex64)
+    decay = np.exp(-np.linspace(0.0, 60.0, shape[0] * shape[1]).reshape(shape[0], shape[1], 1))
+    for field in (psi, (psi * decay).astype(np.complex64), (psi * decay[::-1, ::-1]).astype(np.complex64)):
+        dev = torch.from_numpy(np.ascontiguousarray(field)).cuda()
+        odd = torch.empty(dev.numel() + 1, dtype=dev.dtype, device="cuda")[1:]
+        odd.copy_(dev.reshape(-1))
+        want = exact_moments(field, h, simpson)
+        for t in (dev, odd):   # 16- and 8-byte aligned
+            got = moments(t, shape, h, simpson)
+            if simpson and want[0] == 0:
+                continue
+            assert np.all(np.abs(got - want) <= 2e-15 * np.abs(want)), (got - want) / want
+
+
+def test_moments_of_nonfinite_states():
+    import torch
+    shape, h = (64, 48, 64), (0.3, 0.25, 0.2)
+    psi = inputs.random_psi(shape, seed=2).astype(np.complex64)
+    for bad in (np.inf, np.nan):
+        field = psi.copy()
+        field[3, 4, 17] = bad
+        got = moments(torch.from_numpy(field).cuda(), shape, h, False)
+        assert (np.isinf(got[0]) if np.isinf(bad) else np.isnan(got[0])) and np.all(np.isnan(got[1:]))
+
+
+# every supported length, as the x axis of one grid and the y axis of another
+ALL = [n for n in range(4, 513, 2)
+       if any(n == 2 ** a * 3 ** b * 5 ** c * 7 ** d
+              for a in range(1, 10) for b in range(6) for c in range(4) for d in range(4))]
+
+
+@pytest.mark.parametrize("nx,ny", list(zip(ALL, reversed(ALL))))
+def test_dipolar_potential_of_every_length(orc, nx, ny):
+    """Phi through the x and y transforms of every length.  An FP32 transform's error is a few
+    6e-8 per stage of the field's norm (at most five stages, four transforms): 3e-6."""
+    shape = (nx, ny, 6)
+    h = (9.0 / nx, 8.0 / ny, 1.1)
+    psi = (inputs.random_psi(shape, seed=nx) * 0.3).astype(np.complex64)
+    for cutoff in (0.0, 3.0):
+        gpu = abi.Condensate(shape, h, 0.01, precision=abi.DGPE_MIXED, g=1.0, gdd=1.0, cutoff=cutoff)
+        p = orc.make_params(shape, h, 0.01, orc.IMAG_TIME, (1.0, 1.0, 1.0), 1.0, 1.0, cutoff=cutoff)
+        gpu.set_psi(psi)
+        got = gpu.phi()
+        gpu.close()
+        assert rel(got, orc.dipolar_phi(p, np.abs(psi.astype(np.complex128)) ** 2)) < 3e-6
