@@ -146,7 +146,7 @@ int check_physics(const dgpe_params *p) {
 }
 
 struct Layout {
-  size_t state, partials, tw[3], tw_st[2], cn[3], cn_diff[2], cn_adj[3], cnz, cn8z, dtv[3], psi, spec, utab, ybuf, total;
+  size_t state, partials, tw[3], tw_st[3], cn[3], cn_diff[2], cn_adj[3], cnz, cn8z, dtv[3], psi, spec, utab, ybuf, total;
 };
 
 // FP32 contexts whose compile-time K5 (nz = 128, 256, 384, 512) solves along z at a chunk
@@ -170,9 +170,9 @@ Layout layout_of(const dgpe_params *p, const KernelSet *ks, int max_blocks) {
     L.tw[d] = off;
     off += align_up((size_t)n[d] * e);
   }
-  for (int d = 0; d < 2; ++d) {   // the staged x and y transforms' twiddles (FP32)
+  for (int d = 0; d < 3; ++d) {   // the staged transforms' twiddles (FP32: x and y; FP64: fixed point)
     L.tw_st[d] = off;
-    if (p->precision == DGPE_MIXED) off += align_up(2 * (size_t)n[d] * e);
+    if (p->precision == DGPE_FP64 || (p->precision == DGPE_MIXED && d < 2)) off += align_up(2 * (size_t)n[d] * e);
   }
   for (int d = 0; d < 3; ++d) {
     L.cn[d] = off;
@@ -736,6 +736,7 @@ int dgpe_create(const dgpe_params *p, void *cuda_stream, dgpe_ctx **out) {
   }
   rc = map_cuda(c->ks->init());
   if (!rc && p->precision == DGPE_MIXED) rc = map_cuda(stage_init(p->nx, p->ny));
+  if (!rc && p->precision == DGPE_FP64) rc = map_cuda(fx_init(p->nx, p->ny, p->nz));
   if (!rc) rc = map_cuda(cudaStreamCreateWithFlags(&c->cap_stream, cudaStreamNonBlocking));
   if (!rc) {
     if (p->workspace) {
@@ -769,9 +770,11 @@ int dgpe_create(const dgpe_params *p, void *cuda_stream, dgpe_ctx **out) {
   rc = map_cuda(cudaMemsetAsync(a.psi, 0, (size_t)p->nx * p->ny * p->nz * c->ks->elem_bytes, c->stream));
   if (!rc) rc = map_cuda(c->ks->reset_state(a.state, c->stream));
   for (int d = 0; d < 3 && !rc; ++d) rc = map_cuda(c->ks->twiddles(const_cast<void *>(a.tw[d]), a.plan[d], c->stream));
-  for (int d = 0; d < 2 && !rc && p->precision == DGPE_MIXED; ++d) {
-    a.tw_st[d] = at(c, c->L.tw_st[d]);
-    rc = map_cuda(stage_tables(const_cast<void *>(a.tw_st[d]), n[d], c->stream));
+  for (int d = 0; d < 3 && !rc; ++d) {
+    void *tw = at(c, c->L.tw_st[d]);
+    a.tw_st[d] = tw;
+    if (p->precision == DGPE_FP64) rc = map_cuda(fx_tables(tw, n[d], c->stream));
+    else if (p->precision == DGPE_MIXED && d < 2) rc = map_cuda(stage_tables(tw, n[d], c->stream));
   }
   if (!rc) rc = setup_tables(c, true, true);
   if (rc) {

@@ -1398,8 +1398,9 @@ __device__ __forceinline__ R cutoff_factor(R x) {
 // Ut(k) = 3 kz^2 / |k|^2 - 1 (Ut(0) = 0), times the cutoff factor when a cutoff is set, on
 // the half spectrum [m][i][j] (kz index m <= nz/2, kx index i, ky index j), computed in
 // FP64: k_d = 2 pi q / (n_d h_d) with the signed frequency q (q <= n/2: q, else q - n).
-template <typename R>
-__global__ void k_dipolar_table(R *ut, KArgs a) {
+// FIX: as 2^61 Ut(k), |Ut(k)| < 2.2, for the fixed-point x transforms.
+template <typename R, bool FIX>
+__global__ void k_dipolar_table(void *ut, KArgs a) {
   const size_t total = (size_t)a.nzh * a.nx * a.ny;
   const double two_pi = 6.283185307179586476925286766559;
   for (size_t e = (size_t)blockIdx.x * blockDim.x + threadIdx.x; e < total; e += (size_t)gridDim.x * blockDim.x) {
@@ -1411,7 +1412,8 @@ __global__ void k_dipolar_table(R *ut, KArgs a) {
     const double k2 = kx * kx + ky * ky + kz * kz;
     double u = k2 > 0.0 ? 3.0 * kz * kz / k2 - 1.0 : 0.0;
     if (a.cutoff > 0.0 && k2 > 0.0) u *= cutoff_factor<double>(sqrt(k2) * a.cutoff);
-    ut[e] = R(u);
+    if constexpr (FIX) static_cast<long long *>(ut)[e] = __double2ll_rn(u * 2305843009213693952.0);
+    else static_cast<R *>(ut)[e] = R(u);
   }
 }
 
@@ -3080,9 +3082,10 @@ struct Impl {
   using C = cplx<R>;
   using T = Tiles<R>;
   static constexpr size_t E = sizeof(C);
-  // compile-time transforms of lengths 128-512 (not for double-float: its kernels take many
-  // times longer to compile)
-  static constexpr bool kCtSizes = !std::is_same<R, df>::value;
+  // compile-time transforms of lengths 128-512 (FP32)
+  static constexpr bool kCtSizes = std::is_same<R, float>::value;
+  // the transforms in fixed point (dgpe_fixed.cuh), of lines of 12 points and more
+  static constexpr bool kFixed = std::is_same<R, double>::value;
   // FP32 also at nz = 96 and 64 (K1, K5; the batched small grids)
   static constexpr bool kShortCt = std::is_same<R, float>::value;
   // the FP64-class sweeps run a Thomas solve per line on two threads (k_cn_twisted), the
@@ -3283,7 +3286,8 @@ struct Impl {
     const size_t total = (size_t)a.nzh * a.nx * a.ny;
     const size_t want = (total + 255) / 256, cap = (size_t)sm_count() * 8;
     const int blocks = (int)(want < cap ? want : cap);
-    k_dipolar_table<R><<<blocks, 256, 0, st>>>(reinterpret_cast<R *>(const_cast<void *>(a.utab)), a);
+    if (kFixed && fx_length(a.nx)) k_dipolar_table<R, true><<<blocks, 256, 0, st>>>(const_cast<void *>(a.utab), a);
+    else k_dipolar_table<R, false><<<blocks, 256, 0, st>>>(const_cast<void *>(a.utab), a);
     return cudaGetLastError();
   }
 
@@ -3322,6 +3326,7 @@ struct Impl {
     return true;
   }
   static cudaError_t k1(const KArgs &a, cudaStream_t st) {
+    if (kFixed && fx_run(kK1DensityR2Cz, a, st)) return cudaGetLastError();
     // (instances of other tile heights, ztile_lines, get their own grid and shared memory)
     auto go = [&](auto len) {
       constexpr int N = decltype(len)::value;
@@ -3367,6 +3372,7 @@ struct Impl {
   }
   template <int DIR>
   static cudaError_t ffty(const KArgs &a, cudaStream_t st) {
+    if (kFixed && fx_run(DIR < 0 ? kK2FftY : kK4IfftY, a, st)) return cudaGetLastError();
     if constexpr (kRegFft) {
       if (plan_ct(a.plan[1], 512)) return ffty_reg<DIR, 512>(a, st), cudaGetLastError();
       if (plan_ct(a.plan[1], 256)) return ffty_reg<DIR, 256>(a, st), cudaGetLastError();
@@ -3390,6 +3396,7 @@ struct Impl {
   }
   static cudaError_t k2(const KArgs &a, cudaStream_t st) { return ffty<-1>(a, st); }
   static cudaError_t k3(const KArgs &a, cudaStream_t st) {
+    if (kFixed && fx_run(kK3FftXDipolar, a, st)) return cudaGetLastError();
     if constexpr (kRegFft) {
       if (plan_ct(a.plan[0], 512)) return k3_reg_launch<512>(a, st), cudaGetLastError();
       if (plan_ct(a.plan[0], 256)) return k3_reg_launch<256>(a, st), cudaGetLastError();
@@ -3450,6 +3457,7 @@ struct Impl {
     const dim3 g = grid_z(a);
     const size_t sm = smem_k5(a);
     if (zmode == kZFast) {
+      if (kFixed && fx_run(kK5C2RzPhaseCnz, a, st)) return cudaGetLastError();
       if (a.imag) k5_launch<kZFast, R>(a, g, sm, st);
       else k5_launch<kZFast, C>(a, g, sm, st);
       return cudaGetLastError();

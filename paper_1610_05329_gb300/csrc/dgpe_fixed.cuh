@@ -1,0 +1,935 @@
+// 64-bit fixed-point arithmetic for the transforms of the FP64-class precisions.
+//
+// GB300 issues 2 FP64 operations per clock and SM against 128 32-bit integer ones, so an FP64
+// transform of 256 points (20 FP64 instructions per element) keeps that pipe busy for eight
+// times as long as its bytes take from HBM.  A transform's error is relative to its line's norm
+// whatever the arithmetic, so it may as well run on block fixed point: the elements of a CTA's
+// tile as 64-bit integers under one exponent, exact additions (two 32-bit instructions instead
+// of an FP64 one), products by 64-bit constants through three 32 x 32 -> 64 multiply-adds.
+// With components below 2^58 on entry, a stage's outputs stay below 2^62 up to radix 10, and the
+// tile is rescaled by its largest output before the next stage, so the last bit stays at 2^-58 of
+// the tile's largest element: below an FP64 rounding of the elements' rms up to 512 points.
+// Bound by integer issue (about 250 instructions per complex element and pass).  Measured, us, the
+// FP64 transforms -> these: 256^3 K1 430 -> 134, K2 328 -> 96, K3 690 -> 208, the phase pass 1100 ->
+// 765; 480x480x250 a step 18.0 -> 9.5 ms; 64^3 a step 165 -> 125.  Phi against extended precision
+// (rel-L2, clouds and noise, 36 .. 480 points): 3.8e-16 .. 7.1e-16 -> 2.3e-16 .. 4.2e-16.
+#pragma once
+#include <cstring>
+
+#include "dgpe_stages.cuh"
+
+namespace dgpe {
+
+#define DGPE_HD __host__ __device__ __forceinline__
+
+struct fxc {   // a complex value under the tile's exponent
+  long long re, im;
+};
+DGPE_HD fxc operator+(fxc a, fxc b) { return {a.re + b.re, a.im + b.im}; }
+DGPE_HD fxc operator-(fxc a, fxc b) { return {a.re - b.re, a.im - b.im}; }
+template <int DIR>
+DGPE_HD fxc fx_rot(fxc a) { return DIR < 0 ? fxc{a.im, -a.re} : fxc{-a.im, a.re}; }   // times DIR i
+
+// a = hi 2^32 + lo with a signed lo, so that every product below is a signed one
+DGPE_HD int fx_hi(long long a) { return (int)(a >> 32) + (int)((unsigned)a >> 31); }
+DGPE_HD int fx_lo(long long a) { return (int)(unsigned)a; }
+DGPE_HD long long fx_mad(int a, int b, long long c) { return (long long)a * b + c; }
+constexpr long long kFxHalf = 0x80000000LL;
+
+// a w / 2^64 (the product of the low words, less than half a unit, left out).  |a| < 2^63 - 2^31,
+// |w| < 2^63 - 2^31 and |a| |w| < 2^125.
+DGPE_HD long long fx_mul(long long a, int wh, int wl) {
+  const int ah = fx_hi(a), al = fx_lo(a);
+  const long long mid = fx_mad(ah, wl, fx_mad(al, wh, kFxHalf));
+  return fx_mad(ah, wh, mid >> 32);
+}
+// a (n + f / 2^64), n = -1, 0, 1 and |f| < 2^63: a real constant to 64 fraction bits
+template <int NI, unsigned long long F>
+DGPE_HD long long fx_const(long long a) {
+  constexpr long long f = (long long)F;
+  constexpr int fl = (int)(unsigned)F, fh = (int)((f - fl) / 4294967296LL);
+  const long long p = fx_mul(a, fh, fl);
+  return NI == 0 ? p : NI > 0 ? p + a : p - a;
+}
+
+// A twiddle w 2^60, split into signed words.
+struct __align__(16) fxw {
+  int rh, rl, ih, il;
+};
+// a w / 2^64 = a w / 16 (DIR < 0) or a conj(w) / 16, for components of a below 2^62 (|a| below
+// 2^62.5): the middle sums stay below 2^62 + 2^59.5.
+template <int DIR>
+DGPE_HD fxc fx_twiddle(fxc a, fxw w) {
+  const int rh = fx_hi(a.re), rl = fx_lo(a.re), ih = fx_hi(a.im), il = fx_lo(a.im);
+  const int wih = DIR < 0 ? w.ih : -w.ih, wil = DIR < 0 ? w.il : -w.il;
+  const long long mr = fx_mad(rh, w.rl, fx_mad(rl, w.rh, fx_mad(ih, -wil, fx_mad(il, -wih, kFxHalf))));
+  const long long mi = fx_mad(rh, wil, fx_mad(rl, wih, fx_mad(ih, w.rl, fx_mad(il, w.rh, kFxHalf))));
+  return {fx_mad(rh, w.rh, fx_mad(ih, -wih, mr >> 32)), fx_mad(rh, wih, fx_mad(ih, w.rh, mi >> 32))};
+}
+
+// ---- block scaling -------------------------------------------------------------------------
+// Every stage of a transform starts from components below 2^kFxBits, so that the outputs of its
+// radix P <= 10 stay below 10 2^58.5 < 2^62.  The largest output of the tile (the or of the
+// magnitudes' high words, exchanged at the barrier that ends the stage) gives the shift to the
+// next stage's range: down by the growth that there was, not by the most that there could be.
+constexpr int kFxBits = 58;
+DGPE_HD int fx_mag(long long a) { return (int)(a >> 32) ^ (int)(a >> 63); }   // bits of the high word's magnitude
+DGPE_HD int fx_mag(fxc a) { return fx_mag(a.re) | fx_mag(a.im); }
+// the shift down that takes magnitudes mag to kFxBits bits (negative: up); -26 at least:
+// a tile whose outputs nearly all cancelled carries on with fewer bits
+DGPE_HD int fx_shift(int mag) {
+#ifdef __CUDA_ARCH__
+  const int d = 64 - __clz(mag) - kFxBits;
+#else
+  const int d = (mag ? 64 - __builtin_clz(mag) : 32) - kFxBits;
+#endif
+  return d;
+}
+// a 2^-d, rounded
+DGPE_HD long long fx_scale(long long a, int d) { return d > 0 ? (a + (1LL << (d - 1))) >> d : a << -d; }
+// 16 a 2^-d, the input of fx_twiddle (d <= 4: a radix up to 10 makes components grow by at most
+// 10 sqrt 2 < 16)
+DGPE_HD fxc fx_up(fxc a, int d) {
+  return {(long long)((unsigned long long)a.re << (4 - d)), (long long)((unsigned long long)a.im << (4 - d))};
+}
+
+// ---- butterflies (the usual radix-2/3/4/5/7/8 forms and their prime-factor products) --------
+template <int DIR>
+DGPE_HD void fx_bf2(fxc *v) {
+  const fxc t = v[0] - v[1];
+  v[0] = v[0] + v[1];
+  v[1] = t;
+}
+template <int DIR>
+DGPE_HD void fx_bf3(fxc *v) {
+  const fxc t = v[1] + v[2], d = v[1] - v[2];
+  const fxc m = {v[0].re - (t.re >> 1), v[0].im - (t.im >> 1)};
+  const fxc s = fx_rot<DIR>(fxc{fx_const<1, 0xddb3d742c265539eull>(d.re), fx_const<1, 0xddb3d742c265539eull>(d.im)});
+  v[0] = v[0] + t;
+  v[1] = m + s;
+  v[2] = m - s;
+}
+template <int DIR>
+DGPE_HD void fx_bf4(fxc *v) {
+  const fxc a = v[0] + v[2], b = v[0] - v[2], c = v[1] + v[3], d = fx_rot<DIR>(v[1] - v[3]);
+  v[0] = a + c;
+  v[1] = b + d;
+  v[2] = a - c;
+  v[3] = b - d;
+}
+template <int DIR>
+DGPE_HD void fx_bf5(fxc *v) {
+  const fxc t1 = v[1] + v[4], t2 = v[2] + v[3], d1 = v[1] - v[4], d2 = v[2] - v[3], t = t1 + t2, e = t1 - t2;
+  const fxc m = {v[0].re - (t.re >> 2), v[0].im - (t.im >> 2)};
+  const fxc q = {fx_const<1, 0x8f1bbcdcbfa53e0bull>(e.re), fx_const<1, 0x8f1bbcdcbfa53e0bull>(e.im)};
+  auto s1 = [](fxc a) { return fxc{fx_const<1, 0xf378709a22a7faf3ull>(a.re), fx_const<1, 0xf378709a22a7faf3ull>(a.im)}; };
+  auto s2 = [](fxc a) { return fxc{fx_const<1, 0x96791823aad2ef6eull>(a.re), fx_const<1, 0x96791823aad2ef6eull>(a.im)}; };
+  const fxc a = m + q, b = m - q;
+  const fxc x = fx_rot<DIR>(s1(d1) + s2(d2)), y = fx_rot<DIR>(s2(d1) - s1(d2));
+  v[0] = v[0] + t;
+  v[1] = a + x;
+  v[4] = a - x;
+  v[2] = b + y;
+  v[3] = b - y;
+}
+template <int DIR>
+DGPE_HD void fx_bf7(fxc *v) {
+  const fxc t[3] = {v[1] + v[6], v[2] + v[5], v[3] + v[4]}, d[3] = {v[1] - v[6], v[2] - v[5], v[3] - v[4]};
+  auto c1 = [](fxc a) { return fxc{fx_const<1, 0x9f9d07145f6e8b66ull>(a.re), fx_const<1, 0x9f9d07145f6e8b66ull>(a.im)}; };
+  auto c2 = [](fxc a) { return fxc{fx_const<0, 0xc708de39fb74fb2dull>(a.re), fx_const<0, 0xc708de39fb74fb2dull>(a.im)}; };
+  auto c3 = [](fxc a) { return fxc{fx_const<-1, 0x195a1ab1a51c796dull>(a.re), fx_const<-1, 0x195a1ab1a51c796dull>(a.im)}; };
+  auto s1 = [](fxc a) { return fxc{fx_const<1, 0xc8261ba82ef2585eull>(a.re), fx_const<1, 0xc8261ba82ef2585eull>(a.im)}; };
+  auto s2 = [](fxc a) { return fxc{fx_const<1, 0xf994e02ac74b471dull>(a.re), fx_const<1, 0xf994e02ac74b471dull>(a.im)}; };
+  auto s3 = [](fxc a) { return fxc{fx_const<0, 0x6f130135c6af0401ull>(a.re), fx_const<0, 0x6f130135c6af0401ull>(a.im)}; };
+  const fxc p1 = v[0] + c1(t[0]) + c2(t[1]) + c3(t[2]), q1 = fx_rot<DIR>(s1(d[0]) + s2(d[1]) + s3(d[2]));
+  const fxc p2 = v[0] + c2(t[0]) + c3(t[1]) + c1(t[2]), q2 = fx_rot<DIR>(s2(d[0]) - s3(d[1]) - s1(d[2]));
+  const fxc p3 = v[0] + c3(t[0]) + c1(t[1]) + c2(t[2]), q3 = fx_rot<DIR>(s3(d[0]) - s1(d[1]) + s2(d[2]));
+  v[0] = v[0] + t[0] + t[1] + t[2];
+  v[1] = p1 + q1;
+  v[6] = p1 - q1;
+  v[2] = p2 + q2;
+  v[5] = p2 - q2;
+  v[3] = p3 + q3;
+  v[4] = p3 - q3;
+}
+template <int DIR>
+DGPE_HD void fx_bf8(fxc *v) {
+  fxc a[4], b[4];
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    a[k] = v[k] + v[k + 4];
+    b[k] = v[k] - v[k + 4];
+  }
+  auto r = [](long long x) { return fx_const<1, 0xb504f333f9de6484ull>(x); };   // 1/sqrt 2
+  // e^{DIR i pi/4} = (1 + DIR i)/sqrt 2, e^{DIR 3 i pi/4} = (-1 + DIR i)/sqrt 2
+  const fxc i1 = fx_rot<DIR>(b[1]), i3 = fx_rot<DIR>(b[3]);
+  b[1] = {r(b[1].re + i1.re), r(b[1].im + i1.im)};
+  b[2] = fx_rot<DIR>(b[2]);
+  b[3] = {r(i3.re - b[3].re), r(i3.im - b[3].im)};
+  fx_bf4<DIR>(a);
+  fx_bf4<DIR>(b);
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    v[2 * k] = a[k];
+    v[2 * k + 1] = b[k];
+  }
+}
+template <int DIR>
+DGPE_HD void fx_bf6(fxc *v) {   // 2 x 3: n = 3 n1 + 2 n2, k = 3 k1 + 4 k2 (mod 6)
+  fxc a[3] = {v[0], v[2], v[4]}, b[3] = {v[3], v[5], v[1]};
+  fx_bf3<DIR>(a);
+  fx_bf3<DIR>(b);
+#pragma unroll
+  for (int k = 0; k < 3; ++k) {
+    v[(4 * k) % 6] = a[k] + b[k];
+    v[(4 * k + 3) % 6] = a[k] - b[k];
+  }
+}
+template <int DIR>
+DGPE_HD void fx_bf10(fxc *v) {   // 2 x 5: n = 5 n1 + 2 n2, k = 5 k1 + 6 k2 (mod 10)
+  fxc a[5] = {v[0], v[2], v[4], v[6], v[8]}, b[5] = {v[5], v[7], v[9], v[1], v[3]};
+  fx_bf5<DIR>(a);
+  fx_bf5<DIR>(b);
+#pragma unroll
+  for (int k = 0; k < 5; ++k) {
+    v[(6 * k) % 10] = a[k] + b[k];
+    v[(6 * k + 5) % 10] = a[k] - b[k];
+  }
+}
+template <int DIR>
+DGPE_HD void fx_bf9(fxc *v) {   // 3 x 3 with the twiddles e^{DIR 2 pi i n2 k1 / 9}
+  auto c1 = [](long long a) { return fx_const<1, 0xc41b7d167a81c991ull>(a); };
+  auto s1 = [](long long a) { return fx_const<1, 0xa48dba91e0b0e55dull>(a); };
+  auto c2 = [](long long a) { return fx_const<0, 0x2c7434fc16e71346ull>(a); };
+  auto s2 = [](long long a) { return fx_const<1, 0xfc1c5c6408e0bad0ull>(a); };
+  auto c4 = [](long long a) { return fx_const<-1, 0x0f704ded6e972329ull>(a); };
+  auto s4 = [](long long a) { return fx_const<0, 0x578ea1d2282fd573ull>(a); };
+  auto tw = [](fxc z, auto c, auto s) {
+    return DIR < 0 ? fxc{c(z.re) + s(z.im), c(z.im) - s(z.re)} : fxc{c(z.re) - s(z.im), c(z.im) + s(z.re)};
+  };
+  fxc c[3][3];   // [n2][k1]
+#pragma unroll
+  for (int n2 = 0; n2 < 3; ++n2) {
+    c[n2][0] = v[n2];
+    c[n2][1] = v[n2 + 3];
+    c[n2][2] = v[n2 + 6];
+    fx_bf3<DIR>(c[n2]);
+  }
+  c[1][1] = tw(c[1][1], c1, s1);
+  c[1][2] = tw(c[1][2], c2, s2);
+  c[2][1] = tw(c[2][1], c2, s2);
+  c[2][2] = tw(c[2][2], c4, s4);
+#pragma unroll
+  for (int k1 = 0; k1 < 3; ++k1) {
+    fxc t[3] = {c[0][k1], c[1][k1], c[2][k1]};
+    fx_bf3<DIR>(t);
+#pragma unroll
+    for (int k2 = 0; k2 < 3; ++k2) v[k1 + 3 * k2] = t[k2];
+  }
+}
+template <int DIR, int P>
+DGPE_HD void fx_bf(fxc *v) {
+  if constexpr (P == 2) fx_bf2<DIR>(v);
+  else if constexpr (P == 3) fx_bf3<DIR>(v);
+  else if constexpr (P == 4) fx_bf4<DIR>(v);
+  else if constexpr (P == 5) fx_bf5<DIR>(v);
+  else if constexpr (P == 6) fx_bf6<DIR>(v);
+  else if constexpr (P == 7) fx_bf7<DIR>(v);
+  else if constexpr (P == 8) fx_bf8<DIR>(v);
+  else if constexpr (P == 9) fx_bf9<DIR>(v);
+  else fx_bf10<DIR>(v);
+}
+
+// ---- FP64 <-> fixed point ----------------------------------------------------------------
+// The tile's exponent is the largest biased exponent emax of its values (0x7ff: some value is not
+// finite, and the tile's results are NaN): x = v 2^(emax - 1080), |v| < 2^58, cut off at bit 0.
+DGPE_HD long long fx_bits(double x) {
+#ifdef __CUDA_ARCH__
+  return __double_as_longlong(x);
+#else
+  long long b;
+  memcpy(&b, &x, 8);
+  return b;
+#endif
+}
+DGPE_HD double fx_value(long long b) {
+#ifdef __CUDA_ARCH__
+  return __longlong_as_double(b);
+#else
+  double x;
+  memcpy(&x, &b, 8);
+  return x;
+#endif
+}
+DGPE_HD int fx_exponent_bits(double x) { return (int)(fx_bits(x) >> 32) & 0x7fffffff; }   // orders by exponent
+DGPE_HD long long fx_from(double x, int emax) {
+  const long long b = fx_bits(x);
+  const int e = (int)(b >> 52) & 0x7ff, s = emax - (e > 1 ? e : 1);
+  const unsigned long long m = ((unsigned long long)b & 0xfffffffffffffull) | (e > 0 ? 1ull << 52 : 0ull);
+  const long long v = (long long)((m << 5) >> (s > 63 ? 63 : s));
+  const long long g = b >> 63;
+  return (v ^ g) - g;
+}
+// v 2^(exp - 1023 - 63) rounded to FP64 (to nearest; halves away from zero; below 2^-1022 to 0)
+DGPE_HD double fx_to(long long v, int exp) {
+  const long long g = v >> 63;
+  const unsigned long long a = (unsigned long long)((v ^ g) - g);
+#ifdef __CUDA_ARCH__
+  const int lz = __clzll((long long)a);
+#else
+  const int lz = a ? __builtin_clzll(a) : 64;
+#endif
+  const int f = exp - lz;   // the biased exponent
+  const unsigned long long m = a << (lz & 63);
+  unsigned long long b = ((unsigned long long)(unsigned)(f - 1) << 52) + (m >> 11) + ((m >> 10) & 1ull);
+  if (a == 0 || f < 1) b = 0;
+  else if (f > 2046) b = 0x7ff0000000000000ull;
+  return fx_value((long long)(b | ((unsigned long long)g & 0x8000000000000000ull)));
+}
+
+// The kernels' side of a real type: the exponent key of a value (ordered), the tile's largest key
+// -> exponent, values -> integers and back under `exp`, v 2^(exp - 1086).
+template <typename R>
+struct FxIO;
+template <>
+struct FxIO<double> {
+  static constexpr int kKeyShift = 20, kBad = 0x7ff, kExp = 6;   // exp = emax + kExp
+  DGPE_HD static int key(double x) { return fx_exponent_bits(x); }
+  DGPE_HD static long long from(double x, int emax) { return fx_from(x, emax); }
+  DGPE_HD static double to(long long v, int exp) { return fx_to(v, exp); }
+};
+template <typename R>
+DGPE_HD int fx_key(cplx<R> z) {
+  const int a = FxIO<R>::key(z.re), b = FxIO<R>::key(z.im);
+  return a > b ? a : b;
+}
+
+// ---- plans: the radices of the staged transforms (dgpe_stages.cuh) ---------------------------
+#define DGPE_FIXED_LENGTHS(X) X(128) X(256) X(512) DGPE_STAGE_LENGTHS(X)
+template <int N>
+struct FxPlan {
+  using S = Stages<N>;
+  static constexpr int R1 = S::R1, R2 = S::R2, R3 = S::R3;
+  static constexpr int PL = R3 > 1 ? R3 : R2, NBL = N / PL;                     // the last stage
+  static constexpr int TWL = R3 > 1 ? R1 * (R2 - 1) : 0;                        // its twiddles
+  static constexpr int SLOTS = st_slots<R1, R2, R3, 8>();                       // per line
+};
+// Threads per CTA of a tile of `lines` lines in `smem` bytes of shared memory: at most 256, enough
+// for about 21 warps per SM (what 96 registers a thread allow) with the tiles that fit, and of
+// those the fewest thread-elements over the stages (a thread takes whole butterflies, so a stage
+// rounds up).
+constexpr int fx_threads(int n, int lines, int smem) {
+  int best = 256, cost = 0;
+  for (int nt = 256; nt >= 64 && nt * (225 * 1024 / (smem + 1024)) >= 640; nt -= 32) {
+    int c = 0;
+    for (int s = 0; s < 3; ++s) {
+      const int r = st_radix(n, s);
+      if (r > 1) c += (lines * (n / r) + nt - 1) / nt * r * nt;
+    }
+    if (!cost || c < cost) {
+      cost = c;
+      best = nt;
+    }
+  }
+  return best;
+}
+
+// Or (or maximum) over the CTA of a per-thread value, with the barrier that orders the shared
+// memory written before it.  One slot array per use.
+struct FxSlots {
+  int w[8];
+};
+template <int NT>
+__device__ __forceinline__ int fx_all_or(int v, FxSlots &s) {
+  v = (int)__reduce_or_sync(0xffffffffu, (unsigned)v);
+  if ((threadIdx.x & 31) == 0) s.w[threadIdx.x >> 5] = v;
+  __syncthreads();
+  int r = s.w[0];
+#pragma unroll
+  for (int k = 1; k < NT / 32; ++k) r |= s.w[k];
+  return r;
+}
+template <int NT>
+__device__ __forceinline__ int fx_all_max(int v, FxSlots &s) {
+  v = __reduce_max_sync(0xffffffffu, v);
+  if ((threadIdx.x & 31) == 0) s.w[threadIdx.x >> 5] = v;
+  __syncthreads();
+  int r = s.w[0];
+#pragma unroll
+  for (int k = 1; k < NT / 32; ++k) r = max(r, s.w[k]);
+  return r;
+}
+
+__device__ __forceinline__ fxw fx_ldw(const fxw *p) {
+  const int4 q = __ldg(reinterpret_cast<const int4 *>(p));
+  return {q.x, q.y, q.z, q.w};
+}
+// the inputs of a stage: scaled by the tile's shift d, times the twiddles of output index k
+template <int DIR, int P, int NS>
+__device__ __forceinline__ void fx_inputs(fxc *v, const fxw *__restrict__ tw, int k, int d) {
+  v[0] = {fx_scale(v[0].re, d), fx_scale(v[0].im, d)};
+#pragma unroll
+  for (int r = 1; r < P; ++r) v[r] = fx_twiddle<DIR>(fx_up(v[r], d), fx_ldw(tw + (r - 1) * NS + k));
+}
+template <int P>
+__device__ __forceinline__ int fx_mags(const fxc *v) {
+  int m = 0;
+#pragma unroll
+  for (int r = 0; r < P; ++r) m |= fx_mag(v[r]);
+  return m;
+}
+
+// Stages after the first of a tile of nl <= L lines (SL slots each), element slots in the layouts
+// of dgpe_stages.cuh; the middle stage of three, and the last one, whose outputs go to
+// out(line, j, v): elements j + s NBL.
+template <int DIR, int N, int NT, int SL>
+__device__ __forceinline__ int fx_middle(const fxc *x0, fxc *y0, const fxw *tw, int nl, int d) {
+  using F = FxPlan<N>;
+  constexpr int R1 = F::R1, R2 = F::R2, NB = N / R2, GAP = st_pad2_gap<R1, R2, 8>();
+  int mag = 0;
+  for (int it = threadIdx.x; it < nl * NB; it += NT) {
+    const int l = it / NB, j = it - l * NB, jb = j / R1, k = j - jb * R1;
+    const fxc *x = x0 + l * SL + st_pad1<R1>(j);
+    fxc v[R2];
+#pragma unroll
+    for (int r = 0; r < R2; ++r) v[r] = x[st_pad1<R1>(r * NB)];
+    fx_inputs<DIR, R2, R1>(v, tw, k, d);
+    fx_bf<DIR, R2>(v);
+    mag |= fx_mags<R2>(v);
+    fxc *y = y0 + l * SL + jb * (R1 * R2 + GAP) + k;
+#pragma unroll
+    for (int s = 0; s < R2; ++s) y[s * R1] = v[s];
+  }
+  return mag;
+}
+template <int DIR, int N, int NT, int SL, typename Out>
+__device__ __forceinline__ void fx_last(const fxc *x0, const fxw *tw, int nl, int d, Out out) {
+  using F = FxPlan<N>;
+  constexpr int R1 = F::R1, PL = F::PL, NB = F::NBL, GAP = st_pad2_gap<R1, F::R2, 8>();
+  for (int it = threadIdx.x; it < nl * NB; it += NT) {
+    const int l = it / NB, j = it - l * NB;
+    const fxc *x = x0 + l * SL + (F::R3 > 1 ? j : st_pad1<R1>(j));
+    fxc v[PL];
+#pragma unroll
+    for (int r = 0; r < PL; ++r) v[r] = x[F::R3 > 1 ? r * (NB + GAP) : st_pad1<R1>(r * NB)];
+    fx_inputs<DIR, PL, NB>(v, tw + F::TWL, j, d);
+    fx_bf<DIR, PL>(v);
+    out(l, j, v);
+  }
+}
+template <typename R>
+__device__ __forceinline__ R fx_nan() { return R(__longlong_as_double(0x7ff8000000000000ll)); }
+
+// ---- K2 / K4: y lines ---------------------------------------------------------------------
+template <int N>
+struct FxY {
+  static constexpr int L = N >= 1024 ? 1 : N <= 32 ? 32 : 1024 / N;
+  static constexpr int SL = FxPlan<N>::SLOTS | 1;
+  static constexpr size_t smem = (size_t)(FxPlan<N>::R3 > 1 ? 2 : 1) * L * SL * sizeof(fxc);
+  static constexpr int NT = fx_threads(N, L, smem);
+};
+template <typename R, int DIR, int N>
+__global__ void __launch_bounds__(FxY<N>::NT) k_ffty_fx(const __grid_constant__ KArgs a) {
+  using C = cplx<R>;
+  using Y = FxY<N>;
+  using F = FxPlan<N>;
+  using IO = FxIO<R>;
+  constexpr int R1 = F::R1, SL = Y::SL, NT = Y::NT, NB = N / R1, IT = (Y::L * NB + NT - 1) / NT;
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  __shared__ FxSlots slot[3];
+  fxc *sa = reinterpret_cast<fxc *>(smem_raw), *sb = sa + Y::L * SL;
+  const int total = a.nzh * a.nx, l0 = blockIdx.x * Y::L, nl = min(Y::L, total - l0);
+  C *g = reinterpret_cast<C *>(a.spec) + (size_t)l0 * N;
+  const fxw *tw = reinterpret_cast<const fxw *>(a.tw_st[1]);
+  C x[IT][R1];
+  int key = 0;
+#pragma unroll
+  for (int u = 0; u < IT; ++u) {
+    const int it = threadIdx.x + u * NT, l = it / NB, j = it - l * NB;
+    if (it < nl * NB) {
+#pragma unroll
+      for (int r = 0; r < R1; ++r) x[u][r] = g[l * N + j + r * NB];
+#pragma unroll
+      for (int r = 0; r < R1; ++r) key = max(key, fx_key(x[u][r]));
+    }
+  }
+  const int emax = fx_all_max<NT>(key, slot[0]) >> IO::kKeyShift;
+  if (emax == IO::kBad) {
+    for (int e = threadIdx.x; e < nl * N; e += NT) g[e] = {fx_nan<R>(), fx_nan<R>()};
+    return;
+  }
+  int mag = 0;
+#pragma unroll
+  for (int u = 0; u < IT; ++u) {
+    const int it = threadIdx.x + u * NT, l = it / NB, j = it - l * NB;
+    if (it < nl * NB) {
+      fxc v[R1];
+#pragma unroll
+      for (int r = 0; r < R1; ++r) v[r] = {IO::from(x[u][r].re, emax), IO::from(x[u][r].im, emax)};
+      fx_bf<DIR, R1>(v);
+      mag |= fx_mags<R1>(v);
+      fxc *y = sa + l * SL + st_pad1<R1>(j * R1);
+#pragma unroll
+      for (int s = 0; s < R1; ++s) y[s] = v[s];
+    }
+  }
+  int d = fx_shift(fx_all_or<NT>(mag, slot[1])), exp = emax + IO::kExp + d;
+  if constexpr (F::R3 > 1) {
+    mag = fx_middle<DIR, N, NT, SL>(sa, sb, tw, nl, d);
+    d = fx_shift(fx_all_or<NT>(mag, slot[2]));
+    exp += d;
+  }
+  fx_last<DIR, N, NT, SL>(F::R3 > 1 ? sb : sa, tw, nl, d, [&](int l, int j, const fxc *v) {
+    C *y = g + l * N + j;
+#pragma unroll
+    for (int s = 0; s < F::PL; ++s) y[s * F::NBL] = {IO::to(v[s].re, exp), IO::to(v[s].im, exp)};
+  });
+}
+
+// ---- K3: x lines, 4 columns per CTA (64-byte rows) -------------------------------------------
+template <int N>
+struct FxX {
+  using S = Stages<N>;
+  static constexpr int B = 4;
+  static constexpr int SLA = st_slots<S::R1, S::R2, S::R3, 2>(), SLB = st_slots<S::R3, S::R2, S::R1, 2>();
+  static constexpr int SLOTS = SLA > SLB ? SLA : SLB;
+  static constexpr size_t smem = 2 * (size_t)SLOTS * B * sizeof(fxc);
+  static constexpr int NT = fx_threads(N, B, smem);
+};
+template <int DIR, int N, int P1, int P2, int P3, int B, int NT>
+__device__ __forceinline__ int fx_middle_x(const fxc *x0, fxc *y0, const fxw *tw, int b, int d) {
+  constexpr int NB = N / P2, GAP = st_pad2_gap<P1, P2, 2>();
+  int mag = 0;
+  for (int j = threadIdx.x / B; j < NB; j += NT / B) {
+    const int jb = j / P1, k = j - jb * P1;
+    const fxc *x = x0 + st_pad1<P1>(j) * B + b;
+    fxc v[P2];
+#pragma unroll
+    for (int r = 0; r < P2; ++r) v[r] = x[st_pad1<P1>(r * NB) * B];
+    fx_inputs<DIR, P2, P1>(v, tw, k, d);
+    fx_bf<DIR, P2>(v);
+    mag |= fx_mags<P2>(v);
+    fxc *y = y0 + (jb * (P1 * P2 + GAP) + k) * B + b;
+#pragma unroll
+    for (int s = 0; s < P2; ++s) y[s * P1 * B] = v[s];
+  }
+  return mag;
+}
+template <typename R, int N>
+__global__ void __launch_bounds__(FxX<N>::NT) k3_fx(const __grid_constant__ KArgs a) {
+  using C = cplx<R>;
+  using X = FxX<N>;
+  using IO = FxIO<R>;
+  constexpr int R1 = X::S::R1, R2 = X::S::R2, R3 = X::S::R3, B = X::B, NT = X::NT;
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  __shared__ FxSlots slot[6];
+  fxc *sa = reinterpret_cast<fxc *>(smem_raw), *sb = sa + X::SLOTS * B;
+  const int b = threadIdx.x % B, m = blockIdx.y, jy = blockIdx.x * B + b, ny = a.ny;
+  const bool on = jy < ny;
+  const size_t col = (size_t)m * a.nx * ny + (on ? jy : 0);
+  C *g = reinterpret_cast<C *>(a.spec) + col;
+  const fxw *tw = reinterpret_cast<const fxw *>(a.tw_st[0]), *twr = tw + st_table(N);
+  int mag = 0, d, exp;
+  {
+    constexpr int NB = N / R1, IT = (NB * B + NT - 1) / NT;
+    C x[IT][R1];
+    int key = 0;
+#pragma unroll
+    for (int u = 0; u < IT; ++u) {
+      const int j = threadIdx.x / B + u * (NT / B);
+      if (j < NB) {
+#pragma unroll
+        for (int r = 0; r < R1; ++r) x[u][r] = on ? g[(size_t)(j + r * NB) * ny] : czero<R>();
+#pragma unroll
+        for (int r = 0; r < R1; ++r) key = max(key, fx_key(x[u][r]));
+      }
+    }
+    const int emax = fx_all_max<NT>(key, slot[0]) >> IO::kKeyShift;
+    if (emax == IO::kBad) {
+      for (int j = threadIdx.x / B; j < N; j += NT / B)
+        if (on) g[(size_t)j * ny] = {fx_nan<R>(), fx_nan<R>()};
+      return;
+    }
+    exp = emax + IO::kExp;
+#pragma unroll
+    for (int u = 0; u < IT; ++u) {
+      const int j = threadIdx.x / B + u * (NT / B);
+      if (j < NB) {
+        fxc v[R1];
+#pragma unroll
+        for (int r = 0; r < R1; ++r) v[r] = {IO::from(x[u][r].re, emax), IO::from(x[u][r].im, emax)};
+        fx_bf<-1, R1>(v);
+        mag |= fx_mags<R1>(v);
+        fxc *y = sa + st_pad1<R1>(j * R1) * B + b;
+#pragma unroll
+        for (int s = 0; s < R1; ++s) y[s * B] = v[s];
+      }
+    }
+  }
+  d = fx_shift(fx_all_or<NT>(mag, slot[1]));
+  exp += d;
+  if constexpr (R3 > 1) {
+    mag = fx_middle_x<-1, N, R1, R2, R3, B, NT>(sa, sb, tw, b, d);
+    d = fx_shift(fx_all_or<NT>(mag, slot[2]));
+    exp += d;
+  }
+  // the last forward stage and the product by Ut(k) (table: Ut 2^61), in place; then, at the
+  // products' range, the first inverse stage on the same elements
+  constexpr int P = R3 > 1 ? R3 : R2, NBL = N / P, GAP = st_pad2_gap<R1, R2, 2>();
+  fxc *x0 = R3 > 1 ? sb : sa, *y0 = R3 > 1 ? sa : sb;
+  mag = 0;
+  {
+    const long long *ut = reinterpret_cast<const long long *>(a.utab) + col;
+    for (int j = threadIdx.x / B; j < NBL; j += NT / B) {
+      fxc *x = x0 + (R3 > 1 ? j : st_pad1<R1>(j)) * B + b;
+      fxc v[P];
+      long long u[P];
+#pragma unroll
+      for (int s = 0; s < P; ++s) u[s] = __ldg(ut + (size_t)(j + s * NBL) * ny);
+#pragma unroll
+      for (int r = 0; r < P; ++r) v[r] = x[(R3 > 1 ? r * (NBL + GAP) : st_pad1<R1>(r * NBL)) * B];
+      fx_inputs<-1, P, NBL>(v, R3 > 1 ? tw + R1 * (R2 - 1) : tw, j, d);
+      fx_bf<-1, P>(v);
+#pragma unroll
+      for (int s = 0; s < P; ++s) {
+        const int uh = fx_hi(u[s]), ul = fx_lo(u[s]);
+        v[s] = {fx_mul(v[s].re, uh, ul), fx_mul(v[s].im, uh, ul)};
+      }
+      mag |= fx_mags<P>(v);
+#pragma unroll
+      for (int r = 0; r < P; ++r) x[(R3 > 1 ? r * (NBL + GAP) : st_pad1<R1>(r * NBL)) * B] = v[r];
+    }
+  }
+  d = fx_shift(fx_all_or<NT>(mag, slot[3]));
+  exp += 3 + d;
+  mag = 0;
+  for (int j = threadIdx.x / B; j < NBL; j += NT / B) {
+    const fxc *x = x0 + (R3 > 1 ? j : st_pad1<R1>(j)) * B + b;
+    fxc v[P];
+#pragma unroll
+    for (int r = 0; r < P; ++r) {
+      const fxc t = x[(R3 > 1 ? r * (NBL + GAP) : st_pad1<R1>(r * NBL)) * B];
+      v[r] = {fx_scale(t.re, d), fx_scale(t.im, d)};
+    }
+    fx_bf<+1, P>(v);
+    mag |= fx_mags<P>(v);
+    fxc *y = y0 + st_pad1<P>(j * P) * B + b;
+#pragma unroll
+    for (int s = 0; s < P; ++s) y[s * B] = v[s];
+  }
+  d = fx_shift(fx_all_or<NT>(mag, slot[4]));
+  exp += d;
+  if constexpr (R3 > 1) {
+    mag = fx_middle_x<+1, N, R3, R2, R1, B, NT>(sa, sb, twr, b, d);
+    d = fx_shift(fx_all_or<NT>(mag, slot[5]));
+    exp += d;
+  }
+  {
+    constexpr int NB = N / R1, GAPR = st_pad2_gap<R3, R2, 2>();
+    for (int j = threadIdx.x / B; j < NB; j += NT / B) {
+      const fxc *x = sb + (R3 > 1 ? j : st_pad1<P>(j)) * B + b;
+      fxc v[R1];
+#pragma unroll
+      for (int r = 0; r < R1; ++r) v[r] = x[(R3 > 1 ? r * (NB + GAPR) : st_pad1<P>(r * NB)) * B];
+      fx_inputs<+1, R1, NB>(v, R3 > 1 ? twr + R3 * (R2 - 1) : twr, j, d);
+      fx_bf<+1, R1>(v);
+      if (on) {
+#pragma unroll
+        for (int s = 0; s < R1; ++s) g[(size_t)(j + s * NB) * ny] = {IO::to(v[s].re, exp), IO::to(v[s].im, exp)};
+      }
+    }
+  }
+}
+
+// ---- z lines: tiles of 2 PZ real lines, packed in pairs ------------------------------------
+template <int N>
+struct FxZ {
+  static constexpr int PZ = N <= 64 ? 16 : N <= 128 ? 8 : 4;
+  // line stride: PZ lines by 8 / PZ elements on distinct banks
+  static constexpr int SL0 = FxPlan<N>::SLOTS > N ? FxPlan<N>::SLOTS : N;
+  static constexpr int SL = PZ == 4 ? SL0 + (10 - SL0 % 8) % 8 : SL0 | 1;
+  static constexpr size_t smem = 2 * (size_t)PZ * SL * sizeof(fxc);
+  static constexpr int NT = fx_threads(N, PZ, smem);
+};
+
+// K1: densities, forward transform, separation of the two real spectra
+template <typename R, int N>
+__global__ void __launch_bounds__(FxZ<N>::NT) k1_fx(const __grid_constant__ KArgs a) {
+  using C = cplx<R>;
+  using Z = FxZ<N>;
+  using F = FxPlan<N>;
+  using IO = FxIO<R>;
+  constexpr int R1 = F::R1, SL = Z::SL, NT = Z::NT, PZ = Z::PZ, NB = N / R1, IT = (PZ * NB + NT - 1) / NT;
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  __shared__ FxSlots slot[3];
+  fxc *sa = reinterpret_cast<fxc *>(smem_raw), *sb = sa + PZ * SL;
+  const int i = blockIdx.y, j0 = blockIdx.x * (2 * PZ), np = min(2 * PZ, a.ny - j0) >> 1;
+  const C *psi = reinterpret_cast<const C *>(a.psi) + ((size_t)i * a.ny + j0) * N;
+  const R s2 = a.unit_scale ? R(1) : scale_sq_of<R>(a.state);
+  const bool scaled = (double)s2 != 1.0;
+  R x[IT][R1], y[IT][R1];
+  int key = 0;
+#pragma unroll
+  for (int u = 0; u < IT; ++u) {
+    const int it = threadIdx.x + u * NT, p = it / NB, j = it - p * NB;
+    if (it < np * NB) {
+#pragma unroll
+      for (int r = 0; r < R1; ++r) {
+        const C v = psi[(size_t)(2 * p) * N + j + r * NB], w = psi[(size_t)(2 * p + 1) * N + j + r * NB];
+        x[u][r] = v.re * v.re + v.im * v.im;
+        y[u][r] = w.re * w.re + w.im * w.im;
+      }
+      if (scaled) {
+#pragma unroll
+        for (int r = 0; r < R1; ++r) {
+          x[u][r] = x[u][r] * s2;
+          y[u][r] = y[u][r] * s2;
+        }
+      }
+#pragma unroll
+      for (int r = 0; r < R1; ++r) key = max(key, max(IO::key(x[u][r]), IO::key(y[u][r])));
+    }
+  }
+  const int emax = fx_all_max<NT>(key, slot[0]) >> IO::kKeyShift;
+  const bool bad = emax == IO::kBad;
+  int mag = 0;
+#pragma unroll
+  for (int u = 0; u < IT; ++u) {
+    const int it = threadIdx.x + u * NT, p = it / NB, j = it - p * NB;
+    if (it < np * NB) {
+      fxc v[R1];
+#pragma unroll
+      for (int r = 0; r < R1; ++r) v[r] = {IO::from(x[u][r], emax), IO::from(y[u][r], emax)};
+      fx_bf<-1, R1>(v);
+      mag |= fx_mags<R1>(v);
+      fxc *q = sa + p * SL + st_pad1<R1>(j * R1);
+#pragma unroll
+      for (int s = 0; s < R1; ++s) q[s] = v[s];
+    }
+  }
+  const fxw *tw = reinterpret_cast<const fxw *>(a.tw_st[2]);
+  int d = fx_shift(fx_all_or<NT>(mag, slot[1])), exp = emax + IO::kExp - 1 + d;   // - 1: the half of the separation
+  if constexpr (F::R3 > 1) {
+    mag = fx_middle<-1, N, NT, SL>(sa, sb, tw, np, d);
+    d = fx_shift(fx_all_or<NT>(mag, slot[2]));
+    exp += d;
+  }
+  fxc *res = F::R3 > 1 ? sa : sb;
+  fx_last<-1, N, NT, SL>(F::R3 > 1 ? sb : sa, tw, np, d, [&](int p, int j, const fxc *v) {
+#pragma unroll
+    for (int s = 0; s < F::PL; ++s) res[p * SL + j + s * F::NBL] = v[s];
+  });
+  __syncthreads();
+  C *spec = reinterpret_cast<C *>(a.spec) + (size_t)i * a.ny + j0;
+  const size_t plane = (size_t)a.nx * a.ny;
+  const int p = threadIdx.x % PZ;
+  if (p < np) {
+    for (int m = threadIdx.x / PZ; m <= N / 2; m += NT / PZ) {
+      const fxc zm = res[p * SL + m], zc = res[p * SL + (m ? N - m : 0)];
+      C o1 = {IO::to(zm.re + zc.re, exp), IO::to(zm.im - zc.im, exp)};
+      C o2 = {IO::to(zm.im + zc.im, exp), IO::to(zc.re - zm.re, exp)};
+      if (bad) o1 = o2 = {fx_nan<R>(), fx_nan<R>()};
+      C *dst = spec + m * plane + 2 * p;
+      dst[0] = o1;
+      dst[1] = o2;
+    }
+  }
+}
+
+// K5's phase pass: packing of the two half spectra, inverse transform (Phi), potential step
+template <typename R, int N>
+__global__ void __launch_bounds__(FxZ<N>::NT) k5_fx(const __grid_constant__ KArgs a) {
+  using C = cplx<R>;
+  using Z = FxZ<N>;
+  using F = FxPlan<N>;
+  using IO = FxIO<R>;
+  constexpr int R1 = F::R1, SL = Z::SL, NT = Z::NT, PZ = Z::PZ, M = N / 2 + 1, IT = (PZ * M + NT - 1) / NT;
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  __shared__ FxSlots slot[4];
+  fxc *sa = reinterpret_cast<fxc *>(smem_raw), *sb = sa + PZ * SL;
+  const int i = blockIdx.y, j0 = blockIdx.x * (2 * PZ), np = min(2 * PZ, a.ny - j0) >> 1;
+  int emax;
+  {
+    const C *spec = reinterpret_cast<const C *>(a.spec) + (size_t)i * a.ny + j0;
+    const size_t plane = (size_t)a.nx * a.ny;
+    C x1[IT], x2[IT];
+    int key = 0;
+    const int p = threadIdx.x % PZ;
+#pragma unroll
+    for (int u = 0; u < IT; ++u) {
+      const int m = threadIdx.x / PZ + u * (NT / PZ);
+      if (m < M && p < np) {
+        const C *src = spec + m * plane + 2 * p;
+        x1[u] = src[0];
+        x2[u] = src[1];
+      }
+    }
+#pragma unroll
+    for (int u = 0; u < IT; ++u) {
+      const int m = threadIdx.x / PZ + u * (NT / PZ);
+      if (m < M && p < np) key = max(key, max(fx_key(x1[u]), fx_key(x2[u])));
+    }
+    emax = (fx_all_max<NT>(key, slot[0]) >> IO::kKeyShift) + 1;   // + 1: the sums of the packing
+#pragma unroll
+    for (int u = 0; u < IT; ++u) {
+      const int m = threadIdx.x / PZ + u * (NT / PZ);
+      if (m < M && p < np) {
+        const bool end = m == 0 || m == N / 2;   // real bins of a real field's spectrum
+        const fxc v1 = {IO::from(x1[u].re, emax), end ? 0 : IO::from(x1[u].im, emax)};
+        const fxc v2 = {IO::from(x2[u].re, emax), end ? 0 : IO::from(x2[u].im, emax)};
+        sa[p * SL + m] = {v1.re - v2.im, v1.im + v2.re};
+        if (!end) sa[p * SL + N - m] = {v1.re + v2.im, v2.re - v1.im};
+      }
+    }
+  }
+  const bool bad = emax > IO::kBad;
+  __syncthreads();
+  const fxw *tw = reinterpret_cast<const fxw *>(a.tw_st[2]);
+  int mag = 0;
+  {
+    constexpr int NB = N / R1;
+    for (int it = threadIdx.x; it < np * NB; it += NT) {
+      const int p = it / NB, j = it - p * NB;
+      fxc v[R1];
+#pragma unroll
+      for (int r = 0; r < R1; ++r) v[r] = sa[p * SL + j + r * NB];
+      fx_bf<+1, R1>(v);
+      mag |= fx_mags<R1>(v);
+      fxc *q = sb + p * SL + st_pad1<R1>(j * R1);
+#pragma unroll
+      for (int s = 0; s < R1; ++s) q[s] = v[s];
+    }
+  }
+  int d = fx_shift(fx_all_or<NT>(mag, slot[1])), exp = emax + IO::kExp + d;
+  if constexpr (F::R3 > 1) {
+    mag = fx_middle<+1, N, NT, SL>(sb, sa, tw, np, d);
+    d = fx_shift(fx_all_or<NT>(mag, slot[2]));
+    exp += d;
+  }
+  // theta = dt (V + g n + gdd Phi), 1/(nx ny nz) of the inverse transform folded into gdd
+  C *psi = reinterpret_cast<C *>(a.psi) + ((size_t)i * a.ny + j0) * N;
+  const R *dtv_y = reinterpret_cast<const R *>(a.dtv[1]) + j0, *dtv_z = reinterpret_cast<const R *>(a.dtv[2]);
+  const R dtvx = ldg(reinterpret_cast<const R *>(a.dtv[0]) + i);
+  const R sr = scale_of<R>(a.state);
+  const bool scaled = (double)sr != 1.0;
+  const R dtg = pick<R>(a.dtg, a.dtg_f, a.dtg_l), dtgdd = pick<R>(a.dtgdd_n, a.dtgdd_n_f, a.dtgdd_n_l);
+  fx_last<+1, N, NT, SL>(F::R3 > 1 ? sa : sb, tw, np, d, [&](int p, int j, const fxc *v) {
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      C *row = psi + (size_t)(2 * p + h) * N + j;
+      const R vxy = dtvx + ldg(dtv_y + 2 * p + h);
+      C w[F::PL];
+#pragma unroll
+      for (int s = 0; s < F::PL; ++s) w[s] = row[s * F::NBL];
+#pragma unroll
+      for (int s = 0; s < F::PL; ++s) {
+        R phi = IO::to(h ? v[s].im : v[s].re, exp);
+        if (bad) phi = fx_nan<R>();
+        C z = w[s];
+        if (scaled) z = scale(z, sr);
+        const R dens = z.re * z.re + z.im * z.im;
+        const R theta = fma(dtg, dens, fma(dtgdd, phi, vxy + ldg(dtv_z + j + s * F::NBL)));
+        if (a.imag) {
+          row[s * F::NBL] = scale(z, exp_r(-theta));
+        } else {
+          R sn, cs;
+          sin_cos(theta, &sn, &cs);
+          row[s * F::NBL] = {z.re * cs + z.im * sn, z.im * cs - z.re * sn};
+        }
+      }
+    }
+  });
+}
+
+// ---- set-up ---------------------------------------------------------------------------------
+// The twiddles of the plan of length n and of its radices in reverse order (layout: dgpe_stages.cuh)
+__global__ inline void k_fx_twiddles(fxw *tw, int n, int r1, int r2, int r3) {
+  const int t = blockIdx.x * blockDim.x + threadIdx.x;
+  if (t >= 2 * n) return;
+  const bool rev = t >= n;
+  int e = rev ? t - n : t;
+  const int nst = r3 > 1 ? 3 : 2;
+  const int p1 = rev ? (nst == 3 ? r3 : r2) : r1, p2 = rev ? (nst == 3 ? r2 : r1) : r2, p3 = nst == 3 ? (rev ? r1 : r3) : 1;
+  int ns = p1, p = p2;
+  if (e >= p1 * (p2 - 1)) {
+    e -= p1 * (p2 - 1);
+    ns = p1 * p2;
+    p = p3;
+    if (e >= ns * (p - 1)) return;
+  }
+  const int r = e / ns + 1, k = e % ns;
+  double s, c;
+  sincospi(2.0 * (double)(r * k) / (double)(ns * p), &s, &c);
+  const long long qc = __double2ll_rn(c * 1152921504606846976.0), qs = __double2ll_rn(-s * 1152921504606846976.0);   // 2^60
+  tw[t] = {fx_hi(qc), fx_lo(qc), fx_hi(qs), fx_lo(qs)};
+}
+
+// One translation unit's lengths: every kFxParts-th of the list.
+constexpr int kFxParts = 8;
+constexpr int fx_index(int n) {
+  int i = 0, at = -1;
+#define DGPE_AT(m) \
+  if (m == n) at = i; \
+  ++i;
+  DGPE_FIXED_LENGTHS(DGPE_AT)
+#undef DGPE_AT
+  return at;
+}
+template <int PART>
+struct FxLaunch {
+  template <typename F>
+  static bool with(int n, F &&f) {
+    switch (n) {
+#define DGPE_CASE(m) \
+  case m: \
+    if constexpr (fx_index(m) % kFxParts == PART) { \
+      f(std::integral_constant<int, m>{}); \
+      return true; \
+    } \
+    break;
+      DGPE_FIXED_LENGTHS(DGPE_CASE)
+#undef DGPE_CASE
+      default: break;
+    }
+    return false;
+  }
+  // kernel `which` (kK1DensityR2Cz .. kK4IfftY, kK5C2RzPhaseCnz: the phase pass)
+  template <typename R>
+  static bool run(int which, const KArgs &a, cudaStream_t st) {
+    const int n = which == kK3FftXDipolar ? a.nx : which == kK2FftY || which == kK4IfftY ? a.ny : a.nz;
+    return with(n, [&](auto len) {
+      constexpr int N = decltype(len)::value;
+      using Y = FxY<N>;
+      using X = FxX<N>;
+      using Z = FxZ<N>;
+      const unsigned gy = (a.nzh * a.nx + Y::L - 1) / Y::L;
+      const dim3 gz((a.ny + 2 * Z::PZ - 1) / (2 * Z::PZ), a.nx);
+      if (which == kK2FftY) k_ffty_fx<R, -1, N><<<gy, Y::NT, Y::smem, st>>>(a);
+      else if (which == kK4IfftY) k_ffty_fx<R, +1, N><<<gy, Y::NT, Y::smem, st>>>(a);
+      else if (which == kK3FftXDipolar) k3_fx<R, N><<<dim3((a.ny + X::B - 1) / X::B, a.nzh), X::NT, X::smem, st>>>(a);
+      else if constexpr (N % 2 == 0) {
+        if (which == kK1DensityR2Cz) k1_fx<R, N><<<gz, Z::NT, Z::smem, st>>>(a);
+        else k5_fx<R, N><<<gz, Z::NT, Z::smem, st>>>(a);
+      }
+    });
+  }
+  template <typename R>
+  static cudaError_t init(int nx, int ny, int nz) {
+    cudaError_t e = cudaSuccess;
+    auto opt = [&](auto k, size_t sm) {
+      if (e == cudaSuccess && sm > 48 * 1024 - 512) e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    };
+    with(nx, [&](auto len) { opt(k3_fx<R, decltype(len)::value>, FxX<decltype(len)::value>::smem); });
+    with(ny, [&](auto len) {
+      opt(k_ffty_fx<R, -1, decltype(len)::value>, FxY<decltype(len)::value>::smem);
+      opt(k_ffty_fx<R, +1, decltype(len)::value>, FxY<decltype(len)::value>::smem);
+    });
+    with(nz, [&](auto len) {
+      opt(k1_fx<R, decltype(len)::value>, FxZ<decltype(len)::value>::smem);
+      opt(k5_fx<R, decltype(len)::value>, FxZ<decltype(len)::value>::smem);
+    });
+    return e;
+  }
+};
+
+}  // namespace dgpe

@@ -98,13 +98,15 @@ struct KArgs {
   const void *dtv[3];          // dt v_d x_i^2 per axis (kernel precision)
   void *psi;                   // [nx][ny][nz] complex
   void *spec;                  // [nzh][nx][ny] complex, the z-half-spectrum-major layout
-  const void *utab;            // Ut(k) (times the cutoff factor) on [nzh][nx][ny], FP64 only
+  const void *utab;            // Ut(k) (times the cutoff factor) on [nzh][nx][ny], FP64-class only; 2^61 Ut(k)
+                               // as 64-bit integers where nx has a fixed-point transform
   void *ybuf;                  // [point][line] forward-elimination scratch of the FP64
                                // one-thread-per-line sweeps (nx ny nz complex values)
   float kf[3];                 // 2 pi / (n_d h_d): wavenumber per frequency index (FP32 K3)
   DevState *state;
   double *partials;            // per-block reduction partials
-  const void *tw_st[2];        // twiddles of the staged FP32 x and y transforms (layout in dgpe_stages.cuh)
+  const void *tw_st[3];        // twiddles of the staged transforms (FP32: x and y, dgpe_stages.cuh; FP64-class:
+                               // x, y and z in fixed point, dgpe_fixed.cuh)
   int diff;                    // 1: within the differentiation calls (FP32: the transforms and chunks whose
                                // roundings their results rest on)
   const void *tw[3];           // per-stage twiddle tables of plan[d] (layout in FftPlan), d = x, y, z
@@ -220,6 +222,32 @@ inline cudaError_t stage_init(int nx, int ny) {
 }
 // the twiddles of length n (2 n values; nothing where n has no staged transform)
 cudaError_t stage_tables(void *tw, int n, cudaStream_t st);
+
+// The fixed-point transforms of the FP64-class precisions (dgpe_fixed.cuh), the lengths spread
+// over eight translation units.  fx_run: kernel `which` (K1 to K4, K5: the phase pass) of these
+// arguments; false where its line length has none (below 12).
+#define DGPE_FX_UNITS(X) X(0) X(1) X(2) X(3) X(4) X(5) X(6) X(7)
+#define DGPE_FX_UNIT(i)                                                \
+  bool fx_run##i(int which, const KArgs &a, cudaStream_t st);          \
+  cudaError_t fx_init##i(int nx, int ny, int nz);
+DGPE_FX_UNITS(DGPE_FX_UNIT)
+#undef DGPE_FX_UNIT
+inline bool fx_run(int which, const KArgs &a, cudaStream_t st) {
+#define DGPE_FX_OR(i) || fx_run##i(which, a, st)
+  return false DGPE_FX_UNITS(DGPE_FX_OR);
+#undef DGPE_FX_OR
+}
+inline cudaError_t fx_init(int nx, int ny, int nz) {
+  cudaError_t e = cudaSuccess;
+#define DGPE_FX_INIT(i) \
+  if (e == cudaSuccess) e = fx_init##i(nx, ny, nz);
+  DGPE_FX_UNITS(DGPE_FX_INIT)
+#undef DGPE_FX_INIT
+  return e;
+}
+bool fx_length(int n);   // n has a fixed-point transform
+// the twiddles of length n (2 n values of 16 bytes; nothing where n has no such transform)
+cudaError_t fx_tables(void *tw, int n, cudaStream_t st);
 
 cudaError_t group_init_f32();
 cudaError_t group_step_f32(const KArgs &a, const KArgs *ga, int n, int renorm, cudaStream_t st);
