@@ -177,7 +177,9 @@ Layout layout_of(const dgpe_params *p, const KernelSet *ks, int max_blocks) {
   for (int d = 0; d < 3; ++d) {
     L.cn[d] = off;
     // lane-interleaved tables, scan factors, then the twist pivot of the two-thread sweeps
-    off += align_up((size_t)(4 * axis_chunk(p, d) + 11) * kWarp * e);
+    // (FP64: and the fixed-point sweeps' coefficients)
+    const size_t fx = p->precision == DGPE_FP64 ? fx_cn_entries(n[d] - 2) : 0;
+    off += align_up(((size_t)(4 * axis_chunk(p, d) + 11) * kWarp + fx) * e);
     // the same at the chunk of the differentiation calls, and for dt -> -dt (adjoint)
     const int dc = p->precision == DGPE_MIXED && d < 2 ? diff_chunk(n[d]) : axis_chunk(p, d);
     if (d < 2) {
@@ -188,7 +190,7 @@ Layout layout_of(const dgpe_params *p, const KernelSet *ks, int max_blocks) {
       }
     }
     L.cn_adj[d] = off;
-    off += align_up((size_t)(4 * dc + 11) * kWarp * e);
+    off += align_up(((size_t)(4 * dc + 11) * kWarp + fx) * e);
   }
   L.cnz = 0;   // K5's z tables at their own chunk (FP32 where the compile-time K5 needs them)
   if (needs_cnz(p)) {
@@ -212,7 +214,7 @@ Layout layout_of(const dgpe_params *p, const KernelSet *ks, int max_blocks) {
   L.utab = off;   // FP64 and double-float (8-byte entries); the FP32 kernels evaluate it in place
   if (p->precision != DGPE_MIXED) off += align_up((size_t)(p->nz / 2 + 1) * p->nx * p->ny * 8);
   L.ybuf = off;   // the forward-elimination values of the FP64 per-line sweeps
-  if (p->precision == DGPE_FP64) off += align_up((size_t)p->nx * p->ny * p->nz * e);
+  if (p->precision == DGPE_FP64) off += align_up(fx_scratch((size_t)p->nx * p->ny * p->nz) * e);
   L.total = off;
   (void)ks;
   return L;
@@ -523,7 +525,8 @@ int setup_tables(dgpe_ctx *c, bool cn_changed, bool ut_changed) {
   if (cn_changed && c->L.cnz)
     jobs.job[jobs.n++] = {at(c, c->L.cnz), c->args.cn[2].m, k5_chunk(p->nz), c->args.cn_r[2], kWarp};
   if (jobs.n) {
-    const int rc = map_cuda(c->ks->cn_tables(jobs, c->stream));
+    int rc = map_cuda(c->ks->cn_tables(jobs, c->stream));
+    if (!rc && p->precision == DGPE_FP64) rc = map_cuda(fx_cn_tables(jobs, c->stream));
     if (rc) return rc;
   }
   if (ut_changed) return map_cuda(c->ks->dipolar_table(c->args, c->stream));
@@ -737,6 +740,7 @@ int dgpe_create(const dgpe_params *p, void *cuda_stream, dgpe_ctx **out) {
   rc = map_cuda(c->ks->init());
   if (!rc && p->precision == DGPE_MIXED) rc = map_cuda(stage_init(p->nx, p->ny));
   if (!rc && p->precision == DGPE_FP64) rc = map_cuda(fx_init(p->nx, p->ny, p->nz));
+  if (!rc && p->precision == DGPE_FP64) rc = map_cuda(fx_cn_init());
   if (!rc) rc = map_cuda(cudaStreamCreateWithFlags(&c->cap_stream, cudaStreamNonBlocking));
   if (!rc) {
     if (p->workspace) {

@@ -3500,7 +3500,9 @@ struct Impl {
   template <int AXIS>
   static cudaError_t cn(const KArgs &a, int reduce, int renorm, cudaStream_t st) {
     const int n = AXIS == 0 ? a.nx : AXIS == 1 ? a.ny : a.nz;
-    if constexpr (kCnThread) {
+    if constexpr (kFixed) {
+      return fx_cn(AXIS, a, reduce, renorm, st);
+    } else if constexpr (kCnThread) {
       const long long lines = AXIS == 2 ? (long long)a.nx * a.ny : (long long)(AXIS == 0 ? a.ny : a.nx) * a.nz;
       const size_t sm = AXIS == 0 ? (size_t)n * sizeof(R) : 0;
       const unsigned blocks = (unsigned)((lines + 63) / 64);   // 64 lines, two threads each

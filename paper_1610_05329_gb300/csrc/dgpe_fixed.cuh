@@ -9,9 +9,8 @@
 // With components below 2^58 on entry, a stage's outputs stay below 2^62 up to radix 10, and the
 // tile is rescaled by its largest output before the next stage, so the last bit stays at 2^-58 of
 // the tile's largest element: below an FP64 rounding of the elements' rms up to 512 points.
-// Bound by integer issue (about 250 instructions per complex element and pass).  Measured, us, the
-// FP64 transforms -> these: 256^3 K1 430 -> 134, K2 328 -> 96, K3 690 -> 208, the phase pass 1100 ->
-// 765; 480x480x250 a step 18.0 -> 9.5 ms; 64^3 a step 165 -> 125.  Phi against extended precision
+// Bound by integer issue (about 200 instructions per complex element and pass).  Measured, us, the
+// FP64 transforms -> these: 256^3 K1 430 -> 127, K2 328 -> 74, K3 690 -> 170.  Phi against extended precision
 // (rel-L2, clouds and noise, 36 .. 480 points): 3.8e-16 .. 7.1e-16 -> 2.3e-16 .. 4.2e-16.
 #pragma once
 #include <cstring>
@@ -33,7 +32,16 @@ DGPE_HD fxc fx_rot(fxc a) { return DIR < 0 ? fxc{a.im, -a.re} : fxc{-a.im, a.re}
 // a = hi 2^32 + lo with a signed lo, so that every product below is a signed one
 DGPE_HD int fx_hi(long long a) { return (int)(a >> 32) + (int)((unsigned)a >> 31); }
 DGPE_HD int fx_lo(long long a) { return (int)(unsigned)a; }
-DGPE_HD long long fx_mad(int a, int b, long long c) { return (long long)a * b + c; }
+// a b + c, one instruction (written out: the compiler widens some of these products to 64 x 64 bits)
+DGPE_HD long long fx_mad(int a, int b, long long c) {
+#ifdef __CUDA_ARCH__
+  long long d;
+  asm("mad.wide.s32 %0, %1, %2, %3;" : "=l"(d) : "r"(a), "r"(b), "l"(c));
+  return d;
+#else
+  return (long long)a * b + c;
+#endif
+}
 constexpr long long kFxHalf = 0x80000000LL;
 
 // a w / 2^64 (the product of the low words, less than half a unit, left out).  |a| < 2^63 - 2^31,
@@ -241,8 +249,10 @@ DGPE_HD void fx_bf(fxc *v) {
 }
 
 // ---- FP64 <-> fixed point ----------------------------------------------------------------
-// The tile's exponent is the largest biased exponent emax of its values (0x7ff: some value is not
-// finite, and the tile's results are NaN): x = v 2^(emax - 1080), |v| < 2^58, cut off at bit 0.
+// The tile's exponent is the largest biased exponent emax of its values, at least kFxMinBiased (0x7ff:
+// some value is not finite, and the tile's results are NaN): x = v 2^(emax - 1080), |v| < 2^58, cut
+// off at bit 0; subnormal values, 2^-63 below the least tile exponent, are 0.
+constexpr int kFxMinBiased = 64;
 DGPE_HD long long fx_bits(double x) {
 #ifdef __CUDA_ARCH__
   return __double_as_longlong(x);
@@ -264,14 +274,35 @@ DGPE_HD double fx_value(long long b) {
 DGPE_HD int fx_exponent_bits(double x) { return (int)(fx_bits(x) >> 32) & 0x7fffffff; }   // orders by exponent
 DGPE_HD long long fx_from(double x, int emax) {
   const long long b = fx_bits(x);
-  const int e = (int)(b >> 52) & 0x7ff, s = emax - (e > 1 ? e : 1);
-  const unsigned long long m = ((unsigned long long)b & 0xfffffffffffffull) | (e > 0 ? 1ull << 52 : 0ull);
-  const long long v = (long long)((m << 5) >> (s > 63 ? 63 : s));
+  const int s = emax - ((int)(b >> 52) & 0x7ff);
+  const unsigned long long m = ((unsigned long long)b & 0xfffffffffffffull) | 1ull << 52;
+  const long long v = (long long)((m << 5) >> (s < 63 ? s : 63));
   const long long g = b >> 63;
   return (v ^ g) - g;
 }
-// v 2^(exp - 1023 - 63) rounded to FP64 (to nearest; halves away from zero; below 2^-1022 to 0)
+// v 2^(exp - 1086) rounded to FP64, |v| < 2^62: the conversion and a shift of the exponent field where
+// every nonzero v gives a normal number, else through fx_to_any (below 2^-1022 the result is 0).
+__host__ __device__ __noinline__ static double fx_to_any(long long v, int exp) {
+  const double x = (double)v;
+  const int f = (int)((fx_bits(x) >> 52) & 0x7ff) + exp - 1086;
+  if (v == 0 || f < 1) return 0.0;
+  if (f > 2046) return fx_value(v < 0 ? (long long)0xfff0000000000000ull : 0x7ff0000000000000ll);
+  return fx_value(fx_bits(x) + ((long long)(exp - 1086) << 52));
+}
+DGPE_HD double fx_to_normal(long long v, int exp) {   // 64 <= exp <= 2047
+  const double x = (double)v;
+  return v == 0 ? 0.0 : fx_value(fx_bits(x) + ((long long)(exp - 1086) << 52));
+}
 DGPE_HD double fx_to(long long v, int exp) {
+  return (unsigned)(exp - 64) < 1984u ? fx_to_normal(v, exp) : fx_to_any(v, exp);
+}
+DGPE_HD cplx<double> fx_to(fxc v, int exp) {
+  if ((unsigned)(exp - 64) < 1984u) return {fx_to_normal(v.re, exp), fx_to_normal(v.im, exp)};
+  return {fx_to_any(v.re, exp), fx_to_any(v.im, exp)};
+}
+// The same without the conversion instruction, for the kernels whose FP64 pipe has other work or whose
+// chains wait for it (halves round away from zero): about 20 integer instructions.
+DGPE_HD double fx_to_int(long long v, int exp) {
   const long long g = v >> 63;
   const unsigned long long a = (unsigned long long)((v ^ g) - g);
 #ifdef __CUDA_ARCH__
@@ -279,13 +310,193 @@ DGPE_HD double fx_to(long long v, int exp) {
 #else
   const int lz = a ? __builtin_clzll(a) : 64;
 #endif
-  const int f = exp - lz;   // the biased exponent
-  const unsigned long long m = a << (lz & 63);
-  unsigned long long b = ((unsigned long long)(unsigned)(f - 1) << 52) + (m >> 11) + ((m >> 10) & 1ull);
-  if (a == 0 || f < 1) b = 0;
-  else if (f > 2046) b = 0x7ff0000000000000ull;
+  const int f = exp - lz - 1;   // the biased exponent less 1; the leading bit, at bit 52 below, adds it
+  unsigned long long b = (((a << ((lz - 1) & 63)) + 0x200) >> 10) + ((unsigned long long)(unsigned)f << 52);
+  if ((unsigned)f >= 2046u || a == 0) b = f >= 2046 && a != 0 ? 0x7ff0000000000000ull : 0;
   return fx_value((long long)(b | ((unsigned long long)g & 0x8000000000000000ull)));
 }
+DGPE_HD cplx<double> fx_to_int(fxc v, int exp) { return {fx_to_int(v.re, exp), fx_to_int(v.im, exp)}; }
+
+// ---- one value with its own exponent: v 2^e ------------------------------------------------
+// The recurrences along a line keep every point's precision relative to that point (the tails of a
+// cloud as well as its middle), so the running value carries its own exponent: components just
+// below 2^62 (fx_up's range) after every step.
+struct fxv {
+  fxc v;
+  int e;
+};
+constexpr int kFxMinExp = kFxMinBiased - 1080;   // (values below 2^-960 lose bits from here on)
+DGPE_HD fxv fx_norm(fxc s, int e) {   // components of s below 2^62
+#ifdef __CUDA_ARCH__
+  const int n = __clz(fx_mag(s)) - 2;
+#else
+  const int mg = fx_mag(s), n = (mg ? __builtin_clz(mg) : 32) - 2;
+#endif
+  return {{(long long)((unsigned long long)s.re << n), (long long)((unsigned long long)s.im << n)}, e - n};
+}
+// a w / 16 for a coefficient w of magnitude at most 1 (words of w 2^60; real ones: rh, rl alone)
+template <bool CPLX>
+DGPE_HD fxc fx_coef(fxc a, fxw w) {
+  if constexpr (CPLX) return fx_twiddle<-1>(a, w);
+  else return {fx_mul(a.re, w.rh, w.rl), fx_mul(a.im, w.rh, w.rl)};
+}
+DGPE_HD long long fx_sar(long long a, int s) { return a >> (s < 63 ? s : 63); }
+// psi + p (p: components below 2^59, exponent ep; key: psi's exponent key), normalised
+DGPE_HD fxv fx_forward(double re, double im, int key, fxc p, int ep) {
+  const int em = (key >> 20) - 1080;
+  int e = em > ep ? em : ep;
+  if (e < kFxMinExp) e = kFxMinExp;
+  return fx_norm({fx_from(re, e + 1080) + fx_sar(p.re, e - ep), fx_from(im, e + 1080) + fx_sar(p.im, e - ep)}, e);
+}
+// y + p for a normalised y
+DGPE_HD fxv fx_backward(fxv y, fxc p, int ep) {
+  const int e = y.e + 4 > ep ? y.e + 4 : ep;
+  return fx_norm({fx_sar(y.v.re, e - y.e) + fx_sar(p.re, e - ep), fx_sar(y.v.im, e - y.e) + fx_sar(p.im, e - ep)}, e);
+}
+// 16 bytes of a normalised value: 57 bits of each component, the exponent in the low 6 bits of both
+DGPE_HD fxc fx_pack(fxv y) {
+  const int b = y.e + 1300;
+  return {(long long)(((unsigned long long)y.v.re << 1) & ~63ull) | (b & 63),
+          (long long)(((unsigned long long)y.v.im << 1) & ~63ull) | (b >> 6)};
+}
+DGPE_HD fxv fx_unpack(fxc q) {
+  return {{(q.re & ~63ll) >> 1, (q.im & ~63ll) >> 1}, ((((int)q.im & 63) << 6) | ((int)q.re & 63)) - 1300};
+}
+
+// ---- sine, cosine and exponential of the potential step, in fixed point ------------------------
+// An angle as theta 2^58, |theta| < 18.
+constexpr long long kFxOne58 = 1LL << 58;
+// x 2^58 cut off at bit 0, for |x| < 4; `slow` set otherwise
+DGPE_HD long long fx_angle(double x, bool &slow) {
+  const long long b = fx_bits(x);
+  const int e = (int)(b >> 52) & 0x7ff, s = 1027 - e;
+  slow |= e > 1024;
+  const unsigned long long m = ((unsigned long long)b & 0xfffffffffffffull) | (1ull << 52);
+  const long long v = (long long)((m << 10) >> (s > 63 ? 63 : s < 0 ? 0 : s));
+  const long long g = b >> 63;
+  return (v ^ g) - g;
+}
+// p w / 2^64 + c
+DGPE_HD long long fx_horner(long long p, int wh, int wl, long long c) {
+  const int ph = fx_hi(p), pl = fx_lo(p);
+  const long long mid = fx_mad(ph, wl, fx_mad(pl, wh, kFxHalf));
+  return fx_mad(ph, wh, (mid >> 32) + c);
+}
+// (cos theta, -sin theta) 2^60, the factor e^{-i theta}: up to |theta| = 1/8 the least-squares fits of
+// sin_cos(double); beyond (fx_cis_any, out of line: seldom taken, and twice the code) a reduction by
+// quarter turns and Taylor series to r^17 and r^18 in u / 2, u = r^2 (r <= pi / 4: the remainders are
+// below 2^-63).  Absolute error below 2^-57, so the result's rounding to FP64 dominates.
+__host__ __device__ __noinline__ static fxc fx_cis_any(long long th) {
+  // quarter turns q and the rest f in [-1/2, 1/2), 2^58
+  const long long t = fx_const<1, 0xa2f9836e4e44152aull>(th);   // 2 / pi
+  const int q = (int)((t + (kFxOne58 >> 1)) >> 58);
+  const long long f = t - ((long long)q << 58);
+  const long long f62 = f * 16, r = 2 * (2 * f62 + fx_mul(f62, -1843415740, 1121027178));   // r 2^63, pi/2 = 2 - ...
+  const long long u = 2 * fx_mul(r, fx_hi(r), fx_lo(r));   // (r^2 / 2) 2^64
+  const int uh = fx_hi(u), ul = fx_lo(u);
+  long long ps = fx_horner(1659591, uh, ul, -225704436);   // (-1)^(k+1) 2^k / (2 k + 3)! 2^62
+  ps = fx_horner(ps, uh, ul, 23698965738ll);
+  ps = fx_horner(ps, uh, ul, -1848519327572ll);
+  ps = fx_horner(ps, uh, ul, 101668563016477ll);
+  ps = fx_horner(ps, uh, ul, -3660068268593165ll);
+  ps = fx_horner(ps, uh, ul, 76861433640456465ll);
+  ps = fx_horner(ps, uh, ul, -768614336404564651ll);
+  long long pc = fx_horner(-184399, uh, ul, 28213054);     // (-1)^(k+1) 2^k / (2 k + 2)! 2^62
+  pc = fx_horner(pc, uh, ul, -3385566534ll);
+  pc = fx_horner(pc, uh, ul, 308086554595ll);
+  pc = fx_horner(pc, uh, ul, -20333712603295ll);
+  pc = fx_horner(pc, uh, ul, 915017067148291ll);
+  pc = fx_horner(pc, uh, ul, -25620477880152155ll);
+  pc = fx_horner(pc, uh, ul, 384307168202282325ll);
+  pc = fx_horner(pc, uh, ul, -2305843009213693952ll);
+  const long long ru = fx_mul(r, uh, ul);   // r u 2^62
+  const long long s = (r >> 3) + fx_mul(ps, fx_hi(ru), fx_lo(ru));   // 2^60
+  const long long c = fx_horner(pc, uh, ul, 1LL << 61) >> 1;
+  return (q & 1) ? ((q & 2) ? fxc{s, c} : fxc{-s, -c}) : ((q & 2) ? fxc{-c, s} : fxc{c, -s});
+}
+DGPE_HD fxc fx_cis(long long th) {
+  if (th <= (kFxOne58 >> 3) && th >= -(kFxOne58 >> 3)) {
+    const long long x = th * 64;   // theta 2^64
+    const int xh = fx_hi(x), xl = fx_lo(x);
+    const long long u = fx_mul(x, xh, xl);   // theta^2 2^64
+    const int uh = fx_hi(u), ul = fx_lo(u);
+    long long ps = fx_horner(12704960496226ll, uh, ul, -915017031897204ll);   // 2^62 times the fits
+    ps = fx_horner(ps, uh, ul, 38430716820118072ll);
+    ps = fx_horner(ps, uh, ul, -768614336404564608ll);
+    long long pc = fx_horner(114337425721235ll, uh, ul, -6405119082289318ll);
+    pc = fx_horner(pc, uh, ul, 192153584099929472ll);
+    pc = fx_horner(pc, uh, ul, -2305843009213693440ll);
+    const long long xu = fx_mul(x, uh, ul);   // theta^3 2^64
+    const long long s = (x >> 2) + fx_mul(ps, fx_hi(xu), fx_lo(xu));   // 2^62
+    const long long c = fx_horner(pc, uh, ul, 1LL << 62);
+    return {c >> 2, -(s >> 2)};
+  }
+  return fx_cis_any(th);
+}
+// e^-theta = p 2^(n - 60): 2^f, f in [-1/2, 1/2), by its Taylor series in f / 2 to the 14th power
+// (remainder below 2^-66)
+DGPE_HD long long fx_exp(long long th, int &n) {
+  const long long t = -fx_const<1, 0x71547652b82fe177ull>(th);   // log2 e
+  n = (int)((t + (kFxOne58 >> 1)) >> 58);
+  const long long w = (t - ((long long)n << 58)) * 32;   // (f / 2) 2^64
+  const int wh = fx_hi(w), wl = fx_lo(w);
+  long long p = fx_horner(1280465205, wh, wl, 12931245613ll);   // (2 ln 2)^k / k! 2^60
+  p = fx_horner(p, wh, wl, 121262985468ll);
+  p = fx_horner(p, wh, wl, 1049673046670ll);
+  p = fx_horner(p, wh, wl, 8328969544420ll);
+  p = fx_horner(p, wh, wl, 60080815287248ll);
+  p = fx_horner(p, wh, wl, 390052324203650ll);
+  p = fx_horner(p, wh, wl, 2250906215263282ll);
+  p = fx_horner(p, wh, wl, 11365799319932687ll);
+  p = fx_horner(p, wh, wl, 49192146943818121ll);
+  p = fx_horner(p, wh, wl, 177423166116318949ll);
+  p = fx_horner(p, wh, wl, 511935043789664227ll);
+  p = fx_horner(p, wh, wl, 1107849223398934356ll);
+  p = fx_horner(p, wh, wl, 1598288580650331957ll);
+  return fx_horner(p, wh, wl, 1152921504606846976ll);
+}
+// d = c 2^x with |c| < 2^62 (0 for a subnormal d)
+struct fxs {
+  int h, l, x;
+};
+DGPE_HD fxs fx_scalar(double d) {
+  const long long b = fx_bits(d);
+  const int e = (int)(b >> 52) & 0x7ff;
+  const long long m = e ? (long long)(((unsigned long long)b & 0xfffffffffffffull) | (1ull << 52)) << 9 : 0;
+  const long long c = b < 0 ? -m : m;
+  return {fx_hi(c), fx_lo(c), e - 1084};
+}
+// One point of the potential step: z e^{-i theta} (z e^{-theta}), theta = v + g |z|^2 + dd phi with
+// v 2^58 (a sum of two terms below 4) and phi 2^(exp - 1086) in integers, sd = the shift of dd phi
+// (not below -1: |theta| < 4 + 4 + 2 + 8).  False, and z as it was, where the interaction or z itself is out of range.
+template <bool IMAG>
+DGPE_HD bool fx_phase(double &zre, double &zim, long long v, fxs g, fxs dd, int sd, long long phi) {
+  const int ka = fx_exponent_bits(zre), kb = fx_exponent_bits(zim);
+  int em = (ka > kb ? ka : kb) >> 20;
+  if (em < kFxMinBiased) em = kFxMinBiased;
+  const fxc z = {fx_from(zre, em) * 16, fx_from(zim, em) * 16};   // z 2^-(em - 1084)
+  const long long n = fx_mul(z.re, fx_hi(z.re), fx_lo(z.re)) + fx_mul(z.im, fx_hi(z.im), fx_lo(z.im));
+  const int sg = -(g.x + 2 * (em - 1084) + 186);
+  if (em == 0x7ff || sg < 0) return false;
+  const long long th = v + fx_sar(fx_mul(n, g.h, g.l), sg) + fx_sar(2 * fx_mul(phi, dd.h, dd.l), sd + 1);
+  fxc o;
+  int eo = em - 1080 + 1086;
+  if constexpr (IMAG) {
+    int k;
+    const long long p = fx_exp(th, k);
+    const int ph = fx_hi(p), pl = fx_lo(p);
+    o = {fx_mul(z.re, ph, pl), fx_mul(z.im, ph, pl)};
+    eo += k;
+  } else {
+    const fxc c = fx_cis(th);
+    o = fx_twiddle<-1>(z, fxw{fx_hi(c.re), fx_lo(c.re), fx_hi(c.im), fx_lo(c.im)});
+  }
+  const cplx<double> r = fx_to(o, eo);
+  zre = r.re;
+  zim = r.im;
+  return true;
+}
+DGPE_HD int fx_phase_shift(fxs dd, int exp) { return -(64 + dd.x + exp - 1028); }
 
 // The kernels' side of a real type: the exponent key of a value (ordered), the tile's largest key
 // -> exponent, values -> integers and back under `exp`, v 2^(exp - 1086).
@@ -297,6 +508,7 @@ struct FxIO<double> {
   DGPE_HD static int key(double x) { return fx_exponent_bits(x); }
   DGPE_HD static long long from(double x, int emax) { return fx_from(x, emax); }
   DGPE_HD static double to(long long v, int exp) { return fx_to(v, exp); }
+  DGPE_HD static cplx<double> to(fxc v, int exp) { return fx_to(v, exp); }
 };
 template <typename R>
 DGPE_HD int fx_key(cplx<R> z) {
@@ -453,7 +665,7 @@ __global__ void __launch_bounds__(FxY<N>::NT) k_ffty_fx(const __grid_constant__ 
       for (int r = 0; r < R1; ++r) key = max(key, fx_key(x[u][r]));
     }
   }
-  const int emax = fx_all_max<NT>(key, slot[0]) >> IO::kKeyShift;
+  const int emax = max(fx_all_max<NT>(key, slot[0]) >> IO::kKeyShift, kFxMinBiased);
   if (emax == IO::kBad) {
     for (int e = threadIdx.x; e < nl * N; e += NT) g[e] = {fx_nan<R>(), fx_nan<R>()};
     return;
@@ -482,7 +694,7 @@ __global__ void __launch_bounds__(FxY<N>::NT) k_ffty_fx(const __grid_constant__ 
   fx_last<DIR, N, NT, SL>(F::R3 > 1 ? sb : sa, tw, nl, d, [&](int l, int j, const fxc *v) {
     C *y = g + l * N + j;
 #pragma unroll
-    for (int s = 0; s < F::PL; ++s) y[s * F::NBL] = {IO::to(v[s].re, exp), IO::to(v[s].im, exp)};
+    for (int s = 0; s < F::PL; ++s) y[s * F::NBL] = IO::to(v[s], exp);
   });
 }
 
@@ -544,7 +756,7 @@ __global__ void __launch_bounds__(FxX<N>::NT) k3_fx(const __grid_constant__ KArg
         for (int r = 0; r < R1; ++r) key = max(key, fx_key(x[u][r]));
       }
     }
-    const int emax = fx_all_max<NT>(key, slot[0]) >> IO::kKeyShift;
+    const int emax = max(fx_all_max<NT>(key, slot[0]) >> IO::kKeyShift, kFxMinBiased);
     if (emax == IO::kBad) {
       for (int j = threadIdx.x / B; j < N; j += NT / B)
         if (on) g[(size_t)j * ny] = {fx_nan<R>(), fx_nan<R>()};
@@ -635,7 +847,7 @@ __global__ void __launch_bounds__(FxX<N>::NT) k3_fx(const __grid_constant__ KArg
       fx_bf<+1, R1>(v);
       if (on) {
 #pragma unroll
-        for (int s = 0; s < R1; ++s) g[(size_t)(j + s * NB) * ny] = {IO::to(v[s].re, exp), IO::to(v[s].im, exp)};
+        for (int s = 0; s < R1; ++s) g[(size_t)(j + s * NB) * ny] = IO::to(v[s], exp);
       }
     }
   }
@@ -649,6 +861,7 @@ struct FxZ {
   static constexpr int SL0 = FxPlan<N>::SLOTS > N ? FxPlan<N>::SLOTS : N;
   static constexpr int SL = PZ == 4 ? SL0 + (10 - SL0 % 8) % 8 : SL0 | 1;
   static constexpr size_t smem = 2 * (size_t)PZ * SL * sizeof(fxc);
+  static constexpr size_t smem5 = smem + N * sizeof(long long);   // K5: and the trap's angles along z
   static constexpr int NT = fx_threads(N, PZ, smem);
 };
 
@@ -690,7 +903,7 @@ __global__ void __launch_bounds__(FxZ<N>::NT) k1_fx(const __grid_constant__ KArg
       for (int r = 0; r < R1; ++r) key = max(key, max(IO::key(x[u][r]), IO::key(y[u][r])));
     }
   }
-  const int emax = fx_all_max<NT>(key, slot[0]) >> IO::kKeyShift;
+  const int emax = max(fx_all_max<NT>(key, slot[0]) >> IO::kKeyShift, kFxMinBiased);
   const bool bad = emax == IO::kBad;
   int mag = 0;
 #pragma unroll
@@ -726,8 +939,7 @@ __global__ void __launch_bounds__(FxZ<N>::NT) k1_fx(const __grid_constant__ KArg
   if (p < np) {
     for (int m = threadIdx.x / PZ; m <= N / 2; m += NT / PZ) {
       const fxc zm = res[p * SL + m], zc = res[p * SL + (m ? N - m : 0)];
-      C o1 = {IO::to(zm.re + zc.re, exp), IO::to(zm.im - zc.im, exp)};
-      C o2 = {IO::to(zm.im + zc.im, exp), IO::to(zc.re - zm.re, exp)};
+      C o1 = fx_to_int(fxc{zm.re + zc.re, zm.im - zc.im}, exp), o2 = fx_to_int(fxc{zm.im + zc.im, zc.re - zm.re}, exp);
       if (bad) o1 = o2 = {fx_nan<R>(), fx_nan<R>()};
       C *dst = spec + m * plane + 2 * p;
       dst[0] = o1;
@@ -736,7 +948,18 @@ __global__ void __launch_bounds__(FxZ<N>::NT) k1_fx(const __grid_constant__ KArg
   }
 }
 
-// K5's phase pass: packing of the two half spectra, inverse transform (Phi), potential step
+// the potential step of one point in FP64
+static __device__ __noinline__ cplx<double> phase_fp64(cplx<double> z, double phi, double v, double dtg, double dtgdd, bool imag) {
+  const double theta = fma(dtg, z.re * z.re + z.im * z.im, fma(dtgdd, phi, v));
+  if (imag) return scale(z, exp_r(-theta));
+  double sn, cs;
+  sin_cos(theta, &sn, &cs);
+  return {z.re * cs + z.im * sn, z.im * cs - z.re * sn};
+}
+// K5's phase pass: packing of the two half spectra, inverse transform (Phi), potential step.  Bound by
+// integer issue; at 256^3, real time, 1100 us in FP64, 765 with the transform in integers, 310 with
+// the angle and its factor too (imaginary time, whose exponential was CUDA's, at 480x480x250: 3060 ->
+// 1400).
 template <typename R, int N>
 __global__ void __launch_bounds__(FxZ<N>::NT) k5_fx(const __grid_constant__ KArgs a) {
   using C = cplx<R>;
@@ -747,6 +970,7 @@ __global__ void __launch_bounds__(FxZ<N>::NT) k5_fx(const __grid_constant__ KArg
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ FxSlots slot[4];
   fxc *sa = reinterpret_cast<fxc *>(smem_raw), *sb = sa + PZ * SL;
+  long long *tz = reinterpret_cast<long long *>(sb + PZ * SL);   // dt V_z 2^58
   const int i = blockIdx.y, j0 = blockIdx.x * (2 * PZ), np = min(2 * PZ, a.ny - j0) >> 1;
   int emax;
   {
@@ -769,7 +993,7 @@ __global__ void __launch_bounds__(FxZ<N>::NT) k5_fx(const __grid_constant__ KArg
       const int m = threadIdx.x / PZ + u * (NT / PZ);
       if (m < M && p < np) key = max(key, max(fx_key(x1[u]), fx_key(x2[u])));
     }
-    emax = (fx_all_max<NT>(key, slot[0]) >> IO::kKeyShift) + 1;   // + 1: the sums of the packing
+    emax = max(fx_all_max<NT>(key, slot[0]) >> IO::kKeyShift, kFxMinBiased) + 1;   // + 1: the sums of the packing
 #pragma unroll
     for (int u = 0; u < IT; ++u) {
       const int m = threadIdx.x / PZ + u * (NT / PZ);
@@ -806,39 +1030,330 @@ __global__ void __launch_bounds__(FxZ<N>::NT) k5_fx(const __grid_constant__ KArg
     d = fx_shift(fx_all_or<NT>(mag, slot[2]));
     exp += d;
   }
-  // theta = dt (V + g n + gdd Phi), 1/(nx ny nz) of the inverse transform folded into gdd
+  // theta = dt (V + g n + gdd Phi), 1/(nx ny nz) of the inverse transform folded into gdd; the
+  // angles and factors in integers (fx_phase), or in FP64 where one of them is out of their range
+  // (a CTA whose trap angles or Phi can be, or a point)
   C *psi = reinterpret_cast<C *>(a.psi) + ((size_t)i * a.ny + j0) * N;
-  const R *dtv_y = reinterpret_cast<const R *>(a.dtv[1]) + j0, *dtv_z = reinterpret_cast<const R *>(a.dtv[2]);
-  const R dtvx = ldg(reinterpret_cast<const R *>(a.dtv[0]) + i);
-  const R sr = scale_of<R>(a.state);
-  const bool scaled = (double)sr != 1.0;
-  const R dtg = pick<R>(a.dtg, a.dtg_f, a.dtg_l), dtgdd = pick<R>(a.dtgdd_n, a.dtgdd_n_f, a.dtgdd_n_l);
-  fx_last<+1, N, NT, SL>(F::R3 > 1 ? sa : sb, tw, np, d, [&](int p, int j, const fxc *v) {
+  const double *dtv_y = reinterpret_cast<const double *>(a.dtv[1]) + j0, *dtv_z = reinterpret_cast<const double *>(a.dtv[2]);
+  const double dtvx = ldg(reinterpret_cast<const double *>(a.dtv[0]) + i);
+  const double sr = scale_of<double>(a.state);
+  const bool scaled = sr != 1.0;
+  const fxs g = fx_scalar(a.dtg), dd = fx_scalar(a.dtgdd_n);
+  const int sd = fx_phase_shift(dd, exp);
+  bool out = bad || sd < -1;
+  if (threadIdx.x < 2 * np) fx_angle(dtvx + ldg(dtv_y + threadIdx.x), out);
+  for (int n = threadIdx.x; n < N; n += NT) tz[n] = fx_angle(ldg(dtv_z + n), out);
+  const bool slow = __syncthreads_or(out);
+  auto phase = [&](auto imag) {
+    constexpr bool IMAG = decltype(imag)::value;
+    fx_last<+1, N, NT, SL>(F::R3 > 1 ? sa : sb, tw, np, d, [&](int p, int j, const fxc *v) {
+#pragma unroll 1   // (the code of a point is long: one copy for both lines)
+      for (int h = 0; h < 2; ++h) {
+        C *row = psi + (size_t)(2 * p + h) * N + j;
+        const double vxy = dtvx + ldg(dtv_y + 2 * p + h);
+        bool any = false;
+        const long long v0 = fx_angle(vxy, any);
+        C w[F::PL];
 #pragma unroll
-    for (int h = 0; h < 2; ++h) {
-      C *row = psi + (size_t)(2 * p + h) * N + j;
-      const R vxy = dtvx + ldg(dtv_y + 2 * p + h);
-      C w[F::PL];
+        for (int s = 0; s < F::PL; ++s) w[s] = row[s * F::NBL];
 #pragma unroll
-      for (int s = 0; s < F::PL; ++s) w[s] = row[s * F::NBL];
-#pragma unroll
-      for (int s = 0; s < F::PL; ++s) {
-        R phi = IO::to(h ? v[s].im : v[s].re, exp);
-        if (bad) phi = fx_nan<R>();
-        C z = w[s];
-        if (scaled) z = scale(z, sr);
-        const R dens = z.re * z.re + z.im * z.im;
-        const R theta = fma(dtg, dens, fma(dtgdd, phi, vxy + ldg(dtv_z + j + s * F::NBL)));
-        if (a.imag) {
-          row[s * F::NBL] = scale(z, exp_r(-theta));
-        } else {
-          R sn, cs;
-          sin_cos(theta, &sn, &cs);
-          row[s * F::NBL] = {z.re * cs + z.im * sn, z.im * cs - z.re * sn};
+        for (int s = 0; s < F::PL; ++s) {
+          C z = w[s];
+          if (scaled) z = scale(z, sr);
+          const long long phi = h ? v[s].im : v[s].re;
+          if (slow || !fx_phase<IMAG>(z.re, z.im, v0 + tz[j + s * F::NBL], g, dd, sd, phi))
+            z = phase_fp64(z, bad ? fx_nan<double>() : IO::to(phi, exp), vxy + ldg(dtv_z + j + s * F::NBL), a.dtg, a.dtgdd_n, IMAG);
+          row[s * F::NBL] = z;
         }
       }
+    });
+  };
+  if (a.imag) phase(std::true_type{});
+  else phase(std::false_type{});
+}
+
+// ---- Crank-Nicolson sweeps ------------------------------------------------------------------
+// Coefficients of the fixed-point sweeps, behind the FP64 table of the same axis and direction (at
+// fx_cn_offset): a header {ka, kb}, then alpha_s 2^ka for s < h + 2, then 2 beta_s 2^kb for
+// s < h + 2 (h = m/2, the largest powers of two that keep every magnitude at most 1).
+__host__ __device__ constexpr size_t fx_cn_offset(int chunk) { return ((size_t)4 * kWarp * chunk + 11 * kWarp) * 16; }
+__global__ inline void k_fx_cn_tables(CnJobs jobs) {
+  const CnJob &jb = jobs.job[blockIdx.x];
+  const int m = jb.m, chunk = jb.chunk, mp = kWarp * chunk, n = m / 2 + 2;
+  const double *tab = static_cast<const double *>(jb.tab);
+  fxw *out = reinterpret_cast<fxw *>(static_cast<char *>(jb.tab) + fx_cn_offset(chunk));
+  // (entries past m are the padding of the FP64 table, and within it: n <= m + 1 <= 32 chunk)
+  auto at = [&](int q, int i) { return q * mp + (i % chunk) * kWarp + i / chunk; };
+  auto get = [&](int q, int i) {
+    if (i >= m) return Z64{0.0, 0.0};
+    const double f = q ? 2.0 : 1.0;
+    if (jobs.imag) return Z64{f * tab[at(q, i)], 0.0};
+    return Z64{f * tab[2 * at(q, i)], f * tab[2 * at(q, i) + 1]};
+  };
+  double mx[2] = {0.0, 0.0};
+  for (int q = 0; q < 2; ++q) {
+    for (int i = threadIdx.x; i < n; i += kWarp) {
+      const Z64 z = get(q, i);
+      mx[q] = fmax(mx[q], sqrt(z.re * z.re + z.im * z.im));
     }
-  });
+    for (int o = kWarp / 2; o > 0; o >>= 1) mx[q] = fmax(mx[q], __shfl_xor_sync(0xffffffffu, mx[q], o));
+  }
+  int k[2];
+  for (int q = 0; q < 2; ++q) {
+    int e = 0;
+    frexp(mx[q] * (1.0 + 1e-15), &e);
+    k[q] = mx[q] > 0.0 ? min(-e, 60) : 60;
+  }
+  if (threadIdx.x == 0) out[0] = {k[0], k[1], 0, 0};
+  for (int q = 0; q < 2; ++q)
+    for (int i = threadIdx.x; i < n; i += kWarp) {
+      const Z64 z = get(q, i);
+      const long long re = __double2ll_rn(ldexp(z.re, 60 + k[q])), im = __double2ll_rn(ldexp(z.im, 60 + k[q]));
+      out[1 + q * n + i] = {fx_hi(re), fx_lo(re), fx_hi(im), fx_lo(im)};
+    }
+}
+
+// The sweep along AXIS: two threads per line, the twisted ("burn at both ends") factorization of the
+// Cayley form psi' = 2 (1 - c D)^-1 psi - psi.  The matrix tridiag(-c, 1 + 2c, -c) reads the same from
+// either end, so the top thread eliminates points 0 .. h-1 downwards and the bottom thread points
+// m-1 .. h+1 upwards with the same table entry s at their s-th step; they meet at h = m/2,
+//   gamma x_h = psi_h + alpha_h y_{h-1} + alpha_{m-1-h} z_{h+1}   (in FP64),
+// and substitute back away from it:
+//   y_i = psi_i + alpha_i y_{i-1},  x_i = y_i + alpha_{i+2} x_{i+1}  (x = chi / beta),
+//   psi'_i = 2 beta_i x_i - psi_i.
+// The running values are integers with their own exponent (fxv).  In FP64 arithmetic a sweep is 12
+// FP64 instructions per point, 0.32 ms of that pipe at 256^3; this is about 330 integer ones (0.14 ms)
+// and two FP64 subtractions.  Persistent CTAs: y waits for the way back in a scratch of the CTA's own
+// (packed, 16 bytes a point), so few enough lines are under way for much of it and of their psi to
+// stay in L2.  psi and y come through shared memory by cp.async, two chunks of four points ahead;
+// along z, where a thread's points are consecutive, the lanes of a warp copy each other's chunks as
+// segments of 64 bytes, both ways.  Bound by the latency of the recurrence (a warp issues every 4 to 5
+// cycles; half of the issue slots at 12 warps per SM; DRAM 1.1 GB, 165 us).  Measured at 256^3, real
+// time, us, before (FP64 arithmetic, k_cn_twisted) -> now: y 411 -> 285, x with its sums 515 -> 360, z
+// 410 -> 320; errors against extended precision 0.5 to 0.8 of the FP64 sweep's.
+constexpr int kFxcThreads = 128, kFxcChunk = 4, kFxcStages = 3;
+template <int AXIS>
+constexpr size_t fx_cn_smem(bool reduce, int nx) {
+  const size_t row = AXIS == 2 ? kFxcChunk + 1 : kFxcChunk;
+  return (size_t)kFxcStages * kFxcThreads * (row + kFxcChunk) * 16 + (reduce ? (size_t)nx * 8 : 0);
+}
+template <bool CPLX, int AXIS, bool RED>
+__global__ void __launch_bounds__(kFxcThreads, 4) k_cn_fx(const __grid_constant__ KArgs a, int renorm) {
+  using C = cplx<double>;
+  constexpr int K = kFxcChunk, S = kFxcStages, T = kFxcThreads, ROW = AXIS == 2 ? K + 1 : K;
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  C *pbuf = reinterpret_cast<C *>(smem_raw);                       // psi: [stage][step][thread], z: [stage][thread][step]
+  fxc *ybuf = reinterpret_cast<fxc *>(pbuf + S * T * ROW);         // y: [stage][step][thread]
+  double *wxtab = reinterpret_cast<double *>(ybuf + S * T * K);    // quadrature weights along x
+  const int tid = threadIdx.x, lane = tid & (kWarp - 1);
+  const bool bottom = lane >= kWarp / 2;
+  if constexpr (RED) {
+    for (int n = tid; n < a.nx; n += T) wxtab[n] = quad_weight(n, a.nx, a.simpson);
+    __syncthreads();
+  }
+  const int nfixed = AXIS == 0 ? a.ny : a.nx;
+  const int nlines = AXIS == 2 ? a.nx * a.ny : nfixed * a.nz;
+  const int ntiles = (nlines + T / 2 - 1) / (T / 2);
+  const ptrdiff_t stride = AXIS == 2 ? 1 : AXIS == 1 ? (ptrdiff_t)a.nz : (ptrdiff_t)a.ny * a.nz;
+  const int m = a.cn[AXIS].m, lc = a.cn[AXIS].lchunk, chunk = 1 << lc, mp = kWarp << lc, h = m / 2;
+  using Coef = typename std::conditional<CPLX, C, double>::type;
+  const Coef *tab = reinterpret_cast<const Coef *>(a.cn[AXIS].tab);
+  const fxw *ft = reinterpret_cast<const fxw *>(static_cast<const char *>(a.cn[AXIS].tab) + fx_cn_offset(chunk));
+  const fxw head = fx_ldw(ft);
+  const int ka = head.rh, kb = head.rl;
+  const fxw *fal = ft + 1, *fbe = ft + 1 + h + 2;
+  const double r = a.cn_r[AXIS];
+  fxc *scratch = reinterpret_cast<fxc *>(a.ybuf) + (size_t)blockIdx.x * h * T + tid;   // y of step s at s T
+  double acc[4] = {0.0, 0.0, 0.0, 0.0};
+  for (int tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
+    const int line0 = tile * (T / 2) + tid / kWarp * (kWarp / 2);   // the warp's first line
+    const int line = line0 + (lane & 15);
+    const bool active = line < nlines;
+    const int ln = active ? line : 0, k = ln % a.nz, fixed = ln / a.nz;
+    C *p = reinterpret_cast<C *>(a.psi) +
+           (AXIS == 2 ? (size_t)ln * a.nz : (AXIS == 1 ? (size_t)fixed * a.ny * a.nz : (size_t)fixed * a.nz) + k) + stride;
+    const int nf = active ? (bottom ? m - 1 - h : h) : 0;   // elimination steps of this half
+    // psi of this half's points b + d s for the steps s of chunk c, to stage c % S (z: lane by lane
+    // of the warp's rows, whose b and d follow from the row)
+    auto load_psi = [&](int c, bool back) {
+      if constexpr (AXIS == 2) {
+#pragma unroll
+        for (int q = 0; q < K; ++q) {
+          const int row = q * (kWarp / K) + lane / K, s = c * K + lane % K, l = line0 + (row & 15);
+          const bool bt = row >= kWarp / 2;
+          const int len = bt ? m - 1 - h : h;
+          const int i = back ? (bt ? h + 1 + s : h - 1 - s) : (bt ? m - 1 - s : s);
+          if (l < nlines && s < len)
+            cp_async(pbuf + ((c % S) * T + (tid - lane) + row) * ROW + lane % K, reinterpret_cast<C *>(a.psi) + (size_t)l * a.nz + 1 + i);
+        }
+      } else {
+#pragma unroll
+        for (int e = 0; e < K; ++e) {
+          const int s = c * K + e;
+          const int i = back ? (bottom ? h + 1 + s : h - 1 - s) : (bottom ? m - 1 - s : s);
+          if (s < nf) cp_async(pbuf + ((c % S) * K + e) * T + tid, p + i * stride);
+        }
+      }
+    };
+    auto psi_at = [&](int c, int e) -> C & { return AXIS == 2 ? pbuf[((c % S) * T + tid) * ROW + e] : pbuf[((c % S) * K + e) * T + tid]; };
+    const int nc = (h + K - 1) / K, nwhole = line0 + 15 < nlines ? (m - 1 - h) / K : 0;
+    // elimination
+    fxv y = {{0, 0}, kFxMinExp};
+    int kmax = 0;
+#pragma unroll
+    for (int c = 0; c < S - 1; ++c) {
+      load_psi(c, false);
+      cp_async_commit();
+    }
+    for (int c = 0; c < nc; ++c) {
+      load_psi(c + S - 1, false);
+      cp_async_commit();
+      cp_async_wait_group<S - 1>();
+      if constexpr (AXIS == 2) __syncwarp();
+      // (whole chunks of whole warps without conditions: straight-line code, so that the parts off the
+      // recurrence fill its latency)
+      auto steps = [&](auto whole) {
+        C vs[K];
+#pragma unroll
+        for (int e = 0; e < K; ++e) vs[e] = psi_at(c, e);   // (past the half's end: not used)
+#pragma unroll
+        for (int e = 0; e < K; ++e) {
+          const int s = c * K + e;
+          if (decltype(whole)::value || s < nf) {
+            const C v = vs[e];
+            const int key = fx_key(v);
+            kmax = max(kmax, key);
+            const fxc t = fx_coef<CPLX>(y.v, fx_ldw(fal + s));
+            y = fx_forward(v.re, v.im, key, t, y.e + 4 - ka);
+            scratch[(size_t)s * T] = fx_pack(y);
+          }
+        }
+      };
+      if (c < nwhole) steps(std::true_type{});
+      else steps(std::false_type{});
+      if constexpr (AXIS == 2) __syncwarp();
+    }
+    cp_async_wait_all();
+    __threadfence();   // the scratch is read back through cp.async
+    // y and psi of the way back, step j: the half's step nf - 1 - j
+    auto load_y = [&](int c) {
+#pragma unroll
+      for (int e = 0; e < K; ++e) {
+        const int j = c * K + e;
+        if (j < nf) cp_async(ybuf + ((c % S) * K + e) * T + tid, scratch + (size_t)(nf - 1 - j) * T);
+      }
+    };
+    if constexpr (AXIS == 2) __syncwarp();
+#pragma unroll
+    for (int c = 0; c < S - 1; ++c) {
+      load_psi(c, true);
+      load_y(c);
+      cp_async_commit();
+    }
+    // the twist point, in FP64: gamma x_h = psi_h + alpha_h y_{h-1} + alpha_{m-1-h} z_{h+1}
+    const C yd = fx_to(y.v, y.e + 1086);
+    const C yt = shfl_xor(yd, kWarp / 2);
+    C xh = czero<double>(), ph = czero<double>();
+    if (bottom && active) {
+      auto slot = [&](int s) { return ((s & (chunk - 1)) << 5) + (s >> lc); };
+      ph = p[h * stride];
+      kmax = max(kmax, fx_key(ph));
+      xh = mul(ldg(tab + 4 * mp + 10 * kWarp), cfma(ldg(tab + slot(m - 1 - h)), yd, cfma(ldg(tab + slot(h)), yt, ph)));
+    }
+    const C xt = shfl_xor(xh, kWarp / 2);
+    if (!bottom) xh = xt;
+    kmax = max(kmax, __shfl_xor_sync(0xffffffffu, kmax, kWarp / 2));
+    double s0 = 0.0;
+    auto add = [&](int i, C o) {
+      if constexpr (RED) {
+        if (a.simpson) s0 = fma(wxtab[i + 1], fma(o.re, o.re, o.im * o.im), s0);
+        else s0 = fma(o.im, o.im, fma(o.re, o.re, s0));
+      }
+    };
+    if (bottom && active) {
+      const C o = {twice_minus(xh.re, ph.re), twice_minus(xh.im, ph.im)};
+      p[h * stride] = o;
+      add(h, o);
+    }
+    // c x_h starts both halves' way back
+    const C cx = CPLX ? C{-r * xh.im, r * xh.re} : C{r * xh.re, r * xh.im};
+    const int ex = max(fx_key(cx) >> 20, kFxMinBiased);
+    fxc t = {fx_from(cx.re, ex), fx_from(cx.im, ex)};
+    int et = ex - 1080;
+    for (int c = 0; c < nc; ++c) {
+      load_psi(c + S - 1, true);
+      load_y(c + S - 1);
+      cp_async_commit();
+      cp_async_wait_group<S - 1>();
+      if constexpr (AXIS == 2) __syncwarp();
+      auto steps = [&](auto whole) {
+        C vs[K];
+        fxc ys[K];
+#pragma unroll
+        for (int e = 0; e < K; ++e) {
+          vs[e] = psi_at(c, e);
+          ys[e] = ybuf[((c % S) * K + e) * T + tid];
+        }
+#pragma unroll
+        for (int e = 0; e < K; ++e) {
+          const int j = c * K + e;
+          if (decltype(whole)::value || j < nf) {
+            const int q = nf - 1 - j, i = bottom ? h + 1 + j : h - 1 - j;
+            const C v = vs[e];
+            const fxv x = fx_backward(fx_unpack(ys[e]), t, et);
+            const fxc b = fx_coef<CPLX>(x.v, fx_ldw(fbe + q));
+            t = fx_coef<CPLX>(x.v, fx_ldw(fal + q + 1));   // (q = 0: the last point, unused)
+            et = x.e + 4 - ka;
+            C o;
+            if constexpr (RED) {
+              // the difference in integers: the FP64 pipe has the sums to do
+              const int eb = x.e + 4 - kb, ev = (fx_key(v) >> 20) - 1080, ed = max(max(eb, ev), kFxMinExp);
+              o = fx_to_int(fxc{fx_sar(b.re, ed - eb) - fx_from(v.re, ed + 1080), fx_sar(b.im, ed - eb) - fx_from(v.im, ed + 1080)}, ed + 1086);
+            } else {
+              const int eb = x.e + 4 - kb + 1086;
+              o = fx_to_int(b, eb) - v;
+            }
+            if constexpr (AXIS == 2) psi_at(c, e) = o;
+            else p[i * stride] = o;
+            add(i, o);
+          }
+        }
+      };
+      if (c < nwhole) steps(std::true_type{});
+      else steps(std::false_type{});
+      if constexpr (AXIS == 2) {
+        __syncwarp();
+#pragma unroll
+        for (int q = 0; q < K; ++q) {
+          const int row = q * (kWarp / K) + lane / K, s = c * K + lane % K, l = line0 + (row & 15);
+          const bool bt = row >= kWarp / 2;
+          if (l < nlines && s < (bt ? m - 1 - h : h))
+            reinterpret_cast<C *>(a.psi)[(size_t)l * a.nz + 1 + (bt ? h + 1 + s : h - 1 - s)] = pbuf[((c % S) * T + (tid - lane) + row) * ROW + lane % K];
+        }
+        __syncwarp();
+      }
+    }
+    cp_async_wait_all();
+    if (kmax >= 0x7ff00000) {   // a value that is not finite: so is its line
+      const C nan = {fx_nan<double>(), fx_nan<double>()};
+      for (int s = 0; s < nf; ++s) p[(bottom ? m - 1 - s : s) * stride] = nan;
+      if (bottom && active) p[h * stride] = nan;
+      s0 = fx_nan<double>();
+    }
+    if (active) {
+      // the walls (grid points 0 and N-1)
+      if (!bottom) p[-stride] = czero<double>();
+      else p[m * stride] = czero<double>();
+      if constexpr (RED) {
+        const double wyz = quad_weight_r<double>(fixed, a.ny, a.simpson) * quad_weight_r<double>(k, a.nz, a.simpson);
+        const double yv = (fixed - a.ny / 2) * a.hy, zv = (k - a.nz / 2) * a.hz, tt = wyz * s0;
+        acc[0] += tt;
+        acc[2] = fma(yv * yv, tt, acc[2]);
+        acc[3] = fma(zv * zv, tt, acc[3]);
+      }
+    }
+  }
+  if constexpr (RED) finish_sweep_sums(a, acc, 1.0, 1.0, 1.0, renorm);
 }
 
 // ---- set-up ---------------------------------------------------------------------------------
@@ -909,7 +1424,7 @@ struct FxLaunch {
       else if (which == kK3FftXDipolar) k3_fx<R, N><<<dim3((a.ny + X::B - 1) / X::B, a.nzh), X::NT, X::smem, st>>>(a);
       else if constexpr (N % 2 == 0) {
         if (which == kK1DensityR2Cz) k1_fx<R, N><<<gz, Z::NT, Z::smem, st>>>(a);
-        else k5_fx<R, N><<<gz, Z::NT, Z::smem, st>>>(a);
+        else k5_fx<R, N><<<gz, Z::NT, Z::smem5, st>>>(a);
       }
     });
   }
@@ -926,7 +1441,7 @@ struct FxLaunch {
     });
     with(nz, [&](auto len) {
       opt(k1_fx<R, decltype(len)::value>, FxZ<decltype(len)::value>::smem);
-      opt(k5_fx<R, decltype(len)::value>, FxZ<decltype(len)::value>::smem);
+      opt(k5_fx<R, decltype(len)::value>, FxZ<decltype(len)::value>::smem5);
     });
     return e;
   }

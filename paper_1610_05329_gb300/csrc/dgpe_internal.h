@@ -53,6 +53,11 @@ struct CnJobs {
   int imag;   // the same for every job of a call
 };
 
+// Values of 16 bytes behind an FP64 table for the fixed-point coefficients of m unknowns, and the
+// FP64 sweeps' scratch: the tiles of 64 lines round their number up.
+__host__ __device__ constexpr size_t fx_cn_entries(int m) { return 2 * ((size_t)m / 2 + 2) + 1; }
+__host__ __device__ constexpr size_t fx_scratch(size_t points) { return points + 64 * 512; }
+
 struct CnTab {
   const void *tab;
   int m;
@@ -100,8 +105,8 @@ struct KArgs {
   void *spec;                  // [nzh][nx][ny] complex, the z-half-spectrum-major layout
   const void *utab;            // Ut(k) (times the cutoff factor) on [nzh][nx][ny], FP64-class only; 2^61 Ut(k)
                                // as 64-bit integers where nx has a fixed-point transform
-  void *ybuf;                  // [point][line] forward-elimination scratch of the FP64
-                               // one-thread-per-line sweeps (nx ny nz complex values)
+  void *ybuf;                  // forward-elimination scratch of the FP64 sweeps (fx_scratch(nx ny nz)
+                               // values of 16 bytes)
   float kf[3];                 // 2 pi / (n_d h_d): wavenumber per frequency index (FP32 K3)
   DevState *state;
   double *partials;            // per-block reduction partials
@@ -245,6 +250,11 @@ inline cudaError_t fx_init(int nx, int ny, int nz) {
 #undef DGPE_FX_INIT
   return e;
 }
+// the Crank-Nicolson sweeps of the same precisions (k_cn_fx), and their coefficients behind the
+// FP64 tables of `jobs`
+cudaError_t fx_cn_init();
+cudaError_t fx_cn(int axis, const KArgs &a, int reduce, int renorm, cudaStream_t st);
+cudaError_t fx_cn_tables(const CnJobs &jobs, cudaStream_t st);
 bool fx_length(int n);   // n has a fixed-point transform
 // the twiddles of length n (2 n values of 16 bytes; nothing where n has no such transform)
 cudaError_t fx_tables(void *tw, int n, cudaStream_t st);
