@@ -17,8 +17,7 @@ CSRC = os.path.join(HERE, "csrc")
 OUT_DIR = os.path.join(HERE, "_build")
 LIB = os.path.join(OUT_DIR, "libdgpe.so")
 SOURCES = ["dgpe_api.cu", "kernels_f64.cu", "kernels_f32.cu", "kernels_f32_group.cu", "kernels_df64.cu",
-           "kernels_f32_xy0.cu", "kernels_f32_xy1.cu", "kernels_f32_xy2.cu", "kernels_f32_xy3.cu", "dgpe_noalloc.cu",
-           *("kernels_fx%d.cu" % i for i in range(8))]
+           "dgpe_noalloc.cu", *("kernels_f32_xy%d.cu" % i for i in range(8)), *("kernels_fx%d.cu" % i for i in range(8))]
 HEADERS = ["dgpe_device.cuh", "dgpe_internal.h", "dgpe_df64.cuh", "dgpe_stages.cuh", "dgpe_fixed.cuh"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 FLAGS = ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC", "-I", os.path.join(ROOT, "include")]

@@ -149,11 +149,12 @@ struct Layout {
   size_t state, partials, tw[3], tw_st[3], cn[3], cn_diff[2], cn_adj[3], cnz, cn8z, dtv[3], psi, spec, utab, ybuf, total;
 };
 
-// FP32 contexts whose compile-time K5 (nz = 128, 256, 384, 512) solves along z at a chunk
-// other than the sweeps' power of two (nz = 384: 12 points per lane) get their own tables.
+// FP32 contexts whose K5 is compiled for nz (128, 256, 384, 512 and the staged lengths) and solves
+// along z at a chunk other than the sweeps' power of two (nz = 384: 12 points per lane) get their
+// own tables.
 bool needs_cnz(const dgpe_params *p) {
   const int nz = p->nz;
-  return p->precision == DGPE_MIXED && (nz == 128 || nz == 256 || nz == 384 || nz == 512) &&
+  return p->precision == DGPE_MIXED && (nz == 128 || nz == 256 || nz == 384 || nz == 512 || stage_own_z(nz)) &&
          k5_chunk(nz) != cn_chunk(nz);
 }
 
@@ -170,9 +171,9 @@ Layout layout_of(const dgpe_params *p, const KernelSet *ks, int max_blocks) {
     L.tw[d] = off;
     off += align_up((size_t)n[d] * e);
   }
-  for (int d = 0; d < 3; ++d) {   // the staged transforms' twiddles (FP32: x and y; FP64: fixed point)
+  for (int d = 0; d < 3; ++d) {   // the staged transforms' twiddles (FP64: in fixed point)
     L.tw_st[d] = off;
-    if (p->precision == DGPE_FP64 || (p->precision == DGPE_MIXED && d < 2)) off += align_up(2 * (size_t)n[d] * e);
+    if (p->precision != DGPE_DF64) off += align_up(2 * (size_t)n[d] * e);
   }
   for (int d = 0; d < 3; ++d) {
     L.cn[d] = off;
@@ -268,6 +269,7 @@ void set_physics(KArgs &a, const dgpe_params *p) {
   split_df(a.inv_ntot, &a.inv_ntot_f, &a.inv_ntot_l);
   a.imag = p->mode == DGPE_IMAG_TIME;
   const double h[3] = {p->hx, p->hy, p->hz};
+  for (int d = 0; d < 3; ++d) a.kin_f[d] = (float)(p->kinetic == DGPE_KINETIC_GRADIENT5 ? 1.0 / (12.0 * h[d]) : 1.0 / (h[d] * h[d]));
   for (int d = 0; d < 3; ++d) {
     a.cn_r[d] = p->dt / (4.0 * h[d] * h[d]);
     split_df(a.cn_r[d], &a.cn_rf[d], &a.cn_rl[d]);
@@ -738,7 +740,7 @@ int dgpe_create(const dgpe_params *p, void *cuda_stream, dgpe_ctx **out) {
       c->args.nsm = nsm;
   }
   rc = map_cuda(c->ks->init());
-  if (!rc && p->precision == DGPE_MIXED) rc = map_cuda(stage_init(p->nx, p->ny));
+  if (!rc && p->precision == DGPE_MIXED) rc = map_cuda(stage_init(p->nx, p->ny, p->nz));
   if (!rc && p->precision == DGPE_FP64) rc = map_cuda(fx_init(p->nx, p->ny, p->nz));
   if (!rc && p->precision == DGPE_FP64) rc = map_cuda(fx_cn_init());
   if (!rc) rc = map_cuda(cudaStreamCreateWithFlags(&c->cap_stream, cudaStreamNonBlocking));
@@ -778,7 +780,7 @@ int dgpe_create(const dgpe_params *p, void *cuda_stream, dgpe_ctx **out) {
     void *tw = at(c, c->L.tw_st[d]);
     a.tw_st[d] = tw;
     if (p->precision == DGPE_FP64) rc = map_cuda(fx_tables(tw, n[d], c->stream));
-    else if (p->precision == DGPE_MIXED && d < 2) rc = map_cuda(stage_tables(tw, n[d], c->stream));
+    else if (p->precision == DGPE_MIXED) rc = map_cuda(stage_tables(tw, n[d], c->stream));
   }
   if (!rc) rc = setup_tables(c, true, true);
   if (rc) {

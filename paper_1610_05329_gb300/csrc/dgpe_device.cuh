@@ -1310,6 +1310,16 @@ __global__ void k_cn_tables(CnJobs jobs) {
   // unknowns exactly as they are (the padding only ever multiplies zeros)
   for (int s0 = 0; s0 < L * chunk; s0 += chunk) {
     const int end = s0 + chunk - 1;
+    if (s0 >= m) {   // nothing but padding: no divisions (a short line's tables are mostly this)
+      for (int i = s0; i <= end; ++i) {
+        store_coef<R>(tab, at(0, i), Z64{0.0, 0.0});
+        store_coef<R>(tab, at(1, i), one);
+        store_coef<R>(tab, at(2, i), Z64{0.0, 0.0});
+        store_coef<R>(tab, at(3, i), Z64{0.0, 0.0});
+      }
+      fa[s0 / chunk] = ba[s0 / chunk] = Z64{0.0, 0.0};
+      continue;
+    }
     for (int i = s0; i <= end; ++i) {
       Z64 a = {0.0, 0.0}, e = diag;
       if (i >= m) {
@@ -1854,6 +1864,121 @@ __global__ void __launch_bounds__(8 * RegFft<N>::T, 1024 / (8 * RegFft<N>::T)) k
   else k3_reg_body<N>(a);
 }
 
+// The observables from the totals v over the grid: sums of w n, w kinetic, w V n, w g n^2, w gdd Phi n,
+// w x^2 n, w y^2 n, w z^2 n over the stored values (one thread).
+__device__ __forceinline__ void store_observables(const KArgs &a, double (&v)[8]) {
+  const double dv = a.hx * a.hy * a.hz;
+  DevState *st = a.state;
+  const double s2 = st->s * st->s;
+  for (int q = 0; q < 8; ++q) v[q] *= q == 3 ? s2 * s2 : s2;
+  for (int q = 0; q < 8; ++q) st->sums[q] = v[q];
+  const double norm = dv * v[0];
+  const double ekin = dv * v[1], etrap = dv * v[2], econ = 0.5 * dv * v[3], edd = 0.5 * dv * v[4];
+  st->obs[0] = norm;
+  st->obs[1] = dv * (v[1] + v[2] + v[3] + v[4]) / norm;
+  st->obs[2] = ekin + etrap + econ + edd;
+  st->obs[3] = sqrt(v[5] / v[0]);
+  st->obs[4] = sqrt(v[6] / v[0]);
+  st->obs[5] = sqrt(v[7] / v[0]);
+  st->obs[6] = ekin;
+  st->obs[7] = etrap;
+  st->obs[8] = econ;
+  st->obs[9] = edd;
+  bool finite = true;
+  for (int q = 0; q < 10; ++q) finite = finite && isfinite(st->obs[q]);
+  if (!finite) st->flags |= kFlagNonFinite;
+}
+
+// The observables' sums of FP32 data, one thread's points of z lines (i, j), line by line: each
+// per-point term in FP32 (the state's precision), times the Simpson weight along z (a power of two:
+// exact) or the squared index (an exact integer; FMA exact product), every sum in double-float, as the
+// x sweep's norm; the integer weights and squared indices that a line shares on the line's totals
+// (exact products), h^2, (1/3)^3 and the physical factors in FP64 on the grid's.  The trap term needs
+// no sum of its own: sum w V n = vx sum w x^2 n + vy sum w y^2 n + vz sum w z^2 n.  (A few FP64
+// operations per thread and line bound this pass on GB300's FP64 pipe: 1.0 ms at 384x360x320.)
+struct ObsSums {
+  const KArgs &a;
+  const int i;
+  DFAcc v[8];   // n, the kinetic term, n^2, Phi n, i'^2 n, j'^2 n, k'^2 n (and one unused)
+  // the line: totals of n, the kinetic term, n^2, Phi n, k'^2 n; psi of the line and of its neighbours
+  // (a line outside the grid: this one, times zero)
+  DFAcc t[5];
+  const cplx<float> *line, *nb[8];
+  float in[8];
+  int j;
+  __device__ __forceinline__ ObsSums(const KArgs &k, int x) : a(k), i(x) {}
+  __device__ __forceinline__ void begin(int y) {
+    j = y;
+    const size_t sx = (size_t)a.ny * a.nz;
+    line = reinterpret_cast<const cplx<float> *>(a.psi) + ((size_t)i * a.ny + j) * a.nz;
+    const int off[4] = {-2, -1, 1, 2};
+#pragma unroll
+    for (int d = 0; d < 4; ++d) {
+      const bool x = (unsigned)(i + off[d]) < (unsigned)a.nx, y2 = (unsigned)(j + off[d]) < (unsigned)a.ny;
+      in[d] = x ? 1.0f : 0.0f;
+      in[4 + d] = y2 ? 1.0f : 0.0f;
+      nb[d] = x ? line + (ptrdiff_t)off[d] * (ptrdiff_t)sx : line;
+      nb[4 + d] = y2 ? line + (ptrdiff_t)off[d] * a.nz : line;
+    }
+#pragma unroll
+    for (int q = 0; q < 5; ++q) t[q] = DFAcc();
+  }
+  __device__ __forceinline__ void add(int n, float phi) {
+    using C = cplx<float>;
+    const int nz = a.nz;
+    auto zat = [&](int d) {
+      const bool ok = (unsigned)(n + d) < (unsigned)nz;
+      const C x = line[ok ? n + d : n];
+      return ok ? x : czero<float>();
+    };
+    auto at = [&](int q) { return scale(nb[q][n], in[q]); };
+    const C c = line[n], zm = zat(-1), zp = zat(1), xm = at(1), xp = at(2), ym = at(5), yp = at(6);
+    float kin;   // c . Lap c (the kinetic energy is -1/2 its sum), or |grad c|^2 (+1/2)
+    if (!a.kinetic5) {
+      const float lre = (xm.re - 2.0f * c.re + xp.re) * a.kin_f[0] + (ym.re - 2.0f * c.re + yp.re) * a.kin_f[1] +
+                        (zm.re - 2.0f * c.re + zp.re) * a.kin_f[2];
+      const float lim = (xm.im - 2.0f * c.im + xp.im) * a.kin_f[0] + (ym.im - 2.0f * c.im + yp.im) * a.kin_f[1] +
+                        (zm.im - 2.0f * c.im + zp.im) * a.kin_f[2];
+      kin = fmaf(c.re, lre, c.im * lim);
+    } else {
+      // 4th-order first derivatives (f(-2) - 8 f(-1) + 8 f(1) - f(2)) / (12 h), zero outside
+      const C zm2 = zat(-2), zp2 = zat(2), xm2 = at(0), xp2 = at(3), ym2 = at(4), yp2 = at(7);
+      auto d1 = [](C m2, C m1, C p1, C p2, float f) {
+        const float re = (m2.re - 8.0f * m1.re + 8.0f * p1.re - p2.re) * f;
+        const float im = (m2.im - 8.0f * m1.im + 8.0f * p1.im - p2.im) * f;
+        return fmaf(re, re, im * im);
+      };
+      kin = d1(xm2, xm, xp, xp2, a.kin_f[0]) + d1(ym2, ym, yp, yp2, a.kin_f[1]) + d1(zm2, zm, zp, zp2, a.kin_f[2]);
+    }
+    const float w = (float)quad_weight3(n, nz, a.simpson), d = w * fmaf(c.re, c.re, c.im * c.im);
+    const int kk = n - nz / 2;
+    t[0].add(d);
+    t[1].add(w * kin);
+    t[2].add(d * fmaf(c.re, c.re, c.im * c.im));
+    t[3].add(phi * d);
+    t[4].add_prod((float)(kk * kk), d);
+  }
+  __device__ __forceinline__ void end() {
+    const int jj = j - a.ny / 2, ii = i - a.nx / 2, W = quad_weight3(i, a.nx, a.simpson) * quad_weight3(j, a.ny, a.simpson);
+    const float w = (float)W;   // (W <= 16, the squares <= 2^16: exact)
+#pragma unroll
+    for (int q = 0; q < 4; ++q) v[q].add_scaled(w, t[q]);
+    v[4].add_scaled((float)(ii * ii * W), t[0]);
+    v[5].add_scaled((float)(jj * jj * W), t[0]);
+    v[6].add_scaled(w, t[4]);
+  }
+  __device__ __forceinline__ void finish() {
+    double s[8];
+    if (reduce_across_blocks<8>(v, s, a.partials, &a.state->ticket) && threadIdx.x == 0) {
+      const double ws = a.simpson ? 1.0 / 27.0 : 1.0;
+      const double X = s[4] * ws * a.hx * a.hx, Y = s[5] * ws * a.hy * a.hy, Z = s[6] * ws * a.hz * a.hz;
+      double o[8] = {s[0] * ws, (a.kinetic5 ? 0.5 : -0.5) * s[1] * ws, a.vx * X + a.vy * Y + a.vz * Z, a.g * s[2] * ws,
+                     a.gdd * s[3] * ws, X, Y, Z};
+      store_observables(a, o);
+    }
+  }
+};
+
 // ---------------------------------------------------------------------------------------
 // K5: the z-line kernel.  For kZLines lines (i, j0..): inverse half-spectrum transform
 // along z (C2R, two real lines per complex FFT; the imaginary parts of the kz = 0 and
@@ -2116,79 +2241,19 @@ __device__ __forceinline__ void k5_zline_body(const KArgs &a, const KArgs *ga) {
     const double wxi = quad_weight(i, a.nx, a.simpson);
     const R ihx2 = R(1.0 / (a.hx * a.hx)), ihy2 = R(1.0 / (a.hy * a.hy)), ihz2 = R(1.0 / (a.hz * a.hz));
     const C *gpsi = reinterpret_cast<const C *>(a.psi);
-    const size_t sx = (size_t)a.ny * nz;
+    [[maybe_unused]] const size_t sx = (size_t)a.ny * nz;
     if constexpr (std::is_same<R, float>::value) {
-      // FP32 data: each per-point term in FP32 (the state's precision); the weights exact small
-      // integers (3 x the Simpson weights per axis) and the squared coordinates exact integers
-      // (the signed index squared), every product by them exact (FMA exact product) and every
-      // sum in double-float per thread, as the x sweep's norm; h^2, (1/3)^3 and the physical
-      // factors applied in FP64 to the thread's totals.  The trap term needs no sum of its own:
-      // sum w V n = vx sum w x^2 n + vy sum w y^2 n + vz sum w z^2 n.  (FP64 work per point
-      // would bound this pass on GB300's FP64 pipe.)
-      DFAcc t[7];   // n, the kinetic term, n^2, Phi n, i'^2 n, j'^2 n, k'^2 n
-      const int wx = quad_weight3(i, a.nx, a.simpson), ii = i - a.nx / 2;
-      LinePos pos(threadIdx.x, nz, blockDim.x);
-      for (int e = threadIdx.x; e < nl * nz; e += blockDim.x, pos.next()) {
-        const int b = pos.b, n = pos.k;
-        const int j = j0 + b;
-        const int W = wx * quad_weight3(j, a.ny, a.simpson) * quad_weight3(n, nz, a.simpson);
-        if (W == 0) continue;
-        const C *row = tile + b * LS;
-        const C c = row[cn_slot(n, lc)];
-        const C zm = n > 0 ? row[cn_slot(n - 1, lc)] : czero<R>();
-        const C zp = n < nz - 1 ? row[cn_slot(n + 1, lc)] : czero<R>();
-        const size_t q = (line0 + b) * nz + n;
-        const C ym = j > 0 ? gpsi[q - nz] : czero<R>();
-        const C yp = j < a.ny - 1 ? gpsi[q + nz] : czero<R>();
-        const C xm = i > 0 ? gpsi[q - sx] : czero<R>();
-        const C xp = i < a.nx - 1 ? gpsi[q + sx] : czero<R>();
-        float kin;   // c . Lap c (the kinetic energy is -1/2 its sum), or |grad c|^2 (+1/2)
-        if (!a.kinetic5) {
-          const float lre = (xm.re - 2.0f * c.re + xp.re) * ihx2 + (ym.re - 2.0f * c.re + yp.re) * ihy2 +
-                            (zm.re - 2.0f * c.re + zp.re) * ihz2;
-          const float lim = (xm.im - 2.0f * c.im + xp.im) * ihx2 + (ym.im - 2.0f * c.im + yp.im) * ihy2 +
-                            (zm.im - 2.0f * c.im + zp.im) * ihz2;
-          kin = fmaf(c.re, lre, c.im * lim);
-        } else {
-          // 4th-order first derivatives (f(-2) - 8 f(-1) + 8 f(1) - f(2)) / (12 h), zero outside
-          const C zm2 = n > 1 ? row[cn_slot(n - 2, lc)] : czero<R>();
-          const C zp2 = n < nz - 2 ? row[cn_slot(n + 2, lc)] : czero<R>();
-          const C ym2 = j > 1 ? gpsi[q - 2 * nz] : czero<R>();
-          const C yp2 = j < a.ny - 2 ? gpsi[q + 2 * nz] : czero<R>();
-          const C xm2 = i > 1 ? gpsi[q - 2 * sx] : czero<R>();
-          const C xp2 = i < a.nx - 2 ? gpsi[q + 2 * sx] : czero<R>();
-          auto d1 = [](C m2, C m1, C p1, C p2, float f) {
-            const float re = (m2.re - 8.0f * m1.re + 8.0f * p1.re - p2.re) * f;
-            const float im = (m2.im - 8.0f * m1.im + 8.0f * p1.im - p2.im) * f;
-            return fmaf(re, re, im * im);
-          };
-          kin = d1(xm2, xm, xp, xp2, float(1.0 / (12.0 * a.hx))) + d1(ym2, ym, yp, yp2, float(1.0 / (12.0 * a.hy))) +
-                d1(zm2, zm, zp, zp2, float(1.0 / (12.0 * a.hz)));
+      ObsSums t(a, i);   // (short lines only: the others take dgpe_stages.cuh's kernel)
+      for (int b = threadIdx.x; b < nl; b += blockDim.x) {
+        t.begin(j0 + b);
+        for (int n = 0; n < nz; ++n) {
+          const C z = res[n * SB + (b >> 1)];
+          t.add(n, ((b & 1) ? z.im : z.re) * inv_ntot);
         }
-        const C z = res[n * SB + (b >> 1)];
-        const float phi = ((b & 1) ? z.im : z.re) * inv_ntot;
-        const float d = fmaf(c.re, c.re, c.im * c.im);
-        const int jj = j - a.ny / 2, kk = n - nz / 2;
-        const float wf = (float)W;
-        t[0].add_prod(wf, d);
-        t[1].add_prod(wf, kin);
-        t[2].add_prod(wf, d * d);
-        t[3].add_prod(wf, phi * d);
-        t[4].add_prod((float)(ii * ii * W), d);   // <= 256^2 x 64 = 2^22: exact
-        t[5].add_prod((float)(jj * jj * W), d);
-        t[6].add_prod((float)(kk * kk * W), d);
+        t.end();
       }
-      const double ws = a.simpson ? 1.0 / 27.0 : 1.0;
-      const double X = t[4].value() * ws * a.hx * a.hx, Y = t[5].value() * ws * a.hy * a.hy,
-                   Z = t[6].value() * ws * a.hz * a.hz;
-      v[0] = t[0].value() * ws;
-      v[1] = (a.kinetic5 ? 0.5 : -0.5) * t[1].value() * ws;
-      v[2] = a.vx * X + a.vy * Y + a.vz * Z;
-      v[3] = a.g * t[2].value() * ws;
-      v[4] = a.gdd * t[3].value() * ws;
-      v[5] = X;
-      v[6] = Y;
-      v[7] = Z;
+      t.finish();
+      return;
     } else {
       LinePos pos(threadIdx.x, nz, blockDim.x);
       for (int e = threadIdx.x; e < nl * nz; e += blockDim.x, pos.next()) {
@@ -2242,29 +2307,7 @@ __device__ __forceinline__ void k5_zline_body(const KArgs &a, const KArgs *ga) {
       }
     }
     double tot[8];
-    if (reduce_across_blocks<8>(v, tot, a.partials, &a.state->ticket) && threadIdx.x == 0) {
-      for (int q = 0; q < 8; ++q) v[q] = tot[q];
-      const double dv = a.hx * a.hy * a.hz;
-      DevState *st = a.state;
-      const double s2 = st->s * st->s;
-      for (int q = 0; q < 8; ++q) v[q] *= q == 3 ? s2 * s2 : s2;
-      for (int q = 0; q < 8; ++q) st->sums[q] = v[q];
-      const double norm = dv * v[0];
-      const double ekin = dv * v[1], etrap = dv * v[2], econ = 0.5 * dv * v[3], edd = 0.5 * dv * v[4];
-      st->obs[0] = norm;
-      st->obs[1] = dv * (v[1] + v[2] + v[3] + v[4]) / norm;
-      st->obs[2] = ekin + etrap + econ + edd;
-      st->obs[3] = sqrt(v[5] / v[0]);
-      st->obs[4] = sqrt(v[6] / v[0]);
-      st->obs[5] = sqrt(v[7] / v[0]);
-      st->obs[6] = ekin;
-      st->obs[7] = etrap;
-      st->obs[8] = econ;
-      st->obs[9] = edd;
-      bool finite = true;
-      for (int q = 0; q < 10; ++q) finite = finite && isfinite(st->obs[q]);
-      if (!finite) st->flags |= kFlagNonFinite;
-    }
+    if (reduce_across_blocks<8>(v, tot, a.partials, &a.state->ticket) && threadIdx.x == 0) store_observables(a, tot);
     return;
   }
 
@@ -3327,6 +3370,7 @@ struct Impl {
   }
   static cudaError_t k1(const KArgs &a, cudaStream_t st) {
     if (kFixed && fx_run(kK1DensityR2Cz, a, st)) return cudaGetLastError();
+    if (kRegFft && staged(a, 2) && stage_z(kK1DensityR2Cz, a, nullptr, 1, st)) return cudaGetLastError();
     // (instances of other tile heights, ztile_lines, get their own grid and shared memory)
     auto go = [&](auto len) {
       constexpr int N = decltype(len)::value;
@@ -3354,7 +3398,7 @@ struct Impl {
   }
   // the staged FP32 transforms: where the radix order is the default one, outside the
   // differentiation calls
-  static bool staged(const KArgs &a, int d) { return !a.diff && plan_ct(a.plan[d], d == 0 ? a.nx : a.ny); }
+  static bool staged(const KArgs &a, int d) { return !a.diff && plan_ct(a.plan[d], d == 0 ? a.nx : d == 1 ? a.ny : a.nz); }
   // the register-resident FP32 transforms (default plans of length 128, 256, 512)
   static constexpr bool kRegFft = std::is_same<R, float>::value;
   static constexpr size_t kRegYSmem = 2 * (256 / 64) * (size_t)RegFft<512>::SLOTS * sizeof(cplx<float>);
@@ -3458,6 +3502,7 @@ struct Impl {
     const size_t sm = smem_k5(a);
     if (zmode == kZFast) {
       if (kFixed && fx_run(kK5C2RzPhaseCnz, a, st)) return cudaGetLastError();
+      if (kRegFft && staged(a, 2) && stage_z(kK5C2RzPhaseCnz, a, nullptr, 1, st)) return cudaGetLastError();
       if (a.imag) k5_launch<kZFast, R>(a, g, sm, st);
       else k5_launch<kZFast, C>(a, g, sm, st);
       return cudaGetLastError();
@@ -3475,8 +3520,13 @@ struct Impl {
           else k5_zline<R, C, kZCnOnly, 0><<<g, T::kZThreads, sm, st>>>(a, nullptr);
         }
         break;
-      case kZPhi: k5_zline<R, R, kZPhi, 0><<<g, T::kZThreads, sm, st>>>(a, nullptr); break;
-      case kZObs: k5_zline<R, R, kZObs, 0><<<g, T::kZThreads, sm, st>>>(a, nullptr); break;
+      case kZPhi:
+        if (kRegFft && staged(a, 2) && stage_z(kKMaterialize, a, nullptr, 1, st)) break;
+        k5_zline<R, R, kZPhi, 0><<<g, T::kZThreads, sm, st>>>(a, nullptr);
+        break;
+      case kZObs:
+        if (kRegFft && staged(a, 2) && stage_z(kKObs, a, nullptr, 1, st)) break;
+        k5_zline<R, R, kZObs, 0><<<g, T::kZThreads, sm, st>>>(a, nullptr); break;
       default: return cudaErrorInvalidValue;
     }
     return cudaGetLastError();
@@ -3582,7 +3632,8 @@ struct Impl {
     const int bz = (int)(z.x * z.y);
     const int bx = (a.ny * a.nz + 7) / 8;   // the FP32 x sweep's tiles of at least 8 columns
     const int bt = (int)(((long long)a.ny * a.nz + 63) / 64);   // the two-thread sweep along x
-    return std::max(bz, std::max(bx, bt));
+    const int bo = std::is_same<R, float>::value ? (a.ny + 7) / 8 * a.nx : 0;   // the FP32 observables' tiles
+    return std::max(std::max(bz, bo), std::max(bx, bt));
   }
 
   static const KernelSet *set() {
@@ -3710,7 +3761,7 @@ struct GroupLaunch {
     else if (I::plan_ct(a.plan[2], 128) && a.cn8z_tab) go(integral_constant<int, 128>{});
     else if (I::plan_ct(a.plan[2], 96) && a.cn8z_tab) go(integral_constant<int, 96>{});
     else if (I::plan_ct(a.plan[2], 64) && a.cn8z_tab) go(integral_constant<int, 64>{});
-    else go(integral_constant<int, 0>{});
+    else if (!I::staged(a, 2) || !stage_z(kK5C2RzPhaseCnz, a, ga, n, st)) go(integral_constant<int, 0>{});
   }
   static cudaError_t step(const KArgs &a, const KArgs *ga, int count, int renorm, cudaStream_t st) {
     if (count < 1 || count > 65535) return cudaErrorInvalidValue;
@@ -3730,7 +3781,7 @@ struct GroupLaunch {
       else if (I::plan_ct(a.plan[2], 128)) go(integral_constant<int, 128>{});
       else if (I::plan_ct(a.plan[2], 96)) go(integral_constant<int, 96>{});
       else if (I::plan_ct(a.plan[2], 64)) go(integral_constant<int, 64>{});
-      else go(integral_constant<int, 0>{});
+      else if (!I::staged(a, 2) || !stage_z(kK1DensityR2Cz, a, ga, n, st)) go(integral_constant<int, 0>{});
     }
     ffty<-1>(a, ga, n, st);
     k3(a, ga, n, st);

@@ -517,7 +517,6 @@ DGPE_HD int fx_key(cplx<R> z) {
 }
 
 // ---- plans: the radices of the staged transforms (dgpe_stages.cuh) ---------------------------
-#define DGPE_FIXED_LENGTHS(X) X(128) X(256) X(512) DGPE_STAGE_LENGTHS(X)
 template <int N>
 struct FxPlan {
   using S = Stages<N>;
@@ -1386,7 +1385,7 @@ constexpr int fx_index(int n) {
 #define DGPE_AT(m) \
   if (m == n) at = i; \
   ++i;
-  DGPE_FIXED_LENGTHS(DGPE_AT)
+  DGPE_STAGE_ALL(DGPE_AT)
 #undef DGPE_AT
   return at;
 }
@@ -1402,7 +1401,7 @@ struct FxLaunch {
       return true; \
     } \
     break;
-      DGPE_FIXED_LENGTHS(DGPE_CASE)
+      DGPE_STAGE_ALL(DGPE_CASE)
 #undef DGPE_CASE
       default: break;
     }
@@ -1432,7 +1431,7 @@ struct FxLaunch {
   static cudaError_t init(int nx, int ny, int nz) {
     cudaError_t e = cudaSuccess;
     auto opt = [&](auto k, size_t sm) {
-      if (e == cudaSuccess && sm > 48 * 1024 - 512) e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+      if (e == cudaSuccess && sm > 40 * 1024) e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
     };
     with(nx, [&](auto len) { opt(k3_fx<R, decltype(len)::value>, FxX<decltype(len)::value>::smem); });
     with(ny, [&](auto len) {

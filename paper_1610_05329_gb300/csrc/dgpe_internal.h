@@ -107,18 +107,19 @@ struct KArgs {
                                // as 64-bit integers where nx has a fixed-point transform
   void *ybuf;                  // forward-elimination scratch of the FP64 sweeps (fx_scratch(nx ny nz)
                                // values of 16 bytes)
+  float kin_f[3];              // 1/h_d^2, or 1/(12 h_d) with kinetic5 (FP32 observables)
   float kf[3];                 // 2 pi / (n_d h_d): wavenumber per frequency index (FP32 K3)
   DevState *state;
   double *partials;            // per-block reduction partials
-  const void *tw_st[3];        // twiddles of the staged transforms (FP32: x and y, dgpe_stages.cuh; FP64-class:
-                               // x, y and z in fixed point, dgpe_fixed.cuh)
+  const void *tw_st[3];        // twiddles of the staged transforms (FP32: dgpe_stages.cuh; FP64-class:
+                               // in fixed point, dgpe_fixed.cuh)
   int diff;                    // 1: within the differentiation calls (FP32: the transforms and chunks whose
                                // roundings their results rest on)
   const void *tw[3];           // per-stage twiddle tables of plan[d] (layout in FftPlan), d = x, y, z
   FftPlan plan[3];
   CnTab cn[3];
   const void *cnz_tab;         // K5's z tables at k5_chunk(nz) points per lane, where that is not
-                               // cn[2].chunk (FP32, compile-time nz); else null
+                               // cn[2].chunk (FP32, the kernels compiled for nz); else null
   const void *cn8z_tab;        // K5's z tables in the 8-lane layout (FP32, k5_short_z(nz)); else null
   void *out;                   // optional output (Phi for get_phi)
   // adjoint step
@@ -197,34 +198,44 @@ struct KernelSet {
   cudaError_t (*step_group)(const KArgs &a, const KArgs *ga, int n, int renorm, cudaStream_t st);
 };
 
-// The staged FP32 transforms of the general line lengths (dgpe_stages.cuh), the lengths spread
-// over four translation units: y transforms (dir = -1, +1) and x transforms with the dipolar
-// kernel for `members` condensates (ga their arguments in device memory, or null for one); false
-// where the unit has no kernel of that length.
+// The staged FP32 kernels of the general line lengths (dgpe_stages.cuh), the lengths spread over
+// eight translation units: y transforms (dir = -1, +1), x transforms with the dipolar kernel, and
+// K1, K5's step, the observables or Phi along z (which = kK1DensityR2Cz, kK5C2RzPhaseCnz, kKObs,
+// kKMaterialize), for `members`
+// condensates (ga their arguments in device memory, or null for one); false where there is no
+// kernel of that length.
+#define DGPE_STAGE_UNITS(X) X(0) X(1) X(2) X(3) X(4) X(5) X(6) X(7)
 #define DGPE_STAGE_UNIT(i)                                                                              \
   bool stage_y##i(int dir, const KArgs &a, const KArgs *ga, unsigned members, cudaStream_t st);         \
   bool stage_x##i(const KArgs &a, const KArgs *ga, unsigned members, cudaStream_t st);                  \
-  cudaError_t stage_init##i(int nx, int ny);
-DGPE_STAGE_UNIT(0)
-DGPE_STAGE_UNIT(1)
-DGPE_STAGE_UNIT(2)
-DGPE_STAGE_UNIT(3)
+  bool stage_z##i(int which, const KArgs &a, const KArgs *ga, unsigned members, cudaStream_t st);       \
+  cudaError_t stage_init##i(int nx, int ny, int nz);
+DGPE_STAGE_UNITS(DGPE_STAGE_UNIT)
 #undef DGPE_STAGE_UNIT
 inline bool stage_y(int dir, const KArgs &a, const KArgs *ga, unsigned members, cudaStream_t st) {
-  return stage_y0(dir, a, ga, members, st) || stage_y1(dir, a, ga, members, st) ||
-         stage_y2(dir, a, ga, members, st) || stage_y3(dir, a, ga, members, st);
+#define DGPE_STAGE_OR(i) || stage_y##i(dir, a, ga, members, st)
+  return false DGPE_STAGE_UNITS(DGPE_STAGE_OR);
+#undef DGPE_STAGE_OR
 }
 inline bool stage_x(const KArgs &a, const KArgs *ga, unsigned members, cudaStream_t st) {
-  return stage_x0(a, ga, members, st) || stage_x1(a, ga, members, st) || stage_x2(a, ga, members, st) ||
-         stage_x3(a, ga, members, st);
+#define DGPE_STAGE_OR(i) || stage_x##i(a, ga, members, st)
+  return false DGPE_STAGE_UNITS(DGPE_STAGE_OR);
+#undef DGPE_STAGE_OR
 }
-inline cudaError_t stage_init(int nx, int ny) {
-  cudaError_t e = stage_init0(nx, ny);
-  if (e == cudaSuccess) e = stage_init1(nx, ny);
-  if (e == cudaSuccess) e = stage_init2(nx, ny);
-  if (e == cudaSuccess) e = stage_init3(nx, ny);
+inline bool stage_z(int which, const KArgs &a, const KArgs *ga, unsigned members, cudaStream_t st) {
+#define DGPE_STAGE_OR(i) || stage_z##i(which, a, ga, members, st)
+  return false DGPE_STAGE_UNITS(DGPE_STAGE_OR);
+#undef DGPE_STAGE_OR
+}
+inline cudaError_t stage_init(int nx, int ny, int nz) {
+  cudaError_t e = cudaSuccess;
+#define DGPE_STAGE_INIT(i) \
+  if (e == cudaSuccess) e = stage_init##i(nx, ny, nz);
+  DGPE_STAGE_UNITS(DGPE_STAGE_INIT)
+#undef DGPE_STAGE_INIT
   return e;
 }
+bool stage_own_z(int n);   // K1 and K5's step of z lines of n points are the staged ones
 // the twiddles of length n (2 n values; nothing where n has no staged transform)
 cudaError_t stage_tables(void *tw, int n, cudaStream_t st);
 

@@ -1,6 +1,6 @@
 // FP32 transforms of the general line lengths 2^a 3^b 5^c 7^d (12 .. 512) in two or three
-// stages of radix 2 .. 10, every length its own instance: the y transforms (K2, K4) and the x
-// transforms with the dipolar kernel between them (K3).
+// stages of radix 2 .. 10, every length its own instance: the y transforms (K2, K4), the x
+// transforms with the dipolar kernel between them (K3), and K1 and K5 with the z transforms.
 //
 // The runtime-length transforms of dgpe_device.cuh take four to five radix-2/3/4/5/7/8 stages
 // with every index computed at run time (about 85 instructions per element at 480 = 8 4 3 5),
@@ -103,6 +103,10 @@ __host__ __device__ constexpr int st_radix(int n, int s) {
   X(72) X(80) X(84) X(90) X(96) X(98) X(100) X(108) X(112) X(120) X(126) X(140) X(144) X(150) X(160) X(162) X(168) \
   X(180) X(192) X(196) X(200) X(210) X(216) X(224) X(240) X(250) X(252) X(270) X(280) X(288) X(294) X(300) X(320) \
   X(324) X(336) X(350) X(360) X(378) X(384) X(392) X(400) X(420) X(432) X(448) X(450) X(480) X(486) X(490) X(500) X(504)
+
+// and with those: the lengths of the z kernels
+#define DGPE_STAGE_ALL(X) X(128) X(256) X(512) DGPE_STAGE_LENGTHS(X)
+constexpr bool st_xy(int n) { return n != 128 && n != 256 && n != 512; }
 
 template <int N>
 struct Stages {
@@ -330,6 +334,280 @@ __global__ void __launch_bounds__(StageX<N>::NT) k3_st(const __grid_constant__ K
   }
 }
 
+// ---- K1 and K5 ------------------------------------------------------------------------------
+// z lines (K1 and K5's step: of the lengths that have no kernel in dgpe_device.cuh, 64, 96, 128, 256,
+// 384 and 512 have), in tiles of 2 PZ real lines packed in pairs.
+// Two or three stages instead of the four or five of the runtime lengths, the first one reading global
+// memory and the last one feeding the potential step, Phi or the observables in registers; the L2
+// prefetch of the tile kernels.  Bound by latency at 16 to 24 warps per SM.  us, runtime-length kernels
+// -> these: a step at 480x480x500 (imaginary time) 4.05 -> 3.03 ms, K1 343 there (of 204 at the copy
+// bandwidth), K5 938 (of 340); observables at 384x360x320 (5-point gradient) 829 -> 728, Phi 250 -> 116.
+template <int N>
+struct StageZ {
+  using S = Stages<N>;
+  static constexpr bool kOwn = N != 64 && N != 96 && N != 128 && N != 256 && N != 384 && N != 512;
+  static constexpr int NT = 256;
+  static constexpr int P1 = N <= 64 ? 16 : 8;     // pairs per K1 tile: rows of 128 bytes of the spectrum
+  static constexpr int P5 = N <= 64 ? 16 : N <= 256 ? 8 : 4;   // per K5 tile: two or three CTAs per SM
+  static constexpr int PL = S::R3 > 1 ? S::R3 : S::R2, NBL = N / PL;
+  static constexpr int TWL = S::R3 > 1 ? S::R1 * (S::R2 - 1) : 0;
+  static constexpr int SLOTS = st_slots<S::R1, S::R2, S::R3, 16>() > N ? st_slots<S::R1, S::R2, S::R3, 16>() : N;
+  // line stride: PZ lines by 16 / PZ elements on distinct banks
+  __host__ __device__ static constexpr int stride(int pz) { return pz == 16 ? SLOTS | 1 : SLOTS + (16 / pz - SLOTS % 16 + 16) % 16; }
+  static constexpr size_t smem1 = 2 * (size_t)P1 * stride(P1) * sizeof(cplx<float>);
+  // K5: chunk of the z solve (32 lanes per line, padded to 32 chunks), the solve's tile, which lies
+  // over the second transform buffer
+  static constexpr int CH = k5_chunk(N);
+  static constexpr int LS = (32 * CH + 34) | 1;
+  static constexpr int kTile = 2 * P5 * LS > P5 * stride(P5) ? 2 * P5 * LS : P5 * stride(P5);
+  static constexpr int kRes5 = CH > 10 ? 2 : 3;   // K5 CTAs per SM (registers)
+  static constexpr size_t smem5 = ((size_t)P5 * stride(P5) + kTile + 10 * kWarp) * sizeof(cplx<float>);
+};
+
+// the middle of three stages and the last one of a tile of np <= PZ lines; out(line, j, v): elements
+// j + s NBL of the result
+template <int DIR, int N, int NT, int SL>
+__device__ __forceinline__ void st_middle_z(const cplx<float> *x0, cplx<float> *y0, const cplx<float> *tw, int np) {
+  using C = cplx<float>;
+  using S = Stages<N>;
+  constexpr int R1 = S::R1, R2 = S::R2, NB = N / R2, GAP = st_pad2_gap<R1, R2, 16>();
+  for (int it = threadIdx.x; it < np * NB; it += NT) {
+    const int l = it / NB, j = it - l * NB, jb = j / R1, k = j - jb * R1;
+    const C *x = x0 + l * SL + st_pad1<R1>(j);
+    C v[R2];
+#pragma unroll
+    for (int r = 0; r < R2; ++r) v[r] = x[st_pad1<R1>(r * NB)];
+    st_twiddle<DIR, R2, R1>(v, tw, k);
+    bf<float, DIR, R2>(v);
+    C *y = y0 + l * SL + jb * (R1 * R2 + GAP) + k;
+#pragma unroll
+    for (int s = 0; s < R2; ++s) y[s * R1] = v[s];
+  }
+}
+template <int DIR, int N, int NT, int SL, typename Out>
+__device__ __forceinline__ void st_last_z(const cplx<float> *x0, const cplx<float> *tw, int np, Out out) {
+  using C = cplx<float>;
+  using Z = StageZ<N>;
+  constexpr int R1 = Z::S::R1, PL = Z::PL, NB = Z::NBL, GAP = st_pad2_gap<R1, Z::S::R2, 16>();
+  for (int it = threadIdx.x; it < np * NB; it += NT) {
+    const int l = it / NB, j = it - l * NB;
+    const C *x = x0 + l * SL + (Z::S::R3 > 1 ? j : st_pad1<R1>(j));
+    C v[PL];
+#pragma unroll
+    for (int r = 0; r < PL; ++r) v[r] = x[Z::S::R3 > 1 ? r * (NB + GAP) : st_pad1<R1>(r * NB)];
+    st_twiddle<DIR, PL, NB>(v, tw + Z::TWL, j);
+    bf<float, DIR, PL>(v);
+    out(l, j, v);
+  }
+}
+
+// K1: densities (with a factor 1/2), forward transform, separation of the two real spectra
+template <int N>
+__global__ void __launch_bounds__(StageZ<N>::NT) k1_st(const __grid_constant__ KArgs a0, const KArgs *ga) {
+  using C = cplx<float>;
+  using Z = StageZ<N>;
+  constexpr int R1 = Z::S::R1, PZ = Z::P1, SL = Z::stride(PZ), NT = Z::NT, NB = N / R1;
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  const KArgs &a = ga ? ga[blockIdx.z] : a0;
+  C *sa = reinterpret_cast<C *>(smem_raw), *sb = sa + PZ * SL;
+  const int i = blockIdx.y, j0 = blockIdx.x * (2 * PZ), np = min(2 * PZ, a.ny - j0) >> 1;
+  const C *psi = reinterpret_cast<const C *>(a.psi) + ((size_t)i * a.ny + j0) * N;
+  const float s2 = 0.5f * (a.unit_scale ? 1.0f : scale_sq_of<float>(a.state));
+  const C *tw = reinterpret_cast<const C *>(a.tw_st[2]);
+  {   // the psi rows of the CTA one resident wave ahead into L2
+    constexpr int kRes = (int)(225 * 1024 / (Z::smem1 + 1024)) < 6 ? (int)(225 * 1024 / (Z::smem1 + 1024)) : 6;
+    AheadTile t;
+    if (threadIdx.x == NT - 1 && ahead_tile(a, ga, kRes * a.nsm, t)) {
+      const int j2 = t.bx2 * 2 * PZ;
+      prefetch_l2(reinterpret_cast<const C *>(t.b->psi) + ((size_t)t.i2 * a.ny + j2) * N, min(2 * PZ, a.ny - j2) * N * (unsigned)sizeof(C));
+    }
+  }
+  for (int it = threadIdx.x; it < np * NB; it += NT) {
+    const int p = it / NB, j = it - p * NB;
+    const C *row = psi + (size_t)(2 * p) * N + j;
+    C v[R1];
+#pragma unroll
+    for (int r = 0; r < R1; ++r) {
+      const C x = row[r * NB], y = row[N + r * NB];
+      v[r] = {s2 * (x.re * x.re + x.im * x.im), s2 * (y.re * y.re + y.im * y.im)};
+    }
+    bf<float, -1, R1>(v);
+    C *q = sa + p * SL + st_pad1<R1>(j * R1);
+#pragma unroll
+    for (int s = 0; s < R1; ++s) q[s] = v[s];
+  }
+  __syncthreads();
+  if constexpr (Z::S::R3 > 1) {
+    st_middle_z<-1, N, NT, SL>(sa, sb, tw, np);
+    __syncthreads();
+  }
+  C *res = Z::S::R3 > 1 ? sa : sb;
+  st_last_z<-1, N, NT, SL>(Z::S::R3 > 1 ? sb : sa, tw, np, [&](int p, int j, const C *v) {
+#pragma unroll
+    for (int s = 0; s < Z::PL; ++s) res[p * SL + j + s * Z::NBL] = v[s];
+  });
+  __syncthreads();
+  C *spec = reinterpret_cast<C *>(a.spec) + (size_t)i * a.ny + j0;
+  const size_t plane = (size_t)a.nx * a.ny;
+  const int p = threadIdx.x % PZ;
+  if (p < np) {
+    for (int m = threadIdx.x / PZ; m <= N / 2; m += NT / PZ) {
+      const C zm = res[p * SL + m], zc = res[p * SL + (m ? N - m : 0)];
+      // (16-byte aligned: ny and j0 are even)
+      *reinterpret_cast<float4 *>(spec + m * plane + 2 * p) =
+          make_float4(zm.re + zc.re, zm.im - zc.im, zm.im + zc.im, zc.re - zm.re);
+    }
+  }
+}
+
+// K5: packing of the two half spectra, inverse transform (Phi); then the potential step and
+// Crank-Nicolson along z on the tile, or Phi as the output, or the observables' sums (psi from global
+// memory: a tile's own lines and their neighbours come from L1 and L2)
+enum StageZMode { kStStep, kStPhi, kStObs };
+template <int N, typename Coef, StageZMode MODE>
+__global__ void __launch_bounds__(StageZ<N>::NT, MODE == kStStep ? StageZ<N>::kRes5 : 3) k5_st(const __grid_constant__ KArgs a0, const KArgs *ga) {
+  using C = cplx<float>;
+  using Z = StageZ<N>;
+  constexpr int R1 = Z::S::R1, PZ = Z::P5, SL = Z::stride(PZ), NT = Z::NT, CH = Z::CH, LS = Z::LS;
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  const KArgs &a = ga ? ga[blockIdx.z] : a0;
+  C *sa = reinterpret_cast<C *>(smem_raw), *sb = sa + PZ * SL, *tile = sb;
+  Coef *scan_s = reinterpret_cast<Coef *>(sb + Z::kTile);
+  const int i = blockIdx.y, j0 = blockIdx.x * (2 * PZ), np = min(2 * PZ, a.ny - j0) >> 1;
+  const Coef *tab = reinterpret_cast<const Coef *>(a.cnz_tab ? a.cnz_tab : a.cn[2].tab);
+  if constexpr (MODE == kStStep)
+    for (int q = threadIdx.x; q < 10 * kWarp; q += NT) scan_s[q] = ldg(tab + 4 * kWarp * CH + q);
+  C *z0 = Z::S::R3 > 1 ? sa : sb, *z1 = Z::S::R3 > 1 ? sb : sa;   // the last stage reads sa
+  {
+    const C *spec = reinterpret_cast<const C *>(a.spec) + (size_t)i * a.ny + j0;
+    const size_t plane = (size_t)a.nx * a.ny;
+    const int p = threadIdx.x % PZ;
+    if (p < np) {
+#pragma unroll 4
+      for (int m = threadIdx.x / PZ; m <= N / 2; m += NT / PZ) {
+        const float4 x = *reinterpret_cast<const float4 *>(spec + m * plane + 2 * p);
+        const bool end = m == 0 || m == N / 2;   // real bins of a real field's spectrum
+        const float i1 = end ? 0.0f : x.y, i2 = end ? 0.0f : x.w;
+        z0[p * SL + m] = {x.x - i2, i1 + x.z};
+        if (!end) z0[p * SL + N - m] = {x.x + i2, x.z - i1};
+      }
+    }
+  }
+  {   // the rows of the CTA one resident wave ahead into L2
+    AheadTile t;
+    if (ahead_tile(a, ga, Z::kRes5 * a.nsm, t)) {
+      const int j2 = t.bx2 * 2 * PZ, nl2 = min(2 * PZ, a.ny - j2);
+      const size_t l2 = (size_t)t.i2 * a.ny + j2, plane = (size_t)a.nx * a.ny;
+      const C *sp2 = reinterpret_cast<const C *>(t.b->spec) + l2;
+      for (int m = threadIdx.x; m <= N / 2; m += NT) prefetch_l2(sp2 + m * plane, nl2 * (unsigned)sizeof(C));
+      if (MODE == kStStep && threadIdx.x == NT - 1)
+        prefetch_l2(reinterpret_cast<const C *>(t.b->psi) + l2 * N, nl2 * N * (unsigned)sizeof(C));
+    }
+  }
+  __syncthreads();
+  const C *tw = reinterpret_cast<const C *>(a.tw_st[2]);
+  {
+    constexpr int NB = N / R1;
+    for (int it = threadIdx.x; it < np * NB; it += NT) {
+      const int p = it / NB, j = it - p * NB;
+      C v[R1];
+#pragma unroll
+      for (int r = 0; r < R1; ++r) v[r] = z0[p * SL + j + r * NB];
+      bf<float, +1, R1>(v);
+      C *q = z1 + p * SL + st_pad1<R1>(j * R1);
+#pragma unroll
+      for (int s = 0; s < R1; ++s) q[s] = v[s];
+    }
+  }
+  __syncthreads();
+  if constexpr (Z::S::R3 > 1) {
+    st_middle_z<+1, N, NT, SL>(sb, sa, tw, np);
+    __syncthreads();
+  }
+  if constexpr (MODE == kStPhi) {
+    float *out = reinterpret_cast<float *>(a.out) + ((size_t)i * a.ny + j0) * N;
+    const float f = a.inv_ntot_f;
+    st_last_z<+1, N, NT, SL>(sa, tw, np, [&](int p, int j, const C *v) {
+#pragma unroll
+      for (int s = 0; s < Z::PL; ++s) {
+        out[(size_t)(2 * p) * N + j + s * Z::NBL] = v[s].re * f;
+        out[(size_t)(2 * p + 1) * N + j + s * Z::NBL] = v[s].im * f;
+      }
+    });
+  } else if constexpr (MODE == kStObs) {
+    constexpr int LP = N + 1;
+    float *phi = reinterpret_cast<float *>(sb);
+    const float f = a.inv_ntot_f;
+    st_last_z<+1, N, NT, SL>(sa, tw, np, [&](int p, int j, const C *v) {
+#pragma unroll
+      for (int s = 0; s < Z::PL; ++s) {
+        phi[2 * p * LP + j + s * Z::NBL] = v[s].re * f;
+        phi[(2 * p + 1) * LP + j + s * Z::NBL] = v[s].im * f;
+      }
+    });
+    __syncthreads();
+    ObsSums t(a, i);
+    for (int b = threadIdx.x / kWarp; b < 2 * np; b += NT / kWarp) {   // a warp per line
+      t.begin(j0 + b);
+      for (int n = threadIdx.x % kWarp; n < N; n += kWarp) t.add(n, phi[b * LP + n]);
+      t.end();
+    }
+    t.finish();
+  } else {
+    C *psi = reinterpret_cast<C *>(a.psi) + ((size_t)i * a.ny + j0) * N;
+    const float *dtv_y = reinterpret_cast<const float *>(a.dtv[1]) + j0, *dtv_z = reinterpret_cast<const float *>(a.dtv[2]);
+    const float dtvx = ldg(reinterpret_cast<const float *>(a.dtv[0]) + i);
+    const float sr = scale_of<float>(a.state);
+    const bool scaled = sr != 1.0f;
+    const float dtg = a.dtg_f, dtgdd = a.dtgdd_n_f;
+    constexpr bool IMAG = std::is_same<Coef, float>::value;
+    st_last_z<+1, N, NT, SL>(sa, tw, np, [&](int p, int j, const C *v) {
+      C w[2][Z::PL];
+#pragma unroll
+      for (int h = 0; h < 2; ++h)
+#pragma unroll
+        for (int s = 0; s < Z::PL; ++s) w[h][s] = psi[(size_t)(2 * p + h) * N + j + s * Z::NBL];
+      const float vy[2] = {dtvx + ldg(dtv_y + 2 * p), dtvx + ldg(dtv_y + 2 * p + 1)};
+#pragma unroll
+      for (int s = 0; s < Z::PL; ++s) {
+        const int n = j + s * Z::NBL;
+        const float vz = ldg(dtv_z + n);
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+          C z = w[h][s];
+          if (scaled) z = scale(z, sr);
+          const float dens = z.re * z.re + z.im * z.im;
+          const float theta = fmaf(dtg, dens, fmaf(dtgdd, h ? v[s].im : v[s].re, vy[h] + vz));
+          C o;
+          if constexpr (IMAG) {
+            o = scale(z, exp_r(-theta));
+          } else {
+            float sn, cs;
+            sin_cos(theta, &sn, &cs);
+            o = {z.re * cs + z.im * sn, z.im * cs - z.re * sn};
+          }
+          // slot of grid point n: one pad slot per chunk (the walls are zero)
+          if (n > 0 && n < N - 1) tile[(2 * p + h) * LS + n + (n - 1) / CH] = o;
+        }
+      }
+    });
+    // the padding past the last unknown
+    for (int q = threadIdx.x; q < 2 * np * (32 * CH + 2 - N); q += NT) {
+      const int b = q / (32 * CH + 2 - N > 0 ? 32 * CH + 2 - N : 1), n = N - 1 + q - b * (32 * CH + 2 - N);
+      tile[b * LS + n + (n - 1) / CH] = czero<float>();
+    }
+    __syncthreads();
+    const Coef c = CnCoef<float, Coef>::make(a.cn_rf[2]);
+    for (int b = threadIdx.x / kWarp; b < 2 * np; b += NT / kWarp)
+      cn_line<float, Coef, CH, false, true>(tile + b * LS, 1, kWarp * CH, 0, tab, scan_s, c);
+    __syncthreads();
+    for (int e = threadIdx.x; e < 2 * np * N; e += NT) {
+      const int b = e / N, n = e - b * N;
+      psi[e] = n > 0 && n < N - 1 ? tile[b * LS + n + (n - 1) / CH] : czero<float>();
+    }
+  }
+}
+
 // ---- set-up ---------------------------------------------------------------------------------
 // The twiddles of both orders of the plan of length n (layout above), by sincospi in FP64.
 __global__ inline void k_stage_twiddles(cplx<float> *tw, int n, int r1, int r2, int r3) {
@@ -353,13 +631,13 @@ __global__ inline void k_stage_twiddles(cplx<float> *tw, int n, int r1, int r2, 
 }
 
 // One translation unit's lengths: every kStageParts-th of the list.
-constexpr int kStageParts = 4;
+constexpr int kStageParts = 8;
 constexpr int st_index(int n) {
   int i = 0, at = -1;
 #define DGPE_AT(m) \
   if (m == n) at = i; \
   ++i;
-  DGPE_STAGE_LENGTHS(DGPE_AT)
+  DGPE_STAGE_ALL(DGPE_AT)
 #undef DGPE_AT
   return at;
 }
@@ -377,7 +655,7 @@ struct StageLaunch {
       return true; \
     } \
     break;
-      DGPE_STAGE_LENGTHS(DGPE_CASE)
+      DGPE_STAGE_ALL(DGPE_CASE)
 #undef DGPE_CASE
       default: break;
     }
@@ -388,8 +666,8 @@ struct StageLaunch {
     k<<<g, nt, sm, st>>>(a, ga);
   }
   static bool y(int dir, const KArgs &a, const KArgs *ga, unsigned members, cudaStream_t st) {
-    return with(a.ny, [&](auto len) {
-      constexpr int N = decltype(len)::value;
+    return st_xy(a.ny) && with(a.ny, [&](auto len) {
+      constexpr int N = st_xy(decltype(len)::value) ? decltype(len)::value : 12;
       using Y = StageY<N>;
       const dim3 g((a.nzh * a.nx + Y::L - 1) / Y::L, 1, members);
       if (dir < 0) k_ffty_st<-1, N><<<g, Y::NT, Y::smem, st>>>(a, ga);
@@ -397,22 +675,61 @@ struct StageLaunch {
     });
   }
   static bool x(const KArgs &a, const KArgs *ga, unsigned members, cudaStream_t st) {
-    return with(a.nx, [&](auto len) {
-      constexpr int N = decltype(len)::value;
+    return st_xy(a.nx) && with(a.nx, [&](auto len) {
+      constexpr int N = st_xy(decltype(len)::value) ? decltype(len)::value : 12;
       using X = StageX<N>;
       const dim3 g((a.ny + X::B - 1) / X::B, a.nzh, members);
       k3_st<N><<<g, X::NT, X::smem, st>>>(a, ga);
     });
   }
-  static cudaError_t init(int nx, int ny) {
+  // K1 (which = kK1DensityR2Cz), K5's step (kK5C2RzPhaseCnz), the observables (kKObs) or Phi
+  // (kKMaterialize)
+  static bool z(int which, const KArgs &a, const KArgs *ga, unsigned members, cudaStream_t st) {
+    bool done = false;
+    with(a.nz, [&](auto len) {
+      constexpr int N = decltype(len)::value;
+      using Z = StageZ<N>;
+      const dim3 g1((a.ny + 2 * Z::P1 - 1) / (2 * Z::P1), a.nx, members), g5((a.ny + 2 * Z::P5 - 1) / (2 * Z::P5), a.nx, members);
+      done = true;
+      if (which == kKObs) k5_st<N, float, kStObs><<<g5, Z::NT, Z::smem5, st>>>(a, ga);
+      else if (which == kKMaterialize) k5_st<N, float, kStPhi><<<g5, Z::NT, Z::smem5, st>>>(a, ga);
+      else if constexpr (Z::kOwn) {
+        if (which == kK1DensityR2Cz) k1_st<N><<<g1, Z::NT, Z::smem1, st>>>(a, ga);
+        else if (a.imag) k5_st<N, float, kStStep><<<g5, Z::NT, Z::smem5, st>>>(a, ga);
+        else k5_st<N, cplx<float>, kStStep><<<g5, Z::NT, Z::smem5, st>>>(a, ga);
+      } else {
+        done = false;
+      }
+    });
+    return done;
+  }
+  static cudaError_t init(int nx, int ny, int nz) {
     cudaError_t e = cudaSuccess;
     auto opt = [&](auto k, size_t sm) {
-      if (e == cudaSuccess && sm > 48 * 1024) e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+      // (48 KB less the reductions' static shared memory)
+      if (e == cudaSuccess && sm > 40 * 1024) e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
     };
-    with(nx, [&](auto len) { opt(k3_st<decltype(len)::value>, StageX<decltype(len)::value>::smem); });
+    with(nx, [&](auto len) {
+      constexpr int N = decltype(len)::value;
+      if constexpr (st_xy(N)) opt(k3_st<N>, StageX<N>::smem);
+    });
     with(ny, [&](auto len) {
-      opt(k_ffty_st<-1, decltype(len)::value>, StageY<decltype(len)::value>::smem);
-      opt(k_ffty_st<+1, decltype(len)::value>, StageY<decltype(len)::value>::smem);
+      constexpr int N = decltype(len)::value;
+      if constexpr (st_xy(N)) {
+        opt(k_ffty_st<-1, N>, StageY<N>::smem);
+        opt(k_ffty_st<+1, N>, StageY<N>::smem);
+      }
+    });
+    with(nz, [&](auto len) {
+      using Z = StageZ<decltype(len)::value>;
+      constexpr int N = decltype(len)::value;
+      opt(k5_st<N, float, kStPhi>, Z::smem5);
+      opt(k5_st<N, float, kStObs>, Z::smem5);
+      if constexpr (Z::kOwn) {
+        opt(k1_st<N>, Z::smem1);
+        opt(k5_st<N, float, kStStep>, Z::smem5);
+        opt(k5_st<N, cplx<float>, kStStep>, Z::smem5);
+      }
     });
     return e;
   }

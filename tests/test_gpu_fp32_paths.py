@@ -160,3 +160,33 @@ def test_dipolar_potential_of_every_length(orc, nx, ny):
         got = gpu.phi()
         gpu.close()
         assert rel(got, orc.dipolar_phi(p, np.abs(psi.astype(np.complex128)) ** 2)) < 3e-6
+
+
+@pytest.mark.parametrize("n", ALL)
+def test_z_lines_of_every_length(orc, n):
+    """The density transform, the potential step and z sweep, and the observables along z lines of
+    every length, a last tile of fewer lines among them.  Two steps: two transform chains (3e-6 of
+    Phi, times dt gdd Phi < 0.05), six sweeps (2e-6 each): 1.5e-5; the observables quadratic in it."""
+    shape = (4, 20, n)
+    h = (0.5, 0.4, 8.0 / n)
+    psi = (inputs.gaussian_psi(shape, h, noise=0.05, seed=n)).astype(np.complex64)
+    for mode in (abi.DGPE_REAL_TIME, abi.DGPE_IMAG_TIME):
+        for kinetic in (abi.DGPE_KINETIC_LAPLACIAN3, abi.DGPE_KINETIC_GRADIENT5):
+            # (Simpson in imaginary time: in real time FP32-mixed steps restore that norm, the oracle's do not)
+            simpson = kinetic and mode == abi.DGPE_IMAG_TIME
+            opt = {"integration": abi.DGPE_SIMPSON if simpson else abi.DGPE_RECTANGLE, "kinetic": kinetic}
+            gpu = abi.Condensate(shape, h, 0.004, mode=mode, precision=abi.DGPE_MIXED, nu=(1.0, 1.2, 0.8), g=5.0, gdd=3.0, **opt)
+            gpu.set_psi(psi)
+            gpu.step(2)
+            got, obs = gpu.get_psi(), gpu.observables()
+            gpu.close()
+            p = orc.make_params(shape, h, 0.004, orc.IMAG_TIME if mode else orc.REAL_TIME, (1.0, 1.2, 0.8), 5.0, 3.0, **opt)
+            want = orc.step(p, psi.astype(np.complex128), 2)
+            if mode == abi.DGPE_REAL_TIME:
+                assert rel(got, want) < 1.5e-5
+            else:
+                assert rel(got / np.linalg.norm(got), want / np.linalg.norm(want)) < 1.5e-5
+            ref = orc.observables(p, got.astype(np.complex128))
+            for k in ("norm", "mu", "energy", "e_kin", "e_trap", "e_contact", "rms_x", "rms_y", "rms_z"):
+                if k in obs and k in ref:
+                    assert obs[k] == pytest.approx(ref[k], rel=1e-5), k
