@@ -145,6 +145,16 @@ int check_physics(const dgpe_params *p) {
   return DGPE_OK;
 }
 
+// Double-float contexts of this many points and more run on the FP64 kernels (complex128 is their
+// boundary type too, and the fixed-point kernels keep 53 bits where pairs keep 48): us a step, pairs
+// against FP64, real time: 32^3 66 and 74, 48x64x40 97 and 87, 64^3 111 and 105, 128^3 312 and 268,
+// 256^3 1763 and 1670.
+constexpr size_t kFp64Points = 1 << 16;
+bool fp64_kernels(const dgpe_params *p) {
+  return p->precision == DGPE_FP64 || (p->precision == DGPE_DF64 && (size_t)p->nx * p->ny * p->nz >= kFp64Points);
+}
+bool pairs(const dgpe_params *p) { return p->precision == DGPE_DF64 && !fp64_kernels(p); }
+
 struct Layout {
   size_t state, partials, tw[3], tw_st[3], cn[3], cn_diff[2], cn_adj[3], cnz, cn8z, dtv[3], psi, spec, utab, ybuf, total;
 };
@@ -173,13 +183,13 @@ Layout layout_of(const dgpe_params *p, const KernelSet *ks, int max_blocks) {
   }
   for (int d = 0; d < 3; ++d) {   // the staged transforms' twiddles (FP64: in fixed point)
     L.tw_st[d] = off;
-    if (p->precision != DGPE_DF64) off += align_up(2 * (size_t)n[d] * e);
+    if (!pairs(p)) off += align_up(2 * (size_t)n[d] * e);
   }
   for (int d = 0; d < 3; ++d) {
     L.cn[d] = off;
     // lane-interleaved tables, scan factors, then the twist pivot of the two-thread sweeps
     // (FP64: and the fixed-point sweeps' coefficients)
-    const size_t fx = p->precision == DGPE_FP64 ? fx_cn_entries(n[d] - 2) : 0;
+    const size_t fx = fp64_kernels(p) ? fx_cn_entries(n[d] - 2) : 0;
     off += align_up(((size_t)(4 * axis_chunk(p, d) + 11) * kWarp + fx) * e);
     // the same at the chunk of the differentiation calls, and for dt -> -dt (adjoint)
     const int dc = p->precision == DGPE_MIXED && d < 2 ? diff_chunk(n[d]) : axis_chunk(p, d);
@@ -215,14 +225,14 @@ Layout layout_of(const dgpe_params *p, const KernelSet *ks, int max_blocks) {
   L.utab = off;   // FP64 and double-float (8-byte entries); the FP32 kernels evaluate it in place
   if (p->precision != DGPE_MIXED) off += align_up((size_t)(p->nz / 2 + 1) * p->nx * p->ny * 8);
   L.ybuf = off;   // the forward-elimination values of the FP64 per-line sweeps
-  if (p->precision == DGPE_FP64) off += align_up(fx_scratch((size_t)p->nx * p->ny * p->nz) * e);
+  if (fp64_kernels(p)) off += align_up(fx_scratch((size_t)p->nx * p->ny * p->nz) * e);
   L.total = off;
   (void)ks;
   return L;
 }
 
-const KernelSet *kernel_set(int precision) {
-  return precision == DGPE_FP64 ? kernels_f64() : precision == DGPE_DF64 ? kernels_df64() : kernels_f32();
+const KernelSet *kernel_set(const dgpe_params *p) {
+  return fp64_kernels(p) ? kernels_f64() : pairs(p) ? kernels_df64() : kernels_f32();
 }
 
 // d = f + l: f its FP32 rounding, l = fl32(d - f) (the double-float pair of d)
@@ -528,7 +538,7 @@ int setup_tables(dgpe_ctx *c, bool cn_changed, bool ut_changed) {
     jobs.job[jobs.n++] = {at(c, c->L.cnz), c->args.cn[2].m, k5_chunk(p->nz), c->args.cn_r[2], kWarp};
   if (jobs.n) {
     int rc = map_cuda(c->ks->cn_tables(jobs, c->stream));
-    if (!rc && p->precision == DGPE_FP64) rc = map_cuda(fx_cn_tables(jobs, c->stream));
+    if (!rc && fp64_kernels(p)) rc = map_cuda(fx_cn_tables(jobs, c->stream));
     if (rc) return rc;
   }
   if (ut_changed) return map_cuda(c->ks->dipolar_table(c->args, c->stream));
@@ -705,7 +715,7 @@ int dgpe_workspace_bytes(const dgpe_params *p, size_t *bytes) {
   int rc = check_shape(p);
   if (rc) return rc;
   // the block count of the reducing kernels depends only on shape and precision
-  const KernelSet *ks = kernel_set(p->precision);
+  const KernelSet *ks = kernel_set(p);
   *bytes = layout_of(p, ks, ks->max_blocks(base_args(p))).total;
   return DGPE_OK;
 }
@@ -726,7 +736,7 @@ int dgpe_create(const dgpe_params *p, void *cuda_stream, dgpe_ctx **out) {
   if (!c) return DGPE_ENOMEM;
   c->p = *p;
   c->restore_norm = p->precision == DGPE_MIXED;
-  c->ks = kernel_set(p->precision);
+  c->ks = kernel_set(p);
   c->stream = static_cast<cudaStream_t>(cuda_stream);
   c->args = base_args(p);
   set_physics(c->args, p);
@@ -741,8 +751,8 @@ int dgpe_create(const dgpe_params *p, void *cuda_stream, dgpe_ctx **out) {
   }
   rc = map_cuda(c->ks->init());
   if (!rc && p->precision == DGPE_MIXED) rc = map_cuda(stage_init(p->nx, p->ny, p->nz));
-  if (!rc && p->precision == DGPE_FP64) rc = map_cuda(fx_init(p->nx, p->ny, p->nz));
-  if (!rc && p->precision == DGPE_FP64) rc = map_cuda(fx_cn_init());
+  if (!rc && fp64_kernels(p)) rc = map_cuda(fx_init(p->nx, p->ny, p->nz));
+  if (!rc && fp64_kernels(p)) rc = map_cuda(fx_cn_init());
   if (!rc) rc = map_cuda(cudaStreamCreateWithFlags(&c->cap_stream, cudaStreamNonBlocking));
   if (!rc) {
     if (p->workspace) {
@@ -779,7 +789,7 @@ int dgpe_create(const dgpe_params *p, void *cuda_stream, dgpe_ctx **out) {
   for (int d = 0; d < 3 && !rc; ++d) {
     void *tw = at(c, c->L.tw_st[d]);
     a.tw_st[d] = tw;
-    if (p->precision == DGPE_FP64) rc = map_cuda(fx_tables(tw, n[d], c->stream));
+    if (fp64_kernels(p)) rc = map_cuda(fx_tables(tw, n[d], c->stream));
     else if (p->precision == DGPE_MIXED) rc = map_cuda(stage_tables(tw, n[d], c->stream));
   }
   if (!rc) rc = setup_tables(c, true, true);
@@ -823,7 +833,7 @@ int dgpe_set_psi(dgpe_ctx *c, const void *psi, int where) {
   const size_t n = (size_t)c->p.nx * c->p.ny * c->p.nz;
   const size_t bytes = n * c->ks->elem_bytes;
   int rc;
-  if (c->p.precision == DGPE_DF64) {
+  if (pairs(&c->p)) {
     // complex128 in, double-float pairs (same 16 bytes per value) in the workspace: copy,
     // then split in place
     rc = map_cuda(cudaMemcpyAsync(c->args.psi, psi, bytes,
@@ -845,7 +855,7 @@ int dgpe_get_psi(dgpe_ctx *c, void *out, int where) {
   const size_t bytes = (size_t)c->p.nx * c->p.ny * c->p.nz * c->ks->elem_bytes;
   int rc = launch(c, c->stream, kKMaterialize, [&] { return c->ks->materialize(c->args, c->stream); });
   if (rc) return rc;
-  if (c->p.precision == DGPE_DF64) {
+  if (pairs(&c->p)) {
     // double-float pairs -> complex128, through a stream-ordered temporary for a host buffer
     const size_t n = (size_t)c->p.nx * c->p.ny * c->p.nz;
     if (where == DGPE_DEVICE) {
@@ -1412,7 +1422,7 @@ int host_io_setup(dgpe_ctx *c) {
   // a failed earlier attempt keeps what it created (dgpe_destroy frees it); create the rest
   int rc = DGPE_OK;
   if (!c->psi_alt) rc = map_cuda(cudaMalloc(&c->psi_alt, bytes));
-  if (!rc && c->p.precision == DGPE_DF64 && !c->stage_out) rc = map_cuda(cudaMalloc(&c->stage_out, bytes));
+  if (!rc && pairs(&c->p) && !c->stage_out) rc = map_cuda(cudaMalloc(&c->stage_out, bytes));
   if (!rc && !c->cs_in) rc = map_cuda(cudaStreamCreateWithFlags(&c->cs_in, cudaStreamNonBlocking));
   if (!rc && !c->cs_out) rc = map_cuda(cudaStreamCreateWithFlags(&c->cs_out, cudaStreamNonBlocking));
   cudaEvent_t *ev[7] = {&c->ev_in_ready,    &c->ev_out_ready,   &c->ev_stage_free, &c->ev_main_done[0],
@@ -1451,7 +1461,7 @@ int dgpe_step_host(dgpe_ctx *c, const void *in, void *out, int nsteps) {
   if (rc) return rc;
   c->args.psi = buf[tgt];
   ++c->generation;   // batches holding this context capture its new buffer
-  if (c->p.precision == DGPE_DF64) rc = map_cuda(c->ks->from_c128(buf[tgt], buf[tgt], n, c->stream));
+  if (pairs(&c->p)) rc = map_cuda(c->ks->from_c128(buf[tgt], buf[tgt], n, c->stream));
   if (!rc) rc = map_cuda(c->ks->reset_state(c->args.state, c->stream));
   if (rc) return rc;
   c->latched = DGPE_OK;
@@ -1462,7 +1472,7 @@ int dgpe_step_host(dgpe_ctx *c, const void *in, void *out, int nsteps) {
   if (c->p.mode == DGPE_IMAG_TIME || c->restore_norm)
     rc = launch(c, c->stream, kKMaterialize, [&] { return c->ks->materialize(c->args, c->stream); });
   const void *src = buf[tgt];
-  if (!rc && c->p.precision == DGPE_DF64) {
+  if (!rc && pairs(&c->p)) {
     // pairs -> complex128 into the staging, once the previous output copy has left it
     rc = map_cuda(cudaStreamWaitEvent(c->stream, c->ev_stage_free, 0));
     if (!rc) rc = map_cuda(c->ks->to_c128(buf[tgt], c->stage_out, n, c->stream));
@@ -1473,7 +1483,7 @@ int dgpe_step_host(dgpe_ctx *c, const void *in, void *out, int nsteps) {
   if (!rc) rc = map_cuda(cudaStreamWaitEvent(c->cs_out, c->ev_out_ready, 0));
   if (!rc) rc = map_cuda(cudaMemcpyAsync(out, src, bytes, cudaMemcpyDeviceToHost, c->cs_out));
   if (!rc) rc = map_cuda(cudaEventRecord(c->ev_d2h_done[tgt], c->cs_out));
-  if (!rc && c->p.precision == DGPE_DF64) rc = map_cuda(cudaEventRecord(c->ev_stage_free, c->cs_out));
+  if (!rc && pairs(&c->p)) rc = map_cuda(cudaEventRecord(c->ev_stage_free, c->cs_out));
   return rc;
 }
 

@@ -2726,7 +2726,7 @@ __global__ void __launch_bounds__(kCnrThreads, 1) k_cn_reg(KArgs a, const KArgs 
   else k_cn_reg_body<Coef, AXIS, CH, PAIR>(a, reduce, renorm);
 }
 
-// FP64-class sweeps: two threads per line, the twisted ("burn at both ends") factorization.
+// Double-float sweeps: two threads per line, the twisted ("burn at both ends") factorization.
 // The matrix tridiag(-c, 1 + 2c, -c) reads the same from either end, so its UL factors are
 // its LU factors mirrored: the top thread eliminates points 0 .. h-1 downwards
 // (y_i = psi_i + alpha_i y_{i-1}), the bottom thread points m-1 .. h+1 upwards
@@ -2735,18 +2735,12 @@ __global__ void __launch_bounds__(kCnrThreads, 1) k_cn_reg(KArgs a, const KArgs 
 //   gamma x_h = psi_h + alpha_h y_{h-1} + alpha_{m-1-h} z_{h+1},
 //   gamma = e_h + e_{m-1-h} - (1 + 2c)   (e_i = 1/beta_i, the LU pivots; 1/gamma is stored
 // after the scan factors), then substitute back away from h: chi_i = beta_i (y_i + c chi_{i+1})
-// above, chi_i = beta_{m-1-i} (z_i + c chi_{i-1}) below, psi'_i = 2 chi_i - psi_i.  Twice the
-// threads of one thread per line: at 256^3 a sweep is 4096 warps, 6.7 per SM sub-partition
-// instead of 3.4, so the last partial round of warps idles a sub-partition for about 1/28 of
-// the sweep instead of 1/6.  A warp holds 16 lines: lanes 0-15 their top halves, lanes 16-31
-// their bottom halves.
-// FP64 (12 FP64 instructions per point) writes y and z to the scratch buffer and reads them
-// and psi back; double-float, whose step leans on HBM more, writes them over psi and
-// recovers psi_i = y_i - alpha_i y_{i-1} (z_i - alpha_{m-1-i} z_{i+1}) on the way back.
+// above, chi_i = beta_{m-1-i} (z_i + c chi_{i-1}) below, psi'_i = 2 chi_i - psi_i.  A warp holds 16
+// lines: lanes 0-15 their top halves, lanes 16-31 their bottom halves.  y and z are written over
+// psi, which is recovered on the way back: psi_i = y_i - alpha_i y_{i-1} (z_i - alpha_{m-1-i} z_{i+1}).
 template <typename R, typename Coef, int AXIS>
 __global__ void __launch_bounds__(128, 7) k_cn_twisted(KArgs a, int reduce, int renorm) {
   using C = cplx<R>;
-  constexpr bool kScratch = std::is_same<R, double>::value;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int N = AXIS == 0 ? a.nx : AXIS == 1 ? a.ny : a.nz;
   const int nfixed = AXIS == 0 ? a.ny : a.nx;
@@ -2768,9 +2762,7 @@ __global__ void __launch_bounds__(128, 7) k_cn_twisted(KArgs a, int reduce, int 
   // grid index i + 1 of interior point i
   C *p = reinterpret_cast<C *>(a.psi) +
          (AXIS == 2 ? (size_t)ln * a.nz : (AXIS == 1 ? (size_t)fixed * a.ny * a.nz : (size_t)fixed * a.nz) + k) + stride;
-  // FP64: y_i (z_i) of this line at yb[i * nlines], consecutive lines side by side
-  C *yb = kScratch ? reinterpret_cast<C *>(a.ybuf) + ln : nullptr;
-  auto elim = [&](int i) -> C & { return kScratch ? yb[(size_t)i * (size_t)nlines] : p[(size_t)i * stride]; };
+  auto elim = [&](int i) -> C & { return p[(size_t)i * stride]; };   // y_i (z_i), over psi_i
   const Coef *tab = reinterpret_cast<const Coef *>(a.cn[AXIS].tab);
   const int lc = a.cn[AXIS].lchunk, chunk = 1 << lc, mp = kWarp << lc, m = a.cn[AXIS].m, h = m / 2;
   const Coef c = CnCoef<R, Coef>::make(pick<R>(a.cn_r[AXIS], a.cn_rf[AXIS], a.cn_rl[AXIS]));
@@ -2822,18 +2814,12 @@ __global__ void __launch_bounds__(128, 7) k_cn_twisted(KArgs a, int reduce, int 
   {
     const int ib0 = bottom ? h + 1 : h - 1;
     const int tb0 = bottom ? m - 2 - h : h - 1;
-    // FP64: y_i and psi_i of the coming points; double-float: the eliminated value one point
-    // further on (psi_i is recovered from it), the current one carried in `cur`
-    C yr[kPf], pr[kScratch ? kPf : 1];
+    // the eliminated value one point further on (psi_i is recovered from it), the current one
+    // carried in `cur`
+    C yr[kPf];
 #pragma unroll
     for (int j = 0; j < kPf; ++j) {
-      if constexpr (kScratch) {
-        const int i = ib0 - dir * j;
-        yr[j] = j < nf ? elim(i) : czero<R>();
-        pr[j] = j < nf ? p[(ptrdiff_t)i * (ptrdiff_t)stride] : czero<R>();
-      } else {
-        yr[j] = j + 1 < nf ? elim(ib0 - dir * (j + 1)) : czero<R>();
-      }
+      yr[j] = j + 1 < nf ? elim(ib0 - dir * (j + 1)) : czero<R>();
     }
     C chi = xh, cur = y;
     for (int j0 = 0; j0 < nf; j0 += kPf) {
@@ -2843,22 +2829,10 @@ __global__ void __launch_bounds__(128, 7) k_cn_twisted(KArgs a, int reduce, int 
         if (j < nf) {
           const int i = ib0 - dir * j;
           const int q = slot(tb0 - j);
-          C yi, ps;
-          if constexpr (kScratch) {
-            yi = yr[jj];
-            ps = pr[jj];
-            if (j + kPf < nf) {
-              const int in = ib0 - dir * (j + kPf);
-              yr[jj] = elim(in);
-              pr[jj] = p[(ptrdiff_t)in * (ptrdiff_t)stride];
-            }
-          } else {
-            const C nxt = yr[jj];
-            if (j + 1 + kPf < nf) yr[jj] = elim(ib0 - dir * (j + 1 + kPf));
-            yi = cur;
-            ps = cfma(neg_coef(ldg(tab + q)), nxt, cur);
-            cur = nxt;
-          }
+          const C nxt = yr[jj];
+          if (j + 1 + kPf < nf) yr[jj] = elim(ib0 - dir * (j + 1 + kPf));
+          const C yi = cur, ps = cfma(neg_coef(ldg(tab + q)), nxt, cur);
+          cur = nxt;
           chi = mul(ldg(tab + mp + q), cfma_c(c, chi, yi));
           emit(i, C{twice_minus(chi.re, ps.re), twice_minus(chi.im, ps.im)});
         }
@@ -3131,8 +3105,8 @@ struct Impl {
   static constexpr bool kFixed = std::is_same<R, double>::value;
   // FP32 also at nz = 96 and 64 (K1, K5; the batched small grids)
   static constexpr bool kShortCt = std::is_same<R, float>::value;
-  // the FP64-class sweeps run a Thomas solve per line on two threads (k_cn_twisted), the
-  // FP32 ones the chunked solver in registers (k_cn_reg)
+  // the FP64-class sweeps run a Thomas solve per line on two threads (k_cn_fx, double-float
+  // k_cn_twisted), the FP32 ones the chunked solver in registers (k_cn_reg)
   static constexpr bool kCnThread = Fp64Class<R>::value;
   // and the z sweep too, after a phase-only K5 pass: the per-line solve's fewer arithmetic
   // instructions win over the extra pass through HBM
