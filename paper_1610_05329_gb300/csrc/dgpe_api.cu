@@ -420,8 +420,10 @@ int launch(dgpe_ctx *c, cudaStream_t st, int kernel, F &&f) {
   return DGPE_OK;
 }
 
+KArgs step_args(dgpe_ctx *c);
+
 int enqueue_potential_transforms(dgpe_ctx *c, cudaStream_t st) {
-  const KArgs &a = c->args;
+  const KArgs a = step_args(c);   // (the differentiation calls keep their transforms)
   const KernelSet *ks = c->ks;
   int rc;
   if ((rc = launch(c, st, kK1DensityR2Cz, [&] { return ks->k1(a, st); }))) return rc;
