@@ -365,17 +365,12 @@ def kernel_profile(c, steps, hbm_peak, peak_kind, workload):
     hbm = {"bound": "hbm", "kernel": top["kernel"], "achieved": top["achieved_gbs"], "peak": hbm_peak,
            "unit": "GB/s", "frac": top["frac_hbm"], "traffic": tr,
            "peak_kind": ("measured (MEASURED_PEAKS.json hbm_gbs)" if peak_kind == "measured" else "fallback")}
-    if wl["precision"] == "df64":
-        # FP64-class arithmetic on the FP32 pipe: the same algorithmic FP64 flops, compared
-        # with what the FP64 pipe could do at most
+    if wl["precision"] in ("fp64", "df64"):
+        # FP64-class arithmetic off the FP64 pipe (64-bit integers, or FP32 pairs): the algorithmic
+        # FP64 flops beside what the FP64 pipe could do at most
         roofline = dict(hbm, fp64_equivalent={"achieved": top["fp64_tflops"], "unit": "TFLOP/s",
                                               "fp64_pipe_peak": round(FP64_PEAK_TFLOPS, 4),
                                               "ratio_to_fp64_peak": top["frac_fp64"]})
-    elif wl["precision"] == "fp64":
-        roofline = {"bound": "alu", "kernel": top["kernel"], "achieved": top["fp64_tflops"],
-                    "peak": round(FP64_PEAK_TFLOPS, 4), "unit": "TFLOP/s", "frac": top["frac_fp64"],
-                    "traffic": tr, "peak_kind": "FP64 pipe: 152 SMs x 2 FMA/clk x 2 flops x 2.07 GHz",
-                    "hbm_view": hbm}
     else:
         roofline = hbm
     roofline["instrumented_ms_per_step"] = round(total / steps, 4)
