@@ -65,14 +65,20 @@ struct __align__(16) fxw {
   int rh, rl, ih, il;
 };
 // a w / 2^64 = a w / 16 (DIR < 0) or a conj(w) / 16, for components of a below 2^62 (|a| below
-// 2^62.5): the middle sums stay below 2^62 + 2^59.5.
+// 2^62.5): the middle sums stay below 2^62 + 2^60.  The products that count negative are subtracted
+// in 64 bits (a low word of -2^31 has no negative; a high one, at most 2^28, does).
 template <int DIR>
 DGPE_HD fxc fx_twiddle(fxc a, fxw w) {
   const int rh = fx_hi(a.re), rl = fx_lo(a.re), ih = fx_hi(a.im), il = fx_lo(a.im);
-  const int wih = DIR < 0 ? w.ih : -w.ih, wil = DIR < 0 ? w.il : -w.il;
-  const long long mr = fx_mad(rh, w.rl, fx_mad(rl, w.rh, fx_mad(ih, -wil, fx_mad(il, -wih, kFxHalf))));
-  const long long mi = fx_mad(rh, wil, fx_mad(rl, wih, fx_mad(ih, w.rl, fx_mad(il, w.rh, kFxHalf))));
-  return {fx_mad(rh, w.rh, fx_mad(ih, -wih, mr >> 32)), fx_mad(rh, wih, fx_mad(ih, w.rh, mi >> 32))};
+  if constexpr (DIR < 0) {
+    const long long mr = fx_mad(rh, w.rl, fx_mad(rl, w.rh, kFxHalf)) - fx_mad(ih, w.il, fx_mad(il, w.ih, 0));
+    const long long mi = fx_mad(rh, w.il, fx_mad(rl, w.ih, fx_mad(ih, w.rl, fx_mad(il, w.rh, kFxHalf))));
+    return {fx_mad(rh, w.rh, fx_mad(ih, -w.ih, mr >> 32)), fx_mad(rh, w.ih, fx_mad(ih, w.rh, mi >> 32))};
+  } else {
+    const long long mr = fx_mad(rh, w.rl, fx_mad(rl, w.rh, fx_mad(ih, w.il, fx_mad(il, w.ih, kFxHalf))));
+    const long long mi = fx_mad(ih, w.rl, fx_mad(il, w.rh, kFxHalf)) - fx_mad(rh, w.il, fx_mad(rl, w.ih, 0));
+    return {fx_mad(rh, w.rh, fx_mad(ih, w.ih, mr >> 32)), fx_mad(ih, w.rh, fx_mad(rh, -w.ih, mi >> 32))};
+  }
 }
 
 // ---- block scaling -------------------------------------------------------------------------
