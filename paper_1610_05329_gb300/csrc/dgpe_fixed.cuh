@@ -256,8 +256,8 @@ DGPE_HD void fx_bf(fxc *v) {
 
 // ---- FP64 <-> fixed point ----------------------------------------------------------------
 // The tile's exponent is the largest biased exponent emax of its values, at least kFxMinBiased (0x7ff:
-// some value is not finite, and the tile's results are NaN): x = v 2^(emax - 1080), |v| < 2^58, cut
-// off at bit 0; subnormal values, 2^-63 below the least tile exponent, are 0.
+// some value is not finite, and the tile's results are NaN): x = v 2^(emax - 1075 - UP), |v| < 2^(53 + UP)
+// (a tile's: 2^58), cut off at bit 0; subnormal values, 2^-63 below the least tile exponent, are 0.
 constexpr int kFxMinBiased = 64;
 DGPE_HD long long fx_bits(double x) {
 #ifdef __CUDA_ARCH__
@@ -278,11 +278,12 @@ DGPE_HD double fx_value(long long b) {
 #endif
 }
 DGPE_HD int fx_exponent_bits(double x) { return (int)(fx_bits(x) >> 32) & 0x7fffffff; }   // orders by exponent
+template <int UP = 5>
 DGPE_HD long long fx_from(double x, int emax) {
   const long long b = fx_bits(x);
   const int s = emax - ((int)(b >> 52) & 0x7ff);
   const unsigned long long m = ((unsigned long long)b & 0xfffffffffffffull) | 1ull << 52;
-  const long long v = (long long)((m << 5) >> (s < 63 ? s : 63));
+  const long long v = (long long)((m << UP) >> (s < 63 ? s : 63));
   const long long g = b >> 63;
   return (v ^ g) - g;
 }
@@ -307,7 +308,7 @@ DGPE_HD cplx<double> fx_to(fxc v, int exp) {
   return {fx_to_any(v.re, exp), fx_to_any(v.im, exp)};
 }
 // The same without the conversion instruction, for the kernels whose FP64 pipe has other work or whose
-// chains wait for it (halves round away from zero): about 20 integer instructions.
+// chains wait for it: about 20 integer instructions.
 DGPE_HD double fx_to_int(long long v, int exp) {
   const long long g = v >> 63;
   const unsigned long long a = (unsigned long long)((v ^ g) - g);
@@ -317,7 +318,8 @@ DGPE_HD double fx_to_int(long long v, int exp) {
   const int lz = a ? __builtin_clzll(a) : 64;
 #endif
   const int f = exp - lz - 1;   // the biased exponent less 1; the leading bit, at bit 52 below, adds it
-  unsigned long long b = (((a << ((lz - 1) & 63)) + 0x200) >> 10) + ((unsigned long long)(unsigned)f << 52);
+  const unsigned long long m = a << ((lz - 1) & 63);
+  unsigned long long b = ((m + 0x1ff + (((unsigned)m >> 10) & 1)) >> 10) + ((unsigned long long)(unsigned)f << 52);
   if ((unsigned)f >= 2046u || a == 0) b = f >= 2046 && a != 0 ? 0x7ff0000000000000ull : 0;
   return fx_value((long long)(b | ((unsigned long long)g & 0x8000000000000000ull)));
 }
@@ -327,58 +329,76 @@ DGPE_HD cplx<double> fx_to_int(fxc v, int exp) { return {fx_to_int(v.re, exp), f
 // The recurrences along a line keep every point's precision relative to that point (the tails of a
 // cloud as well as its middle), so the running value carries its own exponent: components just
 // below 2^62 (fx_up's range) after every step.
+// A long run repeats each rounding at each step, so none of them may lean to one side (the packing's
+// cut-off did: the phase of a state turned by 4e-17 a step, coherently).
 struct fxv {
   fxc v;
   int e;
 };
-constexpr int kFxMinExp = kFxMinBiased - 1080;   // (values below 2^-960 lose bits from here on)
+constexpr int kFxMinExp = kFxMinBiased - 1081;   // (values below 2^-960 lose bits from here on)
+DGPE_HD int fx_min(int a, int b) { return a < b ? a : b; }
+DGPE_HD long long fx_shl(long long a, int n) { return (long long)((unsigned long long)a << n); }
 DGPE_HD fxv fx_norm(fxc s, int e) {   // components of s below 2^62
 #ifdef __CUDA_ARCH__
   const int n = __clz(fx_mag(s)) - 2;
 #else
   const int mg = fx_mag(s), n = (mg ? __builtin_clz(mg) : 32) - 2;
 #endif
-  return {{(long long)((unsigned long long)s.re << n), (long long)((unsigned long long)s.im << n)}, e - n};
+  return {{fx_shl(s.re, n), fx_shl(s.im, n)}, e - n};
 }
-// a w / 16 for a coefficient w of magnitude at most 1 (words of w 2^60; real ones: rh, rl alone)
+// a w / 8 for a coefficient w of magnitude at most 1 (words of w 2^61; real ones: rh, rl alone): below
+// 2^59.5 for a normalised a
 template <bool CPLX>
 DGPE_HD fxc fx_coef(fxc a, fxw w) {
   if constexpr (CPLX) return fx_twiddle<-1>(a, w);
   else return {fx_mul(a.re, w.rh, w.rl), fx_mul(a.im, w.rh, w.rl)};
 }
-DGPE_HD long long fx_sar(long long a, int s) { return a >> (s < 63 ? s : 63); }
-// psi + p (p: components below 2^59, exponent ep; key: psi's exponent key), normalised
+constexpr int kFxCoefBits = 61;
+// a 2^-s, s >= 0, rounded (halves up)
+DGPE_HD long long fx_sar(long long a, int s) {
+#ifdef __CUDA_ARCH__
+  long long h;   // 2^(s - 1), 0 for s = 0 (shl.b64 gives 0 for amounts above 63)
+  asm("shl.b64 %0, 1, %1;" : "=l"(h) : "r"(min(s, 63) - 1));
+  return (a + h) >> min(s, 63);
+#else
+  const int k = s < 63 ? s : 63;
+  return (a + (k ? 1LL << (k - 1) : 0)) >> k;
+#endif
+}
+// psi + p (p: components below 2^60, exponent ep; key: psi's exponent key), normalised
 DGPE_HD fxv fx_forward(double re, double im, int key, fxc p, int ep) {
-  const int em = (key >> 20) - 1080;
+  const int em = (key >> 20) - 1081;
   int e = em > ep ? em : ep;
   if (e < kFxMinExp) e = kFxMinExp;
-  return fx_norm({fx_from(re, e + 1080) + fx_sar(p.re, e - ep), fx_from(im, e + 1080) + fx_sar(p.im, e - ep)}, e);
+  return fx_norm({fx_from<6>(re, e + 1081) + fx_sar(p.re, e - ep), fx_from<6>(im, e + 1081) + fx_sar(p.im, e - ep)}, e);
 }
-// y + p for a normalised y
+// y + p for an unpacked y (whose low bits are zero: its shift is exact unless p is far above it)
 DGPE_HD fxv fx_backward(fxv y, fxc p, int ep) {
-  const int e = y.e + 4 > ep ? y.e + 4 : ep;
-  return fx_norm({fx_sar(y.v.re, e - y.e) + fx_sar(p.re, e - ep), fx_sar(y.v.im, e - y.e) + fx_sar(p.im, e - ep)}, e);
+  const int e = y.e + 3 > ep ? y.e + 3 : ep;
+  const int s = fx_min(e - y.e, 63);
+  return fx_norm({(y.v.re >> s) + fx_sar(p.re, e - ep), (y.v.im >> s) + fx_sar(p.im, e - ep)}, e);
 }
-// 16 bytes of a normalised value: 57 bits of each component, the exponent in the low 6 bits of both
+// 16 bytes of a normalised value: 56 bits of each component, rounded to even, the exponent in the low
+// 6 bits of both
 DGPE_HD fxc fx_pack(fxv y) {
   const int b = y.e + 1300;
-  return {(long long)(((unsigned long long)y.v.re << 1) & ~63ull) | (b & 63),
-          (long long)(((unsigned long long)y.v.im << 1) & ~63ull) | (b >> 6)};
+  return {((y.v.re + 31 + ((y.v.re >> 6) & 1)) & ~63ll) | (b & 63), ((y.v.im + 31 + ((y.v.im >> 6) & 1)) & ~63ll) | (b >> 6)};
 }
 DGPE_HD fxv fx_unpack(fxc q) {
-  return {{(q.re & ~63ll) >> 1, (q.im & ~63ll) >> 1}, ((((int)q.im & 63) << 6) | ((int)q.re & 63)) - 1300};
+  return {{q.re & ~63ll, q.im & ~63ll}, ((((int)q.im & 63) << 6) | ((int)q.re & 63)) - 1300};
 }
 
 // ---- sine, cosine and exponential of the potential step, in fixed point ------------------------
 // An angle as theta 2^58, |theta| < 18.
 constexpr long long kFxOne58 = 1LL << 58;
-// x 2^58 cut off at bit 0, for |x| < 4; `slow` set otherwise
+// x 2^58 rounded, for |x| < 4; `slow` set otherwise
 DGPE_HD long long fx_angle(double x, bool &slow) {
   const long long b = fx_bits(x);
   const int e = (int)(b >> 52) & 0x7ff, s = 1027 - e;
   slow |= e > 1024;
   const unsigned long long m = ((unsigned long long)b & 0xfffffffffffffull) | (1ull << 52);
-  const long long v = (long long)((m << 10) >> (s > 63 ? 63 : s < 0 ? 0 : s));
+  const int k = s > 63 ? 63 : s < 0 ? 0 : s;
+  const long long v = (long long)(((m << 10) + ((1ull << k) >> 1)) >> k);
   const long long g = b >> 63;
   return (v ^ g) - g;
 }
@@ -480,7 +500,7 @@ DGPE_HD bool fx_phase(double &zre, double &zim, long long v, fxs g, fxs dd, int 
   const int ka = fx_exponent_bits(zre), kb = fx_exponent_bits(zim);
   int em = (ka > kb ? ka : kb) >> 20;
   if (em < kFxMinBiased) em = kFxMinBiased;
-  const fxc z = {fx_from(zre, em) * 16, fx_from(zim, em) * 16};   // z 2^-(em - 1084)
+  const fxc z = {fx_from<9>(zre, em), fx_from<9>(zim, em)};   // z 2^-(em - 1084)
   const long long n = fx_mul(z.re, fx_hi(z.re), fx_lo(z.re)) + fx_mul(z.im, fx_hi(z.im), fx_lo(z.im));
   const int sg = -(g.x + 2 * (em - 1084) + 186);
   if (em == 0x7ff || sg < 0) return false;
@@ -1080,7 +1100,8 @@ __global__ void __launch_bounds__(FxZ<N>::NT) k5_fx(const __grid_constant__ KArg
 // ---- Crank-Nicolson sweeps ------------------------------------------------------------------
 // Coefficients of the fixed-point sweeps, behind the FP64 table of the same axis and direction (at
 // fx_cn_offset): a header {ka, kb}, then alpha_s 2^ka for s < h + 2, then 2 beta_s 2^kb for
-// s < h + 2 (h = m/2, the largest powers of two that keep every magnitude at most 1).
+// s < h + 2, as words of kFxCoefBits bits (h = m/2, the largest powers of two that keep every magnitude
+// at most 1).
 __host__ __device__ constexpr size_t fx_cn_offset(int chunk) { return ((size_t)4 * kWarp * chunk + 11 * kWarp) * 16; }
 __global__ inline void k_fx_cn_tables(CnJobs jobs) {
   const CnJob &jb = jobs.job[blockIdx.x];
@@ -1113,7 +1134,7 @@ __global__ inline void k_fx_cn_tables(CnJobs jobs) {
   for (int q = 0; q < 2; ++q)
     for (int i = threadIdx.x; i < n; i += kWarp) {
       const Z64 z = get(q, i);
-      const long long re = __double2ll_rn(ldexp(z.re, 60 + k[q])), im = __double2ll_rn(ldexp(z.im, 60 + k[q]));
+      const long long re = __double2ll_rn(ldexp(z.re, kFxCoefBits + k[q])), im = __double2ll_rn(ldexp(z.im, kFxCoefBits + k[q]));
       out[1 + q * n + i] = {fx_hi(re), fx_lo(re), fx_hi(im), fx_lo(im)};
     }
 }
@@ -1229,7 +1250,7 @@ __global__ void __launch_bounds__(kFxcThreads, 4) k_cn_fx(const __grid_constant_
             const int key = fx_key(v);
             kmax = max(kmax, key);
             const fxc t = fx_coef<CPLX>(y.v, fx_ldw(fal + s));
-            y = fx_forward(v.re, v.im, key, t, y.e + 4 - ka);
+            y = fx_forward(v.re, v.im, key, t, y.e + 3 - ka);
             scratch[(size_t)s * T] = fx_pack(y);
           }
         }
@@ -1283,8 +1304,8 @@ __global__ void __launch_bounds__(kFxcThreads, 4) k_cn_fx(const __grid_constant_
     // c x_h starts both halves' way back
     const C cx = CPLX ? C{-r * xh.im, r * xh.re} : C{r * xh.re, r * xh.im};
     const int ex = max(fx_key(cx) >> 20, kFxMinBiased);
-    fxc t = {fx_from(cx.re, ex), fx_from(cx.im, ex)};
-    int et = ex - 1080;
+    fxc t = {fx_from<6>(cx.re, ex), fx_from<6>(cx.im, ex)};
+    int et = ex - 1081;
     for (int c = 0; c < nc; ++c) {
       load_psi(c + S - 1, true);
       load_y(c + S - 1);
@@ -1308,15 +1329,15 @@ __global__ void __launch_bounds__(kFxcThreads, 4) k_cn_fx(const __grid_constant_
             const fxv x = fx_backward(fx_unpack(ys[e]), t, et);
             const fxc b = fx_coef<CPLX>(x.v, fx_ldw(fbe + q));
             t = fx_coef<CPLX>(x.v, fx_ldw(fal + q + 1));   // (q = 0: the last point, unused)
-            et = x.e + 4 - ka;
+            et = x.e + 3 - ka;
+            const int eb = x.e + 3 - kb;
             C o;
             if constexpr (RED) {
               // the difference in integers: the FP64 pipe has the sums to do
-              const int eb = x.e + 4 - kb, ev = (fx_key(v) >> 20) - 1080, ed = max(max(eb, ev), kFxMinExp);
-              o = fx_to_int(fxc{fx_sar(b.re, ed - eb) - fx_from(v.re, ed + 1080), fx_sar(b.im, ed - eb) - fx_from(v.im, ed + 1080)}, ed + 1086);
+              const int ev = (fx_key(v) >> 20) - 1081, ed = max(max(eb, ev), kFxMinExp);
+              o = fx_to_int(fxc{fx_sar(b.re, ed - eb) - fx_from<6>(v.re, ed + 1081), fx_sar(b.im, ed - eb) - fx_from<6>(v.im, ed + 1081)}, ed + 1086);
             } else {
-              const int eb = x.e + 4 - kb + 1086;
-              o = fx_to_int(b, eb) - v;
+              o = fx_to_int(b, eb + 1086) - v;
             }
             if constexpr (AXIS == 2) psi_at(c, e) = o;
             else p[i * stride] = o;

@@ -4,6 +4,7 @@ import ctypes
 import os
 import subprocess
 
+import numpy as np
 import pytest
 
 from paper_1610_05329_gb300 import build
@@ -49,3 +50,78 @@ def test_twiddle_words(lib, dir):
                     want = (a[0] * w[0] - a[1] * wi, a[0] * wi + a[1] * w[0])
                     for got, x in zip(out, want):
                         assert abs((got << 64) - x) <= 2 << 64, (a, w)
+
+
+L, CL = np.longdouble, np.clongdouble
+
+
+def pointer(a):
+    return a.ctypes.data_as(ctypes.POINTER(ctypes.c_double))
+
+
+class Sweep:
+    """The Cayley sweep of m interior points by the kernels' twisted factorization, r = dt / (4 h^2):
+    with the fixed-point functions, and in 64 bits with the same (rounded) coefficients."""
+
+    def __init__(self, lib, m, r, imag):
+        self.lib, self.m, self.r, self.imag = lib, m, r, imag
+        c = CL(L(r) if imag else 1j * L(r))
+        diag, h = 1 + 2 * c, m // 2
+        e, alpha = [1 + 2 * c], [CL(0)]
+        for i in range(1, m):
+            alpha.append(c / e[-1])
+            e.append(diag - c * alpha[-1])
+        self.c = c
+        self.alpha = np.array(alpha).astype(np.complex128)
+        self.beta2 = (2 / np.array(e)).astype(np.complex128)
+        self.ginv = np.array([1 / (e[h] + e[m - 1 - h] - diag)]).astype(np.complex128)
+
+    def fixed(self, psi):   # [m][lines]
+        out = np.ascontiguousarray(psi.T.copy())
+        for line in out:
+            self.lib.host_sweep(int(not self.imag), self.m, ctypes.c_double(self.r), pointer(self.alpha),
+                                pointer(self.beta2), pointer(self.ginv), pointer(line))
+        return out.T.astype(CL)
+
+    def exact(self, psi):
+        m, h, v = self.m, self.m // 2, psi.astype(CL)
+        a, b = self.alpha.astype(CL), self.beta2.astype(CL)
+        y, out = [None] * m, [None] * m
+        for s in range(h):
+            y[s] = v[s] + (a[s] * y[s - 1] if s else 0)
+        for s in range(m - 1 - h):
+            y[m - 1 - s] = v[m - 1 - s] + (a[s] * y[m - s] if s else 0)
+        x_h = self.ginv.astype(CL)[0] * (v[h] + a[h] * y[h - 1] + a[m - 1 - h] * y[h + 1])
+        out[h] = 2 * x_h - v[h]
+        for first, way, n in ((h - 1, -1, h), (h + 1, 1, m - 1 - h)):
+            t = self.c * x_h
+            for j in range(n):
+                i, q = first + way * j, n - 1 - j
+                x = y[i] + t
+                out[i] = b[q] * x - v[i]
+                t = a[q + 1] * x
+        return np.array(out)
+
+
+def clouds(m, lines, seed):
+    rng = np.random.default_rng(seed)
+    x = ((np.arange(m) - m // 2) * 25.0 / m)[:, None]
+    return (np.exp(-0.35 * rng.uniform(0.3, 3, lines) * x * x + 1j * rng.uniform(-0.2, 0.2, lines) * x) *
+            rng.uniform(0.5, 2, lines) + 1e-3 * rng.uniform(-1, 1, (m, lines))).astype(np.complex128)
+
+
+@pytest.mark.parametrize("imag", [True, False])
+@pytest.mark.parametrize("m", [62, 254])
+def test_sweep_roundings_lean_to_no_side(lib, m, imag):
+    """A run of many steps repeats every rounding, so what leans to one side adds up: the error's
+    projection on the result (a change of its norm and phase) must be that of independent roundings,
+    whose standard deviation is sqrt(sum |w|^2 |d|^2) / sum |w|^2 for errors d of results w: within
+    five of them.  The error itself: a few roundings of 2^-53."""
+    s = Sweep(lib, m, 0.0125, imag)
+    psi = clouds(m, 2000, m)
+    want, got = s.exact(psi), s.fixed(psi)
+    d, total = got - want, np.sum(np.abs(want) ** 2)
+    lean = np.sum(np.conj(want) * d) / total
+    noise = np.sqrt(np.sum(np.abs(want) ** 2 * np.abs(d) ** 2)) / total
+    assert abs(lean.real) < 5 * noise and abs(lean.imag) < 5 * noise, (lean, noise)
+    assert np.sqrt(np.sum(np.abs(d) ** 2) / total) < 2.2e-16
