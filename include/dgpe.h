@@ -60,7 +60,13 @@ extern "C" {
 #define DGPE_REAL_TIME 0
 #define DGPE_IMAG_TIME 1
 
-#define DGPE_FP64 0   /* complex128 psi; FFT, phase and CN in FP64 */
+/* complex128 psi; FFT, phase and CN in FP64 or 64-bit fixed point, with an error by the norm no
+ * larger than FP64's (measured against extended precision).  Imaginary time: the real and the
+ * imaginary part of psi each keep 53 bits of their own.  Real time: each is good relative to the
+ * point's magnitude |psi| (one exponent for both; a potential step within 2^-52 of it, a sweep
+ * within a few 2^-52), so a part much smaller than the other keeps fewer bits of its own.
+ * Values below 2^-960 lose bits, and results below 2^-1022 are 0. */
+#define DGPE_FP64 0
 /* complex64 psi; FFT, phase and CN in FP32; the norm and the observables' sums FP64-class
  * (FP32 terms, exact weights, double-float sums per point, FP64 across blocks).  In real time every
  * step restores the norm the real-time run began with (the norm of the state its first step

@@ -328,7 +328,9 @@ DGPE_HD cplx<double> fx_to_int(fxc v, int exp) { return {fx_to_int(v.re, exp), f
 // ---- one value with its own exponent: v 2^e ------------------------------------------------
 // The recurrences along a line keep every point's precision relative to that point (the tails of a
 // cloud as well as its middle), so the running value carries its own exponent: components just
-// below 2^62 (fx_up's range) after every step.
+// below 2^62 (fx_up's range) after every step.  One exponent for both components: complex coefficients
+// (real time) mix them in every product, and each is good to 2^-56 of the point's magnitude.  (Imaginary
+// time, whose real coefficients leave the two parts apart, runs its sweeps in FP64.)
 // A long run repeats each rounding at each step, so none of them may lean to one side (the packing's
 // cut-off did: the phase of a state turned by 4e-17 a step, coherently).
 struct fxv {
@@ -346,13 +348,8 @@ DGPE_HD fxv fx_norm(fxc s, int e) {   // components of s below 2^62
 #endif
   return {{fx_shl(s.re, n), fx_shl(s.im, n)}, e - n};
 }
-// a w / 8 for a coefficient w of magnitude at most 1 (words of w 2^61; real ones: rh, rl alone): below
-// 2^59.5 for a normalised a
-template <bool CPLX>
-DGPE_HD fxc fx_coef(fxc a, fxw w) {
-  if constexpr (CPLX) return fx_twiddle<-1>(a, w);
-  else return {fx_mul(a.re, w.rh, w.rl), fx_mul(a.im, w.rh, w.rl)};
-}
+// a w / 8 for a coefficient w of magnitude at most 1 (words of w 2^61): below 2^59.5 for a normalised a
+DGPE_HD fxc fx_coef(fxc a, fxw w) { return fx_twiddle<-1>(a, w); }
 constexpr int kFxCoefBits = 61;
 // a 2^-s, s >= 0, rounded (halves up)
 DGPE_HD long long fx_sar(long long a, int s) {
@@ -497,29 +494,29 @@ DGPE_HD fxs fx_scalar(double d) {
 // (not below -1: |theta| < 4 + 4 + 2 + 8).  False, and z as it was, where the interaction or z itself is out of range.
 template <bool IMAG>
 DGPE_HD bool fx_phase(double &zre, double &zim, long long v, fxs g, fxs dd, int sd, long long phi) {
-  const int ka = fx_exponent_bits(zre), kb = fx_exponent_bits(zim);
-  int em = (ka > kb ? ka : kb) >> 20;
+  const int ka = fx_exponent_bits(zre) >> 20, kb = fx_exponent_bits(zim) >> 20;
+  int em = ka > kb ? ka : kb;
   if (em < kFxMinBiased) em = kFxMinBiased;
-  const fxc z = {fx_from<9>(zre, em), fx_from<9>(zim, em)};   // z 2^-(em - 1084)
-  const long long n = fx_mul(z.re, fx_hi(z.re), fx_lo(z.re)) + fx_mul(z.im, fx_hi(z.im), fx_lo(z.im));
+  // imaginary time: each component under its own exponent, as its factor is real: it keeps its 53 bits
+  const int er = !IMAG ? em : ka > kFxMinBiased ? ka : kFxMinBiased, ei = !IMAG ? em : kb > kFxMinBiased ? kb : kFxMinBiased;
+  const fxc z = {fx_from<9>(zre, er), fx_from<9>(zim, ei)};   // z.re 2^(er - 1084), ..
+  const long long n = (fx_mul(z.re, fx_hi(z.re), fx_lo(z.re)) >> fx_min(2 * (em - er), 63)) +
+                      (fx_mul(z.im, fx_hi(z.im), fx_lo(z.im)) >> fx_min(2 * (em - ei), 63));
   const int sg = -(g.x + 2 * (em - 1084) + 186);
   if (em == 0x7ff || sg < 0) return false;
   const long long th = v + fx_sar(fx_mul(n, g.h, g.l), sg) + fx_sar(2 * fx_mul(phi, dd.h, dd.l), sd + 1);
-  fxc o;
-  int eo = em - 1080 + 1086;
   if constexpr (IMAG) {
     int k;
     const long long p = fx_exp(th, k);
     const int ph = fx_hi(p), pl = fx_lo(p);
-    o = {fx_mul(z.re, ph, pl), fx_mul(z.im, ph, pl)};
-    eo += k;
+    zre = fx_to(fx_mul(z.re, ph, pl), er + 6 + k);
+    zim = fx_to(fx_mul(z.im, ph, pl), ei + 6 + k);
   } else {
     const fxc c = fx_cis(th);
-    o = fx_twiddle<-1>(z, fxw{fx_hi(c.re), fx_lo(c.re), fx_hi(c.im), fx_lo(c.im)});
+    const cplx<double> r = fx_to(fx_twiddle<-1>(z, fxw{fx_hi(c.re), fx_lo(c.re), fx_hi(c.im), fx_lo(c.im)}), em + 6);
+    zre = r.re;
+    zim = r.im;
   }
-  const cplx<double> r = fx_to(o, eo);
-  zre = r.re;
-  zim = r.im;
   return true;
 }
 DGPE_HD int fx_phase_shift(fxs dd, int exp) { return -(64 + dd.x + exp - 1028); }
@@ -1098,10 +1095,9 @@ __global__ void __launch_bounds__(FxZ<N>::NT) k5_fx(const __grid_constant__ KArg
 }
 
 // ---- Crank-Nicolson sweeps ------------------------------------------------------------------
-// Coefficients of the fixed-point sweeps, behind the FP64 table of the same axis and direction (at
-// fx_cn_offset): a header {ka, kb}, then alpha_s 2^ka for s < h + 2, then 2 beta_s 2^kb for
-// s < h + 2, as words of kFxCoefBits bits (h = m/2, the largest powers of two that keep every magnitude
-// at most 1).
+// Coefficients of the sweeps, behind the FP64 table of the same axis and direction (at fx_cn_offset).
+// Imaginary time: the FP64 values alpha_s for s < h + 2, then 2 beta_s (h = m/2).  Real time: a header {ka, kb}, then alpha_s 2^ka for s < h + 2, then 2 beta_s 2^kb for
+// s < h + 2, as words of kFxCoefBits bits (the largest powers of two that keep every magnitude at most 1).
 __host__ __device__ constexpr size_t fx_cn_offset(int chunk) { return ((size_t)4 * kWarp * chunk + 11 * kWarp) * 16; }
 __global__ inline void k_fx_cn_tables(CnJobs jobs) {
   const CnJob &jb = jobs.job[blockIdx.x];
@@ -1113,9 +1109,13 @@ __global__ inline void k_fx_cn_tables(CnJobs jobs) {
   auto get = [&](int q, int i) {
     if (i >= m) return Z64{0.0, 0.0};
     const double f = q ? 2.0 : 1.0;
-    if (jobs.imag) return Z64{f * tab[at(q, i)], 0.0};
     return Z64{f * tab[2 * at(q, i)], f * tab[2 * at(q, i) + 1]};
   };
+  if (jobs.imag) {
+    for (int q = 0; q < 2; ++q)
+      for (int i = threadIdx.x; i < n; i += kWarp) reinterpret_cast<double *>(out)[q * n + i] = i < m ? (q ? 2.0 : 1.0) * tab[at(q, i)] : 0.0;
+    return;
+  }
   double mx[2] = {0.0, 0.0};
   for (int q = 0; q < 2; ++q) {
     for (int i = threadIdx.x; i < n; i += kWarp) {
@@ -1147,9 +1147,11 @@ __global__ inline void k_fx_cn_tables(CnJobs jobs) {
 // and substitute back away from it:
 //   y_i = psi_i + alpha_i y_{i-1},  x_i = y_i + alpha_{i+2} x_{i+1}  (x = chi / beta),
 //   psi'_i = 2 beta_i x_i - psi_i.
-// The running values are integers with their own exponent (fxv).  In FP64 arithmetic a sweep is 12
-// FP64 instructions per point, 0.32 ms of that pipe at 256^3; this is about 330 integer ones (0.14 ms)
-// and two FP64 subtractions.  Persistent CTAs: y waits for the way back in a scratch of the CTA's own
+// Real time: the running values are integers with their own exponent (fxv).  In FP64 arithmetic a sweep is
+// 12 FP64 instructions per point, 0.32 ms of that pipe at 256^3; this is about 330 integer ones (0.14 ms)
+// and two FP64 subtractions.  Imaginary time: FP64 arithmetic.  Its real coefficients make a sweep 6 FP64
+// instructions per point, no more than the integers take (a step at 480x480x250 6.52 ms with either, at
+// 64^3 104 -> 99 us), and each component of psi keeps its own 53 bits.  Persistent CTAs: y waits for the way back in a scratch of the CTA's own
 // (packed, 16 bytes a point), so few enough lines are under way for much of it and of their psi to
 // stay in L2.  psi and y come through shared memory by cp.async, two chunks of four points ahead;
 // along z, where a thread's points are consecutive, the lanes of a warp copy each other's chunks as
@@ -1185,9 +1187,10 @@ __global__ void __launch_bounds__(kFxcThreads, 4) k_cn_fx(const __grid_constant_
   using Coef = typename std::conditional<CPLX, C, double>::type;
   const Coef *tab = reinterpret_cast<const Coef *>(a.cn[AXIS].tab);
   const fxw *ft = reinterpret_cast<const fxw *>(static_cast<const char *>(a.cn[AXIS].tab) + fx_cn_offset(chunk));
-  const fxw head = fx_ldw(ft);
+  const fxw head = CPLX ? fx_ldw(ft) : fxw{0, 0, 0, 0};
   const int ka = head.rh, kb = head.rl;
   const fxw *fal = ft + 1, *fbe = ft + 1 + h + 2;
+  const double *dal = reinterpret_cast<const double *>(ft), *dbe = dal + h + 2;   // imaginary time
   const double r = a.cn_r[AXIS];
   fxc *scratch = reinterpret_cast<fxc *>(a.ybuf) + (size_t)blockIdx.x * h * T + tid;   // y of step s at s T
   double acc[4] = {0.0, 0.0, 0.0, 0.0};
@@ -1225,6 +1228,7 @@ __global__ void __launch_bounds__(kFxcThreads, 4) k_cn_fx(const __grid_constant_
     const int nc = (h + K - 1) / K, nwhole = line0 + 15 < nlines ? (m - 1 - h) / K : 0;
     // elimination
     fxv y = {{0, 0}, kFxMinExp};
+    C yf = czero<double>();   // imaginary time: in FP64
     int kmax = 0;
 #pragma unroll
     for (int c = 0; c < S - 1; ++c) {
@@ -1247,11 +1251,16 @@ __global__ void __launch_bounds__(kFxcThreads, 4) k_cn_fx(const __grid_constant_
           const int s = c * K + e;
           if (decltype(whole)::value || s < nf) {
             const C v = vs[e];
-            const int key = fx_key(v);
-            kmax = max(kmax, key);
-            const fxc t = fx_coef<CPLX>(y.v, fx_ldw(fal + s));
-            y = fx_forward(v.re, v.im, key, t, y.e + 3 - ka);
-            scratch[(size_t)s * T] = fx_pack(y);
+            if constexpr (CPLX) {
+              const int key = fx_key(v);
+              kmax = max(kmax, key);
+              const fxc t = fx_coef(y.v, fx_ldw(fal + s));
+              y = fx_forward(v.re, v.im, key, t, y.e + 3 - ka);
+              scratch[(size_t)s * T] = fx_pack(y);
+            } else {
+              yf = cfma(__ldg(dal + s), yf, v);
+              reinterpret_cast<C *>(scratch)[(size_t)s * T] = yf;
+            }
           }
         }
       };
@@ -1277,18 +1286,18 @@ __global__ void __launch_bounds__(kFxcThreads, 4) k_cn_fx(const __grid_constant_
       cp_async_commit();
     }
     // the twist point, in FP64: gamma x_h = psi_h + alpha_h y_{h-1} + alpha_{m-1-h} z_{h+1}
-    const C yd = fx_to(y.v, y.e + 1086);
+    const C yd = CPLX ? fx_to(y.v, y.e + 1086) : yf;
     const C yt = shfl_xor(yd, kWarp / 2);
     C xh = czero<double>(), ph = czero<double>();
     if (bottom && active) {
       auto slot = [&](int s) { return ((s & (chunk - 1)) << 5) + (s >> lc); };
       ph = p[h * stride];
-      kmax = max(kmax, fx_key(ph));
+      if constexpr (CPLX) kmax = max(kmax, fx_key(ph));
       xh = mul(ldg(tab + 4 * mp + 10 * kWarp), cfma(ldg(tab + slot(m - 1 - h)), yd, cfma(ldg(tab + slot(h)), yt, ph)));
     }
     const C xt = shfl_xor(xh, kWarp / 2);
     if (!bottom) xh = xt;
-    kmax = max(kmax, __shfl_xor_sync(0xffffffffu, kmax, kWarp / 2));
+    if constexpr (CPLX) kmax = max(kmax, __shfl_xor_sync(0xffffffffu, kmax, kWarp / 2));
     double s0 = 0.0;
     auto add = [&](int i, C o) {
       if constexpr (RED) {
@@ -1306,6 +1315,8 @@ __global__ void __launch_bounds__(kFxcThreads, 4) k_cn_fx(const __grid_constant_
     const int ex = max(fx_key(cx) >> 20, kFxMinBiased);
     fxc t = {fx_from<6>(cx.re, ex), fx_from<6>(cx.im, ex)};
     int et = ex - 1081;
+    C xf = xh;
+    double ap = r;   // imaginary time: x_i = y_i + ap x of the point before
     for (int c = 0; c < nc; ++c) {
       load_psi(c + S - 1, true);
       load_y(c + S - 1);
@@ -1326,18 +1337,24 @@ __global__ void __launch_bounds__(kFxcThreads, 4) k_cn_fx(const __grid_constant_
           if (decltype(whole)::value || j < nf) {
             const int q = nf - 1 - j, i = bottom ? h + 1 + j : h - 1 - j;
             const C v = vs[e];
-            const fxv x = fx_backward(fx_unpack(ys[e]), t, et);
-            const fxc b = fx_coef<CPLX>(x.v, fx_ldw(fbe + q));
-            t = fx_coef<CPLX>(x.v, fx_ldw(fal + q + 1));   // (q = 0: the last point, unused)
-            et = x.e + 3 - ka;
-            const int eb = x.e + 3 - kb;
             C o;
-            if constexpr (RED) {
-              // the difference in integers: the FP64 pipe has the sums to do
-              const int ev = (fx_key(v) >> 20) - 1081, ed = max(max(eb, ev), kFxMinExp);
-              o = fx_to_int(fxc{fx_sar(b.re, ed - eb) - fx_from<6>(v.re, ed + 1081), fx_sar(b.im, ed - eb) - fx_from<6>(v.im, ed + 1081)}, ed + 1086);
+            if constexpr (!CPLX) {
+              xf = cfma(ap, xf, C{__longlong_as_double(ys[e].re), __longlong_as_double(ys[e].im)});
+              o = cfma(__ldg(dbe + q), xf, C{-v.re, -v.im});
+              ap = __ldg(dal + q + 1);
             } else {
-              o = fx_to_int(b, eb + 1086) - v;
+              const fxv x = fx_backward(fx_unpack(ys[e]), t, et);
+              const fxc b = fx_coef(x.v, fx_ldw(fbe + q));
+              t = fx_coef(x.v, fx_ldw(fal + q + 1));   // (q = 0: the last point, unused)
+              et = x.e + 3 - ka;
+              const int eb = x.e + 3 - kb;
+              if constexpr (RED) {
+                // the difference in integers: the FP64 pipe has the sums to do
+                const int ev = (fx_key(v) >> 20) - 1081, ed = max(max(eb, ev), kFxMinExp);
+                o = fx_to_int(fxc{fx_sar(b.re, ed - eb) - fx_from<6>(v.re, ed + 1081), fx_sar(b.im, ed - eb) - fx_from<6>(v.im, ed + 1081)}, ed + 1086);
+              } else {
+                o = fx_to_int(b, eb + 1086) - v;
+              }
             }
             if constexpr (AXIS == 2) psi_at(c, e) = o;
             else p[i * stride] = o;

@@ -9,14 +9,13 @@ using namespace dgpe;
 namespace {
 fxw words(long long re, long long im) { return {fx_hi(re), fx_lo(re), fx_hi(im), fx_lo(im)}; }
 
-// One line of the sweep k_cn_fx, interior points only: al, be = alpha and 2 beta (FP64 pairs) of m
+// One line of the real-time sweep k_cn_fx, interior points only: al, be = alpha and 2 beta (FP64 pairs) of m
 // points, ginv = 1 / gamma, r = dt / (4 h^2).
 struct Z {
   double re, im;
 };
 Z mul(Z a, Z b) { return {a.re * b.re - a.im * b.im, a.re * b.im + a.im * b.re}; }
 Z operator+(Z a, Z b) { return {a.re + b.re, a.im + b.im}; }
-template <bool CPLX>
 void sweep(int m, double r, const Z *al, const Z *be, Z ginv, Z *psi) {
   const int h = m / 2, n = h + 2;
   auto exponent = [&](const Z *t) {
@@ -36,7 +35,7 @@ void sweep(int m, double r, const Z *al, const Z *be, Z ginv, Z *psi) {
     fxv v = {{0, 0}, kFxMinExp};
     for (int s = 0; s < nf; ++s) {
       const int i = bottom ? m - 1 - s : s;
-      const fxc t = fx_coef<CPLX>(v.v, coef(al, s, ka));
+      const fxc t = fx_coef(v.v, coef(al, s, ka));
       v = fx_forward(psi[i].re, psi[i].im, fx_key(cplx<double>{psi[i].re, psi[i].im}), t, v.e + 3 - ka);
       y[i] = fx_pack(v);
     }
@@ -45,7 +44,7 @@ void sweep(int m, double r, const Z *al, const Z *be, Z ginv, Z *psi) {
   const Z yt = forward(false, h), yb = forward(true, m - 1 - h);
   const Z xh = mul(ginv, psi[h] + mul(al[h], yt) + mul(al[m - 1 - h], yb));
   out[h] = {2.0 * xh.re - psi[h].re, 2.0 * xh.im - psi[h].im};
-  const Z cx = CPLX ? Z{-r * xh.im, r * xh.re} : Z{r * xh.re, r * xh.im};
+  const Z cx = {-r * xh.im, r * xh.re};
   const int ex = std::max(fx_key(cplx<double>{cx.re, cx.im}) >> 20, kFxMinBiased);
   for (int bottom = 0; bottom < 2; ++bottom) {
     const int nf = bottom ? m - 1 - h : h;
@@ -54,8 +53,8 @@ void sweep(int m, double r, const Z *al, const Z *be, Z ginv, Z *psi) {
     for (int j = 0; j < nf; ++j) {
       const int q = nf - 1 - j, i = bottom ? h + 1 + j : h - 1 - j;
       const fxv x = fx_backward(fx_unpack(y[i]), t, et);
-      const fxc b = fx_coef<CPLX>(x.v, coef(be, q, kb));
-      t = fx_coef<CPLX>(x.v, coef(al, q + 1, ka));
+      const fxc b = fx_coef(x.v, coef(be, q, kb));
+      t = fx_coef(x.v, coef(al, q + 1, ka));
       et = x.e + 3 - ka;
       out[i] = {fx_to_int(b.re, x.e + 3 - kb + 1086) - psi[i].re, fx_to_int(b.im, x.e + 3 - kb + 1086) - psi[i].im};
     }
@@ -71,9 +70,13 @@ void host_twiddle(int dir, const long long *a, const long long *w, long long *ou
   out[0] = r.re;
   out[1] = r.im;
 }
-void host_sweep(int cplx, int m, double r, const double *al, const double *be, const double *ginv, double *psi) {
+void host_sweep(int m, double r, const double *al, const double *be, const double *ginv, double *psi) {
   auto z = [](const double *p) { return reinterpret_cast<const Z *>(p); };
-  if (cplx) sweep<true>(m, r, z(al), z(be), *z(ginv), reinterpret_cast<Z *>(psi));
-  else sweep<false>(m, r, z(al), z(be), *z(ginv), reinterpret_cast<Z *>(psi));
+  sweep(m, r, z(al), z(be), *z(ginv), reinterpret_cast<Z *>(psi));
+}
+// the potential step of one point, theta = (v + g |z|^2) with v 2^58; 0 where it is out of range
+int host_phase(int imag, double *z, long long v, double g) {
+  const fxs zero = fx_scalar(0.0);
+  return imag ? fx_phase<true>(z[0], z[1], v, fx_scalar(g), zero, 1000, 0) : fx_phase<false>(z[0], z[1], v, fx_scalar(g), zero, 1000, 0);
 }
 }

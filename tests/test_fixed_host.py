@@ -60,12 +60,12 @@ def pointer(a):
 
 
 class Sweep:
-    """The Cayley sweep of m interior points by the kernels' twisted factorization, r = dt / (4 h^2):
+    """The real-time sweep of m interior points by the kernels' twisted factorization, r = dt / (4 h^2):
     with the fixed-point functions, and in 64 bits with the same (rounded) coefficients."""
 
-    def __init__(self, lib, m, r, imag):
-        self.lib, self.m, self.r, self.imag = lib, m, r, imag
-        c = CL(L(r) if imag else 1j * L(r))
+    def __init__(self, lib, m, r):
+        self.lib, self.m, self.r = lib, m, r
+        c = CL(1j * L(r))
         diag, h = 1 + 2 * c, m // 2
         e, alpha = [1 + 2 * c], [CL(0)]
         for i in range(1, m):
@@ -79,8 +79,8 @@ class Sweep:
     def fixed(self, psi):   # [m][lines]
         out = np.ascontiguousarray(psi.T.copy())
         for line in out:
-            self.lib.host_sweep(int(not self.imag), self.m, ctypes.c_double(self.r), pointer(self.alpha),
-                                pointer(self.beta2), pointer(self.ginv), pointer(line))
+            self.lib.host_sweep(self.m, ctypes.c_double(self.r), pointer(self.alpha), pointer(self.beta2),
+                                pointer(self.ginv), pointer(line))
         return out.T.astype(CL)
 
     def exact(self, psi):
@@ -110,14 +110,13 @@ def clouds(m, lines, seed):
             rng.uniform(0.5, 2, lines) + 1e-3 * rng.uniform(-1, 1, (m, lines))).astype(np.complex128)
 
 
-@pytest.mark.parametrize("imag", [True, False])
 @pytest.mark.parametrize("m", [62, 254])
-def test_sweep_roundings_lean_to_no_side(lib, m, imag):
+def test_sweep_roundings_lean_to_no_side(lib, m):
     """A run of many steps repeats every rounding, so what leans to one side adds up: the error's
     projection on the result (a change of its norm and phase) must be that of independent roundings,
     whose standard deviation is sqrt(sum |w|^2 |d|^2) / sum |w|^2 for errors d of results w: within
     five of them.  The error itself: a few roundings of 2^-53."""
-    s = Sweep(lib, m, 0.0125, imag)
+    s = Sweep(lib, m, 0.0125)
     psi = clouds(m, 2000, m)
     want, got = s.exact(psi), s.fixed(psi)
     d, total = got - want, np.sum(np.abs(want) ** 2)
@@ -125,3 +124,47 @@ def test_sweep_roundings_lean_to_no_side(lib, m, imag):
     noise = np.sqrt(np.sum(np.abs(want) ** 2 * np.abs(d) ** 2)) / total
     assert abs(lean.real) < 5 * noise and abs(lean.imag) < 5 * noise, (lean, noise)
     assert np.sqrt(np.sum(np.abs(d) ** 2) / total) < 2.2e-16
+
+
+def phase(lib, imag, z, theta, g):
+    p = (ctypes.c_double * 2)(z.real, z.imag)
+    assert lib.host_phase(int(imag), p, ctypes.c_longlong(round(theta * 2.0 ** 58)), ctypes.c_double(g))
+    return p[0], p[1]
+
+
+@pytest.mark.parametrize("scale", [1.0, 1e-4, 1e-12, 1e-18, 1e-60])
+def test_potential_step_of_a_point(lib, scale):
+    """Imaginary time: each component within 2^-52 of itself (a rounding and an exponential good to
+    2^-56).  Real time: within 2^-52 of the point's magnitude."""
+    rng = np.random.default_rng(3)
+    for _ in range(2000):
+        z = complex(rng.uniform(-1, 1), scale * rng.uniform(-1, 1))
+        theta, g = rng.uniform(0, 0.5), 0.1
+        k = round(theta * 2.0 ** 58)
+        angle = L(k) / L(2) ** 58 + L(g) * (L(z.real) ** 2 + L(z.imag) ** 2)
+        got = phase(lib, True, z, theta, g)
+        for x, q in ((z.real, got[0]), (z.imag, got[1])):
+            want = L(x) * np.exp(-angle)
+            assert abs(L(q) - want) <= L(2) ** -52 * abs(want)
+        got = phase(lib, False, z, theta, g)
+        c, s = np.cos(angle), np.sin(angle)
+        assert abs(L(got[0]) - (L(z.real) * c + L(z.imag) * s)) <= L(2) ** -52 * abs(z)
+        assert abs(L(got[1]) - (L(z.imag) * c - L(z.real) * s)) <= L(2) ** -52 * abs(z)
+
+
+@pytest.mark.parametrize("scale", [1.0, 1e-4, 1e-20])
+@pytest.mark.parametrize("r", [2e-4, 0.0056])
+def test_real_time_sweep_by_magnitude(lib, scale, r):
+    """Complex coefficients mix the parts: a component is good relative to the point's magnitude.  On
+    smooth lines 2 beta x is at most 2.1 of the result, rounded to 53 bits (1.05 eps) and subtracted
+    (0.5 eps): 2 eps.  The twist point has FP64 arithmetic, two complex multiply-adds and a product
+    of two to four roundings each on up to 2.1 of the result: 10 eps."""
+    m = 62
+    s = Sweep(lib, m, r)
+    x = np.exp(-0.002 * (np.arange(m) - m // 2) ** 2)[:, None]
+    psi = x * (1.0 + 1j * scale * np.cos(0.1 * np.arange(200))[None, :])
+    want, got = s.exact(psi), s.fixed(psi)
+    bound = np.full((m, 1), 2.0)
+    bound[m // 2] = 10.0
+    bound = bound * np.finfo(np.float64).eps * np.abs(want)
+    assert np.all(np.abs((got - want).real) <= bound) and np.all(np.abs((got - want).imag) <= bound)

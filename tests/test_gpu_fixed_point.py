@@ -186,3 +186,42 @@ def test_potential_step(mode, shape, dt, g, gdd, scale):
         theta = theta + L(dt) * L(gdd) * exact_phi(psi, h)
     f = np.exp(-theta) if mode == abi.DGPE_IMAG_TIME else np.cos(theta) - 1j * np.sin(theta)
     assert cerror(got, psi * f) < 3e-16 * (1 + float(np.max(np.abs(theta))))
+
+
+# ---- components of very different size ---------------------------------------------------------
+# Imaginary time: the real and imaginary parts are two fields under the same real factors, and each
+# keeps FP64's bits: the tolerances above, of each part by itself.  (Real time mixes the parts: each is
+# good relative to the point's magnitude, test_fixed_host.py.)
+def two_parts(shape, scale):
+    return (inputs.random_psi(shape, seed=3).real + 1j * scale * inputs.random_psi(shape, seed=4).real).astype(np.complex128)
+
+
+@pytest.mark.parametrize("scale", [1e-4, 1e-12, 1e-20])
+@pytest.mark.parametrize("axis,which", [(0, abi.DGPE_SUB_CN_X), (1, abi.DGPE_SUB_CN_Y), (2, abi.DGPE_SUB_CN_Z)])
+def test_imaginary_time_sweep_keeps_each_component(axis, which, scale):
+    for shape in ((20, 14, 36), (6, 50, 18)):
+        psi = two_parts(shape, scale)
+        gpu = abi.Condensate(shape, 0.3, 0.02, mode=abi.DGPE_IMAG_TIME, precision=abi.DGPE_FP64)
+        gpu.set_psi(psi)
+        gpu.substep(which)
+        got = gpu.get_psi()
+        gpu.close()
+        want = exact_sweep(psi, axis, 0.02 / (4 * L(0.3) ** 2), True)
+        assert error(got.real, want.real) < 1e-15 and error(got.imag, want.imag) < 1e-15
+
+
+@pytest.mark.parametrize("scale", [1e-4, 1e-12, 1e-20])
+@pytest.mark.parametrize("shape", [(12, 14, 24), (6, 20, 64)])
+def test_imaginary_time_potential_step_keeps_each_component(shape, scale):
+    psi, dt = two_parts(shape, scale), 0.02
+    h = tuple(8.0 / n for n in shape)
+    gpu = abi.Condensate(shape, h, dt, mode=abi.DGPE_IMAG_TIME, precision=abi.DGPE_FP64, g=5.0, gdd=2.0)
+    gpu.set_psi(psi)
+    gpu.substep(abi.DGPE_SUB_POTENTIAL)
+    got = gpu.get_psi()
+    gpu.close()
+    x = [((np.arange(n) - n // 2).astype(L) * L(d)) for n, d in zip(shape, h)]
+    v = sum((q * q / 2).reshape([-1 if d == e else 1 for e in range(3)]) for d, q in enumerate(x))
+    theta = L(dt) * (v + 5 * (psi.real.astype(L) ** 2 + psi.imag.astype(L) ** 2) + 2 * exact_phi(psi, h))
+    bound = 3e-16 * (1 + float(np.max(np.abs(theta))))
+    assert error(got.real, psi.real * np.exp(-theta)) < bound and error(got.imag, psi.imag * np.exp(-theta)) < bound
