@@ -101,41 +101,56 @@ __global__ void __launch_bounds__(kNoAllocThreads)
 
 // FP32 data.  The kernel above spends six to eight FP64-pipe instructions per point (two
 // conversions among them; GB300 issues 2 per clock per SM): 1.42 ms at 512x512x384 against 0.12 ms
-// of HBM time.  Here the densities and the weighted sums of a warp's lines are FP32 pairs:
-//   - each lane's points are scaled by a power of two taken from the largest of them, so no
-//     square leaves the FP32 range and what underflows is below 2^-100 of the sum;
-//   - re^2 + im^2 is exact to 2^-48 (FMA residuals of both squares and of their sum);
-//   - the weights are exact integers (3 x the quadrature weights, squared signed indices), their
-//     products by the density carry the FMA residual, the sums are TwoSums, renormalised line
-//     by line; a warp passes its pairs on to FP64 once per unit of up to 8 lines
-//     (or where the x index or the scale changes).
-// The result is as near to extended-precision sums as the FP64 kernel's (1e-16).  Lanes that meet an infinity or a NaN take those points in FP64.  Bound by FP32 issue (about 40
-// instructions per point): 1.42 -> 0.245 ms at 512x512x384 (0.49 of HBM).
-constexpr int kMomentPairs = 4;   // pairs of points in a lane's registers
+// of HBM time.  Here a lane sums its points in integers, in units taken from the largest of them:
+//   - a component is m 2^(e - 150) with a 24-bit m; its square, 48 bits, goes to a 64-bit integer
+//     under the lane's exponent E: exact where the component is above 2^-4 of the lane's first
+//     largest, else rounded at 2^-54 of that one's density (E leaves 3 binades for later ones to grow);
+//   - the weights are integers (3 x the quadrature weights, squared signed indices); the sums of
+//     products, of the high and of the low words apart, are exact;
+//   - a lane passes its sums on to FP64 once per unit of up to 8 lines (or where the x index changes
+//     or a point outgrows E).
+// So the sums are better than FP64's own.  Lanes that meet an infinity or a NaN take those points in
+// FP64.  Bound by integer issue (about 35 instructions per point): 1.42 -> 0.29 ms at 512x512x384.  rms error
+// over 36 grids of 2.6e5 to 1.3e6 points, norm and sizes: 1.5e-16, 8e-17 -> 1.05e-16, 7e-17.  (Pairs of FP32
+// in place of the integers take 0.25 ms and leave 2.5e-16, 1.0e-16.)
+constexpr int kMomentPairs = 2;   // pairs of points in a lane's registers (three leave more of a line's end idle)
 
-// a + b, |a| >= |b| or a = 0
-__device__ __forceinline__ void renorm(DFAcc &a) {
-  const float t = __fadd_rn(a.hi, a.lo);
-  a.lo = __fsub_rn(a.lo, __fsub_rn(t, a.hi));
-  a.hi = t;
-}
-// a += w (h + l), exactly up to the rounding of the low part
-__device__ __forceinline__ void add_weighted(DFAcc &a, float w, float h, float l) {
-  const float p = __fmul_rn(w, h);
-  const float e = __fmaf_rn(w, l, __fmaf_rn(w, h, -p));
-  a.add(p);
-  a.lo = __fadd_rn(a.lo, e);
+// A sum of integers 2^32 h + l, and additions of w d and of w times another sum
+struct WideSum {
+  unsigned long long h = 0, l = 0;
+  __device__ __forceinline__ void add(unsigned w, unsigned long long d) {
+    h += (unsigned long long)w * (unsigned)(d >> 32);
+    l += (unsigned long long)w * (unsigned)d;
+  }
+  __device__ __forceinline__ void add(unsigned w, const WideSum &s) {
+    h += w * s.h;
+    l += w * s.l;
+  }
+  __device__ __forceinline__ double value() const { return fma((double)h, 4294967296.0, (double)l); }
+};
+// x^2 in units of 2^(2 (E - 150) - 14) for |x| < 2^(E - 126), rounded (halves up); x comes scaled by a
+// power of two that takes E to `base` (63 at least: a zero's or a subnormal's exponent field, 0, then
+// shifts everything out).  Shifts by the width and more give 0 (shl.b32, shr.u64).
+__device__ __forceinline__ unsigned long long square_units(float x, int base) {
+  const unsigned u = __float_as_uint(x), m = ((u & 0x7fffffu) | 0x800000u) << 7;
+  const unsigned s = 2 * (base - (int)((u >> 23) & 0xff));
+  unsigned lo, hi;   // 2^(s - 1)
+  unsigned long long r;
+  asm("shl.b32 %0, 1, %1;" : "=r"(lo) : "r"(s - 1));
+  asm("shl.b32 %0, 1, %1;" : "=r"(hi) : "r"(s - 33));
+  asm("shr.u64 %0, %1, %2;" : "=l"(r) : "l"((unsigned long long)m * m + ((unsigned long long)hi << 32 | lo)), "r"(s));
+  return r;
 }
 
 template <bool WIDE>
 __global__ void __launch_bounds__(kNoAllocThreads, 3)
     k_moments_f32(const float2 *__restrict__ psi, int nx, int ny, int nz, double hx, double hy, double hz, int simpson,
                   int lines_per_unit, NoAllocScratch *scr, double *out) {
-  __shared__ float4 wz[kNoAllocMaxN / 2];   // W and W k'^2 of two consecutive points
+  __shared__ uint4 wz[kNoAllocMaxN / 2];   // W and W k'^2 of two consecutive points
   for (int p = threadIdx.x; p < nz / 2; p += blockDim.x) {
     const int k0 = 2 * p - nz / 2, k1 = k0 + 1;
-    const float w0 = (float)quad_weight3(2 * p, nz, simpson), w1 = (float)quad_weight3(2 * p + 1, nz, simpson);
-    wz[p] = make_float4(w0, w0 * (float)(k0 * k0), w1, w1 * (float)(k1 * k1));
+    const unsigned w0 = quad_weight3(2 * p, nz, simpson), w1 = quad_weight3(2 * p + 1, nz, simpson);
+    wz[p] = make_uint4(w0, w0 * (unsigned)(k0 * k0), w1, w1 * (unsigned)(k1 * k1));
   }
   __syncthreads();
   const int lane = threadIdx.x & (kWarp - 1), np = nz / 2;
@@ -143,12 +158,12 @@ __global__ void __launch_bounds__(kNoAllocThreads, 3)
   const int nwarps = gridDim.x * (blockDim.x / kWarp);
   const int nunits = (nlines + lines_per_unit - 1) / lines_per_unit;
   double v[4] = {0.0, 0.0, 0.0, 0.0};   // sums of W n, i'^2 W n, j'^2 W n, k'^2 W n
-  // the pairs of one run of lines of equal x index, over 2^-2(sb - 127)
-  DFAcc s0, sy, sz;
-  int sb = 0;   // 0: empty
+  // the sums of one run of lines of equal x index, under E
+  WideSum s0, sy, sz;
+  int E = 0;   // 0: empty
   auto flush = [&](int i) {
-    if (!sb) return;
-    const double un = __hiloint2double((1023 - 2 * (sb - 127)) << 20, 0);
+    if (!E) return;
+    const double un = __hiloint2double((1023 + 2 * (E - 150) - 14) << 20, 0);
     const int ii = i - nx / 2;
     const double wx = (double)quad_weight3(i, nx, simpson) * un;
     const double t = wx * s0.value();
@@ -156,8 +171,8 @@ __global__ void __launch_bounds__(kNoAllocThreads, 3)
     v[1] = fma((double)(ii * ii), t, v[1]);
     v[2] = fma(wx, sy.value(), v[2]);
     v[3] = fma(wx, sz.value(), v[3]);
-    s0 = sy = sz = DFAcc{};
-    sb = 0;
+    s0 = sy = sz = WideSum{};
+    E = 0;
   };
   auto load = [&](int l, int p0, float4 (&c)[kMomentPairs]) {
 #pragma unroll
@@ -182,9 +197,14 @@ __global__ void __launch_bounds__(kNoAllocThreads, 3)
     float4 c[kMomentPairs], nxt[kMomentPairs];
     load(l0, 0, nxt);
     for (int l = l0; l < l1; ++l) {
-      const float wy = (float)quad_weight3(j, ny, simpson);
-      const int jj = j - ny / 2;
-      DFAcc t0, tz;   // this line's sums
+      const unsigned wy = quad_weight3(j, ny, simpson), jj2 = (unsigned)((j - ny / 2) * (j - ny / 2));
+      WideSum t0, tz;   // this line's sums of W_z n, k'^2 W_z n
+      auto fold = [&]() {
+        s0.add(wy, t0);
+        sy.add(wy * jj2, t0);
+        sz.add(wy, tz);
+        t0 = tz = WideSum{};
+      };
       for (int p0 = 0; p0 < np; p0 += kMomentPairs * kWarp) {
 #pragma unroll
         for (int u = 0; u < kMomentPairs; ++u) c[u] = nxt[u];
@@ -197,9 +217,9 @@ __global__ void __launch_bounds__(kNoAllocThreads, 3)
           m = max(max(m, max(__float_as_uint(c[u].x) << 1, __float_as_uint(c[u].y) << 1)),
                   max(__float_as_uint(c[u].z) << 1, __float_as_uint(c[u].w) << 1));
         if (m == 0u) continue;
-        const int e = (int)(m >> 24);
+        const int e = max((int)(m >> 24), 1);
         if (e == 255) {   // an infinity or a NaN: in FP64
-          const int ii = i - nx / 2;
+          const int ii = i - nx / 2, jj = j - ny / 2;
           const double wxy = (double)(quad_weight3(i, nx, simpson) * quad_weight3(j, ny, simpson));
 #pragma unroll 1
           for (int u = 0; u < 2 * kMomentPairs; ++u) {
@@ -215,48 +235,28 @@ __global__ void __launch_bounds__(kNoAllocThreads, 3)
           }
           continue;
         }
-        // scale 2^(sb - 127): the largest magnitude of the run so far in [1, 2), later ones up to
-        // 2^20 larger before the run is passed on
-        const int want = max(254 - e, 1);
-        if (!sb || want < sb - 20) {
-          // the sums of the lines before stay at the old scale: pass them and this line's on
-          s0.add(__fmul_rn(wy, t0.hi));
-          s0.lo = __fadd_rn(s0.lo, __fmul_rn(wy, t0.lo));
-          add_weighted(sy, wy * (float)(jj * jj), t0.hi, t0.lo);
-          add_weighted(sz, wy, tz.hi, tz.lo);
-          t0 = tz = DFAcc{};
+        if (e > E) {   // the first points, or one above E: the sums so far stay at the old unit
+          fold();
           flush(i);
-          sb = want;
+          E = e + 3;
         }
+        // psi scaled so that E becomes base = 200 (by 2^127 at most: base >= 131)
+        const int sb = min(327 - E, 254), base = E + sb - 127;
         const float sc = __int_as_float(sb << 23);
 #pragma unroll
         for (int u = 0; u < kMomentPairs; ++u) {
           const int p = p0 + u * kWarp + lane;
-          const float4 w = wz[min(p, np - 1)];   // (past the line's end the density is zero)
+          const uint4 w = wz[min(p, np - 1)];   // (past the line's end the density is zero)
 #pragma unroll
           for (int h = 0; h < 2; ++h) {
-            const float re = __fmul_rn(h ? c[u].z : c[u].x, sc), im = __fmul_rn(h ? c[u].w : c[u].y, sc);
-            const float a = __fmul_rn(re, re), b = __fmul_rn(im, im);
-            DFAcc d;
-            d.hi = a;
-            d.lo = __fadd_rn(__fmaf_rn(re, re, -a), __fmaf_rn(im, im, -b));
-            d.add(b);
-            const float w0 = h ? w.z : w.x, w2 = h ? w.w : w.y;
-            t0.add(__fmul_rn(w0, d.hi));
-            t0.lo = __fmaf_rn(w0, d.lo, t0.lo);
-            add_weighted(tz, w2, d.hi, d.lo);
+            const unsigned long long d = square_units(__fmul_rn(h ? c[u].z : c[u].x, sc), base) +
+                                         square_units(__fmul_rn(h ? c[u].w : c[u].y, sc), base);
+            t0.add(h ? w.z : w.x, d);
+            tz.add(h ? w.w : w.y, d);
           }
         }
       }
-      renorm(t0);
-      renorm(tz);
-      s0.add(__fmul_rn(wy, t0.hi));   // exact: W_y is 0, 1, 2 or 4
-      s0.lo = __fmaf_rn(wy, t0.lo, s0.lo);
-      add_weighted(sy, wy * (float)(jj * jj), t0.hi, t0.lo);
-      add_weighted(sz, wy, tz.hi, tz.lo);
-      renorm(s0);
-      renorm(sy);
-      renorm(sz);
+      fold();
       if (++j == ny) {
         flush(i);
         j = 0;
@@ -328,9 +328,8 @@ extern "C" int dgpe_moments_noalloc(const void *psi, const dgpe_params *p, doubl
     k_moments_noalloc<double><<<blocks, kNoAllocThreads, 0, st>>>(static_cast<const cplx<double> *>(psi), p->nx,
                                                                   p->ny, p->nz, p->hx, p->hy, p->hz, simpson,
                                                                   scr, out);
-  // FP32 pairs where the time is the arithmetic's.  Below 2^17 points the FP64 kernel takes under
-  // 2 us of its pipe, and the pairs' rounding (2^-48 a point) does not yet average out below the
-  // FP64 sums' own.  Odd lines have no pairs of points.
+  // Integers where the time is the arithmetic's: below 2^17 points the FP64 kernel takes under 2 us of
+  // its pipe.  Odd lines have no pairs of points.
   else if (p->nz % 2 == 0 && nlines * p->nz >= (1 << 17))
     return moments_f32(psi, p, simpson, nlines, scr, out, st);
   else
