@@ -2243,10 +2243,13 @@ __device__ __forceinline__ void k5_zline_body(const KArgs &a, const KArgs *ga) {
     const C *gpsi = reinterpret_cast<const C *>(a.psi);
     [[maybe_unused]] const size_t sx = (size_t)a.ny * nz;
     if constexpr (std::is_same<R, float>::value) {
-      ObsSums t(a, i);   // (short lines only: the others take dgpe_stages.cuh's kernel)
-      for (int b = threadIdx.x; b < nl; b += blockDim.x) {
+      // lines of fewer than 12 points and radix orders other than the default one (the others take
+      // dgpe_stages.cuh's kernel): half a warp or a warp per line
+      const int w = nz > kWarp / 2 ? kWarp : kWarp / 2;
+      ObsSums t(a, i);
+      for (int b = threadIdx.x / w; b < nl; b += blockDim.x / w) {
         t.begin(j0 + b);
-        for (int n = 0; n < nz; ++n) {
+        for (int n = threadIdx.x % w; n < nz; n += w) {
           const C z = res[n * SB + (b >> 1)];
           t.add(n, ((b & 1) ? z.im : z.re) * inv_ntot);
         }
