@@ -290,7 +290,13 @@ int dgpe_batch_sync(dgpe_batch *b);
  * contexts stay owned by the caller and usable.  NULL is safe.  (No paper counterpart.) */
 void dgpe_batch_destroy(dgpe_batch *b);
 
-/* Launch shape of a context's step.  Paper: Summary of revisions, DBEC-GP-MPI (performance
+/* Launch shape of a context's step.  What the step reads of it: in FP64 (and double-float of 2^16
+ * points and more) nothing along lines of 12 points and more, whose kernels have their own radices and
+ * shapes (there plan_style[2] selects the transforms of dgpe_get_phi, dgpe_observables and the
+ * differentiation calls alone); in FP32 plan_style, and ylines and fft_threads where the radix order is
+ * another than 0's (the default order's kernels have their own shapes) and within the differentiation
+ * calls; along lines of fewer than 12 points and in double-float below 2^16 points plan_style, ylines and
+ * fft_threads.  Paper: Summary of revisions, DBEC-GP-MPI (performance
  * depends on the grid sizes and the machine, and configurations should be tried). */
 typedef struct dgpe_tuning {
   int plan_style[3];     /* FFT radix order per axis: 0 radix-8 first, 1 radix-4, 2 radix-3 first */
@@ -302,8 +308,8 @@ typedef struct dgpe_tuning {
 } dgpe_tuning;
 
 /* Time candidate launch shapes on this context's own shape (a few steps each, with CUDA
- * events per kernel), choose the fastest per kernel class (a radix order other than the
- * default only when it is more than 3 % faster), apply it and report it in *out.
+ * events per kernel), choose the fastest per kernel class (a field is varied only where the
+ * step reads it, and changed only for a gain of more than 3 %), apply it and report it in *out.
  * psi and the device state are restored afterwards.  Synchronises; allocates one
  * psi-sized temporary with cudaMallocAsync.  Paper: as dgpe_tuning. */
 int dgpe_autotune(dgpe_ctx *ctx, dgpe_tuning *out);

@@ -674,6 +674,24 @@ int apply_tuning(dgpe_ctx *c, const dgpe_tuning &t) {
   return rc;
 }
 
+FftPlan axis_plan(const dgpe_ctx *c, int d, int style) { return make_plan(d == 0 ? c->p.nx : d == 1 ? c->p.ny : c->p.nz, style); }
+bool same_plan(const FftPlan &a, const FftPlan &b) {
+  if (a.n != b.n || a.nstages != b.nstages) return false;
+  for (int k = 0; k < a.nstages; ++k)
+    if (a.radix[k] != b.radix[k]) return false;
+  return true;
+}
+// What the step's kernels read of a tuning.  The fixed-point kernels (FP64) have their own radices and
+// launch shapes; so have the FP32 kernels of the default radix order; lines of fewer than 12 points and
+// double-float take the runtime ones.
+bool reads_radix_order(const dgpe_ctx *c, int d) {
+  return !(fp64_kernels(&c->p) && fx_length(d == 0 ? c->p.nx : d == 1 ? c->p.ny : c->p.nz));
+}
+bool reads_launch_shape(const dgpe_ctx *c, int d, int style) {
+  if (pairs(&c->p) || !fx_length(d == 0 ? c->p.nx : c->p.ny)) return true;
+  return !fp64_kernels(&c->p) && !same_plan(axis_plan(c, d, style), axis_plan(c, d, 0));
+}
+
 bool tuning_valid(const dgpe_ctx *c, const dgpe_tuning &t) {
   for (int d = 0; d < 3; ++d)
     if (t.plan_style[d] < 0 || t.plan_style[d] > 2) return false;
@@ -1104,87 +1122,97 @@ int dgpe_autotune(dgpe_ctx *c, dgpe_tuning *out) {
     return rc;
   }
   const dgpe_tuning base = current_tuning(c);
-  const int ylines_opts[5] = {2, 4, 8, 16, 32};
-  const int threads_opts[2] = {256, 128};
   const int steps = 3;
-  // per option, the summed time of the kernels it affects
-  double t_style[3][3] = {{1e30, 1e30, 1e30}, {1e30, 1e30, 1e30}, {1e30, 1e30, 1e30}};
-  double t_y[5][2], t_x[2] = {1e30, 1e30}, t_cn[2] = {1e30, 1e30};
-  for (auto &r : t_y) r[0] = r[1] = 1e30;
-  double default_ms = 0;
   const bool timing = c->timing;
   c->timing = true;
-  for (int round = 0; round < 10 && rc == DGPE_OK; ++round) {
-    dgpe_tuning t = base;
-    const int yi = round % 5, ti = (round / 5) % 2, si = round % 3, ci = round % 2;
-    if (round > 0) {
-      t.ylines = ylines_opts[yi];
-      t.fft_threads = threads_opts[ti];
-      for (int d = 0; d < 3; ++d) t.plan_style[d] = si;
-      t.cn_per_sm = 1 + ci;
+  // per-kernel ms of `steps` steps under a tuning: the least of three goes, after a warm-up step
+  double ms[kNumKernels];
+  auto measure = [&](const dgpe_tuning &t) {
+    int r = apply_tuning(c, t);
+    for (int go = -1; go < 3 && !r; ++go) {
+      double now[kNumKernels];
+      for (int s = 0; s < (go < 0 ? 1 : steps) && !r; ++s) r = enqueue_step(c, c->stream);
+      const int rd = drain_kernel_times(c, now);
+      if (!r) r = rd;
+      for (int q = 0; q < kNumKernels && go >= 0; ++q) ms[q] = go ? fmin(ms[q], now[q]) : now[q];
     }
-    if (!tuning_valid(c, t)) continue;
-    rc = apply_tuning(c, t);
-    if (!rc) rc = enqueue_step(c, c->stream);   // warm-up step of this configuration
-    double ms[kNumKernels];
-    if (!rc) rc = drain_kernel_times(c, ms);
-    for (int s = 0; s < steps && rc == DGPE_OK; ++s) rc = enqueue_step(c, c->stream);
-    if (!rc) rc = drain_kernel_times(c, ms);
-    if (rc) break;
-    double total = 0;
-    for (int q = 0; q < kNumKernels; ++q) total += ms[q];
-    if (round == 0) default_ms = total / steps;
-    const double tz = ms[kK1DensityR2Cz] + ms[kK5C2RzPhaseCnz], ty = ms[kK2FftY] + ms[kK4IfftY],
-                 tx = ms[kK3FftXDipolar], tcn = ms[kK6CnY] + ms[kK7CnXReduce];
-    const int sidx[3] = {t.plan_style[0], t.plan_style[1], t.plan_style[2]};
-    t_style[0][sidx[0]] = fmin(t_style[0][sidx[0]], tx);
-    t_style[1][sidx[1]] = fmin(t_style[1][sidx[1]], ty);
-    t_style[2][sidx[2]] = fmin(t_style[2][sidx[2]], tz);
-    int yk = 0;
-    while (ylines_opts[yk] != t.ylines) ++yk;
-    const int tk = t.fft_threads == 256 ? 0 : 1;
-    t_y[yk][tk] = fmin(t_y[yk][tk], ty);
-    t_x[tk] = fmin(t_x[tk], tx);
-    t_cn[t.cn_per_sm - 1] = fmin(t_cn[t.cn_per_sm - 1], tcn);
-  }
+    return r;
+  };
+  auto total = [&] {
+    double s = 0;
+    for (int q = 0; q < kNumKernels; ++q) s += ms[q];
+    return s / steps;
+  };
+  auto transform_ms = [&](int d) {
+    return d == 0 ? ms[kK3FftXDipolar] : d == 1 ? ms[kK2FftY] + ms[kK4IfftY] : ms[kK1DensityR2Cz] + ms[kK5C2RzPhaseCnz];
+  };
+  // A field is varied only where the step's kernels read it, and changed only for a gain of more than
+  // the timing noise (3 %): between equal kernels the clock would decide, and contexts of one shape
+  // that tuned differently would no longer be grouped in a batch.
+  constexpr double kGain = 0.97;
   dgpe_tuning best = base;
-  if (rc == DGPE_OK) {
-    // another radix order only when it is faster by more than the timing noise (3 %): the
-    // default order is the one with compile-time kernels (faster in grouped launches, where
-    // a single context's few-microsecond kernels do not show it)
+  double default_ms = 0, t_axis[3];
+  rc = measure(base);
+  if (!rc) {
+    default_ms = total();
+    for (int d = 0; d < 3; ++d) t_axis[d] = transform_ms(d);
+  }
+  // radix orders, all axes at a time
+  for (int k = 0; k < 3 && !rc; ++k) {
+    dgpe_tuning t = base;
+    bool varied[3], any = false;
     for (int d = 0; d < 3; ++d) {
-      int b = base.plan_style[d];
-      for (int k = 0; k < 3; ++k)
-        if (t_style[d][k] < 0.97 * t_style[d][b]) b = k;
-      best.plan_style[d] = b;
+      varied[d] = reads_radix_order(c, d) && !same_plan(axis_plan(c, d, k), axis_plan(c, d, base.plan_style[d]));
+      if (varied[d]) t.plan_style[d] = k;
+      any |= varied[d];
     }
-    // y-pass shape and transform threads: the (ylines, threads) pair with the least y + x time
-    double bestv = 1e30;
-    for (int yk = 0; yk < 5; ++yk)
-      for (int tk = 0; tk < 2; ++tk) {
-        const double v = t_y[yk][tk] + t_x[tk];
-        if (v < bestv) {
-          bestv = v;
-          best.ylines = ylines_opts[yk];
-          best.fft_threads = threads_opts[tk];
+    if (!any) continue;
+    rc = measure(t);
+    for (int d = 0; d < 3 && !rc; ++d)
+      if (varied[d] && transform_ms(d) < kGain * t_axis[d]) {
+        t_axis[d] = transform_ms(d);
+        best.plan_style[d] = k;
+      }
+  }
+  // lines and threads of the x and y transforms
+  const bool shape[2] = {reads_launch_shape(c, 0, best.plan_style[0]), reads_launch_shape(c, 1, best.plan_style[1])};
+  if (!rc && (shape[0] || shape[1])) {
+    auto xy = [&] { return (shape[0] ? transform_ms(0) : 0.0) + (shape[1] ? transform_ms(1) : 0.0); };
+    const dgpe_tuning at = best;
+    double least = 0;
+    rc = measure(at);
+    if (!rc) least = kGain * xy();
+    for (int threads = 128; threads <= 256; threads += 128)
+      for (int ylines = 2; ylines <= 32 && !rc; ylines *= 2) {
+        dgpe_tuning t = at;
+        t.fft_threads = threads;
+        if (shape[1]) t.ylines = ylines;
+        else if (ylines > 2) continue;
+        if (!tuning_valid(c, t) || (t.ylines == at.ylines && t.fft_threads == at.fft_threads)) continue;
+        rc = measure(t);
+        if (!rc && xy() < least) {
+          least = xy();
+          best.ylines = t.ylines;
+          best.fft_threads = t.fft_threads;
         }
       }
-    best.cn_per_sm = t_cn[1] < t_cn[0] ? 2 : 1;
-    if (!tuning_valid(c, best)) best = base;
-    rc = apply_tuning(c, best);
-    for (int s = 0; s < 1 + steps && rc == DGPE_OK; ++s) {
-      rc = enqueue_step(c, c->stream);
-      if (s == 0 && !rc) {
-        double ms0[kNumKernels];
-        rc = drain_kernel_times(c, ms0);
-      }
-    }
-    double ms[kNumKernels];
-    if (!rc) rc = drain_kernel_times(c, ms);
-    double total = 0;
-    for (int q = 0; q < kNumKernels; ++q) total += ms[q];
+  }
+  // threads of the FP32 sweeps
+  if (!rc && c->p.precision == DGPE_MIXED) {
+    auto sweeps = [&] { return ms[kK6CnY] + ms[kK7CnXReduce]; };
+    dgpe_tuning t = best;
+    t.cn_per_sm = 3 - best.cn_per_sm;
+    rc = measure(best);
+    const double now = sweeps();
+    if (!rc) rc = measure(t);
+    if (!rc && sweeps() < kGain * now) best.cn_per_sm = t.cn_per_sm;
+  }
+  if (!rc) rc = measure(best);
+  if (!rc) {
     best.step_ms_default = default_ms;
-    best.step_ms_tuned = total / steps;
+    best.step_ms_tuned = total();
+  } else {
+    apply_tuning(c, base);
   }
   c->timing = timing;
   // restore the state the tuning steps advanced

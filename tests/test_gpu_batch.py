@@ -161,3 +161,37 @@ def test_grouped_members_equal_individual_steps(mode, shape):
     b.close()
     for c in batched + alone:
         c.close()
+
+
+@pytest.mark.parametrize("precision,shape", [(abi.DGPE_FP64, (32, 48, 24)), (abi.DGPE_FP64, (64, 64, 64)),
+                                             (abi.DGPE_DF64, (48, 64, 40)), (abi.DGPE_MIXED, (24, 36, 48))])
+def test_autotune_leaves_what_no_kernel_reads(precision, shape):
+    """Fields that the step's kernels do not read stay as they are, whatever the clock says: the FP64
+    kernels read none, the FP32 kernels of the default radix order neither lines nor threads.  So
+    contexts of one shape keep one tuning, and are grouped in a batch."""
+    for _ in range(3):
+        c = abi.Condensate(shape, 0.3, 0.005, mode=abi.DGPE_REAL_TIME, precision=precision, g=25.0, gdd=15.0)
+        c.set_psi(inputs.gaussian_psi(shape, 0.3, seed=31).astype(c.np_cdtype))
+        before, after = c.tuning(), c.autotune()
+        c.close()
+        read = set()
+        if precision == abi.DGPE_MIXED:
+            read = {"plan_style", "cn_per_sm"}
+            if after["plan_style"][:2] != before["plan_style"][:2]:   # those orders' kernels read them
+                read |= {"ylines", "fft_threads"}
+        for k in ("plan_style", "ylines", "fft_threads", "cn_per_sm"):
+            assert k in read or after[k] == before[k], (k, before, after)
+
+
+@pytest.mark.parametrize("precision,shape", [(abi.DGPE_FP64, (8, 10, 24)), (abi.DGPE_FP64, (8, 48, 24)),
+                                             (abi.DGPE_DF64, (16, 18, 20)), (abi.DGPE_MIXED, (10, 8, 6))])
+def test_autotune_where_the_shape_is_read(precision, shape):
+    c = abi.Condensate(shape, 0.3, 0.005, mode=abi.DGPE_REAL_TIME, precision=precision, g=25.0, gdd=15.0)
+    psi = inputs.gaussian_psi(shape, 0.3, seed=31).astype(c.np_cdtype)
+    c.set_psi(psi)
+    t = c.autotune()
+    assert t["step_ms_tuned"] > 0 and t["step_ms_default"] > 0
+    assert np.max(np.abs(c.get_psi() - psi)) <= 2.0 ** -47 * np.max(np.abs(psi))
+    c.set_tuning(t)
+    c.step(2)
+    c.close()
