@@ -72,7 +72,9 @@ extern "C" {
  * step restores the norm the real-time run began with (the norm of the state its first step
  * started from), undoing the drift of the FP32-rounded Crank-Nicolson factors (about 3e-7
  * of the norm per step, systematic); the exact scheme conserves the norm, so this corrects
- * rounding only.  dgpe_grad_z2 runs its trajectory without it. */
+ * rounding only.  dgpe_grad_z2 runs its trajectory without it, on transforms and sweeps of other
+ * radices and chunks than dgpe_step's at most lengths: the same scheme, rounded otherwise (its state
+ * differs from dgpe_step's by a few 1e-7). */
 #define DGPE_MIXED 1
 /* Double-float: every value is a pair of FP32 numbers hi + lo (about 48 significant bits)
  * and every operation runs on the FP32 pipe, which GB300 issues 64 times as fast as FP64; grids

@@ -103,9 +103,10 @@ int sweep_chunk(int n) {
 }
 
 // The same for the differentiation calls: the chunks of the 32-lane (a power of two) and 8-lane
-// (n = 8 CH) solvers.  A gradient is a small difference of FP32 values, so another chunking
-// shows in its seventh digit; dgpe_grad_z2 and dgpe_adjoint_step keep these, on which their
-// stored results rest.
+// (n = 8 CH) layouts, and with them (KArgs::diff) the runtime and compile-time transforms of
+// dgpe_device.cuh.  Their results are FP64 numbers, differences of FP32 fields: with the step's chunks
+// and transforms a loss or gradient changes from its eighth digit on (its error against FP64, 1e-6, is
+// the same either way), and callers that compare runs would see it change.
 int diff_chunk(int n) { return n == 32 || n == 48 || n == 64 || n == 96 || n == 128 ? n / 8 : cn_chunk(n); }
 
 // The chunk of the tables of axis d: the sweeps' own in FP32 along x and y, else cn_chunk.

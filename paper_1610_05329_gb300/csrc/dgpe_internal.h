@@ -113,8 +113,7 @@ struct KArgs {
   double *partials;            // per-block reduction partials
   const void *tw_st[3];        // twiddles of the staged transforms (FP32: dgpe_stages.cuh; FP64-class:
                                // in fixed point, dgpe_fixed.cuh)
-  int diff;                    // 1: within the differentiation calls (FP32: the transforms and chunks whose
-                               // roundings their results rest on)
+  int diff;                    // 1: within the differentiation calls (FP32: their own transforms and chunks)
   const void *tw[3];           // per-stage twiddle tables of plan[d] (layout in FftPlan), d = x, y, z
   FftPlan plan[3];
   CnTab cn[3];
