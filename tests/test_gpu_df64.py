@@ -174,3 +174,87 @@ def test_differentiation_is_unsupported():
         gpu.adjoint_step(z, z.clone())
     assert e.value.code == abi.DGPE_EUNSUPPORTED
     gpu.close()
+
+
+# ---- pairs and FP64 kernels on both sides of 2^16 points ---------------------------------------
+# (Contexts of 2^16 points and more run the FP64 kernels: the pairs are held to long runs below that
+# size, the FP64 kernels behind this precision to a reference that shares none of them.)
+@pytest.mark.parametrize("mode", [abi.DGPE_REAL_TIME, abi.DGPE_IMAG_TIME])
+def test_pairs_over_200_steps(orc, mode):
+    """40^3 = 64000 points, pair arithmetic: 200 steps of the oracle and of the FP64 kernels."""
+    shape, h = (40, 40, 40), 0.3
+    psi0 = inputs.gaussian_psi(shape, h, noise=1e-3, seed=1)
+    gpu, p = make(orc, shape, h, 0.004, mode, nu=(1, 1, 1), g=20, gdd=10)
+    f64 = abi.Condensate(shape, h, 0.004, mode=mode, precision=abi.DGPE_FP64, nu=(1, 1, 1), g=20, gdd=10)
+    for c in (gpu, f64):
+        c.set_psi(psi0)
+        c.step(200)
+    want = orc.step(p, psi0, 200)
+    got, other = gpu.get_psi(), f64.get_psi()
+    assert rel(got, want) < DF_STEP_TOL and rel(got, other) < DF_STEP_TOL
+    assert not np.array_equal(got, other)   # (two arithmetics, not one compared with itself)
+    og, ow = gpu.observables(), orc.observables(p, want)
+    for k in ("norm", "mu", "energy", "e_kin", "e_trap", "e_contact", "e_dipolar"):
+        assert og[k] == pytest.approx(ow[k], rel=1e-9, abs=1e-12), k
+    gpu.close()
+    f64.close()
+
+
+@pytest.mark.parametrize("shape", [(32, 64, 30), (40, 40, 40), (32, 64, 32), (40, 42, 40)])
+def test_both_sides_of_the_threshold(orc, shape):
+    """61440 and 64000 points (pairs), 65536 and 67200 (FP64 kernels): every call at the boundary."""
+    h = tuple(10.0 / n for n in shape)
+    psi = state(shape, 0.3)
+    pairs = np.prod(shape) < 1 << 16
+    gpu, p = make(orc, shape, h, 0.004, abi.DGPE_REAL_TIME)
+    gpu.set_psi(psi)
+    got = gpu.get_psi()
+    assert np.max(np.abs(got - psi)) <= (2.0 ** -47 * np.max(np.abs(psi)) if pairs else 0.0)
+    og, ow = gpu.observables(), orc.observables(p, psi)
+    for k in ("norm", "mu", "energy", "e_kin", "e_trap", "e_contact", "e_dipolar"):
+        assert og[k] == pytest.approx(ow[k], rel=1e-11, abs=1e-13), k
+    assert rel(gpu.phi(), orc.dipolar_phi(p, np.abs(psi) ** 2)) < DF_SUB_TOL
+    gpu.step(5)
+    want = orc.step(p, psi, 5)
+    assert rel(gpu.get_psi(), want) < DF_STEP_TOL
+    out = np.empty_like(psi)
+    gpu.step_host(psi, out, 5)
+    gpu.sync()
+    assert rel(out, want) < DF_STEP_TOL
+    gpu.close()
+
+
+def test_full_size_against_library_transforms():
+    """256^3, real time, against plain torch in 64 bits: library FFTs, dense Cayley matrices."""
+    import torch
+    n, h, dt, g, gdd = 256, 0.1, 1e-3, 40.0, 25.0
+    x = (torch.arange(n, device="cuda", dtype=torch.float64) - n // 2) * h
+    line = torch.exp(torch.complex(-0.35 * x * x, 0.1 * x))
+    psi = line[:, None, None] * line[None, :, None] * line[None, None, :]
+    psi = psi / torch.sqrt(h ** 3 * torch.sum(torch.abs(psi) ** 2))
+    gpu = abi.Condensate((n, n, n), h, dt, mode=abi.DGPE_REAL_TIME, precision=abi.DGPE_DF64, nu=(1.0, 1.0, 1.0), g=g, gdd=gdd)
+    gpu.set_psi(psi)
+    gpu.step(3)
+    got = gpu.get_psi(host=False)
+    k = 2.0 * np.pi * torch.fft.fftfreq(n, h, dtype=torch.float64, device="cuda")
+    kz = k[:n // 2 + 1].abs()
+    k2 = k[:, None, None] ** 2 + k[None, :, None] ** 2 + kz[None, None, :] ** 2
+    k2[0, 0, 0] = 1.0
+    u = 3.0 * (kz ** 2)[None, None, :] / k2 - 1.0
+    u[0, 0, 0] = 0.0
+    c, m = 1j * dt / (4.0 * h * h), n - 2
+    eye = torch.eye(m, dtype=torch.complex128, device="cuda")
+    d = torch.diag(torch.ones(m - 1, dtype=torch.complex128, device="cuda"), 1)
+    d = d + d.T - 2.0 * eye
+    cayley = torch.zeros(n, n, dtype=torch.complex128, device="cuda")
+    cayley[1:-1, 1:-1] = torch.linalg.solve(eye - c * d, eye + c * d)
+    v = 0.5 * (x[:, None, None] ** 2 + x[None, :, None] ** 2 + x[None, None, :] ** 2)
+    for _ in range(3):
+        dens = psi.real ** 2 + psi.imag ** 2
+        phi = torch.fft.irfftn(torch.fft.rfftn(dens) * u, s=(n, n, n))
+        psi = psi * torch.exp(-1j * dt * (v + g * dens + gdd * phi))
+        psi = torch.matmul(psi, cayley.T)
+        psi = torch.matmul(cayley, psi)
+        psi = torch.matmul(cayley, psi.reshape(n, -1)).reshape(n, n, n)
+    assert float(torch.linalg.vector_norm(got - psi) / torch.linalg.vector_norm(psi)) < DF_STEP_TOL
+    gpu.close()
