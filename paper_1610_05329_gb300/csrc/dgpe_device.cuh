@@ -2455,29 +2455,18 @@ __global__ void __launch_bounds__(Tiles<R>::kZThreads,
 
 // ---------------------------------------------------------------------------------------
 // K6 / K7: Crank-Nicolson along y (AXIS = 1, lines psi[i][:][k]) or x (AXIS = 0, lines
-// psi[:][j][k]).  K7 (x) also sums
-// n, x^2 n, y^2 n, z^2 n (FP64 totals) and, in the last block, sets the norm and the pending
-// renormalisation factor s = 1/sqrt(norm) (imaginary time) or 1 (real time).  The x^2 n
-// sum is not taken (nothing reads it: the observables take their own FP64 sums).  FP64
-// data: FP64 sums per thread.  FP32 data (k_cn): the terms n = |psi|^2 in FP32 (the state's
-// own precision), and from there every product exact and every sum in double-float, point
-// by point (error about 2^-44 of the total): the weights are exact small integers (3 x the
-// Simpson weights per axis, the squared signed index instead of the squared coordinate),
-// the products by them exact (FMA exact product), the sums Knuth's TwoSum; the factors
-// h_d^2 and (1/3)^3 (Simpson) are applied in FP64 at the end.
+// psi[:][j][k]); FP64 and double-float also along z (K5's second launch).  K7 (x) also sums n, y^2 n
+// and z^2 n and, in the last block, sets the norm and the pending renormalisation factor
+// s = 1/sqrt(norm) (imaginary time) or 1 (real time).  (Nothing reads x^2 n: the observables take
+// their own sums.)  FP64 (k_cn_fx, dgpe_fixed.cuh): FP64 sums per thread.  FP32 (k_cn_reg): the terms
+// n = |psi|^2 in FP32 (the state's own precision), and from there every product exact and every sum in
+// double-float, point by point and over a block (error about 2^-44 of the total): the weights are exact
+// small integers (3 x the Simpson weights per axis, the squared signed index instead of the squared
+// coordinate), the products by them exact (FMA exact product), the sums Knuth's TwoSum; FP64 across
+// blocks; the factors h_d^2 and (1/3)^3 (Simpson) are applied in FP64 at the end.
 // ---------------------------------------------------------------------------------------
-// Running sums of the reduction of the FP64-class per-line sweeps: FP64 for FP64 data,
-// double-float pairs for double-float data.
-template <typename R>
-struct SumAcc;
-template <>
-struct SumAcc<double> {
-  double v = 0.0;
-  __device__ __forceinline__ void add(double t) { v += t; }
-  __device__ __forceinline__ double value() const { return v; }
-};
-template <>
-struct SumAcc<df> {
+// Running sums of the double-float sweeps.
+struct SumAcc {
   df v{0.0f, 0.0f};
   __device__ __forceinline__ void add(df t) { v = v + t; }
   __device__ __forceinline__ double value() const { return (double)v; }
@@ -2758,7 +2747,7 @@ __global__ void __launch_bounds__(128, 7) k_cn_twisted(KArgs a, int reduce, int 
     for (int n = threadIdx.x; n < N; n += blockDim.x) wxtab[n] = R(quad_weight(n, a.nx, a.simpson));
     __syncthreads();
   }
-  SumAcc<R> acc[4];
+  SumAcc acc[4];
   const long long ln = active ? line : 0;
   const int k = (int)(ln % a.nz), fixed = (int)(ln / a.nz);
   const size_t stride = AXIS == 2 ? (size_t)1 : AXIS == 1 ? (size_t)a.nz : (size_t)a.ny * a.nz;
@@ -3238,18 +3227,9 @@ struct Impl {
       chk(allow_smem(k1_density_r2cz<R, 384>));
       chk(allow_smem(k1_density_r2cz<R, 256>));
       chk(allow_smem(k1_density_r2cz<R, 128>));
-      chk(allow_smem(k_ffty<R, -1, 512>));
-      chk(allow_smem(k_ffty<R, +1, 512>));
       chk(allow_smem(k_ffty<R, -1, 384>));
       chk(allow_smem(k_ffty<R, +1, 384>));
-      chk(allow_smem(k_ffty<R, -1, 256>));
-      chk(allow_smem(k_ffty<R, +1, 256>));
-      chk(allow_smem(k_ffty<R, -1, 128>));
-      chk(allow_smem(k_ffty<R, +1, 128>));
-      chk(allow_smem(k3_fftx_dipolar<R, 512>));
       chk(allow_smem(k3_fftx_dipolar<R, 384>));
-      chk(allow_smem(k3_fftx_dipolar<R, 256>));
-      chk(allow_smem(k3_fftx_dipolar<R, 128>));
       chk(allow_smem(k5_zline<R, R, kZFast, 512>));
       chk(allow_smem(k5_zline<R, C, kZFast, 512>));
       chk(allow_smem(k5_zline<R, R, kZFast, 384>));
@@ -3405,10 +3385,7 @@ struct Impl {
     const dim3 g((unsigned)((lines + L - 1) / L));
     const size_t sm = smem_y(a);
     if constexpr (kCtSizes) {
-      if (y_fixed(a, 512)) k_ffty<R, DIR, 512><<<g, kFftThreads, sm, st>>>(a, nullptr);
-      else if (y_fixed(a, 384)) k_ffty<R, DIR, 384><<<g, kFftThreads, sm, st>>>(a, nullptr);
-      else if (y_fixed(a, 256)) k_ffty<R, DIR, 256><<<g, kFftThreads, sm, st>>>(a, nullptr);
-      else if (y_fixed(a, 128)) k_ffty<R, DIR, 128><<<g, kFftThreads, sm, st>>>(a, nullptr);
+      if (y_fixed(a, 384)) k_ffty<R, DIR, 384><<<g, kFftThreads, sm, st>>>(a, nullptr);   // (the differentiation calls)
       else k_ffty<R, DIR, 0><<<g, a.fft_threads, sm, st>>>(a, nullptr);
     } else {
       k_ffty<R, DIR, 0><<<g, a.fft_threads, sm, st>>>(a, nullptr);
@@ -3426,12 +3403,9 @@ struct Impl {
     }
     dim3 grid((a.ny + T::kXCols - 1) / T::kXCols, a.nzh);
     const size_t sm = smem_x(a);
-    const bool fixed = a.fft_threads == kFftThreads;
     if constexpr (kCtSizes) {
-      if (fixed && plan_ct(a.plan[0], 512)) k3_fftx_dipolar<R, 512><<<grid, kFftThreads, sm, st>>>(a, nullptr);
-      else if (fixed && plan_ct(a.plan[0], 384)) k3_fftx_dipolar<R, 384><<<grid, kFftThreads, sm, st>>>(a, nullptr);
-      else if (fixed && plan_ct(a.plan[0], 256)) k3_fftx_dipolar<R, 256><<<grid, kFftThreads, sm, st>>>(a, nullptr);
-      else if (fixed && plan_ct(a.plan[0], 128)) k3_fftx_dipolar<R, 128><<<grid, kFftThreads, sm, st>>>(a, nullptr);
+      if (a.fft_threads == kFftThreads && plan_ct(a.plan[0], 384))   // (the differentiation calls)
+        k3_fftx_dipolar<R, 384><<<grid, kFftThreads, sm, st>>>(a, nullptr);
       else k3_fftx_dipolar<R, 0><<<grid, a.fft_threads, sm, st>>>(a, nullptr);
     } else {
       k3_fftx_dipolar<R, 0><<<grid, a.fft_threads, sm, st>>>(a, nullptr);
@@ -3656,9 +3630,6 @@ struct GroupLaunch {
     attr(k1_density_r2cz<R, 0, true>, e);
     attr(k_ffty<R, -1, 0, true>, e);
     attr(k_ffty<R, +1, 0, true>, e);
-    attr(k_ffty<R, -1, 384, true>, e);
-    attr(k_ffty<R, +1, 384, true>, e);
-    attr(k3_fftx_dipolar<R, 384, true>, e);
     attr(k3_fftx_dipolar<R, 0, true>, e);
     using K = void (*)(KArgs, const KArgs *);
     attr(static_cast<K>(k_ffty_reg<-1, 512, true>), e);
@@ -3703,8 +3674,7 @@ struct GroupLaunch {
     const int L = a.ylines;
     const dim3 g((unsigned)((lines + L - 1) / L), 1, n);
     const size_t sm = I::smem_y(a);
-    if (I::y_fixed(a, 384)) k_ffty<R, DIR, 384, true><<<g, kFftThreads, sm, st>>>(a, ga);
-    else k_ffty<R, DIR, 0, true><<<g, a.fft_threads, sm, st>>>(a, ga);
+    k_ffty<R, DIR, 0, true><<<g, a.fft_threads, sm, st>>>(a, ga);
   }
   static void k3(const KArgs &a, const KArgs *ga, unsigned n, cudaStream_t st) {
     auto reg = [&](auto len) {
@@ -3717,10 +3687,7 @@ struct GroupLaunch {
     if (I::staged(a, 0) && stage_x(a, ga, n, st)) return;
     const dim3 g((a.ny + T::kXCols - 1) / T::kXCols, a.nzh, n);
     const size_t sm = I::smem_x(a);
-    if (a.fft_threads == kFftThreads && I::plan_ct(a.plan[0], 384))
-      k3_fftx_dipolar<R, 384, true><<<g, kFftThreads, sm, st>>>(a, ga);
-    else
-      k3_fftx_dipolar<R, 0, true><<<g, a.fft_threads, sm, st>>>(a, ga);
+    k3_fftx_dipolar<R, 0, true><<<g, a.fft_threads, sm, st>>>(a, ga);
   }
   template <typename Co>
   static void k5(const KArgs &a, const KArgs *ga, unsigned n, cudaStream_t st) {
