@@ -79,4 +79,30 @@ int host_phase(int imag, double *z, long long v, double g) {
   const fxs zero = fx_scalar(0.0);
   return imag ? fx_phase<true>(z[0], z[1], v, fx_scalar(g), zero, 1000, 0) : fx_phase<false>(z[0], z[1], v, fx_scalar(g), zero, 1000, 0);
 }
+// (cos theta, -sin theta) 2^60 of theta 2^58; e^-theta = p 2^(n - 60)
+void host_cis(long long th, long long *out) {
+  const fxc c = fx_cis(th);
+  out[0] = c.re;
+  out[1] = c.im;
+}
+long long host_exp(long long th, int *n) { return fx_exp(th, *n); }
+// the butterfly of radix p in place on p complex values
+void host_butterfly(int dir, int p, long long *v) {
+  fxc *z = reinterpret_cast<fxc *>(v);
+  auto go = [&](auto radix) {
+    constexpr int P = decltype(radix)::value;
+    if (p != P) return;
+    if (dir < 0) fx_bf<-1, P>(z);
+    else fx_bf<+1, P>(z);
+  };
+  go(std::integral_constant<int, 2>{});
+  go(std::integral_constant<int, 3>{});
+  go(std::integral_constant<int, 4>{});
+  go(std::integral_constant<int, 5>{});
+  go(std::integral_constant<int, 6>{});
+  go(std::integral_constant<int, 7>{});
+  go(std::integral_constant<int, 8>{});
+  go(std::integral_constant<int, 9>{});
+  go(std::integral_constant<int, 10>{});
+}
 }

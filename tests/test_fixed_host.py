@@ -168,3 +168,55 @@ def test_real_time_sweep_by_magnitude(lib, scale, r):
     bound[m // 2] = 10.0
     bound = bound * np.finfo(np.float64).eps * np.abs(want)
     assert np.all(np.abs((got - want).real) <= bound) and np.all(np.abs((got - want).imag) <= bound)
+
+
+# ---- the constants ---------------------------------------------------------------------------
+@pytest.mark.parametrize("reach", [1e-3, 0.125, 0.1251, 0.8, 3.2, 17.9])
+def test_cis(lib, reach):
+    """e^{-i theta} in absolute terms within 2^-57 (the fits of the short angles, whose remainder is
+    2^-58, and the rounding of five products at 2^-60; the long ones' reduction by quarter turns)."""
+    mp = pytest.importorskip("mpmath")
+    rng = np.random.default_rng(7)
+    out = pair(0, 0)
+    with mp.workprec(120):
+        for x in np.concatenate([rng.uniform(-reach, reach, 2000), [0.0, reach, -reach]]):
+            th = int(round(x * 2.0 ** 58))
+            lib.host_cis(ctypes.c_longlong(th), out)
+            angle = mp.mpf(th) / 2 ** 58
+            assert abs(mp.mpf(out[0]) / 2 ** 60 - mp.cos(angle)) < mp.mpf(2) ** -57
+            assert abs(mp.mpf(out[1]) / 2 ** 60 + mp.sin(angle)) < mp.mpf(2) ** -57
+
+
+@pytest.mark.parametrize("reach", [1e-3, 0.5, 4.0, 17.9])
+def test_exp(lib, reach):
+    """e^-theta within 2^-56 of itself: theta log2 e, up to 26, rounded twice at 2^-58 of a turn."""
+    mp = pytest.importorskip("mpmath")
+    lib.host_exp.restype = ctypes.c_longlong
+    rng = np.random.default_rng(8)
+    n = ctypes.c_int(0)
+    with mp.workprec(120):
+        for x in np.concatenate([rng.uniform(-reach, reach, 2000), [0.0, reach, -reach]]):
+            th = int(round(x * 2.0 ** 58))
+            p = lib.host_exp(ctypes.c_longlong(th), ctypes.byref(n))
+            want = mp.exp(-mp.mpf(th) / 2 ** 58)
+            assert abs(mp.mpf(p) * mp.mpf(2) ** (n.value - 60) - want) < mp.mpf(2) ** -56 * want
+
+
+@pytest.mark.parametrize("p", range(2, 11))
+@pytest.mark.parametrize("dir", [-1, 1])
+def test_butterflies(lib, p, dir):
+    """Against the discrete Fourier sum.  A product by a constant is off by less than a unit (half of
+    rounding, less than half of the words left out), a halving or quartering by less than one; an
+    output has at most 6 products (radix 7) or two levels of 2 + 2 (radices 9 and 10): 16 units."""
+    mp = pytest.importorskip("mpmath")
+    rng = np.random.default_rng(p)
+    with mp.workprec(140):
+        w = [mp.expjpi(mp.mpf(2 * dir * k) / p) for k in range(p)]
+        for _ in range(50):
+            v = [int(x) for x in rng.integers(-(1 << 58), 1 << 58, 2 * p)]
+            z = [mp.mpc(v[2 * k], v[2 * k + 1]) for k in range(p)]
+            buf = (ctypes.c_longlong * (2 * p))(*v)
+            lib.host_butterfly(dir, p, buf)
+            for k in range(p):
+                want = mp.fsum(z[j] * w[j * k % p] for j in range(p))
+                assert abs(buf[2 * k] - want.real) < 16 and abs(buf[2 * k + 1] - want.imag) < 16, k
