@@ -60,25 +60,25 @@ DGPE_HD long long fx_const(long long a) {
   return NI == 0 ? p : NI > 0 ? p + a : p - a;
 }
 
-// A twiddle w 2^60, split into signed words.
+// A twiddle w 2^60, split into signed words.  The low word of the imaginary part is never -2^31, which
+// has no 32-bit negative: fx_words, by which every factor is made, moves such a value by one unit.
 struct __align__(16) fxw {
   int rh, rl, ih, il;
 };
+DGPE_HD fxw fx_words(long long re, long long im) {
+  if (fx_lo(im) == (int)0x80000000) ++im;
+  return {fx_hi(re), fx_lo(re), fx_hi(im), fx_lo(im)};
+}
 // a w / 2^64 = a w / 16 (DIR < 0) or a conj(w) / 16, for components of a below 2^62 (|a| below
-// 2^62.5): the middle sums stay below 2^62 + 2^60.  The products that count negative are subtracted
-// in 64 bits (a low word of -2^31 has no negative; a high one, at most 2^28, does).
+// 2^62.5): the middle sums stay below 2^62 + 2^60.  (The negatives in 32 bits cost nothing; with sums
+// subtracted in 64 bits K3 at 256^3 took 191 us instead of 171.)
 template <int DIR>
 DGPE_HD fxc fx_twiddle(fxc a, fxw w) {
   const int rh = fx_hi(a.re), rl = fx_lo(a.re), ih = fx_hi(a.im), il = fx_lo(a.im);
-  if constexpr (DIR < 0) {
-    const long long mr = fx_mad(rh, w.rl, fx_mad(rl, w.rh, kFxHalf)) - fx_mad(ih, w.il, fx_mad(il, w.ih, 0));
-    const long long mi = fx_mad(rh, w.il, fx_mad(rl, w.ih, fx_mad(ih, w.rl, fx_mad(il, w.rh, kFxHalf))));
-    return {fx_mad(rh, w.rh, fx_mad(ih, -w.ih, mr >> 32)), fx_mad(rh, w.ih, fx_mad(ih, w.rh, mi >> 32))};
-  } else {
-    const long long mr = fx_mad(rh, w.rl, fx_mad(rl, w.rh, fx_mad(ih, w.il, fx_mad(il, w.ih, kFxHalf))));
-    const long long mi = fx_mad(ih, w.rl, fx_mad(il, w.rh, kFxHalf)) - fx_mad(rh, w.il, fx_mad(rl, w.ih, 0));
-    return {fx_mad(rh, w.rh, fx_mad(ih, w.ih, mr >> 32)), fx_mad(ih, w.rh, fx_mad(rh, -w.ih, mi >> 32))};
-  }
+  const int wih = DIR < 0 ? w.ih : -w.ih, wil = DIR < 0 ? w.il : -w.il;
+  const long long mr = fx_mad(rh, w.rl, fx_mad(rl, w.rh, fx_mad(ih, -wil, fx_mad(il, -wih, kFxHalf))));
+  const long long mi = fx_mad(rh, wil, fx_mad(rl, wih, fx_mad(ih, w.rl, fx_mad(il, w.rh, kFxHalf))));
+  return {fx_mad(rh, w.rh, fx_mad(ih, -wih, mr >> 32)), fx_mad(rh, wih, fx_mad(ih, w.rh, mi >> 32))};
 }
 
 // ---- block scaling -------------------------------------------------------------------------
@@ -513,7 +513,7 @@ DGPE_HD bool fx_phase(double &zre, double &zim, long long v, fxs g, fxs dd, int 
     zim = fx_to(fx_mul(z.im, ph, pl), ei + 6 + k);
   } else {
     const fxc c = fx_cis(th);
-    const cplx<double> r = fx_to(fx_twiddle<-1>(z, fxw{fx_hi(c.re), fx_lo(c.re), fx_hi(c.im), fx_lo(c.im)}), em + 6);
+    const cplx<double> r = fx_to(fx_twiddle<-1>(z, fx_words(c.re, c.im)), em + 6);
     zre = r.re;
     zim = r.im;
   }
@@ -979,9 +979,9 @@ static __device__ __noinline__ cplx<double> phase_fp64(cplx<double> z, double ph
   return {z.re * cs + z.im * sn, z.im * cs - z.re * sn};
 }
 // K5's phase pass: packing of the two half spectra, inverse transform (Phi), potential step.  Bound by
-// integer issue; at 256^3, real time, 1100 us in FP64, 765 with the transform in integers, 310 with
+// integer issue; at 256^3, real time, 1100 us in FP64, 765 with the transform in integers, 295 with
 // the angle and its factor too (imaginary time, whose exponential was CUDA's, at 480x480x250: 3060 ->
-// 1400).
+// 1500, 80 of them for an exponent per component).
 template <typename R, int N>
 __global__ void __launch_bounds__(FxZ<N>::NT) k5_fx(const __grid_constant__ KArgs a) {
   using C = cplx<R>;
@@ -1135,7 +1135,7 @@ __global__ inline void k_fx_cn_tables(CnJobs jobs) {
     for (int i = threadIdx.x; i < n; i += kWarp) {
       const Z64 z = get(q, i);
       const long long re = __double2ll_rn(ldexp(z.re, kFxCoefBits + k[q])), im = __double2ll_rn(ldexp(z.im, kFxCoefBits + k[q]));
-      out[1 + q * n + i] = {fx_hi(re), fx_lo(re), fx_hi(im), fx_lo(im)};
+      out[1 + q * n + i] = fx_words(re, im);
     }
 }
 
@@ -1150,15 +1150,15 @@ __global__ inline void k_fx_cn_tables(CnJobs jobs) {
 // Real time: the running values are integers with their own exponent (fxv).  In FP64 arithmetic a sweep is
 // 12 FP64 instructions per point, 0.32 ms of that pipe at 256^3; this is about 330 integer ones (0.14 ms)
 // and two FP64 subtractions.  Imaginary time: FP64 arithmetic.  Its real coefficients make a sweep 6 FP64
-// instructions per point, no more than the integers take (a step at 480x480x250 6.52 ms with either, at
-// 64^3 104 -> 99 us), and each component of psi keeps its own 53 bits.  Persistent CTAs: y waits for the way back in a scratch of the CTA's own
+// instructions per point, no more than the integers take (us at 256^3, integers -> FP64: y 254 -> 238, x with
+// its sums 341 -> 381, z 296 -> 272; a step at 64^3 104 -> 98), and each component of psi keeps its own 53 bits.  Persistent CTAs: y waits for the way back in a scratch of the CTA's own
 // (packed, 16 bytes a point), so few enough lines are under way for much of it and of their psi to
 // stay in L2.  psi and y come through shared memory by cp.async, two chunks of four points ahead;
 // along z, where a thread's points are consecutive, the lanes of a warp copy each other's chunks as
 // segments of 64 bytes, both ways.  Bound by the latency of the recurrence (a warp issues every 4 to 5
 // cycles; half of the issue slots at 12 warps per SM; DRAM 1.1 GB, 165 us).  Measured at 256^3, real
-// time, us, before (FP64 arithmetic, k_cn_twisted) -> now: y 411 -> 285, x with its sums 515 -> 360, z
-// 410 -> 320; errors against extended precision 0.5 to 0.8 of the FP64 sweep's.
+// time, us, FP64 arithmetic (without these pipelines) -> now: y 411 -> 292, x with its sums 515 -> 378, z
+// 410 -> 325; errors against extended precision 0.7 of the FP64 sweep's (1.1e-16 and 1.6e-16).
 constexpr int kFxcThreads = 128, kFxcChunk = 4, kFxcStages = 3;
 template <int AXIS>
 constexpr size_t fx_cn_smem(bool reduce, int nx) {
@@ -1419,7 +1419,7 @@ __global__ inline void k_fx_twiddles(fxw *tw, int n, int r1, int r2, int r3) {
   double s, c;
   sincospi(2.0 * (double)(r * k) / (double)(ns * p), &s, &c);
   const long long qc = __double2ll_rn(c * 1152921504606846976.0), qs = __double2ll_rn(-s * 1152921504606846976.0);   // 2^60
-  tw[t] = {fx_hi(qc), fx_lo(qc), fx_hi(qs), fx_lo(qs)};
+  tw[t] = fx_words(qc, qs);
 }
 
 // One translation unit's lengths: every kFxParts-th of the list.

@@ -7,8 +7,6 @@
 using namespace dgpe;
 
 namespace {
-fxw words(long long re, long long im) { return {fx_hi(re), fx_lo(re), fx_hi(im), fx_lo(im)}; }
-
 // One line of the real-time sweep k_cn_fx, interior points only: al, be = alpha and 2 beta (FP64 pairs) of m
 // points, ginv = 1 / gamma, r = dt / (4 h^2).
 struct Z {
@@ -27,7 +25,7 @@ void sweep(int m, double r, const Z *al, const Z *be, Z ginv, Z *psi) {
   };
   const int ka = exponent(al), kb = exponent(be);
   auto coef = [&](const Z *t, int i, int k) {
-    return i < m ? words(std::llrint(std::ldexp(t[i].re, kFxCoefBits + k)), std::llrint(std::ldexp(t[i].im, kFxCoefBits + k))) : fxw{0, 0, 0, 0};
+    return i < m ? fx_words(std::llrint(std::ldexp(t[i].re, kFxCoefBits + k)), std::llrint(std::ldexp(t[i].im, kFxCoefBits + k))) : fxw{0, 0, 0, 0};
   };
   std::vector<fxc> y(m);
   std::vector<Z> out(m);
@@ -66,7 +64,7 @@ void sweep(int m, double r, const Z *al, const Z *be, Z ginv, Z *psi) {
 extern "C" {
 // a w / 2^64 (dir < 0) or a conj(w) / 2^64
 void host_twiddle(int dir, const long long *a, const long long *w, long long *out) {
-  const fxc r = dir < 0 ? fx_twiddle<-1>({a[0], a[1]}, words(w[0], w[1])) : fx_twiddle<+1>({a[0], a[1]}, words(w[0], w[1]));
+  const fxc r = dir < 0 ? fx_twiddle<-1>({a[0], a[1]}, fx_words(w[0], w[1])) : fx_twiddle<+1>({a[0], a[1]}, fx_words(w[0], w[1]));
   out[0] = r.re;
   out[1] = r.im;
 }
