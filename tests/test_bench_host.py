@@ -76,3 +76,27 @@ def test_reference_arm_prints_the_contract_line():
     assert line["cpu_baseline"]["value"] == line["value"]
     assert line["e2e"] == {"value": line["value"], "unit": line["unit"], "h2d_bytes_per_step": 0,
                            "d2h_bytes_per_step": 0}
+
+
+def test_traffic_key_covers_every_kernel_header(monkeypatch):
+    """A stored traffic figure must not outlive a change of any kernel: the key changes with each of
+    the headers that the kernels stand in."""
+    import builtins
+    import io
+    import os
+    csrc = os.path.join(bench.ROOT, "paper_1610_05329_gb300", "csrc")
+    headers = sorted(f for f in os.listdir(csrc) if f.endswith(".cuh"))
+    key, plain = bench.kernel_source_sha1(), builtins.open
+    for changed in headers:
+        def other(path, *a, **k):
+            return io.BytesIO(b"changed") if os.path.basename(str(path)) == changed else plain(path, *a, **k)
+        monkeypatch.setattr(builtins, "open", other)
+        assert bench.kernel_source_sha1() != key, changed
+        monkeypatch.undo()
+
+
+def test_arithmetic_of_double_float_by_size():
+    assert bench.arithmetic(bench.WORKLOADS["real256_df64"]) == "fp64"
+    assert bench.arithmetic({"shape": (40, 40, 40), "precision": "df64"}) == "df64"
+    assert bench.arithmetic({"shape": (32, 64, 32), "precision": "df64"}) == "fp64"
+    assert bench.arithmetic(bench.WORKLOADS["real512x512x384_mixed"]) == "mixed"
