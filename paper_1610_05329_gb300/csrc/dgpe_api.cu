@@ -148,8 +148,8 @@ int check_physics(const dgpe_params *p) {
 
 // Double-float contexts of this many points and more run on the FP64 kernels (complex128 is their
 // boundary type too, and the fixed-point kernels keep 53 bits where pairs keep 48): us a step, pairs
-// against FP64, real time: 32^3 66 and 74, 48x64x40 97 and 87, 64^3 111 and 105, 128^3 312 and 268,
-// 256^3 1763 and 1670.
+// against FP64, real time: 32^3 66 and 72, 40^3 78 and 78, 48x64x40 97 and 87, 64^3 111 and 106, 128^3 312
+// and 276, 256^3 1763 and 1710.
 constexpr size_t kFp64Points = 1 << 16;
 bool fp64_kernels(const dgpe_params *p) {
   return p->precision == DGPE_FP64 || (p->precision == DGPE_DF64 && (size_t)p->nx * p->ny * p->nz >= kFp64Points);
