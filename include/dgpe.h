@@ -68,7 +68,7 @@ extern "C" {
  * Values below 2^-960 lose bits, and results below 2^-1022 are 0. */
 #define DGPE_FP64 0
 /* complex64 psi; FFT, phase and CN in FP32; the norm and the observables' sums FP64-class
- * (FP32 terms, exact weights, double-float sums per point, FP64 across blocks).  In real time every
+ * (FP32 terms, exact weights, double-float sums per point and over a block, FP64 across blocks).  In real time every
  * step restores the norm the real-time run began with (the norm of the state its first step
  * started from), undoing the drift of the FP32-rounded Crank-Nicolson factors (about 3e-7
  * of the norm per step, systematic); the exact scheme conserves the norm, so this corrects
@@ -195,8 +195,8 @@ int dgpe_step(dgpe_ctx *ctx, int nsteps);
  * dgpe_set_psi), run nsteps steps, copy the result (as dgpe_get_psi) to host memory `out`.
  * Asynchronous: the copies run on two internal streams, and successive calls alternate the
  * state between the workspace's psi buffer and a second one of the same size (allocated at
- * the first call with cudaMalloc, outside the workspace, freed by dgpe_destroy; double-float
- * also stages its converted output), so the input copy of one call overlaps the previous
+ * the first call with cudaMalloc, outside the workspace, freed by dgpe_destroy; double-float pairs
+ * also stage their converted output), so the input copy of one call overlaps the previous
  * call's steps and its output copy the next call's, with no device-side copy.  `in` must stay
  * unchanged and `out` unread until dgpe_sync (which waits for the copies too); later calls
  * that change psi on this context wait for the output copy by themselves.  Pinned host
